@@ -8,6 +8,14 @@ namespace vt {
 cudaError_t launch_clip_f32(const ClipArgs& a, int t, cudaStream_t s);
 cudaError_t launch_clip_f64(const ClipArgs& a, int t, cudaStream_t s);
 cudaError_t launch_clip_big(const ClipArgs& a, cudaStream_t s);
+cudaError_t launch_trace_f32(const TraceArgs& a, cudaStream_t s);
+cudaError_t launch_trace_f64(const TraceArgs& a, cudaStream_t s);
+
+cudaError_t launch_trace(const TraceArgs& a, int precision, cudaStream_t s)
+{
+    if (a.nq <= 0) return cudaSuccess;
+    return precision == VT_FP64 ? launch_trace_f64(a, s) : launch_trace_f32(a, s);
+}
 
 size_t clip_state_pos_offset(int precision)
 {

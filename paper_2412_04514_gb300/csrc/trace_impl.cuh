@@ -1,0 +1,1136 @@
+// trace_impl.cuh -- stage 3 of the list schedule: whole cells by edge tracing.
+//
+// The cell of a generator is the intersection of the half-spaces of its walls
+// and of the bisectors with its nearest generators (votess paper, Summary).
+// Clipping plane by plane builds and discards about four vertices for every
+// one that stays, and each cut is a chain of dependent topology updates. Here
+// the final polyhedron of the whole list is found at once, vertex by vertex:
+// from a vertex (a, b, c) the edge on planes a and b ends at the plane h that
+// the ray along it meets first, which is the vertex (b, a, h). The midpoint to
+// the nearest generator lies on the cell, so two such rays from it reach a
+// first vertex, and every further vertex costs one ray. An edge whose other
+// end was met already is closed by a search among the open ends instead of a
+// ray, so a cell of V vertices takes V + 1 rays of one plane test per plane.
+//
+// Work split: 8 lanes build one cell, four cells of a warp in lockstep (every
+// warp collective names all 32 lanes; a group that is done idles until the
+// others are). Each lane holds every eighth plane in registers; a ray is NR
+// plane tests per lane and a minimum over the 8 lanes. Wider groups repeat the
+// per-ray bookkeeping on more lanes, narrower ones hold more of the planes and
+// of shared memory per warp. Bound by instruction issue (4,400 warp
+// instructions per cell of the first round against 14,900 of the clipper) and
+// by instruction fetch. 1M points on a GB300, list and last pass with
+// neighbours: uniform 17.0 -> 7.3 ms, half in clumps 20.2 -> 11.0 ms in the
+// FP32 form, 126 -> 22.6 and 141 -> 35.4 ms in the FP64 form.
+//
+// Certificate. The rays run in float32 and decide nothing by themselves: the
+// vertices are solved again from their three planes, and the cell is accepted
+// only when every vertex lies inside every other plane by more than the
+// float32 error of that test (a bound that grows with the conditioning of the
+// vertex) and every edge has both its ends. Such vertices are vertices of the
+// exact polyhedron, and a set of them that is closed under its edges is all of
+// them, so an accepted topology is the exact one. A cell that fails (vertices
+// within round-off of a further plane, ill-conditioned or more than 48 of
+// them) is handed to the plane-by-plane clipper with its FP64 rechecks.
+//
+// Security radius. A cell whose 4 R^2 is within the list's reach is final.
+// Otherwise its results are written all the same and a second kernel (a warp
+// per cell) walks the generators beyond the list and within 2R, row by row of
+// the grid: one that cuts no vertex changes nothing, so without a cutting
+// generator the results stand. The other cells are built again from their
+// faces and the nearest cutting generators, in the next round; what a further
+// generator still cuts after the last round goes to the clipper as well.
+#pragma once
+#include "clip_impl.cuh"
+
+namespace vt {
+
+namespace {
+
+constexpr unsigned TFULL = 0xffffffffu;
+constexpr int TT = 8;              // lanes per cell
+constexpr int TG = 32 / TT;        // cells per warp
+constexpr int TRACE_V = 48;        // vertices of a cell (its polyhedron has V / 2 + 2 faces)
+constexpr int TRACE_E = 3 * TRACE_V / 2;  // its edges
+constexpr int TRACE_SLOTS = 16;    // open edge ends of a cell (two per lane)
+constexpr int TRACE_KEEP = 12;     // cutting generators handed to the next round
+constexpr int PAD_PLANE = INT_MIN;
+
+// 8-lane primitives of a warp in lockstep
+struct Sub {
+    int lane, gl, base, gi;
+    __device__ __forceinline__ Sub()
+    {
+        lane = threadIdx.x & 31;
+        gl = lane & (TT - 1);
+        base = lane & ~(TT - 1);
+        gi = lane / TT;
+    }
+    __device__ __forceinline__ unsigned ballot(bool p) const
+    {
+        return (__ballot_sync(TFULL, p) >> base) & ((1u << TT) - 1u);
+    }
+    __device__ __forceinline__ bool any(bool p) const { return ballot(p) != 0; }
+    template <typename V>
+    __device__ __forceinline__ V bcast(V v, int src) const { return __shfl_sync(TFULL, v, src, TT); }
+    __device__ __forceinline__ float max(float v) const
+    {
+#pragma unroll
+        for (int o = TT / 2; o >= 1; o >>= 1) v = fmaxf(v, __shfl_xor_sync(TFULL, v, o));
+        return v;
+    }
+    __device__ __forceinline__ float min(float v) const
+    {
+#pragma unroll
+        for (int o = TT / 2; o >= 1; o >>= 1) v = fminf(v, __shfl_xor_sync(TFULL, v, o));
+        return v;
+    }
+    __device__ __forceinline__ double maxd(double v) const
+    {
+#pragma unroll
+        for (int o = TT / 2; o >= 1; o >>= 1) {
+            const double u = __shfl_xor_sync(TFULL, v, o);
+            v = u > v ? u : v;
+        }
+        return v;
+    }
+    __device__ __forceinline__ int incl_scan(int v) const
+    {
+#pragma unroll
+        for (int d = 1; d < TT; d <<= 1) {
+            const int u = __shfl_up_sync(TFULL, v, d, TT);
+            if (gl >= d) v += u;
+        }
+        return v;
+    }
+};
+
+// reciprocal, square root and its reciprocal to 1e-6 or better, flushing
+// denormals: the tests' margins cover them, no result is formed from them
+__device__ __forceinline__ float rcp_fast(float x)
+{
+    float y;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+__device__ __forceinline__ float rsqrt_fast(float x)
+{
+    float y;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+__device__ __forceinline__ float sqrt_fast(float x)
+{
+    float y;
+    asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+
+// vertex positions and planes in the arithmetic of the results. The FP32
+// form solves and integrates with the float planes; the FP64 form keeps double
+// planes and positions beside the float ones that the tests use.
+template <typename Real, int NP>
+struct TraceReal {};
+template <int NP>
+struct TraceReal<double, NP> {
+    double pn[NP][3];  // n
+    double ps[NP];     // b / |n|^2
+    double v[TRACE_V][3];
+};
+
+template <typename Real, int NP>
+struct alignas(16) TraceSmem : TraceReal<Real, NP> {
+    float4 pl[NP];            // n, b of n.x <= b
+    float4 vp[TRACE_V];       // position; its error bound relative to R
+    int32_t src[NP];          // sorted index (with image code), -1..-6 walls, PAD_PLANE
+    uint8_t vid[TRACE_V][4];  // planes (ccw from outside)
+    // edges: planes a | b << 8, vertices s << 16 | t << 24; (a, b) follow one
+    // another in vid[s], so s -> t runs ccw around b and t -> s around a
+    uint32_t ed[TRACE_E];
+    union {
+        float nl[NP];         // |n| (until the vertices are solved)
+        int32_t f[NP];        // the finish: each plane's area sum, then the faces' neighbour keys
+    } u;
+};
+// stride of a group's block: the four groups of a warp read the same member
+// at once (float4 broadcasts), so their blocks start 32 bytes apart modulo the
+// 128 bytes of the banks
+template <typename Real, int NP>
+constexpr size_t trace_stride()
+{
+    return (sizeof(TraceSmem<Real, NP>) + 95) / 128 * 128 + 32;
+}
+
+// the ray v + t d against this lane's planes (unit normals): (t bits with the
+// plane index in the low six) of the first plane met over the group; a value
+// of 0x7f800000 or more when none is met. A plane counts when the ray closes in
+// on it faster than `least`, which leaves out the planes that hold the ray
+// (their rate is round-off) together with those whose vertex would be too
+// ill-conditioned to accept. The six low bits of t only order hits that agree
+// to 8e-6, whose vertices the certificate would refuse anyway.
+template <int NR>
+__device__ __forceinline__ uint32_t hit_rows(const float* nx, const float* ny, const float* nz, const float* nb, float vx,
+                                             float vy, float vz, float dx, float dy, float dz, float least)
+{
+    uint32_t key = 0xffffffffu;
+#pragma unroll
+    for (int r = 0; r < NR; ++r) {
+        const float s = fmaf(-nx[r], vx, fmaf(-ny[r], vy, fmaf(-nz[r], vz, nb[r])));
+        const float nd = fmaf(nx[r], dx, fmaf(ny[r], dy, nz[r] * dz));
+        const uint32_t k = (__float_as_uint(s * rcp_fast(nd)) & ~63u) | (uint32_t)(r * TT);
+        key = nd > least ? ::min(key, k) : key;
+    }
+    return key;
+}
+// rows: the rows of planes in use over the warp (two unrolled forms: the
+// lists fill all NR, most later rounds three)
+template <int NR>
+__device__ __forceinline__ uint32_t first_hit(const float (&nx)[NR], const float (&ny)[NR], const float (&nz)[NR],
+                                              const float (&nb)[NR], int rows, float vx, float vy, float vz, float dx,
+                                              float dy, float dz, float least, int gl)
+{
+    uint32_t key = rows <= 3 ? hit_rows<3>(nx, ny, nz, nb, vx, vy, vz, dx, dy, dz, least)
+                             : hit_rows<NR>(nx, ny, nz, nb, vx, vy, vz, dx, dy, dz, least);
+    key |= (uint32_t)gl;
+#pragma unroll
+    for (int o = TT / 2; o >= 1; o >>= 1) key = ::min(key, __shfl_xor_sync(TFULL, key, o));
+    return key;
+}
+// planes of the lane's first NR rows closer than thr to v (or behind it)
+template <int NR>
+__device__ __forceinline__ int near_rows(const float* nx, const float* ny, const float* nz, const float* nb, float4 v,
+                                         float thr)
+{
+    int near = 0;
+#pragma unroll
+    for (int r = 0; r < NR; ++r)
+        near += fmaf(-nx[r], v.x, fmaf(-ny[r], v.y, fmaf(-nz[r], v.z, nb[r]))) < thr ? 1 : 0;
+    return near;
+}
+
+// below this |det| of the unit normals (about 1 in 3,000 vertices) the FP32
+// form solves a vertex in FP64
+constexpr float UNIT_F64 = 1e-2f;
+template <bool PER>
+__device__ VT_RARE bool solve_vertex64(int a, int b, int c, const float4* __restrict__ sorted, float4 pi,
+                                       const GridDesc& grid, float& x, float& y, float& z)
+{
+    double dx = 0, dy = 0, dz = 0;
+    const bool ok = vertex64(plane64<PER>(a, sorted, pi, grid), plane64<PER>(b, sorted, pi, grid),
+                             plane64<PER>(c, sorted, pi, grid), dx, dy, dz);
+    x = (float)dx;
+    y = (float)dy;
+    z = (float)dz;
+    return ok;
+}
+
+// the i-th (0-based) plane of a face mask
+__device__ __forceinline__ int nth_face(uint32_t lo, uint32_t hi, int i)
+{
+    const int c = __popc(lo);
+    return i < c ? nth_bit32(lo, i) : 32 + nth_bit32(hi, i - c);
+}
+
+// moments, neighbours and geometry of the group's cell (the quantities of
+// finish_cell); every lane of the warp calls, groups with V = 0 write nothing.
+// (fl, fh): the planes that are faces. A lane per edge: the two triangles of
+// an edge share its cross product. Areas only decide which faces are above
+// the neighbour threshold: they add up in fixed point (integers add in any
+// order alike), and a face below 1e-4 R^2 is added up again in the arithmetic
+// of the form, edge by edge.
+template <typename Real, int NP, bool PER>
+__device__ __forceinline__ void trace_finish(TraceSmem<Real, NP>& sm, const Sub& G, int V, uint32_t fl, uint32_t fh,
+                                             float R2, float4 pi, int64_t out_idx, const TraceArgs& A)
+{
+    constexpr bool F64 = sizeof(Real) == 8;
+    const int gl = G.gl;
+    const bool act = V > 0;
+    const int F = act ? __popc(fl) + __popc(fh) : 0;
+    const int E = 3 * V / 2;
+    if (A.rec) {
+        for (int f = gl; f < NP; f += TT) sm.u.f[f] = 0;
+        __syncwarp();
+    }
+    auto plane = [&](int f, Real& x, Real& y, Real& z, Real& sc) {
+        if constexpr (F64) {
+            x = sm.pn[f][0];
+            y = sm.pn[f][1];
+            z = sm.pn[f][2];
+            sc = sm.ps[f];
+        } else {
+            const float4 p = sm.pl[f];
+            x = p.x;
+            y = p.y;
+            z = p.z;
+            sc = sm.src[f] < 0 ? p.w : 0.5f;  // b / |n|^2
+        }
+    };
+    auto vert = [&](int s, Real& x, Real& y, Real& z) {
+        if constexpr (F64) {
+            x = sm.v[s][0];
+            y = sm.v[s][1];
+            z = sm.v[s][2];
+        } else {
+            const float4 p = sm.vp[s];
+            x = p.x;
+            y = p.y;
+            z = p.z;
+        }
+    };
+    // tetrahedra (0, foot of face, v, next(v around the face))
+    Real vol = 0, mx = 0, my = 0, mz = 0, m2 = 0;
+    const float fix = 1048576.0f * rcp_fast(R2);
+#pragma unroll 1
+    for (int e = gl; e < E; e += TT) {
+        const uint32_t ed = sm.ed[e];
+        Real ax, ay, az, bx, by, bz;
+        vert((ed >> 16) & 0xff, ax, ay, az);
+        vert(ed >> 24, bx, by, bz);
+        const Real cx = ay * bz - az * by, cy = az * bx - ax * bz, cz = ax * by - ay * bx;
+        const Real ab2 = ax * ax + ay * ay + az * az + bx * bx + by * by + bz * bz;
+        const Real tx = ax + bx, ty = ay + by, tz = az + bz;
+#pragma unroll
+        for (int t = 0; t < 2; ++t) {
+            const int f = vt_ck((ed >> (8 * t)) & 0xff, NP, CK_PLANE, A.st);
+            Real px, py, pz, sc;
+            plane(f, px, py, pz, sc);
+            const Real qx = px * sc, qy = py * sc, qz = pz * sc;
+            const Real qc = qx * cx + qy * cy + qz * cz;
+            const Real dv = qc * (Real)(t ? 1.0 / 6.0 : -1.0 / 6.0);
+            const Real sx = qx + tx, sy = qy + ty, sz = qz + tz;
+            const Real q2 = qx * qx + qy * qy + qz * qz;
+            vol += dv;
+            mx += dv * sx;
+            my += dv * sy;
+            mz += dv * sz;
+            m2 += dv * (q2 + ab2 + sx * sx + sy * sy + sz * sz);
+            if (A.rec) {  // twice the triangle's signed area is q.c / |q|
+                const float a2 = (float)qc * rsqrt_fast((float)q2) * fix;
+                atomicAdd(&sm.u.f[f], __float2int_rn(t ? a2 : -a2));
+            }
+        }
+    }
+    // FP64 sums over the 8 lanes by reduce-scatter: 7 additions instead of 15
+    double w;
+    {
+        const double s0[8] = {(double)vol, (double)mx, (double)my, (double)mz, (double)m2, 0.0, 0.0, 0.0};
+        double t4[4], t2[2];
+        const bool hi1 = (gl & 4) != 0, hi2 = (gl & 2) != 0, hi3 = (gl & 1) != 0;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const double send = hi1 ? s0[i] : s0[4 + i];
+            t4[i] = (hi1 ? s0[4 + i] : s0[i]) + __shfl_xor_sync(TFULL, send, 4);
+        }
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+            const double send = hi2 ? t4[i] : t4[2 + i];
+            t2[i] = (hi2 ? t4[2 + i] : t4[i]) + __shfl_xor_sync(TFULL, send, 2);
+        }
+        w = (hi3 ? t2[1] : t2[0]) + __shfl_xor_sync(TFULL, hi3 ? t2[0] : t2[1], 1);
+    }
+    // lane 0 holds V, 1 M_x, 2 M_y, 3 M_z, 4 M2
+    const double vol_t = G.bcast(w, 0);
+    if (act) {
+        if (gl == 0 && A.vol) A.vol[out_idx] = vol_t;
+        if (gl >= 1 && gl <= 3 && A.cen) {
+            const float pc = gl == 1 ? pi.x : (gl == 2 ? pi.y : pi.z);
+            A.cen[3 * out_idx + gl - 1] = (double)pc + 0.25 * w / vol_t;
+        }
+        if (gl == 4 && A.m2) A.m2[out_idx] = 0.05 * w;
+    }
+    if (!A.rec) return;
+    __syncwarp();  // the area sums are complete
+    uint8_t* rec = A.rec + (size_t)out_idx * A.rec_stride;
+    const bool geom = (A.emit & VT_EMIT_GEOM) != 0;
+    int32_t* rfn = reinterpret_cast<int32_t*>(rec + REC_FNBR_OFF);
+    int kept = 0;
+    const int Fmax = __reduce_max_sync(TFULL, F);
+#pragma unroll 1
+    for (int i0 = 0; i0 < Fmax; i0 += TT) {
+        const int i = i0 + gl;
+        int key = INT_MAX;
+        if (i < F) {
+            const int f = nth_face(fl, fh, i);
+            const int src = sm.src[f];
+            int oid = src;  // wall ids stay
+            if (PER) {
+                if (src < 0)
+                    oid = (int)out_idx;
+                else
+                    oid = A.index_space == VT_INDEX_ORIGINAL ? __float_as_int(A.sorted[src & IMG_INDEX_MASK].w)
+                                                             : (src & IMG_INDEX_MASK);
+            } else if (src >= 0 && A.index_space == VT_INDEX_ORIGINAL) {
+                oid = __float_as_int(A.sorted[src].w);
+            }
+            if (geom) rfn[i] = oid;
+            bool nb = true;
+            if (sm.u.f[f] < 210) {  // 2e-4 R^2 of doubled area
+                Real fnx, fny, fnz, sc, area = 0, tau;
+                plane(f, fnx, fny, fnz, sc);
+                const Real qx = fnx * sc, qy = fny * sc, qz = fnz * sc;
+#pragma unroll 1
+                for (int e = 0; e < E; ++e) {
+                    const uint32_t ed = sm.ed[e];
+                    const bool on_a = (ed & 0xff) == (uint32_t)f;
+                    if (!on_a && ((ed >> 8) & 0xff) != (uint32_t)f) continue;
+                    Real ux, uy, uz, wx, wy, wz;
+                    vert(on_a ? ed >> 24 : (ed >> 16) & 0xff, ux, uy, uz);
+                    vert(on_a ? (ed >> 16) & 0xff : ed >> 24, wx, wy, wz);
+                    ux -= qx; uy -= qy; uz -= qz;
+                    wx -= qx; wy -= qy; wz -= qz;
+                    area += (uy * wz - uz * wy) * fnx + (uz * wx - ux * wz) * fny + (ux * wy - uy * wx) * fnz;
+                }
+                area *= (Real)0.5 / sqrt(fnx * fnx + fny * fny + fnz * fnz);
+                if (!F64) {
+                    const float cv = cbrtf((float)vol_t);
+                    tau = (Real)((float)Tol<float>::area_rel * cv * cv);
+                } else {
+                    tau = (Real)(Tol<double>::area_rel * cbrt(vol_t * vol_t));
+                }
+                nb = area > tau;
+            }
+            nb = nb && (src >= 0 || PER);
+            kept += nb;
+            // (periodic ids may repeat; the plane makes the key unique)
+            if (nb) key = PER ? oid * 64 + f : oid;
+        }
+        __syncwarp();  // (the i-th face is plane i or a later one: its area is read before this)
+        if (i < F) sm.u.f[i] = key;
+    }
+    __syncwarp();
+    int32_t* rnbr = reinterpret_cast<int32_t*>(rec + REC_NBR_OFF);
+#pragma unroll 1
+    for (int i = gl; i < F; i += TT) {  // neighbours ascending: each key's rank
+        const int key = sm.u.f[i];
+        if (key == INT_MAX) continue;
+        int rank = 0;
+#pragma unroll 4
+        for (int k = 0; k < F; ++k) rank += sm.u.f[k] < key ? 1 : 0;
+        rnbr[rank] = PER ? key / 64 : key;
+    }
+    const int nn = G.bcast(G.incl_scan(kept), TT - 1);
+    if (geom) {
+        double* rv = reinterpret_cast<double*>(rec + REC_VTX_OFF);
+        float* rv32 = reinterpret_cast<float*>(rec + REC_VTX_OFF);
+        for (int s = gl; s < V; s += TT) {
+            Real x, y, z;
+            vert(s, x, y, z);
+            if (A.rec_f32) {
+                rv32[3 * s] = (float)x;
+                rv32[3 * s + 1] = (float)y;
+                rv32[3 * s + 2] = (float)z;
+            } else {
+                rv[3 * s] = (double)pi.x + (double)x;
+                rv[3 * s + 1] = (double)pi.y + (double)y;
+                rv[3 * s + 2] = (double)pi.z + (double)z;
+            }
+        }
+        // loops of the faces: the vertex after vertex s around the t-th of its
+        // planes at byte 4 s + t, and each plane's lowest vertex and degree,
+        // over the planes (not needed any more)
+        __syncwarp();
+        uint8_t* next = reinterpret_cast<uint8_t*>(sm.pl);
+        int32_t* first = reinterpret_cast<int32_t*>(sm.pl) + TRACE_V;
+        int32_t* degree = first + NP;
+        static_assert(4 * TRACE_V + 8 * NP <= 16 * NP, "the loops fit the planes");
+        for (int f = gl; f < NP; f += TT) {
+            first[f] = TRACE_V;
+            degree[f] = 0;
+        }
+        __syncwarp();
+#pragma unroll 1
+        for (int e = gl; e < E; e += TT) {
+            const uint32_t ed = sm.ed[e];
+            const int s = (ed >> 16) & 0xff, t = ed >> 24;
+#pragma unroll
+            for (int k = 0; k < 2; ++k) {  // k = 0: plane a, t -> s; 1: plane b, s -> t
+                const int f = (ed >> (8 * k)) & 0xff, u = k ? s : t, v = k ? t : s;
+                const uint32_t ids = *reinterpret_cast<const uint32_t*>(sm.vid[u]);
+                const int at = (ids & 0xff) == (uint32_t)f ? 0 : (((ids >> 8) & 0xff) == (uint32_t)f ? 1 : 2);
+                next[4 * u + at] = (uint8_t)v;
+                atomicMin(&first[f], u);
+                atomicAdd(&degree[f], 1);
+            }
+        }
+        __syncwarp();
+        uint8_t* rdeg = rec + REC_FDEG_OFF;
+        uint8_t* rfv = rec + REC_FVTX_OFF;
+        int base = 0;
+#pragma unroll 1
+        for (int i0 = 0; i0 < Fmax; i0 += TT) {
+            const int i = i0 + gl;
+            const int f = i < F ? nth_face(fl, fh, i) : 0;
+            const int deg = i < F ? degree[f] : 0;
+            const int inc = G.incl_scan(deg);
+            const int pos = base + inc - deg;
+            base += G.bcast(inc, TT - 1);
+            if (i < F) {
+                rdeg[i] = (uint8_t)deg;
+                int cur = first[f];
+#pragma unroll 1
+                for (int k = 0; k < deg; ++k) {
+                    const uint32_t ids = *reinterpret_cast<const uint32_t*>(sm.vid[cur]);
+                    const int at = (ids & 0xff) == (uint32_t)f ? 0 : (((ids >> 8) & 0xff) == (uint32_t)f ? 1 : 2);
+                    rfv[vt_ck(pos + k, 3 * REC_VERTS, CK_RECORD, A.st)] = (uint8_t)cur;
+                    cur = next[4 * cur + at];
+                }
+            }
+        }
+    }
+    if (act && gl == 0) {
+        RecHeader* hd = reinterpret_cast<RecHeader*>(rec);
+        hd->nnbr = nn;
+        hd->nface = geom ? F : 0;
+        hd->nvtx = geom ? V : 0;
+        hd->nfv = geom ? 3 * V : 0;
+        hd->p[0] = pi.x;
+        hd->p[1] = pi.y;
+        hd->p[2] = pi.z;
+    }
+    __syncwarp();
+}
+
+// appends q of the lanes with `on` to a device list, one counter update per warp
+__device__ __forceinline__ void append(int32_t* list, int32_t* ctr, bool on, int q, int lane)
+{
+    const unsigned m = __ballot_sync(TFULL, on);
+    if (!m) return;
+    int at = 0;
+    if (lane == __ffs(m) - 1) at = atomicAdd(ctr, __popc(m));
+    at = __shfl_sync(TFULL, at, __ffs(m) - 1);
+    if (on) list[at + __popc(m & ((1u << lane) - 1u))] = q;
+}
+
+// an open cell between the two kernels of a round, in its state slot
+struct alignas(16) OpenCell {
+    int32_t np, nf;
+    float reach;              // generators with a float key below this are behind it
+    float all2;               // (2R)^2
+    float band;               // error bound of the vertex positions
+    int32_t pad[3];
+    int32_t src[40];          // planes of the next round: its faces, then what cuts it
+    float4 far[TRACE_V];      // vertices a generator at `reach` or beyond can cut
+};
+static_assert(TRACE_V / 2 + 2 + TRACE_KEEP <= 40, "the planes of the next round");
+static_assert(sizeof(OpenCell) <= StateLayout<float, 64, 64>::BYTES, "an open cell fits the state slot");
+
+constexpr int CUT_BLOCK = 256;
+constexpr int CUT_LIST = TRACE_KEEP + 32;
+
+// the nearest `cap` of the warp's ns candidates, in order of (key, id)
+__device__ __forceinline__ int keep_nearest(float* key, int32_t* id, int ns, int cap, int lane)
+{
+    __syncwarp();
+    const float k0 = lane < ns ? key[lane] : FLT_MAX, k1 = lane + 32 < ns ? key[lane + 32] : FLT_MAX;
+    const int j0 = lane < ns ? id[lane] : INT_MAX, j1 = lane + 32 < ns ? id[lane + 32] : INT_MAX;
+    int r0 = 0, r1 = 0;
+#pragma unroll 1
+    for (int i = 0; i < ns; ++i) {
+        const float k = key[i];
+        const int j = id[i];
+        r0 += k < k0 || (k == k0 && j < j0);
+        r1 += k < k1 || (k == k1 && j < j1);
+    }
+    __syncwarp();
+    if (lane < ns && r0 < cap) {
+        key[r0] = k0;
+        id[r0] = j0;
+    }
+    if (lane + 32 < ns && r1 < cap) {
+        key[r1] = k1;
+        id[r1] = j1;
+    }
+    __syncwarp();
+    return ns < cap ? ns : cap;
+}
+
+// The walk of the open cells, a warp per cell: the generators with keys of at
+// least the cell's reach and within 2R that cut one of its vertices, the
+// nearest TRACE_KEEP of them. It takes the rows of the grid that meet the box
+// of the far vertices' balls and the ball of the current limit, less the grid
+// cells the list covered; the limit grows from the reach by half its radius at
+// a time, and the walk ends at the first limit that met a cutting generator
+// (the cell it leaves is smaller). A lane per row finds the row's runs, then
+// the lanes share the rows' generators.
+template <bool PER>
+__global__ void __launch_bounds__(CUT_BLOCK) k_cutters(const __grid_constant__ TraceArgs A)
+{
+    __shared__ float4 s_far[CUT_BLOCK / 32][TRACE_V];
+    __shared__ float s_key[CUT_BLOCK / 32][CUT_LIST];
+    __shared__ int32_t s_id[CUT_BLOCK / 32][CUT_LIST];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    float4* far = s_far[warp];
+    float* key = s_key[warp];
+    int32_t* id = s_id[warp];
+    const int have = *A.nq_dev;
+    const int nq = have < (int)A.nq ? have : (int)A.nq;
+    unsigned cells = 0, cands = 0;
+    for (;;) {
+        int c = 0;
+        if (lane == 0) c = atomicAdd(A.queue, 1);
+        c = __shfl_sync(TFULL, c, 0);
+        if (c >= nq) break;
+        const int q = A.queries[c];
+        const GridDesc& grid = grid_of(A.g, A.sets, A.set_of, q);
+        const float4 pi = A.sorted[q];
+        OpenCell* h = reinterpret_cast<OpenCell*>(A.state + (size_t)q * A.state_stride);
+        const int np = h->np, nf = h->nf;
+        const float all2 = h->all2, band = h->band;
+        float reach = h->reach;
+        // the box of the far vertices' balls, around the generator
+        float l0 = 0, l1 = 0, l2 = 0, h0 = 0, h1 = 0, h2 = 0;
+        for (int s = lane; s < nf; s += 32) {
+            const float4 v = h->far[s];
+            const float r = sqrt_fast(v.w) * (1.0f + 1e-4f);
+            l0 = fminf(l0, v.x - r); h0 = fmaxf(h0, v.x + r);
+            l1 = fminf(l1, v.y - r); h1 = fmaxf(h1, v.y + r);
+            l2 = fminf(l2, v.z - r); h2 = fmaxf(h2, v.z + r);
+            far[s] = v;
+        }
+#pragma unroll
+        for (int o = 16; o >= 1; o >>= 1) {
+            l0 = fminf(l0, __shfl_xor_sync(TFULL, l0, o)); h0 = fmaxf(h0, __shfl_xor_sync(TFULL, h0, o));
+            l1 = fminf(l1, __shfl_xor_sync(TFULL, l1, o)); h1 = fmaxf(h1, __shfl_xor_sync(TFULL, h1, o));
+            l2 = fminf(l2, __shfl_xor_sync(TFULL, l2, o)); h2 = fmaxf(h2, __shfl_xor_sync(TFULL, h2, o));
+        }
+        __syncwarp();
+        const int Gr = grid.G;
+        const int32_t* coff = A.cell_off + grid.cell_base;
+        const float m = (float)grid.margin;
+        const float cx = (float)grid.cw[0], cy = (float)grid.cw[1];
+        // periodic: unwrapped grid coordinates, and each row once per z image
+        const float lim_lo = PER ? -2.0f * (float)Gr : 0.0f,
+                    lim_hi = PER ? 3.0f * (float)Gr - 1.0f : (float)Gr - 1.0f;
+        auto clamp = [&](float t) { return (int)floorf(fminf(fmaxf(t, lim_lo), lim_hi)); };
+        int ns = 0;
+        bool more = false, end = nf == 0;
+        // (40 steps of 2.25 cover every ratio of float32 keys that differ; the
+        // last one takes the whole ball)
+#pragma unroll 1
+        for (int it = 0; !end && ns == 0; ++it) {
+            const float lim2 = it < 40 ? fminf(all2, 2.25f * reach) : all2;
+            const float r_out2 = lim2 * (1.0f + 1e-4f), r_in2 = reach * (1.0f - 1e-4f);
+            const float rr = sqrt_fast(r_out2) * (1.0f + 1e-5f);
+            const float z_lo = pi.z + fmaxf(l2, -rr) - m, z_hi = pi.z + fminf(h2, rr) + m;
+            const int x0 = clamp((pi.x + fmaxf(l0, -rr) - m - grid.lo[0]) * grid.scale[0] - 1e-3f);
+            const int x1 = clamp((pi.x + fminf(h0, rr) + m - grid.lo[0]) * grid.scale[0] + 1e-3f);
+            const int y0 = clamp((pi.y + fmaxf(l1, -rr) - m - grid.lo[1]) * grid.scale[1] - 1e-3f);
+            const int y1 = clamp((pi.y + fminf(h1, rr) + m - grid.lo[1]) * grid.scale[1] + 1e-3f);
+            int t0 = 0, nt = 1;
+            if (PER) {
+                t0 = floordiv(clamp((z_lo - grid.lo[2]) * grid.scale[2] - 1e-3f), Gr);
+                nt = floordiv(clamp((z_hi - grid.lo[2]) * grid.scale[2] + 1e-3f), Gr) - t0 + 1;
+            }
+            const int wy = y1 - y0 + 1, nrow = (x1 - x0 + 1) * wy * nt;
+#pragma unroll 1
+            for (int e0 = 0; e0 < nrow; e0 += 32) {
+                const int e = e0 + lane;
+                int sa = 0, la = 0, sb = 0, lb = 0, code = IMG_NONE;
+                if (e < nrow) {
+                    const int e2 = PER ? e / nt : e;
+                    const int tz = PER ? t0 + (e - e2 * nt) : 0;
+                    const int ex = e2 / wy, x = x0 + ex, y = y0 + (e2 - ex * wy);
+                    const int tx = PER ? floordiv(x, Gr) : 0, ty = PER ? floordiv(y, Gr) : 0;
+                    const float gx0 = grid.lo[0] + (float)x * cx - m, gx1 = grid.lo[0] + (float)(x + 1) * cx + m;
+                    const float gy0 = grid.lo[1] + (float)y * cy - m, gy1 = grid.lo[1] + (float)(y + 1) * cy + m;
+                    const float dxn = fmaxf(fmaxf(gx0 - pi.x, pi.x - gx1), 0.0f),
+                                dyn = fmaxf(fmaxf(gy0 - pi.y, pi.y - gy1), 0.0f);
+                    const float dxf = fmaxf(pi.x - gx0, gx1 - pi.x), dyf = fmaxf(pi.y - gy0, gy1 - pi.y);
+                    const float dn2 = dxn * dxn + dyn * dyn, df2 = dxf * dxf + dyf * dyf;
+                    if (dn2 <= r_out2) {
+                        const float zr = sqrtf(r_out2 - dn2) + m;
+                        int za = clamp((fmaxf(pi.z - zr, z_lo) - grid.lo[2]) * grid.scale[2] - 1e-3f);
+                        int zb = clamp((fminf(pi.z + zr, z_hi) - grid.lo[2]) * grid.scale[2] + 1e-3f);
+                        if (PER) {
+                            za = za > tz * Gr ? za : tz * Gr;
+                            zb = zb < tz * Gr + Gr - 1 ? zb : tz * Gr + Gr - 1;
+                        }
+                        // grid cells wholly inside the ball that is behind: [i0, i1]
+                        int i0 = zb + 1, i1 = zb;
+                        if (r_in2 > df2) {
+                            const float zi = sqrtf(r_in2 - df2) - m;
+                            i0 = (int)ceilf(fminf(fmaxf((pi.z - zi - grid.lo[2]) * grid.scale[2] + 1e-3f, lim_lo - 1.0f),
+                                                  lim_hi + 2.0f));
+                            i1 = (int)floorf(fminf(fmaxf((pi.z + zi - grid.lo[2]) * grid.scale[2] - 1e-3f, lim_lo - 1.0f),
+                                                   lim_hi + 2.0f)) - 1;
+                            if (i0 > i1 || i1 < za || i0 > zb) {
+                                i0 = zb + 1;
+                                i1 = zb;
+                            }
+                        }
+                        const int base = ((x - tx * Gr) * Gr + (y - ty * Gr)) * Gr - tz * Gr;
+                        const int ea = i0 - 1, fb = i1 + 1 > za ? i1 + 1 : za;
+                        if (za <= ea) {
+                            sa = coff[base + za];
+                            la = coff[base + ea + 1] - sa;
+                        }
+                        if (i0 <= zb && fb <= zb) {
+                            sb = coff[base + fb];
+                            lb = coff[base + zb + 1] - sb;
+                        }
+                        if (PER) code = img_code(tx, ty, tz);
+                    }
+                }
+                int incl = la + lb;
+#pragma unroll
+                for (int d = 1; d < 32; d <<= 1) {
+                    const int u = __shfl_up_sync(TFULL, incl, d);
+                    if (lane >= d) incl += u;
+                }
+                const int total = __shfl_sync(TFULL, incl, 31);
+                const int start = incl - la - lb;
+                cands += (unsigned)total;
+#pragma unroll 1
+                for (int c0 = 0; c0 < total; c0 += 32) {
+                    const int i = c0 + lane;
+                    int seg = 0;  // rows ending at or before i
+#pragma unroll
+                    for (int step = 16; step >= 1; step >>= 1)
+                        if (__shfl_sync(TFULL, incl, (seg + step - 1) & 31) <= i) seg += step;
+                    seg &= 31;
+                    const int off = i - __shfl_sync(TFULL, start, seg), na = __shfl_sync(TFULL, la, seg);
+                    const int ja = __shfl_sync(TFULL, sa, seg), jb = __shfl_sync(TFULL, sb, seg);
+                    const int cd = PER ? __shfl_sync(TFULL, code, seg) : IMG_NONE;
+                    const int j = off < na ? ja + off : jb + (off - na);
+                    const int jj = PER ? img_pack(j, cd) : j;
+                    float3 o = make_float3(0.0f, 0.0f, 0.0f);
+                    const bool in = i < total && j != q;
+                    if (in) o = img_off_t<PER>(pi, A.sorted[j], cd, grid);
+                    const float d2 = fmaf(o.z, o.z, fmaf(o.y, o.y, o.x * o.x));
+                    bool cuts = in && d2 >= reach && d2 <= r_out2;
+                    if (!__any_sync(TFULL, cuts)) continue;
+                    float top = -FLT_MAX;
+#pragma unroll 2
+                    for (int k = 0; k < nf; ++k) {
+                        const float4 v = far[k];
+                        top = fmaxf(top, fmaf(o.x, v.x, fmaf(o.y, v.y, o.z * v.z)));
+                    }
+                    cuts = cuts && 0.5f * d2 - top <= band * sqrt_fast(d2);
+                    if (cuts)  // (the cell's own faces touch their vertices)
+                        for (int p = 0; p < np; ++p)
+                            if (h->src[p] == jj) cuts = false;
+                    const unsigned cm = __ballot_sync(TFULL, cuts);
+                    if (cuts) {
+                        const int at = ns + __popc(cm & ((1u << lane) - 1u));
+                        key[at] = d2;
+                        id[at] = jj;
+                    }
+                    ns += __popc(cm);
+                    if (ns > TRACE_KEEP) {
+                        more = true;
+                        ns = keep_nearest(key, id, ns, TRACE_KEEP, lane);
+                    }
+                }
+            }
+            end = lim2 >= all2;
+            if (!more) reach = lim2;  // (all of it is behind)
+        }
+        ++cells;
+        if (ns > 0) {
+            ns = keep_nearest(key, id, ns, TRACE_KEEP, lane);
+            if (more) reach = key[ns - 1];  // what the next round need not look at again
+            if (lane < ns) h->src[np + lane] = id[lane];
+            if (lane == 0) {
+                h->np = np + ns;
+                h->reach = reach;
+                A.next_list[atomicAdd(A.next_ctr, 1)] = q;
+            }
+        }
+        __syncwarp();
+    }
+    if (lane == 0 && cells) {
+        // (one walk per cell: later rounds continue it)
+        if (A.round == 0) atomicAdd(&A.st->walk_cells, (unsigned long long)cells);
+        atomicAdd(&A.st->walk_cands, (unsigned long long)cands);
+    }
+}
+
+// Blocks of 128 threads build 16 cells at a time, their warps aligned by a
+// barrier before the rays and one after them: the rays, the certificate and the
+// finish are 70 KB of code, and warps that drift apart wait for instructions
+// (uniform 1M points, neighbours: 7.58 ms of the list pass against 9.07 without
+// barriers; blocks of 256 threads 7.69 and of 64 threads 7.18 against 7.29 ms,
+// the latter 0.4 ms slower with geometry). Five blocks per SM (96 registers, no
+// spills) against six: 7.29 and 7.41 ms.
+constexpr int TRACE_BLOCK = 128;
+constexpr int TRACE_MINB = 5;
+
+template <typename Real, int NR, bool PER>
+__global__ void __launch_bounds__(TRACE_BLOCK, (sizeof(Real) == 4 ? TRACE_MINB : 4)) k_trace(const __grid_constant__ TraceArgs A)
+{
+    constexpr int NP = NR * TT;
+    constexpr bool F64 = sizeof(Real) == 8;
+    // smallest |det| of a vertex's three unit normals, above the rounding of the
+    // rates of approach (worse vertices are left to the clipper)
+    constexpr float UNIT_MIN = F64 ? 2e-5f : 2e-4f;
+    using S = TraceSmem<Real, NP>;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const Sub G;
+    const int gl = G.gl;
+    S& sm = *reinterpret_cast<S*>(smem_raw + (threadIdx.x / TT) * trace_stride<Real, NP>());
+    int nq = (int)A.nq;
+    if (A.nq_dev) {
+        const int have = *A.nq_dev;
+        nq = have < nq ? have : nq;
+    }
+    unsigned n_open = 0, n_second = 0;  // added once per group
+    __shared__ int s_first;
+    for (;;) {
+        if (threadIdx.x == 0) s_first = atomicAdd(A.queue, TRACE_BLOCK / TT);
+        __syncthreads();
+        const int c_block = s_first;
+        if (c_block >= nq) break;
+        const int c4 = c_block + (threadIdx.x / 32) * TG;
+        const bool act = c4 + G.gi < nq;  // a group past the end repeats the last cell and writes nothing
+        const int c = act ? c4 + G.gi : nq - 1;
+        const int q = A.queries ? A.queries[c] : c;
+        const GridDesc& grid = grid_of(A.g, A.sets, A.set_of, q);
+        const float4 pi = A.sorted[q];
+        uint8_t* state = A.state + (size_t)q * A.state_stride;
+        // ---- planes: unit normals in registers, the planes themselves in shared memory
+        float nx[NR], ny[NR], nz[NR], nb[NR];
+        int P;
+        float reach;  // every generator with a float key below this was in the lists so far
+        bool end = false;
+        const int32_t* srcs;
+        const Real* keys = nullptr;
+        if (A.round == 0) {
+            const int64_t li = (int64_t)c * A.kstride;
+            srcs = A.nbr + li - 6;
+            keys = reinterpret_cast<const Real*>(A.d2) + li;
+            P = 6 + A.kc;
+            reach = (float)keys[A.kc - 1] * (F64 ? 1.0f - 1e-6f : 1.0f);  // (FP64 keys round)
+        } else {
+            const OpenCell* h = reinterpret_cast<const OpenCell*>(state);
+            srcs = h->src;
+            P = h->np;
+            reach = h->reach;
+        }
+        const int rows = __reduce_max_sync(TFULL, (P + TT - 1) / TT);
+#pragma unroll
+        for (int r = 0; r < NR; ++r) {
+            const int p = r * TT + gl;
+            int src = PAD_PLANE;
+            if (p < P) {
+                if (A.round == 0 && p < 6) {
+                    src = -(p + 1);
+                } else {
+                    src = srcs[p];
+                    if (A.round == 0 && src < 0) {  // the list holds every other generator
+                        src = PAD_PLANE;
+                        end = true;
+                    }
+                }
+            }
+            float x = 0.0f, y = 0.0f, z = 0.0f, b = 1.0f, len = 0.0f, inv = 0.0f;
+            if (src >= 0) {
+                const float3 o = img_off_t<PER>(pi, A.sorted[img_index_t<PER>(src)], img_code_t<PER>(src), grid);
+                x = o.x;
+                y = o.y;
+                z = o.z;
+                const float nn = x * x + y * y + z * z;
+                b = 0.5f * nn;
+                len = sqrt_fast(nn);
+                inv = rsqrt_fast(nn);
+            } else if (src != PAD_PLANE) {
+                const int w = -src - 1, axis = w >> 1, upper = w & 1;
+                const float one = upper ? 1.0f : -1.0f;
+                x = axis == 0 ? one : 0.0f;
+                y = axis == 1 ? one : 0.0f;
+                z = axis == 2 ? one : 0.0f;
+                const float pc = axis == 0 ? pi.x : (axis == 1 ? pi.y : pi.z);
+                b = PER ? (float)(0.5 * ((double)grid.hi[axis] - (double)grid.lo[axis]))
+                        : (upper ? grid.hi[axis] - pc : pc - grid.lo[axis]);
+                len = inv = 1.0f;
+            }
+            nx[r] = x * inv;
+            ny[r] = y * inv;
+            nz[r] = z * inv;
+            nb[r] = src != PAD_PLANE ? b * inv : FLT_MAX;
+            sm.pl[p] = make_float4(x, y, z, b);
+            sm.u.nl[p] = len;
+            sm.src[p] = src;
+            if constexpr (F64) {
+                if (src != PAD_PLANE) {
+                    const P64 d = plane64<PER>(src, A.sorted, pi, grid);
+                    sm.pn[p][0] = d.x;
+                    sm.pn[p][1] = d.y;
+                    sm.pn[p][2] = d.z;
+                    sm.ps[p] = src >= 0 ? 0.5 : d.b;  // b / |n|^2
+                }
+            }
+        }
+        __syncwarp();
+        const bool all = G.any(end);
+        const unsigned gen0 = G.ballot(sm.src[gl] >= 0);
+        bool ok = gen0 != 0;  // a nearest generator to start from
+        const int f0 = gen0 ? __ffs(gen0) - 1 : 0;
+        // ---- first vertex --------------------------------------------------
+        int V = 0;
+        int E = 0;
+        // open edge ends (an edge of ed without its second vertex; -1: free)
+        int r0 = -1, r1 = -1;
+        unsigned live = 0;
+        {
+            const float4 n0 = sm.pl[f0];
+            float vx = 0.5f * n0.x, vy = 0.5f * n0.y, vz = 0.5f * n0.z;
+            // a direction in plane f0: n0 x the axis it is least along
+            const float ax = fabsf(n0.x), ay = fabsf(n0.y), az = fabsf(n0.z);
+            float dx, dy, dz;
+            if (ax <= ay && ax <= az) { dx = 0.0f; dy = n0.z; dz = -n0.y; }
+            else if (ay <= az) { dx = -n0.z; dy = 0.0f; dz = n0.x; }
+            else { dx = n0.y; dy = -n0.x; dz = 0.0f; }
+            int f1 = f0, h = f0;
+#pragma unroll 1
+            for (int e = 0; e < 2; ++e) {
+                // (the second ray runs along f0 and f1: n0 x n1 ends at (f0, f1, h))
+                const uint32_t key = first_hit<NR>(nx, ny, nz, nb, rows, vx, vy, vz, dx, dy, dz,
+                                                   e == 0 ? 1e-3f * sm.u.nl[f0] : UNIT_MIN * sm.u.nl[f0] * sm.u.nl[f1], gl);
+                ok = ok && key < 0x7f800000u;
+                h = ok ? (int)(key & 63u) : f0;
+                const float4 nh = sm.pl[h];
+                const float t = (nh.w - (nh.x * vx + nh.y * vy + nh.z * vz)) * rcp_fast(nh.x * dx + nh.y * dy + nh.z * dz);
+                vx = fmaf(t, dx, vx);
+                vy = fmaf(t, dy, vy);
+                vz = fmaf(t, dz, vz);
+                if (e == 0) {
+                    f1 = h;
+                    dx = n0.y * nh.z - n0.z * nh.y;
+                    dy = n0.z * nh.x - n0.x * nh.z;
+                    dz = n0.x * nh.y - n0.y * nh.x;
+                }
+            }
+            if (gl == 0) {
+                sm.vp[0] = make_float4(vx, vy, vz, 0.0f);
+                *reinterpret_cast<uint32_t*>(sm.vid[0]) = (uint32_t)f0 | ((uint32_t)f1 << 8) | ((uint32_t)h << 16);
+            }
+            V = 1;
+            if (gl == 0) r0 = f0 | (f1 << 8);
+            if (gl == 1) r0 = f1 | (h << 8);
+            if (gl == 2) r0 = h | (f0 << 8);
+            live = 7u;
+        }
+        __syncwarp();
+        // ---- one ray per further vertex ------------------------------------
+        bool run = ok;
+#pragma unroll 1
+        while (__any_sync(TFULL, run)) {
+            // the lowest slot: new ends take the lowest free ones, so the newest go
+            // first (oldest first leaves more ends open: 1.7% of the cells of
+            // uniform points ran out of the slots, against 0.4%)
+            const int slot = __ffs(live) - 1;
+            const int got = G.bcast(slot < TT ? r0 : r1, slot & (TT - 1));
+            r0 = gl == slot ? -1 : r0;
+            r1 = gl + TT == slot ? -1 : r1;
+            const int ent = run ? got : 0;
+            const int a = ent & 0xff, b = (ent >> 8) & 0xff, w = ent >> 16;
+            const float4 v = sm.vp[w], na = sm.pl[a], nbp = sm.pl[b];
+            // the edge on a and b leaves (a, b, c) along n_b x n_a
+            const float dx = nbp.y * na.z - nbp.z * na.y, dy = nbp.z * na.x - nbp.x * na.z,
+                        dz = nbp.x * na.y - nbp.y * na.x;
+            const uint32_t key = first_hit<NR>(nx, ny, nz, nb, rows, v.x, v.y, v.z, dx, dy, dz,
+                                               UNIT_MIN * sm.u.nl[a] * sm.u.nl[b], gl);
+            if (key >= 0x7f800000u || V >= TRACE_V || E > TRACE_E - 3) {
+                ok = ok && !run;
+                run = false;
+            }
+            const int h = run ? (int)(key & 63u) : 0;
+            const float4 nh = sm.pl[h];
+            const float t = fmaf(-nh.x, v.x, fmaf(-nh.y, v.y, fmaf(-nh.z, v.z, nh.w))) *
+                            rcp_fast(fmaf(nh.x, dx, fmaf(nh.y, dy, nh.z * dz)));
+            // its other two edges, (a, h) and (h, b): close them against an open
+            // end of the same edge, (h, a) or (b, h), or leave them open
+            const int k1 = run ? h | (a << 8) : 0xfffe, k2 = run ? b | (h << 8) : 0xfffe;
+            const int e0 = r0 & 0xffff, e1 = r1 & 0xffff;
+            const bool p1 = e0 == k1, p2 = e0 == k2, q1 = e1 == k1, q2 = e1 == k2;
+            const bool c1 = G.any(p1 || q1), c2 = G.any(p2 || q2);
+            if (p1 || p2) {
+                sm.ed[E + (p1 ? 1 : 1 + c1)] = (uint32_t)r0 | ((uint32_t)V << 24);
+                r0 = -1;
+            }
+            if (q1 || q2) {
+                sm.ed[E + (q1 ? 1 : 1 + c1)] = (uint32_t)r1 | ((uint32_t)V << 24);
+                r1 = -1;
+            }
+            live = G.ballot(r0 >= 0) | (G.ballot(r1 >= 0) << TT);
+            if (run) {
+                if (gl == 0) {
+                    sm.vp[V] = make_float4(fmaf(t, dx, v.x), fmaf(t, dy, v.y), fmaf(t, dz, v.z), 0.0f);
+                    *reinterpret_cast<uint32_t*>(sm.vid[V]) = (uint32_t)b | ((uint32_t)a << 8) | ((uint32_t)h << 16);
+                    sm.ed[E] = (uint32_t)ent | ((uint32_t)V << 24);
+                }
+                // the lowest free slots take what stays open
+                const unsigned free1 = ~live;
+                const unsigned free2 = c1 ? free1 : free1 & (free1 - 1u);
+                const int s1 = c1 ? 31 : __ffs(free1) - 1, s2 = c2 ? 31 : __ffs(free2) - 1;
+                r0 = gl == s1 ? a | (h << 8) | (V << 16) : (gl == s2 ? h | (b << 8) | (V << 16) : r0);
+                r1 = gl + TT == s1 ? a | (h << 8) | (V << 16) : (gl + TT == s2 ? h | (b << 8) | (V << 16) : r1);
+                live |= (1u << s1) | (1u << s2);
+                if (live & 0x7fff0000u) ok = run = false;  // more open ends than slots
+                live &= 0xffffu;
+                E += 1 + c1 + c2;
+                ++V;
+                run = run && live != 0;
+            }
+            __syncwarp();
+        }
+        __syncthreads();
+        // ---- vertices from their planes -------------------------------------
+        double R2d = 0.0;
+        float R2 = 0.0f, emax = 0.0f;
+        uint32_t fl = 0, fh = 0;  // the planes that are faces
+#pragma unroll 1
+        for (int s = gl; s < V; s += TT) {
+            const uint32_t ids = *reinterpret_cast<const uint32_t*>(sm.vid[s]);
+            const int a = ids & 0xff, b = (ids >> 8) & 0xff, cc = (ids >> 16) & 0xff;
+            fl |= (a < 32 ? 1u << a : 0u) | (b < 32 ? 1u << b : 0u) | (cc < 32 ? 1u << cc : 0u);
+            fh |= (a < 32 ? 0u : 1u << (a - 32)) | (b < 32 ? 0u : 1u << (b - 32)) | (cc < 32 ? 0u : 1u << (cc - 32));
+            const float4 p = sm.pl[a], o = sm.pl[b], h = sm.pl[cc];
+            const float bcx = o.y * h.z - o.z * h.y, bcy = o.z * h.x - o.x * h.z, bcz = o.x * h.y - o.y * h.x;
+            const float det = p.x * bcx + p.y * bcy + p.z * bcz;
+            // |det| of the unit normals: the vertex moves by (rounding) / this
+            const float unit = fabsf(det) * rcp_fast(sm.u.nl[a] * sm.u.nl[b] * sm.u.nl[cc]);
+            if (!(unit > UNIT_MIN)) ok = false;
+            float x, y, z, err;
+            if constexpr (F64) {
+                const double ax = sm.pn[a][0], ay = sm.pn[a][1], az = sm.pn[a][2];
+                const double bx = sm.pn[b][0], by = sm.pn[b][1], bz = sm.pn[b][2];
+                const double cx = sm.pn[cc][0], cy = sm.pn[cc][1], cz = sm.pn[cc][2];
+                const double ab = sm.ps[a] * (sm.src[a] < 0 ? 1.0 : (ax * ax + ay * ay) + az * az);
+                const double bb = sm.ps[b] * (sm.src[b] < 0 ? 1.0 : (bx * bx + by * by) + bz * bz);
+                const double cb = sm.ps[cc] * (sm.src[cc] < 0 ? 1.0 : (cx * cx + cy * cy) + cz * cz);
+                double dx = 0, dy = 0, dz = 0;
+                if (!solve3<double>(ax, ay, az, ab, bx, by, bz, bb, cx, cy, cz, cb, dx, dy, dz)) ok = false;
+                sm.v[s][0] = dx;
+                sm.v[s][1] = dy;
+                sm.v[s][2] = dz;
+                const double d = (dx * dx + dy * dy) + dz * dz;
+                R2d = d > R2d ? d : R2d;
+                x = (float)dx;
+                y = (float)dy;
+                z = (float)dz;
+                err = 1e-6f;  // float rounding of the position, of the plane and of the test
+            } else {
+                const float cax = h.y * p.z - h.z * p.y, cay = h.z * p.x - h.x * p.z, caz = h.x * p.y - h.y * p.x;
+                const float abx = p.y * o.z - p.z * o.y, aby = p.z * o.x - p.x * o.z, abz = p.x * o.y - p.y * o.x;
+                const float inv = rcp(det);
+                x = (p.w * bcx + o.w * cax + h.w * abx) * inv;
+                y = (p.w * bcy + o.w * cay + h.w * aby) * inv;
+                z = (p.w * bcz + o.w * caz + h.w * abz) * inv;
+                err = 1e-6f + 1.5e-6f * rcp_fast(unit);
+                if (unit < UNIT_F64) {  // ill-conditioned: float32 would lose digits
+                    if (!solve_vertex64<PER>(sm.src[a], sm.src[b], sm.src[cc], A.sorted, pi, grid, x, y, z)) ok = false;
+                    err = 1e-6f;
+                }
+            }
+            const float d = x * x + y * y + z * z;
+            if (!isfinite(d)) ok = false;
+            R2 = fmaxf(R2, d);
+            emax = fmaxf(emax, err);
+            sm.vp[s] = make_float4(x, y, z, err);
+        }
+        R2 = G.max(R2);
+        emax = G.max(emax);
+        if (F64) R2d = G.maxd(R2d);
+#pragma unroll
+        for (int o = TT / 2; o >= 1; o >>= 1) {
+            fl |= __shfl_xor_sync(TFULL, fl, o);
+            fh |= __shfl_xor_sync(TFULL, fh, o);
+        }
+        __syncwarp();
+        // ---- the certificate: every vertex clearly inside all planes but its three
+        const float R = sqrtf(R2);
+        {
+            int near = 0;
+            const int vmax = __reduce_max_sync(TFULL, ok ? V : 0);
+#pragma unroll 2
+            for (int s = 0; s < vmax; ++s) {
+                const float4 v = sm.vp[s];
+                const float thr = s < V ? v.w * R : -INFINITY;  // (other slots hold anything)
+                near += rows <= 3 ? near_rows<3>(nx, ny, nz, nb, v, thr) : near_rows<NR>(nx, ny, nz, nb, v, thr);
+            }
+            near = G.bcast(G.incl_scan(near), TT - 1);
+            ok = !G.any(!ok) && near == 3 * V && 2 * E == 3 * V;
+        }
+        // ---- security radius, and the generators beyond the list -------------
+        bool valid = all;
+        if (A.round == 0 && !all)
+            valid = F64 ? 4.0 * R2d <= (double)keys[A.kc - 1] : 4.0f * R2 <= reach * (1.0f - 1e-5f);
+        const bool open = ok && !valid;
+        if (A.round == 0 && act && ok && gl == 0) {
+            n_open += open;
+            if (A.k_first > 0 && srcs[6 + A.k_first] >= 0)
+                n_second += F64 ? 4.0 * R2d > (double)keys[A.k_first] : 4.0f * R2 > (float)keys[A.k_first];
+        }
+        // ---- results: those of an open cell stand unless a generator beyond the
+        // list turns out to cut it
+        {
+            const int64_t out_idx = A.index_space == VT_INDEX_ORIGINAL ? (int64_t)__float_as_int(pi.w) : (int64_t)q;
+            trace_finish<Real, NP, PER>(sm, G, act && ok ? V : 0, fl, fh, R2, pi, out_idx, A);
+        }
+        append(A.slow_list, A.slow_ctr, act && !ok && gl == 0, q, G.lane);
+        if (__any_sync(TFULL, act && open)) {
+            append(A.open_list, A.open_ctr, act && open && gl == 0, q, G.lane);
+            OpenCell* h = reinterpret_cast<OpenCell*>(state);
+            const int F = __popc(fl) + __popc(fh);
+            if (act && open)
+                for (int i = gl; i < F; i += TT) h->src[i] = sm.src[nth_face(fl, fh, i)];
+            // the vertices beyond half the reach: a generator cuts a vertex v only
+            // from inside the ball of radius |v| around v
+            int nf = 0;
+            const int vmax = __reduce_max_sync(TFULL, act && open ? V : 0);
+            const float half = 0.25f * reach * (1.0f - 1e-4f);
+#pragma unroll 1
+            for (int s0 = 0; s0 < vmax; s0 += TT) {
+                const float4 v = sm.vp[s0 + gl];
+                const float d = v.x * v.x + v.y * v.y + v.z * v.z;
+                const bool far = act && open && s0 + gl < V && d >= half;
+                const unsigned m = G.ballot(far);
+                if (far) h->far[nf + __popc(m & ((1u << gl) - 1u))] = make_float4(v.x, v.y, v.z, d);
+                nf += __popc(m);
+            }
+            if (act && open && gl == 0) {
+                h->np = F;
+                h->nf = nf;
+                h->reach = reach;
+                h->all2 = 4.0f * R2 * (1.0f + 2e-5f);
+                h->band = emax * R;
+            }
+        }
+        __syncwarp();
+    }
+    if (gl == 0 && n_open) atomicAdd(&A.st->n_open, (int)n_open);
+    if (gl == 0 && n_second) atomicAdd(&A.st->n_second, (int)n_second);
+}
+
+// as many blocks as are resident at once (they take cells from the queue)
+template <typename K>
+cudaError_t resident_blocks(K kern, int block, size_t smem, int64_t cells, int per_block, unsigned& blocks)
+{
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    int dev = 0, sms = 0, per_sm = 0;
+    if (e == cudaSuccess) e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, block, smem);
+    if (e != cudaSuccess) return e;
+    const int64_t want = (cells + per_block - 1) / per_block, resident = (int64_t)sms * (per_sm > 0 ? per_sm : 1);
+    blocks = (unsigned)(want < resident ? (want > 0 ? want : 1) : resident);
+    return cudaSuccess;
+}
+
+template <typename Real, int NR>
+cudaError_t launch_trace_t(const TraceArgs& a, cudaStream_t s)
+{
+    const size_t smem = trace_stride<Real, NR * TT>() * (TRACE_BLOCK / TT);
+    auto kern = a.g.periodic ? k_trace<Real, NR, true> : k_trace<Real, NR, false>;
+    unsigned blocks = 1;
+    const cudaError_t e = resident_blocks(kern, TRACE_BLOCK, smem, a.nq, TRACE_BLOCK / TT, blocks);
+    if (e != cudaSuccess) return e;
+    kern<<<blocks, TRACE_BLOCK, smem, s>>>(a);
+    count_launch();
+    return cudaGetLastError();
+}
+
+}  // namespace
+
+}  // namespace vt

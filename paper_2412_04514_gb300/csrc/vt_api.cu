@@ -238,7 +238,7 @@ Layout make_layout(const vt_params* p, int64_t n, int64_t cells, bool batch)
     L.rob_nbr = take(sizeof(int32_t) * L.rob_cap);
     L.rob_d2 = take(sizeof(double) * L.rob_cap);
     L.set_of = batch ? take(sizeof(int32_t) * nn) : 0;
-    L.ctr = take(sizeof(int32_t) * (4 * VT_MAX_PASSES + 8));
+    L.ctr = take(sizeof(int32_t) * CTR_COUNT);
     L.rlen = take(sizeof(int32_t) * nn);
     L.total = off;
     return L;
@@ -478,6 +478,90 @@ int clip_pass(const Ctx& c, const vt_params* p, const int32_t* list, int64_t m, 
     return VT_OK;
 }
 
+// Whether the list pass with lists of `kl` entries builds whole cells by edge
+// tracing (trace_impl.cuh): the pass after it would be the last one anyway (the
+// tracing finishes every open cell by its own walk, so a caller's further
+// doubling passes stay as they are), and the list is long enough that what it
+// leaves to the walk is small.
+bool traced_pass(const vt_params* p, const Layout& L, int kl)
+{
+    return L.state_stride > 0 && kl >= 12 && 2 * kl > p->k_max;
+}
+
+// The list pass over all n cells by edge tracing: kNN with k_list entries,
+// the lists' cells, further rounds for the cells that farther generators cut,
+// and the plane-by-plane clipper for the cells whose certificate failed or that
+// are still cut after the last round. Every count stays on the device. open,
+// next: scratch lists of n cells, free after the pass.
+int trace_pass(const Ctx& c, const vt_params* p, int64_t n, int k, int k_list, int variant, vt_cells_out* out,
+               int32_t* slow, int32_t* open, int32_t* next, int32_t* fail_next, int32_t* ctr_next,
+               int32_t* fail_robust, int32_t* ctr_robust)
+{
+    const Layout& L = c.L;
+    StageTimer dummy;
+    StageTimer& T = c.timer ? *c.timer : dummy;
+    int32_t* ctr = c.at<int32_t>(L.ctr);
+    T.begin(StageTimer::KNNL);
+    cudaError_t e = launch_knn(c.at<float4>(L.sorted), c.at<int32_t>(L.cell_off), c.g, n, nullptr, n, k_list,
+                               p->precision, c.at<int32_t>(L.knn_nbr), c.at<void>(L.knn_d2), c.st, c.s, c.sets,
+                               c.set_of(), nullptr, 0, c.at<int32_t>(L.ctr) + CTR_QUEUE);
+    T.end();
+    if (c.knn_launches) ++*c.knn_launches;
+    if (e != cudaSuccess) return cuda_fail(e, "knn launch");
+    TraceArgs a{};
+    a.sorted = c.at<float4>(L.sorted);
+    a.cell_off = c.at<int32_t>(L.cell_off);
+    a.g = c.g;
+    a.sets = c.sets;
+    a.set_of = c.set_of();
+    a.nq = n;
+    a.nbr = c.at<int32_t>(L.knn_nbr);
+    a.d2 = c.at<void>(L.knn_d2);
+    a.kstride = k_list;
+    a.kc = k_list < TRACE_LIST ? k_list : TRACE_LIST;
+    a.k_first = k < a.kc ? k : 0;
+    a.emit = p->emit;
+    a.index_space = p->index_space;
+    a.rec_f32 = p->precision != VT_FP64 ? 1 : 0;
+    a.vol = (p->emit & VT_EMIT_VOL) ? out->vol : nullptr;
+    a.cen = (p->emit & VT_EMIT_CEN) ? out->cen : nullptr;
+    a.m2 = (p->emit & VT_EMIT_M2) ? out->m2 : nullptr;
+    a.rec = L.rec_stride ? c.at<uint8_t>(L.rec) : nullptr;
+    a.rec_stride = L.rec_stride;
+    a.state = c.at<uint8_t>(L.state);
+    a.state_stride = L.state_stride;
+    a.slow_list = slow;
+    a.slow_ctr = ctr + CTR_SLOW;
+    a.st = c.st;
+    for (int round = 0; round < TRACE_ROUNDS; ++round) {
+        // the cells (all, or those the walk before sent back), then the walk over
+        // the open ones among them
+        a.round = round;
+        a.queries = round == 0 ? nullptr : next;
+        a.nq_dev = round == 0 ? nullptr : &ctr[CTR_TRACE + 2 * round - 1];
+        a.open_list = open;
+        a.open_ctr = &ctr[CTR_TRACE + 2 * round];
+        a.queue = &ctr[CTR_TQUEUE + 2 * round];
+        T.begin(StageTimer::CLIP);
+        e = launch_trace(a, p->precision, c.s);
+        T.end();
+        if (c.clip_launches) ++*c.clip_launches;
+        if (e != cudaSuccess) return cuda_fail(e, "trace launch");
+        a.queries = open;
+        a.nq_dev = a.open_ctr;
+        a.next_list = round == TRACE_ROUNDS - 1 ? slow : next;
+        a.next_ctr = round == TRACE_ROUNDS - 1 ? a.slow_ctr : &ctr[CTR_TRACE + 2 * round + 1];
+        a.queue = &ctr[CTR_TQUEUE + 2 * round + 1];
+        T.begin(StageTimer::KNN);
+        e = launch_cutters(a, c.s);
+        T.end();
+        if (c.knn_launches) ++*c.knn_launches;
+        if (e != cudaSuccess) return cuda_fail(e, "walk launch");
+    }
+    return clip_pass(c, p, slow, n, ctr + CTR_SLOW, k, false, 0, variant, p->precision, out, fail_next, ctr_next, fail_robust,
+                     ctr_robust, k_list, true, k_list > k ? k_list : 0);
+}
+
 // the last pass for resumed regular cells (`list`, m cells or *m_dev): range
 // lists of every generator that can still cut, sorted nearest first, clipped
 // as complete lists; cells with more candidates than a list holds go to
@@ -669,7 +753,7 @@ int tessellate_run(Ctx& c, const float* pts, int64_t n, const vt_params* p, vt_c
     c.clip_launches = &S.clip_launches;
     c.knn_launches = &S.knn_launches;
     cudaError_t ce = cudaMemsetAsync(c.st, 0, sizeof(DevStatus), c.s);
-    if (ce == cudaSuccess) ce = cudaMemsetAsync(c.at<int32_t>(L.ctr), 0, sizeof(int32_t) * (4 * VT_MAX_PASSES + 8), c.s);
+    if (ce == cudaSuccess) ce = cudaMemsetAsync(c.at<int32_t>(L.ctr), 0, sizeof(int32_t) * CTR_COUNT, c.s);
     if (ce != cudaSuccess) return cuda_fail(ce, "status reset");
     if (n > 0) {
         timer.begin(StageTimer::GRID);
@@ -743,6 +827,9 @@ int tessellate_run(Ctx& c, const float* pts, int64_t n, const vt_params* p, vt_c
             if (last && pi > 0)
                 r = range_pass(c, p, q, n, qn, k_prev, variant_reg, out, regl[(pi + 1) % 2], &ctr_reg[pi], rob_new,
                                &ctr_new[pi], unval, &c.st->n_unval);
+            else if (pi == 0 && !last && traced_pass(p, L, kk))
+                r = trace_pass(c, p, n, merged ? p->k0 : kk, kk, variant_reg, out, regl[0], robl[0], robl[1], rn,
+                               rc, rob_new, &ctr_new[pi]);
             else
                 r = clip_pass(c, p, q, n, qn, merged ? p->k0 : kk, last, k_prev, variant_reg, p->precision, out, rn,
                               rc, rob_new, &ctr_new[pi], merged ? kk : 0, false, merged ? kk : 0);
@@ -780,6 +867,7 @@ int tessellate_run(Ctx& c, const float* pts, int64_t n, const vt_params* p, vt_c
     bool implicit = true;  // the first pass runs over all cells without a list
     int k = fused ? p->k_max + 1 : p->k0;  // fused: the exhaustive walk is the first pass
     int k_prev = 0;  // regular cells resume from their saved state after list entry k_prev
+    int64_t n_open = 0;  // cells that a traced list pass left open and finished itself
 
     while (m_reg + m_rob > 0) {
         const bool exhaustive = k > p->k_max;
@@ -787,11 +875,11 @@ int tessellate_run(Ctx& c, const float* pts, int64_t n, const vt_params* p, vt_c
         const bool merged = implicit && !exhaustive && 2 * k <= p->k_max && (int64_t)2 * k * m_reg <= L.knn_cap;
         if (S.passes < VT_MAX_PASSES) {
             S.k_of_pass[S.passes] = kk;
-            S.cells_of_pass[S.passes] = m_reg + m_rob;
+            S.cells_of_pass[S.passes] = m_reg + m_rob + (exhaustive ? n_open : 0);
         }
         timer.pass = S.passes;
         ++S.passes;
-        if (exhaustive) S.exhaustive_cells = m_reg + m_rob;
+        if (exhaustive) S.exhaustive_cells = m_reg + m_rob + n_open;
         int64_t got_next = 0, got_rob = 0;
         if (m_reg > 0) {
             if ((r = zero_counters(c))) return r;
@@ -805,6 +893,9 @@ int tessellate_run(Ctx& c, const float* pts, int64_t n, const vt_params* p, vt_c
             if (by_range)
                 r = range_pass(c, p, reg_cur, m_reg, nullptr, k_prev, variant_reg, out, reg_nxt, &c.st->n_range_over,
                                rob_new, &c.st->n_fail_robust, unval + n_unval, &c.st->n_fail_next);
+            else if (implicit && !exhaustive && traced_pass(p, L, merged ? 2 * kk : kk))
+                r = trace_pass(c, p, m_reg, kk, merged ? 2 * kk : kk, variant_reg, out, reg_cur, rob_cur, rob_nxt,
+                               reg_nxt, &c.st->n_fail_next, rob_new, &c.st->n_fail_robust);
             else
                 // the first two list passes (k and 2 k) run as one launch over
                 // the 2 k list when 2 k <= k_max: a cell the first k entries
@@ -818,6 +909,7 @@ int tessellate_run(Ctx& c, const float* pts, int64_t n, const vt_params* p, vt_c
             if ((r = status_errors(h))) return r;
             got_next = h.n_fail_next;
             got_rob = h.n_fail_robust;
+            n_open = h.n_open;
             if (exhaustive && got_next > 0) {
                 // the exhaustive pass concludes every cell; what it hands on
                 // is unvalidated (range lists write it to unval + n_unval)
@@ -882,6 +974,12 @@ int tessellate_run(Ctx& c, const float* pts, int64_t n, const vt_params* p, vt_c
         }
         k_prev = k;
         k *= 2;
+    }
+    if (n_open > 0 && S.exhaustive_cells == 0 && S.passes < VT_MAX_PASSES) {
+        // every open cell was finished inside the list pass: its last part
+        S.k_of_pass[S.passes] = 0;
+        S.cells_of_pass[S.passes] = S.exhaustive_cells = n_open;
+        ++S.passes;
     }
     S.unvalidated = n_unval;
     if (n_unval > 0) {

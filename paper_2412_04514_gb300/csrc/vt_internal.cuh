@@ -459,7 +459,8 @@ struct DevStatus {
     int32_t pad0;
     unsigned long long walk_cells;  // last-pass walks over the shells within 2R (range lists, clipper)
     unsigned long long walk_cands;  // generators of the grid runs those walks examined
-    int32_t pad[6];
+    int32_t n_open;           // cells the traced list left open (stats)
+    int32_t pad[5];
 };
 static_assert(sizeof(DevStatus) % 64 == 0, "status block must stay 64-byte sized");
 
@@ -549,6 +550,13 @@ enum : int8_t { CELL_DONE = 0, CELL_NEED_K = 1, CELL_NEED_ROBUST = 2, CELL_UNVAL
 // ---------------------------------------------------------------------------
 // the cell counter of a clip launch, in the workspace's counter region
 constexpr int CTR_QUEUE = 4 * VT_MAX_PASSES + 4;
+// the traced pass: the lists of its rounds, and the cells left to the
+// plane-by-plane clipper
+constexpr int TRACE_ROUNDS = 4;
+constexpr int CTR_TRACE = CTR_QUEUE + 1;            // open and next list of each round
+constexpr int CTR_SLOW = CTR_TRACE + 2 * TRACE_ROUNDS;
+constexpr int CTR_TQUEUE = CTR_SLOW + 1;            // a cell counter per launch of the pass
+constexpr int CTR_COUNT = CTR_TQUEUE + 2 * TRACE_ROUNDS;
 
 struct Layout {
     int G;
@@ -652,6 +660,39 @@ struct ClipArgs {
 // variant: 0 = FP32 regular, 1 = FP64 regular, 2 = FP64 robust (bigger capacity),
 // 3 = FP32 with the robust capacity (the FP32 form's first fallback)
 cudaError_t launch_clip(const ClipArgs& a, int variant, int threads_per_cell, cudaStream_t s);
+// whole cells by edge tracing (trace_impl.cuh): one round over lists or over
+// the plane sets saved by the round before
+struct TraceArgs {
+    const float4* sorted;
+    const int32_t* cell_off;
+    GridDesc g;
+    const GridDesc* sets;
+    const int32_t* set_of;
+    int64_t nq;               // cells (the bound when nq_dev is set)
+    const int32_t* nq_dev;
+    const int32_t* queries;   // sorted indices (NULL = 0..nq-1, with lists)
+    const int32_t* nbr;       // round 0: lists, kstride entries per cell, the first kc used
+    const void* d2;
+    int kstride, kc;
+    int k_first;              // > 0: count the cells still open at this entry (statistics)
+    int round;                // 0: lists; > 0: the planes left by the round before
+    int emit, index_space, rec_f32;
+    double *vol, *cen, *m2;
+    uint8_t* rec;
+    size_t rec_stride;
+    uint8_t* state;
+    size_t state_stride;
+    int32_t *open_list, *open_ctr;  // cells the walk has to look at
+    int32_t *next_list, *next_ctr;  // cells to build again (the walk's output)
+    int32_t *slow_list, *slow_ctr;  // cells for the plane-by-plane clipper
+    DevStatus* st;
+    int32_t* queue;           // the launch's cell counter (zero)
+};
+// lists used per cell at most: with the six walls they fill the planes of a group
+constexpr int TRACE_LIST = 34;
+cudaError_t launch_trace(const TraceArgs& a, int precision, cudaStream_t s);
+// the walk of a round: a.queries / a.nq_dev are the round's open cells
+cudaError_t launch_cutters(const TraceArgs& a, cudaStream_t s);
 size_t clip_state_bytes(int precision);       // per-cell state of the regular variant (64 slots)
 size_t clip_state_pos_offset(int precision);  // offset of its vertex positions: Real[3][64], x, y, z rows
 

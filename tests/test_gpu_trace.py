@@ -1,0 +1,116 @@
+"""Cells by edge tracing (csrc/trace_impl.cuh) at the sizes where they can go
+wrong: lists that hold every other generator, lists shorter and longer than the
+planes of a group, cells with more vertices than its slots, cells that every
+round leaves open, degenerate vertices (the certificate refuses them), point
+counts that leave groups and blocks partly empty, and small sets in a batch.
+Both forms against the FP64 oracle, to the tolerances of the other parity tests
+(FP32: 1e-5 relative, about 150 roundings of the volume's terms; FP64: 1e-12,
+the oracle's own bound on cells of clumps)."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+
+import oracle
+import paper_2412_04514_gb300 as vt
+from paper_2412_04514_gb300 import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+TOL = {"fp32": 1e-5, "fp64": 1e-12}
+
+
+def check(pts, prec, want=None, periodic=False, **kw):
+    if want is None:
+        want = oracle.tessellate(pts, periodic=periodic)
+    cells = vt.tessellate(torch.from_numpy(pts).cuda(),
+                          vt.Params(precision=prec, emit=("nbr", "vol", "cen", "geom"), periodic=periodic, **kw))
+    np.testing.assert_allclose(cells.vol.cpu().numpy(), want["vol"], rtol=TOL[prec])
+    np.testing.assert_allclose(cells.cen.cpu().numpy(), want["cen"], rtol=TOL[prec], atol=TOL[prec] * 1e-2)
+    if prec == "fp64":
+        assert np.array_equal(cells.nbr_off.cpu().numpy(), want["nbr_off"])
+        assert np.array_equal(cells.nbr.cpu().numpy(), want["nbr"])
+    # every cell is a simple polyhedron: V = 2 F - 4, three faces at each vertex
+    v, f = torch.diff(cells.vtx_off), torch.diff(cells.face_off)
+    assert torch.equal(v, 2 * f - 4)
+    deg = torch.diff(cells.face_vtx_off)
+    assert int(deg.min()) >= 3 and int(deg.sum()) == 3 * int(v.sum())
+    return cells
+
+
+@pytest.mark.parametrize("prec", ["fp32", "fp64"])
+@pytest.mark.parametrize("n", [1, 2, 3, 5, 31, 32, 33, 34, 35, 63, 65, 127, 129, 515])
+def test_small_counts(n, prec):
+    check(W.uniform(n, 100 + n), prec)
+
+
+@pytest.mark.parametrize("prec", ["fp32", "fp64"])
+@pytest.mark.parametrize("k0,k_max", [(6, 12), (12, 12), (16, 31), (17, 34), (17, 40), (18, 36), (40, 70), (64, 64)])
+def test_list_lengths(k0, k_max, prec):
+    check(W.mixed(3001, 5, n_clumps=3), prec, k0=k0, k_max=k_max)
+
+
+@pytest.mark.parametrize("prec", ["fp32", "fp64"])
+@pytest.mark.parametrize("n", [40, 300, 1201])
+def test_periodic(n, prec):
+    check(W.mixed(n, 9, n_clumps=2, periodic=True), prec, periodic=True)
+
+
+@pytest.mark.parametrize("prec", ["fp32", "fp64"])
+@pytest.mark.parametrize("around", [20, 26, 27, 40, 60])
+def test_many_faced_cells(around, prec):
+    # a generator inside a shell of `around` others at about one distance: its
+    # cell has up to around faces (26 fill the vertex slots of a group)
+    rng = np.random.default_rng(around)
+    d = rng.standard_normal((around, 3))
+    shell = 0.5 + (0.2 + 1e-3 * rng.random((around, 1))) * d / np.linalg.norm(d, axis=1, keepdims=True)
+    far = rng.random((400, 3))
+    far = far[np.linalg.norm(far - 0.5, axis=1) > 0.4]
+    check(np.concatenate([[[0.5, 0.5, 0.5]], shell, far]).astype(np.float32), prec)
+
+
+@pytest.mark.parametrize("prec", ["fp32", "fp64"])
+def test_sparse_cells_beside_a_dense_clump(prec):
+    # the lists of the sparse points end inside the clump; thousands of its
+    # points lie within twice their radius and the rounds cut them back
+    rng = np.random.default_rng(4)
+    clump = 0.5 + 2e-3 * rng.standard_normal((6000, 3))
+    check(np.concatenate([clump, rng.random((60, 3))]).astype(np.float32), prec)
+
+
+@pytest.mark.parametrize("prec", ["fp32", "fp64"])
+@pytest.mark.parametrize("make", [lambda: W.cubic_lattice(8), lambda: W.bcc_lattice(6)])
+def test_lattices(make, prec):
+    # every vertex of the cubic lattice and the walls' of the BCC lattice have
+    # more than three planes: the certificate sends the cells to the clipper
+    pts = make()
+    want = oracle.tessellate(pts)
+    cells = vt.tessellate(torch.from_numpy(pts).cuda(), vt.Params(precision=prec, emit=("nbr", "vol", "cen")))
+    np.testing.assert_allclose(cells.vol.cpu().numpy(), want["vol"], rtol=TOL[prec])
+    np.testing.assert_allclose(cells.cen.cpu().numpy(), want["cen"], rtol=TOL[prec])
+
+
+@pytest.mark.parametrize("prec", ["fp32", "fp64"])
+def test_batch_of_small_sets(prec):
+    sizes = [1, 2, 0, 7, 33, 34, 35, 200, 1, 1500]
+    parts = [W.uniform(n, 40 + i) for i, n in enumerate(sizes)]
+    off = np.concatenate([[0], np.cumsum(sizes)])
+    b = vt.Batch(torch.from_numpy(np.concatenate(parts)).cuda(), off, vt.Params(precision=prec, emit=("nbr", "vol", "cen")))
+    b.capture()
+    b.replay()
+    cells = b.result()
+    vol = cells.vol.cpu().numpy()
+    for i, p in enumerate(parts):
+        if len(p):
+            np.testing.assert_allclose(vol[off[i]:off[i + 1]], oracle.tessellate(p)["vol"], rtol=TOL[prec])
+
+
+def test_repeats_bit_for_bit():
+    pts = torch.from_numpy(W.mixed(30_011, 33, n_clumps=20)).cuda()
+    for prec in ("fp32", "fp64"):
+        p = vt.Params(precision=prec, emit=("nbr", "vol", "cen", "m2", "geom"))
+        a = vt.tessellate(pts, p)
+        for _ in range(3):
+            b = vt.tessellate(pts, p)
+            for name in ("vol", "cen", "m2", "nbr", "vtx", "face_nbr", "face_vtx"):
+                assert torch.equal(getattr(a, name), getattr(b, name)), (prec, name)
