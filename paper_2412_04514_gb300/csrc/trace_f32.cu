@@ -3,7 +3,7 @@
 
 namespace vt {
 
-cudaError_t launch_trace_f32(const TraceArgs& a, cudaStream_t s) { return launch_trace_t<float, 5>(a, s); }
+cudaError_t launch_trace_f32(const TraceArgs& a, cudaStream_t s) { return launch_trace_t<float>(a, s); }
 
 cudaError_t launch_cutters(const TraceArgs& a, cudaStream_t s)
 {

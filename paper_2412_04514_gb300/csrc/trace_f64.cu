@@ -3,6 +3,6 @@
 
 namespace vt {
 
-cudaError_t launch_trace_f64(const TraceArgs& a, cudaStream_t s) { return launch_trace_t<double, 5>(a, s); }
+cudaError_t launch_trace_f64(const TraceArgs& a, cudaStream_t s) { return launch_trace_t<double>(a, s); }
 
 }  // namespace vt

@@ -30,16 +30,20 @@
 // vertex) and every edge has both its ends. Such vertices are vertices of the
 // exact polyhedron, and a set of them that is closed under its edges is all of
 // them, so an accepted topology is the exact one. A cell that fails (vertices
-// within round-off of a further plane, ill-conditioned or more than 48 of
-// them) is handed to the plane-by-plane clipper with its FP64 rechecks.
+// within round-off of a further plane, ill-conditioned or too many of them) is
+// built again by other means, in the end by the plane-by-plane clipper with its
+// FP64 rechecks.
 //
 // Security radius. A cell whose 4 R^2 is within the list's reach is final.
 // Otherwise its results are written all the same and a second kernel (a warp
 // per cell) walks the generators beyond the list and within 2R, row by row of
 // the grid: one that cuts no vertex changes nothing, so without a cutting
 // generator the results stand. The other cells are built again from their
-// faces and the nearest cutting generators, in the next round; what a further
-// generator still cuts after the last round goes to the clipper as well.
+// faces and the nearest cutting generators, once more by groups of 8 lanes and
+// then, with the cells that failed, by a warp per cell that rebuilds and walks
+// until nothing cuts. That kernel holds more planes, vertices and open edges
+// and solves more vertices in FP64; what its certificate refuses too goes to
+// the plane-by-plane clipper.
 #pragma once
 #include "clip_impl.cuh"
 
@@ -48,15 +52,11 @@ namespace vt {
 namespace {
 
 constexpr unsigned TFULL = 0xffffffffu;
-constexpr int TT = 8;              // lanes per cell
-constexpr int TG = 32 / TT;        // cells per warp
-constexpr int TRACE_V = 48;        // vertices of a cell (its polyhedron has V / 2 + 2 faces)
-constexpr int TRACE_E = 3 * TRACE_V / 2;  // its edges
-constexpr int TRACE_SLOTS = 16;    // open edge ends of a cell (two per lane)
 constexpr int TRACE_KEEP = 12;     // cutting generators handed to the next round
 constexpr int PAD_PLANE = INT_MIN;
 
-// 8-lane primitives of a warp in lockstep
+// groups of TT lanes of a warp in lockstep
+template <int TT>
 struct Sub {
     int lane, gl, base, gi;
     __device__ __forceinline__ Sub()
@@ -68,7 +68,8 @@ struct Sub {
     }
     __device__ __forceinline__ unsigned ballot(bool p) const
     {
-        return (__ballot_sync(TFULL, p) >> base) & ((1u << TT) - 1u);
+        const unsigned b = __ballot_sync(TFULL, p);
+        return TT == 32 ? b : (b >> base) & ((1u << (TT & 31)) - 1u);
     }
     __device__ __forceinline__ bool any(bool p) const { return ballot(p) != 0; }
     template <typename V>
@@ -77,12 +78,6 @@ struct Sub {
     {
 #pragma unroll
         for (int o = TT / 2; o >= 1; o >>= 1) v = fmaxf(v, __shfl_xor_sync(TFULL, v, o));
-        return v;
-    }
-    __device__ __forceinline__ float min(float v) const
-    {
-#pragma unroll
-        for (int o = TT / 2; o >= 1; o >>= 1) v = fminf(v, __shfl_xor_sync(TFULL, v, o));
         return v;
     }
     __device__ __forceinline__ double maxd(double v) const
@@ -126,91 +121,43 @@ __device__ __forceinline__ float sqrt_fast(float x)
     return y;
 }
 
-// vertex positions and planes in the arithmetic of the results. The FP32
-// form solves and integrates with the float planes; the FP64 form keeps double
-// planes and positions beside the float ones that the tests use.
-template <typename Real, int NP>
+// positions and planes in the arithmetic of the results. The FP32 form solves
+// and integrates with the float planes; the FP64 form keeps double planes and
+// positions beside the float ones that the tests use.
+template <typename Real, int NP, int NV>
 struct TraceReal {};
-template <int NP>
-struct TraceReal<double, NP> {
+template <int NP, int NV>
+struct TraceReal<double, NP, NV> {
     double pn[NP][3];  // n
     double ps[NP];     // b / |n|^2
-    double v[TRACE_V][3];
+    double v[NV][3];
 };
 
-template <typename Real, int NP>
-struct alignas(16) TraceSmem : TraceReal<Real, NP> {
-    float4 pl[NP];            // n, b of n.x <= b
-    float4 vp[TRACE_V];       // position; its error bound relative to R
-    int32_t src[NP];          // sorted index (with image code), -1..-6 walls, PAD_PLANE
-    uint8_t vid[TRACE_V][4];  // planes (ccw from outside)
+// shared memory of a group: NP planes, NV vertices
+template <typename Real, int NP, int NV>
+struct alignas(16) TraceSmem : TraceReal<Real, NP, NV> {
+    float4 pl[NP];       // n, b of n.x <= b
+    float4 vp[NV];       // position; its error bound relative to R
+    int32_t src[NP];     // sorted index (with image code), -1..-6 walls, PAD_PLANE
+    uint8_t vid[NV][4];  // planes (ccw from outside)
     // edges: planes a | b << 8, vertices s << 16 | t << 24; (a, b) follow one
     // another in vid[s], so s -> t runs ccw around b and t -> s around a
-    uint32_t ed[TRACE_E];
+    uint32_t ed[3 * NV / 2];
     union {
-        float nl[NP];         // |n| (until the vertices are solved)
-        int32_t f[NP];        // the finish: each plane's area sum, then the faces' neighbour keys
+        float nl[NP];    // |n| (until the vertices are solved)
+        int32_t f[NP];   // the finish: each plane's area sum, then the faces' neighbour keys
     } u;
 };
 // stride of a group's block: the four groups of a warp read the same member
 // at once (float4 broadcasts), so their blocks start 32 bytes apart modulo the
 // 128 bytes of the banks
-template <typename Real, int NP>
+template <typename S>
 constexpr size_t trace_stride()
 {
-    return (sizeof(TraceSmem<Real, NP>) + 95) / 128 * 128 + 32;
+    return (sizeof(S) + 95) / 128 * 128 + 32;
 }
 
-// the ray v + t d against this lane's planes (unit normals): (t bits with the
-// plane index in the low six) of the first plane met over the group; a value
-// of 0x7f800000 or more when none is met. A plane counts when the ray closes in
-// on it faster than `least`, which leaves out the planes that hold the ray
-// (their rate is round-off) together with those whose vertex would be too
-// ill-conditioned to accept. The six low bits of t only order hits that agree
-// to 8e-6, whose vertices the certificate would refuse anyway.
-template <int NR>
-__device__ __forceinline__ uint32_t hit_rows(const float* nx, const float* ny, const float* nz, const float* nb, float vx,
-                                             float vy, float vz, float dx, float dy, float dz, float least)
-{
-    uint32_t key = 0xffffffffu;
-#pragma unroll
-    for (int r = 0; r < NR; ++r) {
-        const float s = fmaf(-nx[r], vx, fmaf(-ny[r], vy, fmaf(-nz[r], vz, nb[r])));
-        const float nd = fmaf(nx[r], dx, fmaf(ny[r], dy, nz[r] * dz));
-        const uint32_t k = (__float_as_uint(s * rcp_fast(nd)) & ~63u) | (uint32_t)(r * TT);
-        key = nd > least ? ::min(key, k) : key;
-    }
-    return key;
-}
-// rows: the rows of planes in use over the warp (two unrolled forms: the
-// lists fill all NR, most later rounds three)
-template <int NR>
-__device__ __forceinline__ uint32_t first_hit(const float (&nx)[NR], const float (&ny)[NR], const float (&nz)[NR],
-                                              const float (&nb)[NR], int rows, float vx, float vy, float vz, float dx,
-                                              float dy, float dz, float least, int gl)
-{
-    uint32_t key = rows <= 3 ? hit_rows<3>(nx, ny, nz, nb, vx, vy, vz, dx, dy, dz, least)
-                             : hit_rows<NR>(nx, ny, nz, nb, vx, vy, vz, dx, dy, dz, least);
-    key |= (uint32_t)gl;
-#pragma unroll
-    for (int o = TT / 2; o >= 1; o >>= 1) key = ::min(key, __shfl_xor_sync(TFULL, key, o));
-    return key;
-}
-// planes of the lane's first NR rows closer than thr to v (or behind it)
-template <int NR>
-__device__ __forceinline__ int near_rows(const float* nx, const float* ny, const float* nz, const float* nb, float4 v,
-                                         float thr)
-{
-    int near = 0;
-#pragma unroll
-    for (int r = 0; r < NR; ++r)
-        near += fmaf(-nx[r], v.x, fmaf(-ny[r], v.y, fmaf(-nz[r], v.z, nb[r]))) < thr ? 1 : 0;
-    return near;
-}
-
-// below this |det| of the unit normals (about 1 in 3,000 vertices) the FP32
-// form solves a vertex in FP64
-constexpr float UNIT_F64 = 1e-2f;
+// FP64 position of the vertex of three planes (out of line: rarely needed)
 template <bool PER>
 __device__ VT_RARE bool solve_vertex64(int a, int b, int c, const float4* __restrict__ sorted, float4 pi,
                                        const GridDesc& grid, float& x, float& y, float& z)
@@ -224,28 +171,429 @@ __device__ VT_RARE bool solve_vertex64(int a, int b, int c, const float4* __rest
     return ok;
 }
 
-// the i-th (0-based) plane of a face mask
-__device__ __forceinline__ int nth_face(uint32_t lo, uint32_t hi, int i)
-{
-    const int c = __popc(lo);
-    return i < c ? nth_bit32(lo, i) : 32 + nth_bit32(hi, i - c);
-}
+// a set of planes
+template <int W>
+struct Faces {
+    uint32_t w[W];
+    __device__ __forceinline__ void clear()
+    {
+#pragma unroll
+        for (int i = 0; i < W; ++i) w[i] = 0;
+    }
+    __device__ __forceinline__ void add(int p)
+    {
+#pragma unroll
+        for (int i = 0; i < W; ++i) w[i] |= p >> 5 == i ? 1u << (p & 31) : 0u;
+    }
+    __device__ __forceinline__ int count() const
+    {
+        int c = 0;
+#pragma unroll
+        for (int i = 0; i < W; ++i) c += __popc(w[i]);
+        return c;
+    }
+    // the n-th (0-based) of them
+    __device__ __forceinline__ int nth(int n) const
+    {
+        int at = 0;
+        uint32_t x = w[0];
+#pragma unroll
+        for (int i = 1; i < W; ++i) {
+            const int c = __popc(x);
+            if (n >= c && at == 32 * (i - 1)) {
+                n -= c;
+                at = 32 * i;
+                x = w[i];
+            }
+        }
+        return at + nth_bit32(x, n);
+    }
+};
+
+// One cell per group of TT lanes: its planes (unit normals in registers, plane
+// r * TT + lane in row r), then its polyhedron in shared memory. Every member
+// is called by the whole warp; groups without work pass through.
+template <typename Real, int TT, int NR, int NV, bool PER>
+struct Tracer {
+    static constexpr int NP = NR * TT;
+    static constexpr bool F64 = sizeof(Real) == 8;
+    static constexpr int NE = 3 * NV / 2;
+    using S = TraceSmem<Real, NP, NV>;
+    // smallest |det| of a vertex's three unit normals, above the rounding of the
+    // rates of approach (worse vertices are left to the clipper)
+    static constexpr float UNIT_MIN = F64 ? 2e-5f : 2e-4f;
+    // below this |det| the FP32 form solves a vertex in FP64 (about 1 vertex in
+    // 3,000), and below the other when a cell's error bounds failed it
+    static constexpr float UNIT_F64 = 1e-2f, UNIT_F64_AGAIN = 0.3f;
+    static constexpr int SR = TT == 8 ? 2 : 1;       // registers of open edge ends per lane
+    static constexpr int SLOTS = TT == 32 ? 31 : SR * TT;  // (bit 31 marks a closed edge)
+
+    float nx[NR], ny[NR], nz[NR], nb[NR];
+    int rows;               // rows of planes in use over the warp
+    bool ok;
+    int V, E;
+    float R2, R, emax;      // max |v|^2, its root, largest error bound relative to R
+    double R2d;
+    Faces<(NP + 31) / 32> faces;  // the planes that are faces
+
+    // plane row r of the lane from its source
+    __device__ __forceinline__ void set_plane(S& sm, int r, int p, int src, float4 pi, const GridDesc& grid,
+                                              const float4* __restrict__ sorted)
+    {
+        float x = 0.0f, y = 0.0f, z = 0.0f, b = 1.0f, len = 0.0f, inv = 0.0f;
+        if (src >= 0) {
+            const float3 o = img_off_t<PER>(pi, sorted[img_index_t<PER>(src)], img_code_t<PER>(src), grid);
+            x = o.x;
+            y = o.y;
+            z = o.z;
+            const float nn = x * x + y * y + z * z;
+            b = 0.5f * nn;
+            len = sqrt_fast(nn);
+            inv = rsqrt_fast(nn);
+        } else if (src != PAD_PLANE) {
+            const int w = -src - 1, axis = w >> 1, upper = w & 1;
+            const float one = upper ? 1.0f : -1.0f;
+            x = axis == 0 ? one : 0.0f;
+            y = axis == 1 ? one : 0.0f;
+            z = axis == 2 ? one : 0.0f;
+            const float pc = axis == 0 ? pi.x : (axis == 1 ? pi.y : pi.z);
+            b = PER ? (float)(0.5 * ((double)grid.hi[axis] - (double)grid.lo[axis]))
+                    : (upper ? grid.hi[axis] - pc : pc - grid.lo[axis]);
+            len = inv = 1.0f;
+        }
+        nx[r] = x * inv;
+        ny[r] = y * inv;
+        nz[r] = z * inv;
+        nb[r] = src != PAD_PLANE ? b * inv : FLT_MAX;
+        sm.pl[p] = make_float4(x, y, z, b);
+        sm.u.nl[p] = len;
+        sm.src[p] = src;
+        if constexpr (F64) {
+            if (src != PAD_PLANE) {
+                const P64 d = plane64<PER>(src, sorted, pi, grid);
+                sm.pn[p][0] = d.x;
+                sm.pn[p][1] = d.y;
+                sm.pn[p][2] = d.z;
+                sm.ps[p] = src >= 0 ? 0.5 : d.b;  // b / |n|^2
+            }
+        }
+    }
+
+    template <int N>
+    __device__ __forceinline__ uint32_t hit_rows(float vx, float vy, float vz, float dx, float dy, float dz,
+                                                 float least) const
+    {
+        uint32_t key = 0xffffffffu;
+#pragma unroll
+        for (int r = 0; r < N; ++r) {
+            const float s = fmaf(-nx[r], vx, fmaf(-ny[r], vy, fmaf(-nz[r], vz, nb[r])));
+            const float nd = fmaf(nx[r], dx, fmaf(ny[r], dy, nz[r] * dz));
+            const uint32_t k = (__float_as_uint(s * rcp_fast(nd)) & ~63u) | (uint32_t)(r * TT);
+            key = nd > least ? ::min(key, k) : key;
+        }
+        return key;
+    }
+    // the ray v + t d against the planes (unit normals): the first plane met, -1
+    // when none is. A plane counts when the ray closes in on it faster than
+    // `least`, which leaves out the planes that hold the ray (their rate is
+    // round-off) together with those whose vertex would be too ill-conditioned.
+    // Groups of 8 lanes carry the plane index in the low six bits of t, which
+    // orders hits that agree to 8e-6 by index: the certificate refuses the wrong
+    // ones. A warp per cell compares all of t. Two unrolled forms of the former:
+    // the lists fill all rows, most later rounds three.
+    __device__ __forceinline__ int first_hit(const Sub<TT>& G, float vx, float vy, float vz, float dx, float dy, float dz,
+                                             float least) const
+    {
+        if constexpr (TT == 32) {
+            uint32_t key = 0xffffffffu;
+            int row = 0;
+#pragma unroll
+            for (int r = 0; r < NR; ++r) {
+                const float s = fmaf(-nx[r], vx, fmaf(-ny[r], vy, fmaf(-nz[r], vz, nb[r])));
+                const float nd = fmaf(nx[r], dx, fmaf(ny[r], dy, nz[r] * dz));
+                const uint32_t k = __float_as_uint(s * rcp_fast(nd));
+                const bool take = nd > least && k < key;
+                key = take ? k : key;
+                row = take ? r : row;
+            }
+            const uint32_t first = __reduce_min_sync(TFULL, key);
+            const int lane = __ffs(__ballot_sync(TFULL, key == first)) - 1;
+            row = __shfl_sync(TFULL, row, lane);
+            return first < 0x7f800000u ? row * TT + lane : -1;
+        } else {
+            uint32_t key;
+            if (NR > 3 && rows <= 3) key = hit_rows<(NR > 3 ? 3 : NR)>(vx, vy, vz, dx, dy, dz, least);
+            else key = hit_rows<NR>(vx, vy, vz, dx, dy, dz, least);
+            key |= (uint32_t)G.gl;
+#pragma unroll
+            for (int o = TT / 2; o >= 1; o >>= 1) key = ::min(key, __shfl_xor_sync(TFULL, key, o));
+            return key < 0x7f800000u ? (int)(key & 63u) : -1;
+        }
+    }
+
+    // vertices (as triples of planes) and edges, one ray per vertex. f0: the
+    // plane of the nearest generator; on: the group has a cell
+    __device__ __forceinline__ void trace(const Sub<TT>& G, S& sm, bool on, int f0)
+    {
+        const int gl = G.gl;
+        ok = on;
+        V = 1;
+        E = 0;
+        int o[SR];  // open edge ends (an edge of ed without its second vertex; -1: free)
+#pragma unroll
+        for (int i = 0; i < SR; ++i) o[i] = -1;
+        {
+            const float4 n0 = sm.pl[f0];
+            float vx = 0.5f * n0.x, vy = 0.5f * n0.y, vz = 0.5f * n0.z;
+            // a direction in plane f0: n0 x the axis it is least along
+            const float ax = fabsf(n0.x), ay = fabsf(n0.y), az = fabsf(n0.z);
+            float dx, dy, dz;
+            if (ax <= ay && ax <= az) { dx = 0.0f; dy = n0.z; dz = -n0.y; }
+            else if (ay <= az) { dx = -n0.z; dy = 0.0f; dz = n0.x; }
+            else { dx = n0.y; dy = -n0.x; dz = 0.0f; }
+            int f1 = f0, h = f0;
+#pragma unroll 1
+            for (int e = 0; e < 2; ++e) {
+                // (the second ray runs along f0 and f1: n0 x n1 ends at (f0, f1, h))
+                const int hit = first_hit(G, vx, vy, vz, dx, dy, dz,
+                                          e == 0 ? 1e-3f * sm.u.nl[f0] : UNIT_MIN * sm.u.nl[f0] * sm.u.nl[f1]);
+                ok = ok && hit >= 0;
+                h = ok ? hit : f0;
+                const float4 nh = sm.pl[h];
+                const float t = (nh.w - (nh.x * vx + nh.y * vy + nh.z * vz)) *
+                                rcp_fast(nh.x * dx + nh.y * dy + nh.z * dz);
+                vx = fmaf(t, dx, vx);
+                vy = fmaf(t, dy, vy);
+                vz = fmaf(t, dz, vz);
+                if (e == 0) {
+                    f1 = h;
+                    dx = n0.y * nh.z - n0.z * nh.y;
+                    dy = n0.z * nh.x - n0.x * nh.z;
+                    dz = n0.x * nh.y - n0.y * nh.x;
+                }
+            }
+            if (gl == 0) {
+                sm.vp[0] = make_float4(vx, vy, vz, 0.0f);
+                *reinterpret_cast<uint32_t*>(sm.vid[0]) = (uint32_t)f0 | ((uint32_t)f1 << 8) | ((uint32_t)h << 16);
+            }
+            if (gl == 0) o[0] = f0 | (f1 << 8);
+            if (gl == 1) o[0] = f1 | (h << 8);
+            if (gl == 2) o[0] = h | (f0 << 8);
+        }
+        unsigned live = 7u;
+        __syncwarp();
+        bool run = ok;
+#pragma unroll 1
+        while (__any_sync(TFULL, run)) {
+            // the lowest slot: new ends take the lowest free ones, so the newest go
+            // first (oldest first leaves more ends open: 1.7% of the cells of
+            // uniform points ran out of 16 slots, against 0.4%)
+            const int slot = __ffs(live) - 1;
+            const int got = G.bcast(SR == 1 || slot < TT ? o[0] : o[SR - 1], slot & (TT - 1));
+#pragma unroll
+            for (int i = 0; i < SR; ++i) o[i] = gl + i * TT == slot ? -1 : o[i];
+            const int ent = run ? got : 0;
+            const int a = ent & 0xff, b = (ent >> 8) & 0xff, w = ent >> 16;
+            const float4 v = sm.vp[w], na = sm.pl[a], nbp = sm.pl[b];
+            // the edge on a and b leaves (a, b, c) along n_b x n_a
+            const float dx = nbp.y * na.z - nbp.z * na.y, dy = nbp.z * na.x - nbp.x * na.z,
+                        dz = nbp.x * na.y - nbp.y * na.x;
+            const int hit = first_hit(G, v.x, v.y, v.z, dx, dy, dz, UNIT_MIN * sm.u.nl[a] * sm.u.nl[b]);
+            if (hit < 0 || V >= NV || E > NE - 3) {
+                ok = ok && !run;
+                run = false;
+            }
+            const int h = run ? hit : 0;
+            const float4 nh = sm.pl[h];
+            const float t = fmaf(-nh.x, v.x, fmaf(-nh.y, v.y, fmaf(-nh.z, v.z, nh.w))) *
+                            rcp_fast(fmaf(nh.x, dx, fmaf(nh.y, dy, nh.z * dz)));
+            // the vertex (b, a, h): its other two edges, (a, h) and (h, b), close
+            // against an open end of the same edge, (h, a) or (b, h), or stay open
+            const int k1 = run ? h | (a << 8) : 0xfffe, k2 = run ? b | (h << 8) : 0xfffe;
+            bool m1 = false, m2 = false;
+#pragma unroll
+            for (int i = 0; i < SR; ++i) {
+                m1 = m1 || (o[i] & 0xffff) == k1;
+                m2 = m2 || (o[i] & 0xffff) == k2;
+            }
+            const bool c1 = G.any(m1), c2 = G.any(m2);
+#pragma unroll
+            for (int i = 0; i < SR; ++i) {
+                const int k = o[i] & 0xffff;
+                if (k == k1 || k == k2) {
+                    sm.ed[E + (k == k1 ? 1 : 1 + c1)] = (uint32_t)o[i] | ((uint32_t)V << 24);
+                    o[i] = -1;
+                }
+            }
+            if (SR == 1) live = G.ballot(o[0] >= 0);
+            else live = G.ballot(o[0] >= 0) | (G.ballot(o[SR - 1] >= 0) << (TT & 31));
+            if (run) {
+                if (gl == 0) {
+                    sm.vp[V] = make_float4(fmaf(t, dx, v.x), fmaf(t, dy, v.y), fmaf(t, dz, v.z), 0.0f);
+                    *reinterpret_cast<uint32_t*>(sm.vid[V]) = (uint32_t)b | ((uint32_t)a << 8) | ((uint32_t)h << 16);
+                    sm.ed[E] = (uint32_t)ent | ((uint32_t)V << 24);
+                }
+                // the lowest free slots take what stays open
+                const unsigned free1 = ~live, free2 = c1 ? free1 : free1 & (free1 - 1u);
+                const int s1 = c1 ? 31 : __ffs(free1) - 1, s2 = c2 ? 31 : __ffs(free2) - 1;
+#pragma unroll
+                for (int i = 0; i < SR; ++i) {
+                    const int at = gl + i * TT;
+                    o[i] = at == s1 ? a | (h << 8) | (V << 16) : (at == s2 ? h | (b << 8) | (V << 16) : o[i]);
+                }
+                if ((!c1 && s1 >= SLOTS) || (!c2 && (unsigned)s2 >= (unsigned)SLOTS)) ok = run = false;
+                live = (live | (1u << s1) | (1u << (s2 & 31))) & ((1u << SLOTS) - 1u);
+                E += 1 + c1 + c2;
+                ++V;
+                run = run && live != 0;
+            }
+            __syncwarp();
+        }
+    }
+
+    // the vertices from their planes (in the arithmetic of the form), R, the faces
+    __device__ __forceinline__ void solve(const Sub<TT>& G, S& sm, float4 pi, const GridDesc& grid,
+                                          const float4* __restrict__ sorted, float unit_f64)
+    {
+        R2d = 0.0;
+        R2 = emax = 0.0f;
+        faces.clear();
+#pragma unroll 1
+        for (int s = G.gl; s < V; s += TT) {
+            const uint32_t ids = *reinterpret_cast<const uint32_t*>(sm.vid[s]);
+            const int a = ids & 0xff, b = (ids >> 8) & 0xff, c = (ids >> 16) & 0xff;
+            faces.add(a);
+            faces.add(b);
+            faces.add(c);
+            const float4 p = sm.pl[a], o = sm.pl[b], h = sm.pl[c];
+            const float bcx = o.y * h.z - o.z * h.y, bcy = o.z * h.x - o.x * h.z, bcz = o.x * h.y - o.y * h.x;
+            const float det = p.x * bcx + p.y * bcy + p.z * bcz;
+            // |det| of the unit normals: the vertex moves by (rounding) / this
+            const float unit = fabsf(det) * rcp_fast(sm.u.nl[a] * sm.u.nl[b] * sm.u.nl[c]);
+            if (!(unit > UNIT_MIN)) ok = false;
+            float x, y, z, err;
+            if constexpr (F64) {
+                const double ax = sm.pn[a][0], ay = sm.pn[a][1], az = sm.pn[a][2];
+                const double bx = sm.pn[b][0], by = sm.pn[b][1], bz = sm.pn[b][2];
+                const double cx = sm.pn[c][0], cy = sm.pn[c][1], cz = sm.pn[c][2];
+                const double ab = sm.ps[a] * (sm.src[a] < 0 ? 1.0 : (ax * ax + ay * ay) + az * az);
+                const double bb = sm.ps[b] * (sm.src[b] < 0 ? 1.0 : (bx * bx + by * by) + bz * bz);
+                const double cb = sm.ps[c] * (sm.src[c] < 0 ? 1.0 : (cx * cx + cy * cy) + cz * cz);
+                double dx = 0, dy = 0, dz = 0;
+                if (!solve3<double>(ax, ay, az, ab, bx, by, bz, bb, cx, cy, cz, cb, dx, dy, dz)) ok = false;
+                sm.v[s][0] = dx;
+                sm.v[s][1] = dy;
+                sm.v[s][2] = dz;
+                const double d = (dx * dx + dy * dy) + dz * dz;
+                R2d = d > R2d ? d : R2d;
+                x = (float)dx;
+                y = (float)dy;
+                z = (float)dz;
+                err = 1e-6f;  // float rounding of the position, of the plane and of the test
+            } else {
+                const float cax = h.y * p.z - h.z * p.y, cay = h.z * p.x - h.x * p.z, caz = h.x * p.y - h.y * p.x;
+                const float abx = p.y * o.z - p.z * o.y, aby = p.z * o.x - p.x * o.z, abz = p.x * o.y - p.y * o.x;
+                const float inv = rcp(det);
+                x = (p.w * bcx + o.w * cax + h.w * abx) * inv;
+                y = (p.w * bcy + o.w * cay + h.w * aby) * inv;
+                z = (p.w * bcz + o.w * caz + h.w * abz) * inv;
+                err = 1e-6f + 1.5e-6f * rcp_fast(unit);
+                if (unit < unit_f64) {  // ill-conditioned: float32 would lose digits
+                    if (!solve_vertex64<PER>(sm.src[a], sm.src[b], sm.src[c], sorted, pi, grid, x, y, z)) ok = false;
+                    err = 1e-6f;
+                }
+            }
+            const float d = x * x + y * y + z * z;
+            if (!isfinite(d)) ok = false;
+            R2 = fmaxf(R2, d);
+            emax = fmaxf(emax, err);
+            sm.vp[s] = make_float4(x, y, z, err);
+        }
+        R2 = G.max(R2);
+        emax = G.max(emax);
+        if (F64) R2d = G.maxd(R2d);
+#pragma unroll
+        for (int i = 0; i < (NP + 31) / 32; ++i)
+#pragma unroll
+            for (int o = TT / 2; o >= 1; o >>= 1) faces.w[i] |= __shfl_xor_sync(TFULL, faces.w[i], o);
+        R = sqrtf(R2);
+        __syncwarp();
+    }
+
+    // planes of the lane's first N rows closer than thr to v (or behind it)
+    template <int N>
+    __device__ __forceinline__ int near_rows(float4 v, float thr) const
+    {
+        int near = 0;
+#pragma unroll
+        for (int r = 0; r < N; ++r)
+            near += fmaf(-nx[r], v.x, fmaf(-ny[r], v.y, fmaf(-nz[r], v.z, nb[r]))) < thr ? 1 : 0;
+        return near;
+    }
+    // every vertex clearly inside all planes but its three, every edge closed
+    __device__ __forceinline__ void certify(const Sub<TT>& G, const S& sm)
+    {
+        int near = 0;
+        const int vmax = __reduce_max_sync(TFULL, ok ? V : 0);
+#pragma unroll 2
+        for (int s = 0; s < vmax; ++s) {
+            const float4 v = sm.vp[s];
+            const float thr = s < V ? v.w * R : -INFINITY;  // (other slots hold anything)
+            if (NR > 3 && rows <= 3) near += near_rows<(NR > 3 ? 3 : NR)>(v, thr);
+            else near += near_rows<NR>(v, thr);
+        }
+        near = G.bcast(G.incl_scan(near), TT - 1);
+        ok = !G.any(!ok) && near == 3 * V && 2 * E == 3 * V;
+    }
+    // the same with FP64 where float32 does not decide: a plane too close to a
+    // vertex passes when the vertex, solved in FP64, is inside it by 1e-10 |n| R
+    // (a warp per cell only)
+    __device__ __forceinline__ void certify64(const Sub<TT>& G, const S& sm, float4 pi, const GridDesc& grid,
+                                              const float4* __restrict__ sorted)
+    {
+        bool fine = ok && 2 * E == 3 * V;
+        const int vmax = __any_sync(TFULL, !ok) ? 0 : V;
+#pragma unroll 1
+        for (int s = 0; s < vmax; ++s) {
+            const float4 v = sm.vp[s];
+            const uint32_t ids = *reinterpret_cast<const uint32_t*>(sm.vid[s]);
+#pragma unroll 1
+            for (int r = 0; r < NR; ++r) {
+                const int p = r * TT + G.gl;
+                const float4 n = sm.pl[p];
+                const float len = sqrt_fast(n.x * n.x + n.y * n.y + n.z * n.z);
+                const float d = fmaf(-n.x, v.x, fmaf(-n.y, v.y, fmaf(-n.z, v.z, n.w)));
+                const bool own = p == (int)(ids & 0xff) || p == (int)((ids >> 8) & 0xff) || p == (int)((ids >> 16) & 0xff);
+                if (own || !(d < v.w * R * len)) continue;
+                double x, y, z;
+                const P64 h = plane64<PER>(sm.src[p], sorted, pi, grid);
+                const bool solved = vertex64(plane64<PER>(sm.src[ids & 0xff], sorted, pi, grid),
+                                             plane64<PER>(sm.src[(ids >> 8) & 0xff], sorted, pi, grid),
+                                             plane64<PER>(sm.src[(ids >> 16) & 0xff], sorted, pi, grid), x, y, z);
+                if (!solved || !(h.b - ((h.x * x + h.y * y) + h.z * z) > 1e-10 * (double)len * (double)R)) fine = false;
+            }
+        }
+        ok = !__any_sync(TFULL, !fine);
+    }
+};
 
 // moments, neighbours and geometry of the group's cell (the quantities of
 // finish_cell); every lane of the warp calls, groups with V = 0 write nothing.
-// (fl, fh): the planes that are faces. A lane per edge: the two triangles of
+// A lane per edge (eight lanes also of a warp per cell, so that the float sums
+// are the same whichever kernel built the cell): the two triangles of
 // an edge share its cross product. Areas only decide which faces are above
 // the neighbour threshold: they add up in fixed point (integers add in any
 // order alike), and a face below 1e-4 R^2 is added up again in the arithmetic
 // of the form, edge by edge.
-template <typename Real, int NP, bool PER>
-__device__ __forceinline__ void trace_finish(TraceSmem<Real, NP>& sm, const Sub& G, int V, uint32_t fl, uint32_t fh,
-                                             float R2, float4 pi, int64_t out_idx, const TraceArgs& A)
+template <typename Real, int TT, int NP, int NV, bool PER>
+__device__ __forceinline__ void trace_finish(TraceSmem<Real, NP, NV>& sm, const Sub<TT>& G, int V,
+                                             const Faces<(NP + 31) / 32>& faces, float R2, float4 pi, int64_t out_idx,
+                                             const TraceArgs& A)
 {
     constexpr bool F64 = sizeof(Real) == 8;
     const int gl = G.gl;
     const bool act = V > 0;
-    const int F = act ? __popc(fl) + __popc(fh) : 0;
+    const int F = act ? faces.count() : 0;
     const int E = 3 * V / 2;
     if (A.rec) {
         for (int f = gl; f < NP; f += TT) sm.u.f[f] = 0;
@@ -281,7 +629,7 @@ __device__ __forceinline__ void trace_finish(TraceSmem<Real, NP>& sm, const Sub&
     Real vol = 0, mx = 0, my = 0, mz = 0, m2 = 0;
     const float fix = 1048576.0f * rcp_fast(R2);
 #pragma unroll 1
-    for (int e = gl; e < E; e += TT) {
+    for (int e = gl < 8 ? gl : E; e < E; e += 8) {
         const uint32_t ed = sm.ed[e];
         Real ax, ay, az, bx, by, bz;
         vert((ed >> 16) & 0xff, ax, ay, az);
@@ -350,7 +698,7 @@ __device__ __forceinline__ void trace_finish(TraceSmem<Real, NP>& sm, const Sub&
         const int i = i0 + gl;
         int key = INT_MAX;
         if (i < F) {
-            const int f = nth_face(fl, fh, i);
+            const int f = faces.nth(i);
             const int src = sm.src[f];
             int oid = src;  // wall ids stay
             if (PER) {
@@ -392,7 +740,7 @@ __device__ __forceinline__ void trace_finish(TraceSmem<Real, NP>& sm, const Sub&
             nb = nb && (src >= 0 || PER);
             kept += nb;
             // (periodic ids may repeat; the plane makes the key unique)
-            if (nb) key = PER ? oid * 64 + f : oid;
+            if (nb) key = PER ? oid * 128 + f : oid;
         }
         __syncwarp();  // (the i-th face is plane i or a later one: its area is read before this)
         if (i < F) sm.u.f[i] = key;
@@ -406,7 +754,7 @@ __device__ __forceinline__ void trace_finish(TraceSmem<Real, NP>& sm, const Sub&
         int rank = 0;
 #pragma unroll 4
         for (int k = 0; k < F; ++k) rank += sm.u.f[k] < key ? 1 : 0;
-        rnbr[rank] = PER ? key / 64 : key;
+        rnbr[rank] = PER ? key / 128 : key;
     }
     const int nn = G.bcast(G.incl_scan(kept), TT - 1);
     if (geom) {
@@ -430,11 +778,11 @@ __device__ __forceinline__ void trace_finish(TraceSmem<Real, NP>& sm, const Sub&
         // over the planes (not needed any more)
         __syncwarp();
         uint8_t* next = reinterpret_cast<uint8_t*>(sm.pl);
-        int32_t* first = reinterpret_cast<int32_t*>(sm.pl) + TRACE_V;
+        int32_t* first = reinterpret_cast<int32_t*>(sm.pl) + NV;
         int32_t* degree = first + NP;
-        static_assert(4 * TRACE_V + 8 * NP <= 16 * NP, "the loops fit the planes");
+        static_assert(4 * NV + 8 * NP <= 16 * NP, "the loops fit the planes");
         for (int f = gl; f < NP; f += TT) {
-            first[f] = TRACE_V;
+            first[f] = NV;
             degree[f] = 0;
         }
         __syncwarp();
@@ -459,7 +807,7 @@ __device__ __forceinline__ void trace_finish(TraceSmem<Real, NP>& sm, const Sub&
 #pragma unroll 1
         for (int i0 = 0; i0 < Fmax; i0 += TT) {
             const int i = i0 + gl;
-            const int f = i < F ? nth_face(fl, fh, i) : 0;
+            const int f = i < F ? faces.nth(i) : 0;
             const int deg = i < F ? degree[f] : 0;
             const int inc = G.incl_scan(deg);
             const int pos = base + inc - deg;
@@ -501,21 +849,20 @@ __device__ __forceinline__ void append(int32_t* list, int32_t* ctr, bool on, int
     if (on) list[at + __popc(m & ((1u << lane) - 1u))] = q;
 }
 
-// an open cell between the two kernels of a round, in its state slot
+// an open or failed cell between two kernels of the pass, in its state slot
 struct alignas(16) OpenCell {
     int32_t np, nf;
     float reach;              // generators with a float key below this are behind it
     float all2;               // (2R)^2
     float band;               // error bound of the vertex positions
     int32_t pad[3];
-    int32_t src[40];          // planes of the next round: its faces, then what cuts it
-    float4 far[TRACE_V];      // vertices a generator at `reach` or beyond can cut
+    int32_t src[40];          // its planes: the faces, then what cuts it
+    float4 far[48];           // vertices a generator at `reach` or beyond can cut
 };
-static_assert(TRACE_V / 2 + 2 + TRACE_KEEP <= 40, "the planes of the next round");
 static_assert(sizeof(OpenCell) <= StateLayout<float, 64, 64>::BYTES, "an open cell fits the state slot");
 
-constexpr int CUT_BLOCK = 256;
-constexpr int CUT_LIST = TRACE_KEEP + 32;
+// a warp's list of cutting generators: the ones kept, and a batch
+constexpr int CUT_LIST = 64;
 
 // the nearest `cap` of the warp's ns candidates, in order of (key, id)
 __device__ __forceinline__ int keep_nearest(float* key, int32_t* id, int ns, int cap, int lane)
@@ -544,24 +891,206 @@ __device__ __forceinline__ int keep_nearest(float* key, int32_t* id, int ns, int
     return ns < cap ? ns : cap;
 }
 
-// The walk of the open cells, a warp per cell: the generators with keys of at
-// least the cell's reach and within 2R that cut one of its vertices, the
-// nearest TRACE_KEEP of them. It takes the rows of the grid that meet the box
-// of the far vertices' balls and the ball of the current limit, less the grid
-// cells the list covered; the limit grows from the reach by half its radius at
-// a time, and the walk ends at the first limit that met a cutting generator
-// (the cell it leaves is smaller). A lane per row finds the row's runs, then
-// the lanes share the rows' generators.
+// The walk of a cell, by a warp: the generators with keys of at least `reach`
+// and within 2R (all2) that cut one of the nf far vertices (x, y, z, |v|^2;
+// shared memory, as the lists key and id), the nearest `keep` of them in order;
+// returns their count. own[0, np): the cell's planes. It takes the rows of the
+// grid that meet the box of the far vertices' balls and the ball of the current
+// limit, less the grid cells that are behind; the limit grows from the reach by
+// half its radius at a time, and the walk ends at the first limit that met a
+// cutting generator (the cell it leaves is smaller). A lane per row finds the
+// row's runs, then the lanes share the rows' generators. reach becomes what a
+// later walk of the cell need not look at again.
+template <bool PER>
+__device__ __forceinline__ int walk(const TraceArgs& A, const GridDesc& grid, int q, float4 pi, const float4* far, int nf,
+                                    const int32_t* own, int np, float all2, float band, int keep, float& reach,
+                                    float* key, int32_t* id, unsigned& cands)
+{
+    const int lane = threadIdx.x & 31;
+    // the box of the far vertices' balls, around the generator
+    float l0 = 0, l1 = 0, l2 = 0, h0 = 0, h1 = 0, h2 = 0;
+    for (int s = lane; s < nf; s += 32) {
+        const float4 v = far[s];
+        const float r = sqrt_fast(v.w) * (1.0f + 1e-4f);
+        l0 = fminf(l0, v.x - r); h0 = fmaxf(h0, v.x + r);
+        l1 = fminf(l1, v.y - r); h1 = fmaxf(h1, v.y + r);
+        l2 = fminf(l2, v.z - r); h2 = fmaxf(h2, v.z + r);
+    }
+#pragma unroll
+    for (int o = 16; o >= 1; o >>= 1) {
+        l0 = fminf(l0, __shfl_xor_sync(TFULL, l0, o)); h0 = fmaxf(h0, __shfl_xor_sync(TFULL, h0, o));
+        l1 = fminf(l1, __shfl_xor_sync(TFULL, l1, o)); h1 = fmaxf(h1, __shfl_xor_sync(TFULL, h1, o));
+        l2 = fminf(l2, __shfl_xor_sync(TFULL, l2, o)); h2 = fmaxf(h2, __shfl_xor_sync(TFULL, h2, o));
+    }
+    const int Gr = grid.G;
+    const int32_t* coff = A.cell_off + grid.cell_base;
+    const float m = (float)grid.margin;
+    const float cx = (float)grid.cw[0], cy = (float)grid.cw[1];
+    // periodic: unwrapped grid coordinates, and each row once per z image
+    const float lim_lo = PER ? -2.0f * (float)Gr : 0.0f,
+                lim_hi = PER ? 3.0f * (float)Gr - 1.0f : (float)Gr - 1.0f;
+    auto clamp = [&](float t) { return (int)floorf(fminf(fmaxf(t, lim_lo), lim_hi)); };
+    int ns = 0;
+    bool more = false, end = nf == 0;
+    // (40 steps of 2.25 cover every ratio of float32 keys that differ; the
+    // last one takes the whole ball)
+#pragma unroll 1
+    for (int it = 0; !end && ns == 0; ++it) {
+        const float lim2 = it < 40 ? fminf(all2, 2.25f * reach) : all2;
+        const float r_out2 = lim2 * (1.0f + 1e-4f), r_in2 = reach * (1.0f - 1e-4f);
+        const float rr = sqrt_fast(r_out2) * (1.0f + 1e-5f);
+        const float z_lo = pi.z + fmaxf(l2, -rr) - m, z_hi = pi.z + fminf(h2, rr) + m;
+        const int x0 = clamp((pi.x + fmaxf(l0, -rr) - m - grid.lo[0]) * grid.scale[0] - 1e-3f);
+        const int x1 = clamp((pi.x + fminf(h0, rr) + m - grid.lo[0]) * grid.scale[0] + 1e-3f);
+        const int y0 = clamp((pi.y + fmaxf(l1, -rr) - m - grid.lo[1]) * grid.scale[1] - 1e-3f);
+        const int y1 = clamp((pi.y + fminf(h1, rr) + m - grid.lo[1]) * grid.scale[1] + 1e-3f);
+        int t0 = 0, nt = 1;
+        if (PER) {
+            t0 = floordiv(clamp((z_lo - grid.lo[2]) * grid.scale[2] - 1e-3f), Gr);
+            nt = floordiv(clamp((z_hi - grid.lo[2]) * grid.scale[2] + 1e-3f), Gr) - t0 + 1;
+        }
+        const int wy = y1 - y0 + 1, nrow = (x1 - x0 + 1) * wy * nt;
+#pragma unroll 1
+        for (int e0 = 0; e0 < nrow; e0 += 32) {
+            const int e = e0 + lane;
+            int sa = 0, la = 0, sb = 0, lb = 0, code = IMG_NONE;
+            if (e < nrow) {
+                const int e2 = PER ? e / nt : e;
+                const int tz = PER ? t0 + (e - e2 * nt) : 0;
+                const int ex = e2 / wy, x = x0 + ex, y = y0 + (e2 - ex * wy);
+                const int tx = PER ? floordiv(x, Gr) : 0, ty = PER ? floordiv(y, Gr) : 0;
+                const float gx0 = grid.lo[0] + (float)x * cx - m, gx1 = grid.lo[0] + (float)(x + 1) * cx + m;
+                const float gy0 = grid.lo[1] + (float)y * cy - m, gy1 = grid.lo[1] + (float)(y + 1) * cy + m;
+                const float dxn = fmaxf(fmaxf(gx0 - pi.x, pi.x - gx1), 0.0f),
+                            dyn = fmaxf(fmaxf(gy0 - pi.y, pi.y - gy1), 0.0f);
+                const float dxf = fmaxf(pi.x - gx0, gx1 - pi.x), dyf = fmaxf(pi.y - gy0, gy1 - pi.y);
+                const float dn2 = dxn * dxn + dyn * dyn, df2 = dxf * dxf + dyf * dyf;
+                if (dn2 <= r_out2) {
+                    const float zr = sqrtf(r_out2 - dn2) + m;
+                    int za = clamp((fmaxf(pi.z - zr, z_lo) - grid.lo[2]) * grid.scale[2] - 1e-3f);
+                    int zb = clamp((fminf(pi.z + zr, z_hi) - grid.lo[2]) * grid.scale[2] + 1e-3f);
+                    if (PER) {
+                        za = za > tz * Gr ? za : tz * Gr;
+                        zb = zb < tz * Gr + Gr - 1 ? zb : tz * Gr + Gr - 1;
+                    }
+                    // grid cells wholly inside the ball that is behind: [i0, i1]
+                    int i0 = zb + 1, i1 = zb;
+                    if (r_in2 > df2) {
+                        const float zi = sqrtf(r_in2 - df2) - m;
+                        i0 = (int)ceilf(fminf(fmaxf((pi.z - zi - grid.lo[2]) * grid.scale[2] + 1e-3f, lim_lo - 1.0f),
+                                              lim_hi + 2.0f));
+                        i1 = (int)floorf(fminf(fmaxf((pi.z + zi - grid.lo[2]) * grid.scale[2] - 1e-3f, lim_lo - 1.0f),
+                                               lim_hi + 2.0f)) - 1;
+                        if (i0 > i1 || i1 < za || i0 > zb) {
+                            i0 = zb + 1;
+                            i1 = zb;
+                        }
+                    }
+                    const int base = ((x - tx * Gr) * Gr + (y - ty * Gr)) * Gr - tz * Gr;
+                    const int ea = i0 - 1, fb = i1 + 1 > za ? i1 + 1 : za;
+                    if (za <= ea) {
+                        sa = coff[base + za];
+                        la = coff[base + ea + 1] - sa;
+                    }
+                    if (i0 <= zb && fb <= zb) {
+                        sb = coff[base + fb];
+                        lb = coff[base + zb + 1] - sb;
+                    }
+                    if (PER) code = img_code(tx, ty, tz);
+                }
+            }
+            int incl = la + lb;
+#pragma unroll
+            for (int d = 1; d < 32; d <<= 1) {
+                const int u = __shfl_up_sync(TFULL, incl, d);
+                if (lane >= d) incl += u;
+            }
+            const int total = __shfl_sync(TFULL, incl, 31);
+            const int start = incl - la - lb;
+            cands += (unsigned)total;
+#pragma unroll 1
+            for (int c0 = 0; c0 < total; c0 += 32) {
+                const int i = c0 + lane;
+                int seg = 0;  // rows ending at or before i
+#pragma unroll
+                for (int step = 16; step >= 1; step >>= 1)
+                    if (__shfl_sync(TFULL, incl, (seg + step - 1) & 31) <= i) seg += step;
+                seg &= 31;
+                const int off = i - __shfl_sync(TFULL, start, seg), na = __shfl_sync(TFULL, la, seg);
+                const int ja = __shfl_sync(TFULL, sa, seg), jb = __shfl_sync(TFULL, sb, seg);
+                const int cd = PER ? __shfl_sync(TFULL, code, seg) : IMG_NONE;
+                const int j = off < na ? ja + off : jb + (off - na);
+                const int jj = PER ? img_pack(j, cd) : j;
+                float3 o = make_float3(0.0f, 0.0f, 0.0f);
+                const bool in = i < total && j != q;
+                if (in) o = img_off_t<PER>(pi, A.sorted[j], cd, grid);
+                const float d2 = fmaf(o.z, o.z, fmaf(o.y, o.y, o.x * o.x));
+                bool cuts = in && d2 >= reach && d2 <= r_out2;
+                if (!__any_sync(TFULL, cuts)) continue;
+                float top = -FLT_MAX;
+#pragma unroll 2
+                for (int k = 0; k < nf; ++k) {
+                    const float4 v = far[k];
+                    top = fmaxf(top, fmaf(o.x, v.x, fmaf(o.y, v.y, o.z * v.z)));
+                }
+                cuts = cuts && 0.5f * d2 - top <= band * sqrt_fast(d2);
+                if (cuts)  // (the cell's own faces touch their vertices)
+                    for (int p = 0; p < np; ++p)
+                        if (own[p] == jj) cuts = false;
+                const unsigned cm = __ballot_sync(TFULL, cuts);
+                if (cuts) {
+                    const int at = ns + __popc(cm & ((1u << lane) - 1u));
+                    key[at] = d2;
+                    id[at] = jj;
+                }
+                ns += __popc(cm);
+                if (ns > keep) {
+                    more = true;
+                    ns = keep_nearest(key, id, ns, keep, lane);
+                }
+            }
+        }
+        end = lim2 >= all2;
+        if (!more) reach = lim2;  // (all of it is behind)
+    }
+    if (ns > 0) {
+        ns = keep_nearest(key, id, ns, keep, lane);
+        if (more) reach = key[ns - 1];
+    }
+    return ns;
+}
+
+// vertices beyond half the reach into far (x, y, z, |v|^2): a generator cuts a
+// vertex v only from inside the ball of radius |v| around v
+template <int TT, typename S>
+__device__ __forceinline__ int far_vertices(const Sub<TT>& G, const S& sm, bool on, int V, float reach, float4* far)
+{
+    int nf = 0;
+    const int vmax = __reduce_max_sync(TFULL, on ? V : 0);
+    const float half = 0.25f * reach * (1.0f - 1e-4f);
+#pragma unroll 1
+    for (int s0 = 0; s0 < vmax; s0 += TT) {
+        const int s = s0 + G.gl;  // (the slots are a multiple of TT)
+        const float4 v = sm.vp[s];
+        const float d = v.x * v.x + v.y * v.y + v.z * v.z;
+        const bool is = on && s < V && d >= half;
+        const unsigned m = G.ballot(is);
+        if (is) far[nf + __popc(m & ((1u << G.gl) - 1u))] = make_float4(v.x, v.y, v.z, d);
+        nf += __popc(m);
+    }
+    return nf;
+}
+
+// the walk of a round's open cells, a warp per cell
+constexpr int CUT_BLOCK = 256;
 template <bool PER>
 __global__ void __launch_bounds__(CUT_BLOCK) k_cutters(const __grid_constant__ TraceArgs A)
 {
-    __shared__ float4 s_far[CUT_BLOCK / 32][TRACE_V];
+    __shared__ float4 s_far[CUT_BLOCK / 32][48];
     __shared__ float s_key[CUT_BLOCK / 32][CUT_LIST];
     __shared__ int32_t s_id[CUT_BLOCK / 32][CUT_LIST];
+    static_assert(48 / 2 + 2 + TRACE_KEEP <= 40, "the planes of the next round");
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    float4* far = s_far[warp];
-    float* key = s_key[warp];
-    int32_t* id = s_id[warp];
     const int have = *A.nq_dev;
     const int nq = have < (int)A.nq ? have : (int)A.nq;
     unsigned cells = 0, cands = 0;
@@ -575,161 +1104,14 @@ __global__ void __launch_bounds__(CUT_BLOCK) k_cutters(const __grid_constant__ T
         const float4 pi = A.sorted[q];
         OpenCell* h = reinterpret_cast<OpenCell*>(A.state + (size_t)q * A.state_stride);
         const int np = h->np, nf = h->nf;
-        const float all2 = h->all2, band = h->band;
         float reach = h->reach;
-        // the box of the far vertices' balls, around the generator
-        float l0 = 0, l1 = 0, l2 = 0, h0 = 0, h1 = 0, h2 = 0;
-        for (int s = lane; s < nf; s += 32) {
-            const float4 v = h->far[s];
-            const float r = sqrt_fast(v.w) * (1.0f + 1e-4f);
-            l0 = fminf(l0, v.x - r); h0 = fmaxf(h0, v.x + r);
-            l1 = fminf(l1, v.y - r); h1 = fmaxf(h1, v.y + r);
-            l2 = fminf(l2, v.z - r); h2 = fmaxf(h2, v.z + r);
-            far[s] = v;
-        }
-#pragma unroll
-        for (int o = 16; o >= 1; o >>= 1) {
-            l0 = fminf(l0, __shfl_xor_sync(TFULL, l0, o)); h0 = fmaxf(h0, __shfl_xor_sync(TFULL, h0, o));
-            l1 = fminf(l1, __shfl_xor_sync(TFULL, l1, o)); h1 = fmaxf(h1, __shfl_xor_sync(TFULL, h1, o));
-            l2 = fminf(l2, __shfl_xor_sync(TFULL, l2, o)); h2 = fmaxf(h2, __shfl_xor_sync(TFULL, h2, o));
-        }
+        for (int s = lane; s < nf; s += 32) s_far[warp][s] = h->far[s];
         __syncwarp();
-        const int Gr = grid.G;
-        const int32_t* coff = A.cell_off + grid.cell_base;
-        const float m = (float)grid.margin;
-        const float cx = (float)grid.cw[0], cy = (float)grid.cw[1];
-        // periodic: unwrapped grid coordinates, and each row once per z image
-        const float lim_lo = PER ? -2.0f * (float)Gr : 0.0f,
-                    lim_hi = PER ? 3.0f * (float)Gr - 1.0f : (float)Gr - 1.0f;
-        auto clamp = [&](float t) { return (int)floorf(fminf(fmaxf(t, lim_lo), lim_hi)); };
-        int ns = 0;
-        bool more = false, end = nf == 0;
-        // (40 steps of 2.25 cover every ratio of float32 keys that differ; the
-        // last one takes the whole ball)
-#pragma unroll 1
-        for (int it = 0; !end && ns == 0; ++it) {
-            const float lim2 = it < 40 ? fminf(all2, 2.25f * reach) : all2;
-            const float r_out2 = lim2 * (1.0f + 1e-4f), r_in2 = reach * (1.0f - 1e-4f);
-            const float rr = sqrt_fast(r_out2) * (1.0f + 1e-5f);
-            const float z_lo = pi.z + fmaxf(l2, -rr) - m, z_hi = pi.z + fminf(h2, rr) + m;
-            const int x0 = clamp((pi.x + fmaxf(l0, -rr) - m - grid.lo[0]) * grid.scale[0] - 1e-3f);
-            const int x1 = clamp((pi.x + fminf(h0, rr) + m - grid.lo[0]) * grid.scale[0] + 1e-3f);
-            const int y0 = clamp((pi.y + fmaxf(l1, -rr) - m - grid.lo[1]) * grid.scale[1] - 1e-3f);
-            const int y1 = clamp((pi.y + fminf(h1, rr) + m - grid.lo[1]) * grid.scale[1] + 1e-3f);
-            int t0 = 0, nt = 1;
-            if (PER) {
-                t0 = floordiv(clamp((z_lo - grid.lo[2]) * grid.scale[2] - 1e-3f), Gr);
-                nt = floordiv(clamp((z_hi - grid.lo[2]) * grid.scale[2] + 1e-3f), Gr) - t0 + 1;
-            }
-            const int wy = y1 - y0 + 1, nrow = (x1 - x0 + 1) * wy * nt;
-#pragma unroll 1
-            for (int e0 = 0; e0 < nrow; e0 += 32) {
-                const int e = e0 + lane;
-                int sa = 0, la = 0, sb = 0, lb = 0, code = IMG_NONE;
-                if (e < nrow) {
-                    const int e2 = PER ? e / nt : e;
-                    const int tz = PER ? t0 + (e - e2 * nt) : 0;
-                    const int ex = e2 / wy, x = x0 + ex, y = y0 + (e2 - ex * wy);
-                    const int tx = PER ? floordiv(x, Gr) : 0, ty = PER ? floordiv(y, Gr) : 0;
-                    const float gx0 = grid.lo[0] + (float)x * cx - m, gx1 = grid.lo[0] + (float)(x + 1) * cx + m;
-                    const float gy0 = grid.lo[1] + (float)y * cy - m, gy1 = grid.lo[1] + (float)(y + 1) * cy + m;
-                    const float dxn = fmaxf(fmaxf(gx0 - pi.x, pi.x - gx1), 0.0f),
-                                dyn = fmaxf(fmaxf(gy0 - pi.y, pi.y - gy1), 0.0f);
-                    const float dxf = fmaxf(pi.x - gx0, gx1 - pi.x), dyf = fmaxf(pi.y - gy0, gy1 - pi.y);
-                    const float dn2 = dxn * dxn + dyn * dyn, df2 = dxf * dxf + dyf * dyf;
-                    if (dn2 <= r_out2) {
-                        const float zr = sqrtf(r_out2 - dn2) + m;
-                        int za = clamp((fmaxf(pi.z - zr, z_lo) - grid.lo[2]) * grid.scale[2] - 1e-3f);
-                        int zb = clamp((fminf(pi.z + zr, z_hi) - grid.lo[2]) * grid.scale[2] + 1e-3f);
-                        if (PER) {
-                            za = za > tz * Gr ? za : tz * Gr;
-                            zb = zb < tz * Gr + Gr - 1 ? zb : tz * Gr + Gr - 1;
-                        }
-                        // grid cells wholly inside the ball that is behind: [i0, i1]
-                        int i0 = zb + 1, i1 = zb;
-                        if (r_in2 > df2) {
-                            const float zi = sqrtf(r_in2 - df2) - m;
-                            i0 = (int)ceilf(fminf(fmaxf((pi.z - zi - grid.lo[2]) * grid.scale[2] + 1e-3f, lim_lo - 1.0f),
-                                                  lim_hi + 2.0f));
-                            i1 = (int)floorf(fminf(fmaxf((pi.z + zi - grid.lo[2]) * grid.scale[2] - 1e-3f, lim_lo - 1.0f),
-                                                   lim_hi + 2.0f)) - 1;
-                            if (i0 > i1 || i1 < za || i0 > zb) {
-                                i0 = zb + 1;
-                                i1 = zb;
-                            }
-                        }
-                        const int base = ((x - tx * Gr) * Gr + (y - ty * Gr)) * Gr - tz * Gr;
-                        const int ea = i0 - 1, fb = i1 + 1 > za ? i1 + 1 : za;
-                        if (za <= ea) {
-                            sa = coff[base + za];
-                            la = coff[base + ea + 1] - sa;
-                        }
-                        if (i0 <= zb && fb <= zb) {
-                            sb = coff[base + fb];
-                            lb = coff[base + zb + 1] - sb;
-                        }
-                        if (PER) code = img_code(tx, ty, tz);
-                    }
-                }
-                int incl = la + lb;
-#pragma unroll
-                for (int d = 1; d < 32; d <<= 1) {
-                    const int u = __shfl_up_sync(TFULL, incl, d);
-                    if (lane >= d) incl += u;
-                }
-                const int total = __shfl_sync(TFULL, incl, 31);
-                const int start = incl - la - lb;
-                cands += (unsigned)total;
-#pragma unroll 1
-                for (int c0 = 0; c0 < total; c0 += 32) {
-                    const int i = c0 + lane;
-                    int seg = 0;  // rows ending at or before i
-#pragma unroll
-                    for (int step = 16; step >= 1; step >>= 1)
-                        if (__shfl_sync(TFULL, incl, (seg + step - 1) & 31) <= i) seg += step;
-                    seg &= 31;
-                    const int off = i - __shfl_sync(TFULL, start, seg), na = __shfl_sync(TFULL, la, seg);
-                    const int ja = __shfl_sync(TFULL, sa, seg), jb = __shfl_sync(TFULL, sb, seg);
-                    const int cd = PER ? __shfl_sync(TFULL, code, seg) : IMG_NONE;
-                    const int j = off < na ? ja + off : jb + (off - na);
-                    const int jj = PER ? img_pack(j, cd) : j;
-                    float3 o = make_float3(0.0f, 0.0f, 0.0f);
-                    const bool in = i < total && j != q;
-                    if (in) o = img_off_t<PER>(pi, A.sorted[j], cd, grid);
-                    const float d2 = fmaf(o.z, o.z, fmaf(o.y, o.y, o.x * o.x));
-                    bool cuts = in && d2 >= reach && d2 <= r_out2;
-                    if (!__any_sync(TFULL, cuts)) continue;
-                    float top = -FLT_MAX;
-#pragma unroll 2
-                    for (int k = 0; k < nf; ++k) {
-                        const float4 v = far[k];
-                        top = fmaxf(top, fmaf(o.x, v.x, fmaf(o.y, v.y, o.z * v.z)));
-                    }
-                    cuts = cuts && 0.5f * d2 - top <= band * sqrt_fast(d2);
-                    if (cuts)  // (the cell's own faces touch their vertices)
-                        for (int p = 0; p < np; ++p)
-                            if (h->src[p] == jj) cuts = false;
-                    const unsigned cm = __ballot_sync(TFULL, cuts);
-                    if (cuts) {
-                        const int at = ns + __popc(cm & ((1u << lane) - 1u));
-                        key[at] = d2;
-                        id[at] = jj;
-                    }
-                    ns += __popc(cm);
-                    if (ns > TRACE_KEEP) {
-                        more = true;
-                        ns = keep_nearest(key, id, ns, TRACE_KEEP, lane);
-                    }
-                }
-            }
-            end = lim2 >= all2;
-            if (!more) reach = lim2;  // (all of it is behind)
-        }
+        const int ns = walk<PER>(A, grid, q, pi, s_far[warp], nf, h->src, np, h->all2, h->band, TRACE_KEEP, reach,
+                                 s_key[warp], s_id[warp], cands);
         ++cells;
         if (ns > 0) {
-            ns = keep_nearest(key, id, ns, TRACE_KEEP, lane);
-            if (more) reach = key[ns - 1];  // what the next round need not look at again
-            if (lane < ns) h->src[np + lane] = id[lane];
+            if (lane < ns) h->src[np + lane] = s_id[warp][lane];
             if (lane == 0) {
                 h->np = np + ns;
                 h->reach = reach;
@@ -755,40 +1137,39 @@ __global__ void __launch_bounds__(CUT_BLOCK) k_cutters(const __grid_constant__ T
 constexpr int TRACE_BLOCK = 128;
 constexpr int TRACE_MINB = 5;
 
-template <typename Real, int NR, bool PER>
+// the lists' cells, or the cells sent back by the walk of the round before, by
+// groups of 8 lanes
+template <typename Real, bool PER>
 __global__ void __launch_bounds__(TRACE_BLOCK, (sizeof(Real) == 4 ? TRACE_MINB : 4)) k_trace(const __grid_constant__ TraceArgs A)
 {
-    constexpr int NP = NR * TT;
-    constexpr bool F64 = sizeof(Real) == 8;
-    // smallest |det| of a vertex's three unit normals, above the rounding of the
-    // rates of approach (worse vertices are left to the clipper)
-    constexpr float UNIT_MIN = F64 ? 2e-5f : 2e-4f;
-    using S = TraceSmem<Real, NP>;
+    constexpr int TT = 8, NR = 5, NV = 48;
+    using T = Tracer<Real, TT, NR, NV, PER>;
+    using S = typename T::S;
+    constexpr bool F64 = T::F64;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    const Sub G;
+    __shared__ int s_first;
+    const Sub<TT> G;
     const int gl = G.gl;
-    S& sm = *reinterpret_cast<S*>(smem_raw + (threadIdx.x / TT) * trace_stride<Real, NP>());
+    S& sm = *reinterpret_cast<S*>(smem_raw + (threadIdx.x / TT) * trace_stride<S>());
     int nq = (int)A.nq;
     if (A.nq_dev) {
         const int have = *A.nq_dev;
         nq = have < nq ? have : nq;
     }
     unsigned n_open = 0, n_second = 0;  // added once per group
-    __shared__ int s_first;
     for (;;) {
         if (threadIdx.x == 0) s_first = atomicAdd(A.queue, TRACE_BLOCK / TT);
         __syncthreads();
         const int c_block = s_first;
         if (c_block >= nq) break;
-        const int c4 = c_block + (threadIdx.x / 32) * TG;
-        const bool act = c4 + G.gi < nq;  // a group past the end repeats the last cell and writes nothing
-        const int c = act ? c4 + G.gi : nq - 1;
+        const int c0 = c_block + threadIdx.x / TT;
+        const bool act = c0 < nq;  // a group past the end repeats the last cell and writes nothing
+        const int c = act ? c0 : nq - 1;
         const int q = A.queries ? A.queries[c] : c;
         const GridDesc& grid = grid_of(A.g, A.sets, A.set_of, q);
         const float4 pi = A.sorted[q];
-        uint8_t* state = A.state + (size_t)q * A.state_stride;
-        // ---- planes: unit normals in registers, the planes themselves in shared memory
-        float nx[NR], ny[NR], nz[NR], nb[NR];
+        OpenCell* h = reinterpret_cast<OpenCell*>(A.state + (size_t)q * A.state_stride);
+        T t;
         int P;
         float reach;  // every generator with a float key below this was in the lists so far
         bool end = false;
@@ -801,12 +1182,11 @@ __global__ void __launch_bounds__(TRACE_BLOCK, (sizeof(Real) == 4 ? TRACE_MINB :
             P = 6 + A.kc;
             reach = (float)keys[A.kc - 1] * (F64 ? 1.0f - 1e-6f : 1.0f);  // (FP64 keys round)
         } else {
-            const OpenCell* h = reinterpret_cast<const OpenCell*>(state);
             srcs = h->src;
             P = h->np;
             reach = h->reach;
         }
-        const int rows = __reduce_max_sync(TFULL, (P + TT - 1) / TT);
+        t.rows = __reduce_max_sync(TFULL, (P + TT - 1) / TT);
 #pragma unroll
         for (int r = 0; r < NR; ++r) {
             const int p = r * TT + gl;
@@ -822,285 +1202,184 @@ __global__ void __launch_bounds__(TRACE_BLOCK, (sizeof(Real) == 4 ? TRACE_MINB :
                     }
                 }
             }
-            float x = 0.0f, y = 0.0f, z = 0.0f, b = 1.0f, len = 0.0f, inv = 0.0f;
-            if (src >= 0) {
-                const float3 o = img_off_t<PER>(pi, A.sorted[img_index_t<PER>(src)], img_code_t<PER>(src), grid);
-                x = o.x;
-                y = o.y;
-                z = o.z;
-                const float nn = x * x + y * y + z * z;
-                b = 0.5f * nn;
-                len = sqrt_fast(nn);
-                inv = rsqrt_fast(nn);
-            } else if (src != PAD_PLANE) {
-                const int w = -src - 1, axis = w >> 1, upper = w & 1;
-                const float one = upper ? 1.0f : -1.0f;
-                x = axis == 0 ? one : 0.0f;
-                y = axis == 1 ? one : 0.0f;
-                z = axis == 2 ? one : 0.0f;
-                const float pc = axis == 0 ? pi.x : (axis == 1 ? pi.y : pi.z);
-                b = PER ? (float)(0.5 * ((double)grid.hi[axis] - (double)grid.lo[axis]))
-                        : (upper ? grid.hi[axis] - pc : pc - grid.lo[axis]);
-                len = inv = 1.0f;
-            }
-            nx[r] = x * inv;
-            ny[r] = y * inv;
-            nz[r] = z * inv;
-            nb[r] = src != PAD_PLANE ? b * inv : FLT_MAX;
-            sm.pl[p] = make_float4(x, y, z, b);
-            sm.u.nl[p] = len;
-            sm.src[p] = src;
-            if constexpr (F64) {
-                if (src != PAD_PLANE) {
-                    const P64 d = plane64<PER>(src, A.sorted, pi, grid);
-                    sm.pn[p][0] = d.x;
-                    sm.pn[p][1] = d.y;
-                    sm.pn[p][2] = d.z;
-                    sm.ps[p] = src >= 0 ? 0.5 : d.b;  // b / |n|^2
-                }
-            }
+            t.set_plane(sm, r, p, src, pi, grid, A.sorted);
         }
         __syncwarp();
         const bool all = G.any(end);
-        const unsigned gen0 = G.ballot(sm.src[gl] >= 0);
-        bool ok = gen0 != 0;  // a nearest generator to start from
-        const int f0 = gen0 ? __ffs(gen0) - 1 : 0;
-        // ---- first vertex --------------------------------------------------
-        int V = 0;
-        int E = 0;
-        // open edge ends (an edge of ed without its second vertex; -1: free)
-        int r0 = -1, r1 = -1;
-        unsigned live = 0;
-        {
-            const float4 n0 = sm.pl[f0];
-            float vx = 0.5f * n0.x, vy = 0.5f * n0.y, vz = 0.5f * n0.z;
-            // a direction in plane f0: n0 x the axis it is least along
-            const float ax = fabsf(n0.x), ay = fabsf(n0.y), az = fabsf(n0.z);
-            float dx, dy, dz;
-            if (ax <= ay && ax <= az) { dx = 0.0f; dy = n0.z; dz = -n0.y; }
-            else if (ay <= az) { dx = -n0.z; dy = 0.0f; dz = n0.x; }
-            else { dx = n0.y; dy = -n0.x; dz = 0.0f; }
-            int f1 = f0, h = f0;
-#pragma unroll 1
-            for (int e = 0; e < 2; ++e) {
-                // (the second ray runs along f0 and f1: n0 x n1 ends at (f0, f1, h))
-                const uint32_t key = first_hit<NR>(nx, ny, nz, nb, rows, vx, vy, vz, dx, dy, dz,
-                                                   e == 0 ? 1e-3f * sm.u.nl[f0] : UNIT_MIN * sm.u.nl[f0] * sm.u.nl[f1], gl);
-                ok = ok && key < 0x7f800000u;
-                h = ok ? (int)(key & 63u) : f0;
-                const float4 nh = sm.pl[h];
-                const float t = (nh.w - (nh.x * vx + nh.y * vy + nh.z * vz)) * rcp_fast(nh.x * dx + nh.y * dy + nh.z * dz);
-                vx = fmaf(t, dx, vx);
-                vy = fmaf(t, dy, vy);
-                vz = fmaf(t, dz, vz);
-                if (e == 0) {
-                    f1 = h;
-                    dx = n0.y * nh.z - n0.z * nh.y;
-                    dy = n0.z * nh.x - n0.x * nh.z;
-                    dz = n0.x * nh.y - n0.y * nh.x;
-                }
-            }
-            if (gl == 0) {
-                sm.vp[0] = make_float4(vx, vy, vz, 0.0f);
-                *reinterpret_cast<uint32_t*>(sm.vid[0]) = (uint32_t)f0 | ((uint32_t)f1 << 8) | ((uint32_t)h << 16);
-            }
-            V = 1;
-            if (gl == 0) r0 = f0 | (f1 << 8);
-            if (gl == 1) r0 = f1 | (h << 8);
-            if (gl == 2) r0 = h | (f0 << 8);
-            live = 7u;
-        }
-        __syncwarp();
-        // ---- one ray per further vertex ------------------------------------
-        bool run = ok;
-#pragma unroll 1
-        while (__any_sync(TFULL, run)) {
-            // the lowest slot: new ends take the lowest free ones, so the newest go
-            // first (oldest first leaves more ends open: 1.7% of the cells of
-            // uniform points ran out of the slots, against 0.4%)
-            const int slot = __ffs(live) - 1;
-            const int got = G.bcast(slot < TT ? r0 : r1, slot & (TT - 1));
-            r0 = gl == slot ? -1 : r0;
-            r1 = gl + TT == slot ? -1 : r1;
-            const int ent = run ? got : 0;
-            const int a = ent & 0xff, b = (ent >> 8) & 0xff, w = ent >> 16;
-            const float4 v = sm.vp[w], na = sm.pl[a], nbp = sm.pl[b];
-            // the edge on a and b leaves (a, b, c) along n_b x n_a
-            const float dx = nbp.y * na.z - nbp.z * na.y, dy = nbp.z * na.x - nbp.x * na.z,
-                        dz = nbp.x * na.y - nbp.y * na.x;
-            const uint32_t key = first_hit<NR>(nx, ny, nz, nb, rows, v.x, v.y, v.z, dx, dy, dz,
-                                               UNIT_MIN * sm.u.nl[a] * sm.u.nl[b], gl);
-            if (key >= 0x7f800000u || V >= TRACE_V || E > TRACE_E - 3) {
-                ok = ok && !run;
-                run = false;
-            }
-            const int h = run ? (int)(key & 63u) : 0;
-            const float4 nh = sm.pl[h];
-            const float t = fmaf(-nh.x, v.x, fmaf(-nh.y, v.y, fmaf(-nh.z, v.z, nh.w))) *
-                            rcp_fast(fmaf(nh.x, dx, fmaf(nh.y, dy, nh.z * dz)));
-            // its other two edges, (a, h) and (h, b): close them against an open
-            // end of the same edge, (h, a) or (b, h), or leave them open
-            const int k1 = run ? h | (a << 8) : 0xfffe, k2 = run ? b | (h << 8) : 0xfffe;
-            const int e0 = r0 & 0xffff, e1 = r1 & 0xffff;
-            const bool p1 = e0 == k1, p2 = e0 == k2, q1 = e1 == k1, q2 = e1 == k2;
-            const bool c1 = G.any(p1 || q1), c2 = G.any(p2 || q2);
-            if (p1 || p2) {
-                sm.ed[E + (p1 ? 1 : 1 + c1)] = (uint32_t)r0 | ((uint32_t)V << 24);
-                r0 = -1;
-            }
-            if (q1 || q2) {
-                sm.ed[E + (q1 ? 1 : 1 + c1)] = (uint32_t)r1 | ((uint32_t)V << 24);
-                r1 = -1;
-            }
-            live = G.ballot(r0 >= 0) | (G.ballot(r1 >= 0) << TT);
-            if (run) {
-                if (gl == 0) {
-                    sm.vp[V] = make_float4(fmaf(t, dx, v.x), fmaf(t, dy, v.y), fmaf(t, dz, v.z), 0.0f);
-                    *reinterpret_cast<uint32_t*>(sm.vid[V]) = (uint32_t)b | ((uint32_t)a << 8) | ((uint32_t)h << 16);
-                    sm.ed[E] = (uint32_t)ent | ((uint32_t)V << 24);
-                }
-                // the lowest free slots take what stays open
-                const unsigned free1 = ~live;
-                const unsigned free2 = c1 ? free1 : free1 & (free1 - 1u);
-                const int s1 = c1 ? 31 : __ffs(free1) - 1, s2 = c2 ? 31 : __ffs(free2) - 1;
-                r0 = gl == s1 ? a | (h << 8) | (V << 16) : (gl == s2 ? h | (b << 8) | (V << 16) : r0);
-                r1 = gl + TT == s1 ? a | (h << 8) | (V << 16) : (gl + TT == s2 ? h | (b << 8) | (V << 16) : r1);
-                live |= (1u << s1) | (1u << s2);
-                if (live & 0x7fff0000u) ok = run = false;  // more open ends than slots
-                live &= 0xffffu;
-                E += 1 + c1 + c2;
-                ++V;
-                run = run && live != 0;
-            }
-            __syncwarp();
-        }
+        const unsigned gen0 = G.ballot(sm.src[gl] >= 0);  // the nearest generator's plane follows the walls
+        t.trace(G, sm, gen0 != 0, gen0 ? __ffs(gen0) - 1 : 0);
         __syncthreads();
-        // ---- vertices from their planes -------------------------------------
-        double R2d = 0.0;
-        float R2 = 0.0f, emax = 0.0f;
-        uint32_t fl = 0, fh = 0;  // the planes that are faces
-#pragma unroll 1
-        for (int s = gl; s < V; s += TT) {
-            const uint32_t ids = *reinterpret_cast<const uint32_t*>(sm.vid[s]);
-            const int a = ids & 0xff, b = (ids >> 8) & 0xff, cc = (ids >> 16) & 0xff;
-            fl |= (a < 32 ? 1u << a : 0u) | (b < 32 ? 1u << b : 0u) | (cc < 32 ? 1u << cc : 0u);
-            fh |= (a < 32 ? 0u : 1u << (a - 32)) | (b < 32 ? 0u : 1u << (b - 32)) | (cc < 32 ? 0u : 1u << (cc - 32));
-            const float4 p = sm.pl[a], o = sm.pl[b], h = sm.pl[cc];
-            const float bcx = o.y * h.z - o.z * h.y, bcy = o.z * h.x - o.x * h.z, bcz = o.x * h.y - o.y * h.x;
-            const float det = p.x * bcx + p.y * bcy + p.z * bcz;
-            // |det| of the unit normals: the vertex moves by (rounding) / this
-            const float unit = fabsf(det) * rcp_fast(sm.u.nl[a] * sm.u.nl[b] * sm.u.nl[cc]);
-            if (!(unit > UNIT_MIN)) ok = false;
-            float x, y, z, err;
-            if constexpr (F64) {
-                const double ax = sm.pn[a][0], ay = sm.pn[a][1], az = sm.pn[a][2];
-                const double bx = sm.pn[b][0], by = sm.pn[b][1], bz = sm.pn[b][2];
-                const double cx = sm.pn[cc][0], cy = sm.pn[cc][1], cz = sm.pn[cc][2];
-                const double ab = sm.ps[a] * (sm.src[a] < 0 ? 1.0 : (ax * ax + ay * ay) + az * az);
-                const double bb = sm.ps[b] * (sm.src[b] < 0 ? 1.0 : (bx * bx + by * by) + bz * bz);
-                const double cb = sm.ps[cc] * (sm.src[cc] < 0 ? 1.0 : (cx * cx + cy * cy) + cz * cz);
-                double dx = 0, dy = 0, dz = 0;
-                if (!solve3<double>(ax, ay, az, ab, bx, by, bz, bb, cx, cy, cz, cb, dx, dy, dz)) ok = false;
-                sm.v[s][0] = dx;
-                sm.v[s][1] = dy;
-                sm.v[s][2] = dz;
-                const double d = (dx * dx + dy * dy) + dz * dz;
-                R2d = d > R2d ? d : R2d;
-                x = (float)dx;
-                y = (float)dy;
-                z = (float)dz;
-                err = 1e-6f;  // float rounding of the position, of the plane and of the test
-            } else {
-                const float cax = h.y * p.z - h.z * p.y, cay = h.z * p.x - h.x * p.z, caz = h.x * p.y - h.y * p.x;
-                const float abx = p.y * o.z - p.z * o.y, aby = p.z * o.x - p.x * o.z, abz = p.x * o.y - p.y * o.x;
-                const float inv = rcp(det);
-                x = (p.w * bcx + o.w * cax + h.w * abx) * inv;
-                y = (p.w * bcy + o.w * cay + h.w * aby) * inv;
-                z = (p.w * bcz + o.w * caz + h.w * abz) * inv;
-                err = 1e-6f + 1.5e-6f * rcp_fast(unit);
-                if (unit < UNIT_F64) {  // ill-conditioned: float32 would lose digits
-                    if (!solve_vertex64<PER>(sm.src[a], sm.src[b], sm.src[cc], A.sorted, pi, grid, x, y, z)) ok = false;
-                    err = 1e-6f;
-                }
-            }
-            const float d = x * x + y * y + z * z;
-            if (!isfinite(d)) ok = false;
-            R2 = fmaxf(R2, d);
-            emax = fmaxf(emax, err);
-            sm.vp[s] = make_float4(x, y, z, err);
-        }
-        R2 = G.max(R2);
-        emax = G.max(emax);
-        if (F64) R2d = G.maxd(R2d);
-#pragma unroll
-        for (int o = TT / 2; o >= 1; o >>= 1) {
-            fl |= __shfl_xor_sync(TFULL, fl, o);
-            fh |= __shfl_xor_sync(TFULL, fh, o);
-        }
-        __syncwarp();
-        // ---- the certificate: every vertex clearly inside all planes but its three
-        const float R = sqrtf(R2);
-        {
-            int near = 0;
-            const int vmax = __reduce_max_sync(TFULL, ok ? V : 0);
-#pragma unroll 2
-            for (int s = 0; s < vmax; ++s) {
-                const float4 v = sm.vp[s];
-                const float thr = s < V ? v.w * R : -INFINITY;  // (other slots hold anything)
-                near += rows <= 3 ? near_rows<3>(nx, ny, nz, nb, v, thr) : near_rows<NR>(nx, ny, nz, nb, v, thr);
-            }
-            near = G.bcast(G.incl_scan(near), TT - 1);
-            ok = !G.any(!ok) && near == 3 * V && 2 * E == 3 * V;
-        }
-        // ---- security radius, and the generators beyond the list -------------
+        t.solve(G, sm, pi, grid, A.sorted, T::UNIT_F64);
+        t.certify(G, sm);
+        // security radius
         bool valid = all;
         if (A.round == 0 && !all)
-            valid = F64 ? 4.0 * R2d <= (double)keys[A.kc - 1] : 4.0f * R2 <= reach * (1.0f - 1e-5f);
-        const bool open = ok && !valid;
-        if (A.round == 0 && act && ok && gl == 0) {
+            valid = F64 ? 4.0 * t.R2d <= (double)keys[A.kc - 1] : 4.0f * t.R2 <= reach * (1.0f - 1e-5f);
+        const bool open = act && t.ok && !valid;
+        if (A.round == 0 && act && t.ok && gl == 0) {
             n_open += open;
             if (A.k_first > 0 && srcs[6 + A.k_first] >= 0)
-                n_second += F64 ? 4.0 * R2d > (double)keys[A.k_first] : 4.0f * R2 > (float)keys[A.k_first];
+                n_second += F64 ? 4.0 * t.R2d > (double)keys[A.k_first] : 4.0f * t.R2 > (float)keys[A.k_first];
         }
-        // ---- results: those of an open cell stand unless a generator beyond the
-        // list turns out to cut it
-        {
-            const int64_t out_idx = A.index_space == VT_INDEX_ORIGINAL ? (int64_t)__float_as_int(pi.w) : (int64_t)q;
-            trace_finish<Real, NP, PER>(sm, G, act && ok ? V : 0, fl, fh, R2, pi, out_idx, A);
-        }
-        append(A.slow_list, A.slow_ctr, act && !ok && gl == 0, q, G.lane);
-        if (__any_sync(TFULL, act && open)) {
-            append(A.open_list, A.open_ctr, act && open && gl == 0, q, G.lane);
-            OpenCell* h = reinterpret_cast<OpenCell*>(state);
-            const int F = __popc(fl) + __popc(fh);
-            if (act && open)
-                for (int i = gl; i < F; i += TT) h->src[i] = sm.src[nth_face(fl, fh, i)];
-            // the vertices beyond half the reach: a generator cuts a vertex v only
-            // from inside the ball of radius |v| around v
-            int nf = 0;
-            const int vmax = __reduce_max_sync(TFULL, act && open ? V : 0);
-            const float half = 0.25f * reach * (1.0f - 1e-4f);
-#pragma unroll 1
-            for (int s0 = 0; s0 < vmax; s0 += TT) {
-                const float4 v = sm.vp[s0 + gl];
-                const float d = v.x * v.x + v.y * v.y + v.z * v.z;
-                const bool far = act && open && s0 + gl < V && d >= half;
-                const unsigned m = G.ballot(far);
-                if (far) h->far[nf + __popc(m & ((1u << gl) - 1u))] = make_float4(v.x, v.y, v.z, d);
-                nf += __popc(m);
-            }
-            if (act && open && gl == 0) {
-                h->np = F;
-                h->nf = nf;
-                h->reach = reach;
-                h->all2 = 4.0f * R2 * (1.0f + 2e-5f);
-                h->band = emax * R;
-            }
+        // the results of an open cell stand unless a generator beyond the list
+        // turns out to cut it
+        const int64_t out_idx = A.index_space == VT_INDEX_ORIGINAL ? (int64_t)__float_as_int(pi.w) : (int64_t)q;
+        trace_finish<Real, TT, T::NP, NV, PER>(sm, G, act && t.ok ? t.V : 0, t.faces, t.R2, pi, out_idx, A);
+        const bool failed = act && !t.ok;
+        if (!__any_sync(TFULL, open || failed)) continue;
+        append(A.open_list, A.open_ctr, open && gl == 0, q, G.lane);
+        append(A.tail_list, A.tail_ctr, failed && gl == 0, q, G.lane);
+        // its faces, or all planes of a failed one
+        const int F = t.faces.count();
+        if (open)
+            for (int i = gl; i < F; i += TT) h->src[i] = sm.src[t.faces.nth(i)];
+        if (failed && A.round == 0)
+            for (int p = gl; p < P; p += TT) h->src[p] = sm.src[p];
+        const int nf = far_vertices<TT>(G, sm, open, t.V, reach, h->far);
+        if ((open || failed) && gl == 0) {
+            h->np = open ? F : P;
+            h->nf = nf;
+            // (a failed list that holds every other generator has no beyond)
+            h->reach = failed && all ? FLT_MAX : reach;
+            h->all2 = 4.0f * t.R2 * (1.0f + 2e-5f);
+            h->band = t.emax * t.R;
         }
         __syncwarp();
     }
     if (gl == 0 && n_open) atomicAdd(&A.st->n_open, (int)n_open);
     if (gl == 0 && n_second) atomicAdd(&A.st->n_second, (int)n_second);
+}
+
+// Whole cells by a warp each: traced, walked, and traced again with what cut
+// them until nothing does. The cells that k_trace failed or that are still cut
+// after its rounds, and every cell of a small call, whose time is the latency
+// of one cell: one launch where the rounds take five, and rays over three rows
+// of 32 planes instead of five of 8. A cell comes out the same bit for bit from
+// either kernel.
+constexpr int TAIL_BLOCK = 128;
+template <typename Real, bool PER>
+struct TailSmem {
+    typename Tracer<Real, 32, 3, 96, PER>::S t;
+    float4 far[96];
+    int32_t src[96];
+    float key[CUT_LIST];
+    int32_t id[CUT_LIST];
+};
+template <typename Real, bool PER>
+__global__ void __launch_bounds__(TAIL_BLOCK, 4) k_trace_tail(const __grid_constant__ TraceArgs A)
+{
+    constexpr int TT = 32, NR = 3, NV = 96;
+    using T = Tracer<Real, TT, NR, NV, PER>;
+    constexpr bool F64 = T::F64;
+    static_assert(NV / 2 + 2 + TRACE_KEEP <= T::NP && NV / 2 + 2 <= REC_FACES && NV <= REC_VERTS, "capacities");
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const Sub<TT> G;
+    const int lane = G.lane;
+    TailSmem<Real, PER>& m = reinterpret_cast<TailSmem<Real, PER>*>(smem_raw)[threadIdx.x / 32];
+    int nq = (int)A.nq;
+    if (A.nq_dev) {
+        const int have = *A.nq_dev;
+        nq = have < nq ? have : nq;
+    }
+    unsigned walks = 0, cands = 0, n_open = 0, n_second = 0;
+    for (;;) {
+        int c = 0;
+        if (lane == 0) c = atomicAdd(A.queue, 1);
+        c = __shfl_sync(TFULL, c, 0);
+        if (c >= nq) break;
+        const int q = A.queries ? A.queries[c] : c;
+        const GridDesc& grid = grid_of(A.g, A.sets, A.set_of, q);
+        const float4 pi = A.sorted[q];
+        const OpenCell* h = reinterpret_cast<const OpenCell*>(A.state + (size_t)q * A.state_stride);
+        int P;
+        float reach;
+        bool all = false;
+        const Real* keys = nullptr;
+        if (A.round == 0) {
+            const int64_t li = (int64_t)c * A.kstride;
+            keys = reinterpret_cast<const Real*>(A.d2) + li;
+            P = 6 + A.kc;
+            reach = (float)keys[A.kc - 1] * (F64 ? 1.0f - 1e-6f : 1.0f);
+            bool end = false;
+            for (int p = lane; p < P; p += TT) {
+                int src = p < 6 ? -(p + 1) : A.nbr[li + p - 6];
+                if (p >= 6 && src < 0) {
+                    src = PAD_PLANE;
+                    end = true;
+                }
+                m.src[p] = src;
+            }
+            all = __any_sync(TFULL, end);
+        } else {
+            P = h->np;
+            reach = h->reach;
+            all = reach == FLT_MAX;
+            for (int p = lane; p < P; p += TT) m.src[p] = h->src[p];
+        }
+        __syncwarp();
+        T t;
+        t.rows = NR;
+        bool done = false;
+        // (every turn adds a generator that cuts; the bound only ends what float
+        // round-off could keep turning)
+#pragma unroll 1
+        for (int turn = 0; turn < 200 && !done; ++turn) {
+#pragma unroll
+            for (int r = 0; r < NR; ++r) {
+                const int p = r * TT + lane;
+                t.set_plane(m.t, r, p, p < P ? m.src[p] : PAD_PLANE, pi, grid, A.sorted);
+            }
+            __syncwarp();
+            const unsigned gen0 = G.ballot(m.t.src[lane] >= 0);
+            t.trace(G, m.t, gen0 != 0, gen0 ? __ffs(gen0) - 1 : 0);
+            const bool traced = t.ok;
+            t.solve(G, m.t, pi, grid, A.sorted, T::UNIT_F64);
+            t.certify(G, m.t);
+            if (!t.ok && traced) {
+                t.ok = true;
+                t.solve(G, m.t, pi, grid, A.sorted, T::UNIT_F64_AGAIN);
+                t.certify64(G, m.t, pi, grid, A.sorted);
+            }
+            if (!t.ok) break;
+            bool valid = all;
+            if (A.round == 0 && turn == 0) {
+                if (!all) valid = F64 ? 4.0 * t.R2d <= (double)keys[A.kc - 1] : 4.0f * t.R2 <= reach * (1.0f - 1e-5f);
+                n_open += !valid;
+                if (A.k_first > 0 && m.t.src[6 + A.k_first] >= 0)
+                    n_second += F64 ? 4.0 * t.R2d > (double)keys[A.k_first] : 4.0f * t.R2 > (float)keys[A.k_first];
+            }
+            const float all2 = 4.0f * t.R2 * (1.0f + 2e-5f);
+            if (!valid && all2 > reach) {
+                const int F = t.faces.count();
+                const int nf = far_vertices<TT>(G, m.t, true, t.V, reach, m.far);
+                __syncwarp();
+                if (turn == 0 && A.round == 0) ++walks;
+                const int ns = walk<PER>(A, grid, q, pi, m.far, nf, m.t.src, P, all2, t.emax * t.R, TRACE_KEEP, reach,
+                                         m.key, m.id, cands);
+                if (ns > 0) {
+                    __syncwarp();
+                    for (int i = lane; i < F; i += TT) m.src[i] = m.t.src[t.faces.nth(i)];
+                    if (lane < ns) m.src[F + lane] = m.id[lane];
+                    P = F + ns;
+                    __syncwarp();
+                    continue;
+                }
+            }
+            done = true;
+        }
+        const int64_t out_idx = A.index_space == VT_INDEX_ORIGINAL ? (int64_t)__float_as_int(pi.w) : (int64_t)q;
+        if (done)
+            trace_finish<Real, TT, T::NP, NV, PER>(m.t, G, t.V, t.faces, t.R2, pi, out_idx, A);
+        else if (lane == 0)
+            A.slow_list[atomicAdd(A.slow_ctr, 1)] = q;
+        __syncwarp();
+    }
+    if (lane == 0) {
+        if (walks) atomicAdd(&A.st->walk_cells, (unsigned long long)walks);
+        if (cands) atomicAdd(&A.st->walk_cands, (unsigned long long)cands);
+        if (n_open) atomicAdd(&A.st->n_open, (int)n_open);
+        if (n_second) atomicAdd(&A.st->n_second, (int)n_second);
+    }
 }
 
 // as many blocks as are resident at once (they take cells from the queue)
@@ -1118,15 +1397,23 @@ cudaError_t resident_blocks(K kern, int block, size_t smem, int64_t cells, int p
     return cudaSuccess;
 }
 
-template <typename Real, int NR>
+template <typename Real>
 cudaError_t launch_trace_t(const TraceArgs& a, cudaStream_t s)
 {
-    const size_t smem = trace_stride<Real, NR * TT>() * (TRACE_BLOCK / TT);
-    auto kern = a.g.periodic ? k_trace<Real, NR, true> : k_trace<Real, NR, false>;
     unsigned blocks = 1;
-    const cudaError_t e = resident_blocks(kern, TRACE_BLOCK, smem, a.nq, TRACE_BLOCK / TT, blocks);
-    if (e != cudaSuccess) return e;
-    kern<<<blocks, TRACE_BLOCK, smem, s>>>(a);
+    if (a.tail) {
+        auto kern = a.g.periodic ? k_trace_tail<Real, true> : k_trace_tail<Real, false>;
+        const size_t smem = sizeof(TailSmem<Real, false>) * (TAIL_BLOCK / 32);
+        const cudaError_t e = resident_blocks(kern, TAIL_BLOCK, smem, a.nq, TAIL_BLOCK / 32, blocks);
+        if (e != cudaSuccess) return e;
+        kern<<<blocks, TAIL_BLOCK, smem, s>>>(a);
+    } else {
+        auto kern = a.g.periodic ? k_trace<Real, true> : k_trace<Real, false>;
+        const size_t smem = trace_stride<typename Tracer<Real, 8, 5, 48, false>::S>() * (TRACE_BLOCK / 8);
+        const cudaError_t e = resident_blocks(kern, TRACE_BLOCK, smem, a.nq, TRACE_BLOCK / 8, blocks);
+        if (e != cudaSuccess) return e;
+        kern<<<blocks, TRACE_BLOCK, smem, s>>>(a);
+    }
     count_launch();
     return cudaGetLastError();
 }

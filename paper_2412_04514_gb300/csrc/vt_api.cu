@@ -488,13 +488,19 @@ bool traced_pass(const vt_params* p, const Layout& L, int kl)
     return L.state_stride > 0 && kl >= 12 && 2 * kl > p->k_max;
 }
 
+// point counts up to which every cell goes to the warp-per-cell kernel at once
+#ifndef VT_TRACE_SMALL
+#define VT_TRACE_SMALL 16384
+#endif
+constexpr int64_t TRACE_SMALL = VT_TRACE_SMALL;
+
 // The list pass over all n cells by edge tracing: kNN with k_list entries,
-// the lists' cells, further rounds for the cells that farther generators cut,
-// and the plane-by-plane clipper for the cells whose certificate failed or that
-// are still cut after the last round. Every count stays on the device. open,
-// next: scratch lists of n cells, free after the pass.
+// two rounds of groups of 8 lanes and the walk, a warp per cell for what they
+// leave, and the plane-by-plane clipper for the cells whose certificate failed
+// there too. Every count stays on the device. slow, open, next, tail: lists of n
+// cells, scratch of the pass (slow until its clipper launch).
 int trace_pass(const Ctx& c, const vt_params* p, int64_t n, int k, int k_list, int variant, vt_cells_out* out,
-               int32_t* slow, int32_t* open, int32_t* next, int32_t* fail_next, int32_t* ctr_next,
+               int32_t* slow, int32_t* open, int32_t* next, int32_t* tail, int32_t* fail_next, int32_t* ctr_next,
                int32_t* fail_robust, int32_t* ctr_robust)
 {
     const Layout& L = c.L;
@@ -533,14 +539,18 @@ int trace_pass(const Ctx& c, const vt_params* p, int64_t n, int k, int k_list, i
     a.slow_list = slow;
     a.slow_ctr = ctr + CTR_SLOW;
     a.st = c.st;
-    for (int round = 0; round < TRACE_ROUNDS; ++round) {
+    const bool small = n <= TRACE_SMALL;
+    for (int round = 0; !small && round < TRACE_ROUNDS; ++round) {
         // the cells (all, or those the walk before sent back), then the walk over
         // the open ones among them
+        const bool last = round == TRACE_ROUNDS - 1;
         a.round = round;
         a.queries = round == 0 ? nullptr : next;
         a.nq_dev = round == 0 ? nullptr : &ctr[CTR_TRACE + 2 * round - 1];
         a.open_list = open;
         a.open_ctr = &ctr[CTR_TRACE + 2 * round];
+        a.tail_list = tail;
+        a.tail_ctr = &ctr[CTR_TAIL];
         a.queue = &ctr[CTR_TQUEUE + 2 * round];
         T.begin(StageTimer::CLIP);
         e = launch_trace(a, p->precision, c.s);
@@ -549,8 +559,8 @@ int trace_pass(const Ctx& c, const vt_params* p, int64_t n, int k, int k_list, i
         if (e != cudaSuccess) return cuda_fail(e, "trace launch");
         a.queries = open;
         a.nq_dev = a.open_ctr;
-        a.next_list = round == TRACE_ROUNDS - 1 ? slow : next;
-        a.next_ctr = round == TRACE_ROUNDS - 1 ? a.slow_ctr : &ctr[CTR_TRACE + 2 * round + 1];
+        a.next_list = last ? tail : next;
+        a.next_ctr = last ? &ctr[CTR_TAIL] : &ctr[CTR_TRACE + 2 * round + 1];
         a.queue = &ctr[CTR_TQUEUE + 2 * round + 1];
         T.begin(StageTimer::KNN);
         e = launch_cutters(a, c.s);
@@ -558,6 +568,16 @@ int trace_pass(const Ctx& c, const vt_params* p, int64_t n, int k, int k_list, i
         if (c.knn_launches) ++*c.knn_launches;
         if (e != cudaSuccess) return cuda_fail(e, "walk launch");
     }
+    a.round = small ? 0 : TRACE_ROUNDS;
+    a.tail = 1;
+    a.queries = small ? nullptr : tail;
+    a.nq_dev = small ? nullptr : &ctr[CTR_TAIL];
+    a.queue = &ctr[CTR_TQUEUE + 2 * TRACE_ROUNDS];
+    T.begin(StageTimer::CLIP);
+    e = launch_trace(a, p->precision, c.s);
+    T.end();
+    if (c.clip_launches) ++*c.clip_launches;
+    if (e != cudaSuccess) return cuda_fail(e, "trace launch");
     return clip_pass(c, p, slow, n, ctr + CTR_SLOW, k, false, 0, variant, p->precision, out, fail_next, ctr_next, fail_robust,
                      ctr_robust, k_list, true, k_list > k ? k_list : 0);
 }
@@ -828,7 +848,7 @@ int tessellate_run(Ctx& c, const float* pts, int64_t n, const vt_params* p, vt_c
                 r = range_pass(c, p, q, n, qn, k_prev, variant_reg, out, regl[(pi + 1) % 2], &ctr_reg[pi], rob_new,
                                &ctr_new[pi], unval, &c.st->n_unval);
             else if (pi == 0 && !last && traced_pass(p, L, kk))
-                r = trace_pass(c, p, n, merged ? p->k0 : kk, kk, variant_reg, out, regl[0], robl[0], robl[1], rn,
+                r = trace_pass(c, p, n, merged ? p->k0 : kk, kk, variant_reg, out, regl[0], robl[0], robl[1], rob64, rn,
                                rc, rob_new, &ctr_new[pi]);
             else
                 r = clip_pass(c, p, q, n, qn, merged ? p->k0 : kk, last, k_prev, variant_reg, p->precision, out, rn,
@@ -895,7 +915,7 @@ int tessellate_run(Ctx& c, const float* pts, int64_t n, const vt_params* p, vt_c
                                rob_new, &c.st->n_fail_robust, unval + n_unval, &c.st->n_fail_next);
             else if (implicit && !exhaustive && traced_pass(p, L, merged ? 2 * kk : kk))
                 r = trace_pass(c, p, m_reg, kk, merged ? 2 * kk : kk, variant_reg, out, reg_cur, rob_cur, rob_nxt,
-                               reg_nxt, &c.st->n_fail_next, rob_new, &c.st->n_fail_robust);
+                               rob64, reg_nxt, &c.st->n_fail_next, rob_new, &c.st->n_fail_robust);
             else
                 // the first two list passes (k and 2 k) run as one launch over
                 // the 2 k list when 2 k <= k_max: a cell the first k entries

@@ -552,11 +552,12 @@ enum : int8_t { CELL_DONE = 0, CELL_NEED_K = 1, CELL_NEED_ROBUST = 2, CELL_UNVAL
 constexpr int CTR_QUEUE = 4 * VT_MAX_PASSES + 4;
 // the traced pass: the lists of its rounds, and the cells left to the
 // plane-by-plane clipper
-constexpr int TRACE_ROUNDS = 4;
+constexpr int TRACE_ROUNDS = 2;
 constexpr int CTR_TRACE = CTR_QUEUE + 1;            // open and next list of each round
-constexpr int CTR_SLOW = CTR_TRACE + 2 * TRACE_ROUNDS;
+constexpr int CTR_TAIL = CTR_TRACE + 2 * TRACE_ROUNDS - 1;  // (the last next list)
+constexpr int CTR_SLOW = CTR_TAIL + 1;
 constexpr int CTR_TQUEUE = CTR_SLOW + 1;            // a cell counter per launch of the pass
-constexpr int CTR_COUNT = CTR_TQUEUE + 2 * TRACE_ROUNDS;
+constexpr int CTR_COUNT = CTR_TQUEUE + 2 * TRACE_ROUNDS + 1;
 
 struct Layout {
     int G;
@@ -675,7 +676,8 @@ struct TraceArgs {
     const void* d2;
     int kstride, kc;
     int k_first;              // > 0: count the cells still open at this entry (statistics)
-    int round;                // 0: lists; > 0: the planes left by the round before
+    int round;                // 0: lists; > 0: the planes in the cells' state slots
+    int tail;                 // 1: a warp per cell, until nothing cuts it
     int emit, index_space, rec_f32;
     double *vol, *cen, *m2;
     uint8_t* rec;
@@ -684,6 +686,7 @@ struct TraceArgs {
     size_t state_stride;
     int32_t *open_list, *open_ctr;  // cells the walk has to look at
     int32_t *next_list, *next_ctr;  // cells to build again (the walk's output)
+    int32_t *tail_list, *tail_ctr;  // cells that failed: for the warp per cell
     int32_t *slow_list, *slow_ctr;  // cells for the plane-by-plane clipper
     DevStatus* st;
     int32_t* queue;           // the launch's cell counter (zero)
