@@ -137,7 +137,7 @@ struct TraceReal<double, NP, NV> {
 template <typename Real, int NP, int NV>
 struct alignas(16) TraceSmem : TraceReal<Real, NP, NV> {
     float4 pl[NP];       // n, b of n.x <= b
-    float4 vp[NV];       // position; its error bound relative to R
+    float4 vp[NV];       // position; a bound of its error and that of a plane test, as a length
     int32_t src[NP];     // sorted index (with image code), -1..-6 walls, PAD_PLANE
     uint8_t vid[NV][4];  // planes (ccw from outside)
     // edges: planes a | b << 8, vertices s << 16 | t << 24; (a, b) follow one
@@ -160,15 +160,16 @@ constexpr size_t trace_stride()
 // FP64 position of the vertex of three planes (out of line: rarely needed)
 template <bool PER>
 __device__ VT_RARE bool solve_vertex64(int a, int b, int c, const float4* __restrict__ sorted, float4 pi,
-                                       const GridDesc& grid, float& x, float& y, float& z)
+                                       const GridDesc& grid, double& x, double& y, double& z)
 {
-    double dx = 0, dy = 0, dz = 0;
-    const bool ok = vertex64(plane64<PER>(a, sorted, pi, grid), plane64<PER>(b, sorted, pi, grid),
-                             plane64<PER>(c, sorted, pi, grid), dx, dy, dz);
-    x = (float)dx;
-    y = (float)dy;
-    z = (float)dz;
-    return ok;
+    x = y = z = 0.0;
+    return vertex64(plane64<PER>(a, sorted, pi, grid), plane64<PER>(b, sorted, pi, grid),
+                    plane64<PER>(c, sorted, pi, grid), x, y, z);
+}
+// the low halves of a position in FP64 beside its float32 value
+__device__ __forceinline__ float4 low_half(double x, double y, double z)
+{
+    return make_float4((float)(x - (double)(float)x), (float)(y - (double)(float)y), (float)(z - (double)(float)z), 0.0f);
 }
 
 // a set of planes
@@ -210,6 +211,18 @@ struct Faces {
     }
 };
 
+// mask of a group's open edge ends
+template <int TT>
+struct LiveMask {
+    using T = uint32_t;
+};
+template <>
+struct LiveMask<32> {
+    using T = uint64_t;
+};
+__device__ __forceinline__ int lowest(uint32_t x) { return __ffs(x) - 1; }
+__device__ __forceinline__ int lowest(uint64_t x) { return __ffsll((long long)x) - 1; }
+
 // One cell per group of TT lanes: its planes (unit normals in registers, plane
 // r * TT + lane in row r), then its polyhedron in shared memory. Every member
 // is called by the whole warp; groups without work pass through.
@@ -220,19 +233,20 @@ struct Tracer {
     static constexpr int NE = 3 * NV / 2;
     using S = TraceSmem<Real, NP, NV>;
     // smallest |det| of a vertex's three unit normals, above the rounding of the
-    // rates of approach (worse vertices are left to the clipper)
-    static constexpr float UNIT_MIN = F64 ? 2e-5f : 2e-4f;
-    // below this |det| the FP32 form solves a vertex in FP64 (about 1 vertex in
-    // 3,000), and below the other when a cell's error bounds failed it
-    static constexpr float UNIT_F64 = 1e-2f, UNIT_F64_AGAIN = 0.3f;
-    static constexpr int SR = TT == 8 ? 2 : 1;       // registers of open edge ends per lane
-    static constexpr int SLOTS = TT == 32 ? 31 : SR * TT;  // (bit 31 marks a closed edge)
+    // rates of approach in float32, and in FP64
+    static constexpr float UNIT_MIN = F64 ? 2e-5f : 2e-4f, UNIT_MIN64 = 1e-7f;
+    // below this |det| the FP32 form solves a vertex in FP64 (about 1 in 3,000)
+    static constexpr float UNIT_F64 = 1e-2f;
+    static constexpr int SR = 2;                     // registers of open edge ends per lane
+    using Live = typename LiveMask<TT>::T;           // a bit per slot; the top bit marks a closed edge
+    static constexpr int CLOSED = 8 * sizeof(Live) - 1;
+    static constexpr int SLOTS = SR * TT < CLOSED ? SR * TT : CLOSED;
 
     float nx[NR], ny[NR], nz[NR], nb[NR];
     int rows;               // rows of planes in use over the warp
     bool ok;
     int V, E;
-    float R2, R, emax;      // max |v|^2, its root, largest error bound relative to R
+    float R2;               // max |v|^2
     double R2d;
     Faces<(NP + 31) / 32> faces;  // the planes that are faces
 
@@ -331,10 +345,40 @@ struct Tracer {
         }
     }
 
-    // vertices (as triples of planes) and edges, one ray per vertex. f0: the
-    // plane of the nearest generator; on: the group has a cell
-    __device__ __forceinline__ void trace(const Sub<TT>& G, S& sm, bool on, int f0)
+    // the first plane met in FP64 (a warp per cell, its planes (n, b) in pd): for
+    // cells whose far walls leave float32 positions too coarse for the near planes
+    __device__ __forceinline__ int first_hit64(const S& sm, const double (*pd)[4], double vx, double vy, double vz,
+                                               double dx, double dy, double dz, float least) const
     {
+        const int lane = threadIdx.x & 31;
+        uint32_t key = 0xffffffffu;
+        int row = 0;
+#pragma unroll
+        for (int r = 0; r < NR; ++r) {
+            const int p = r * TT + lane;
+            const double* h = pd[p];
+            const float s = (float)(h[3] - ((h[0] * vx + h[1] * vy) + h[2] * vz));
+            const float nd = (float)((h[0] * dx + h[1] * dy) + h[2] * dz);
+            const uint32_t k = __float_as_uint(s * rcp_fast(nd));
+            const bool take = nd > least * sm.u.nl[p] && k < key;  // (no plane: nd = 0)
+            key = take ? k : key;
+            row = take ? r : row;
+        }
+        const uint32_t first = __reduce_min_sync(TFULL, key);
+        const int from = __ffs(__ballot_sync(TFULL, key == first)) - 1;
+        row = __shfl_sync(TFULL, row, from);
+        return first < 0x7f800000u ? row * TT + from : -1;
+    }
+
+    // vertices (as triples of planes) and edges, one ray per vertex. f0: the
+    // plane of the nearest generator; on: the group has a cell. W: the rays'
+    // arithmetic (double: a warp per cell, its planes in pd; lo holds the low
+    // halves of the positions)
+    template <typename W>
+    __device__ __forceinline__ void trace(const Sub<TT>& G, S& sm, bool on, int f0, const double (*pd)[4], float4* lo)
+    {
+        constexpr bool DBL = sizeof(W) == 8;
+        constexpr float LEAST = DBL ? UNIT_MIN64 : UNIT_MIN;
         const int gl = G.gl;
         ok = on;
         V = 1;
@@ -342,45 +386,82 @@ struct Tracer {
         int o[SR];  // open edge ends (an edge of ed without its second vertex; -1: free)
 #pragma unroll
         for (int i = 0; i < SR; ++i) o[i] = -1;
+        auto plane = [&](int p, W& x, W& y, W& z, W& b) {
+            if constexpr (DBL) {
+                x = pd[p][0];
+                y = pd[p][1];
+                z = pd[p][2];
+                b = pd[p][3];
+            } else {
+                const float4 h = sm.pl[p];
+                x = h.x;
+                y = h.y;
+                z = h.z;
+                b = h.w;
+            }
+        };
+        auto hit_of = [&](W vx, W vy, W vz, W dx, W dy, W dz, float least) {
+            if constexpr (DBL) return first_hit64(sm, pd, vx, vy, vz, dx, dy, dz, least);
+            else return first_hit(G, vx, vy, vz, dx, dy, dz, least);
+        };
+        // v + t d on plane h
+        auto advance = [&](W& vx, W& vy, W& vz, W dx, W dy, W dz, int h) {
+            W hx, hy, hz, hb;
+            plane(h, hx, hy, hz, hb);
+            const W s = hb - (hx * vx + hy * vy + hz * vz), nd = hx * dx + hy * dy + hz * dz;
+            W t;
+            if constexpr (DBL) {  // (one Newton step from float32: 1e-13)
+                const double r = rcp_fast((float)nd);
+                t = s * r;
+                t += (s - t * nd) * r;
+            } else {
+                t = s * rcp_fast(nd);
+            }
+            vx += t * dx;
+            vy += t * dy;
+            vz += t * dz;
+        };
+        auto put = [&](int s, W x, W y, W z) {
+            sm.vp[s] = make_float4((float)x, (float)y, (float)z, 0.0f);
+            if constexpr (DBL) lo[s] = low_half(x, y, z);
+        };
         {
-            const float4 n0 = sm.pl[f0];
-            float vx = 0.5f * n0.x, vy = 0.5f * n0.y, vz = 0.5f * n0.z;
+            W n0x, n0y, n0z, n0b;
+            plane(f0, n0x, n0y, n0z, n0b);
+            W vx = (W)0.5 * n0x, vy = (W)0.5 * n0y, vz = (W)0.5 * n0z;
             // a direction in plane f0: n0 x the axis it is least along
-            const float ax = fabsf(n0.x), ay = fabsf(n0.y), az = fabsf(n0.z);
-            float dx, dy, dz;
-            if (ax <= ay && ax <= az) { dx = 0.0f; dy = n0.z; dz = -n0.y; }
-            else if (ay <= az) { dx = -n0.z; dy = 0.0f; dz = n0.x; }
-            else { dx = n0.y; dy = -n0.x; dz = 0.0f; }
+            const W ax = n0x < 0 ? -n0x : n0x, ay = n0y < 0 ? -n0y : n0y, az = n0z < 0 ? -n0z : n0z;
+            W dx, dy, dz;
+            if (ax <= ay && ax <= az) { dx = 0; dy = n0z; dz = -n0y; }
+            else if (ay <= az) { dx = -n0z; dy = 0; dz = n0x; }
+            else { dx = n0y; dy = -n0x; dz = 0; }
             int f1 = f0, h = f0;
 #pragma unroll 1
             for (int e = 0; e < 2; ++e) {
                 // (the second ray runs along f0 and f1: n0 x n1 ends at (f0, f1, h))
-                const int hit = first_hit(G, vx, vy, vz, dx, dy, dz,
-                                          e == 0 ? 1e-3f * sm.u.nl[f0] : UNIT_MIN * sm.u.nl[f0] * sm.u.nl[f1]);
+                const int hit = hit_of(vx, vy, vz, dx, dy, dz,
+                                       e == 0 ? 1e-3f * sm.u.nl[f0] : LEAST * sm.u.nl[f0] * sm.u.nl[f1]);
                 ok = ok && hit >= 0;
                 h = ok ? hit : f0;
-                const float4 nh = sm.pl[h];
-                const float t = (nh.w - (nh.x * vx + nh.y * vy + nh.z * vz)) *
-                                rcp_fast(nh.x * dx + nh.y * dy + nh.z * dz);
-                vx = fmaf(t, dx, vx);
-                vy = fmaf(t, dy, vy);
-                vz = fmaf(t, dz, vz);
+                advance(vx, vy, vz, dx, dy, dz, h);
                 if (e == 0) {
                     f1 = h;
-                    dx = n0.y * nh.z - n0.z * nh.y;
-                    dy = n0.z * nh.x - n0.x * nh.z;
-                    dz = n0.x * nh.y - n0.y * nh.x;
+                    W hx, hy, hz, hb;
+                    plane(h, hx, hy, hz, hb);
+                    dx = n0y * hz - n0z * hy;
+                    dy = n0z * hx - n0x * hz;
+                    dz = n0x * hy - n0y * hx;
                 }
             }
             if (gl == 0) {
-                sm.vp[0] = make_float4(vx, vy, vz, 0.0f);
+                put(0, vx, vy, vz);
                 *reinterpret_cast<uint32_t*>(sm.vid[0]) = (uint32_t)f0 | ((uint32_t)f1 << 8) | ((uint32_t)h << 16);
             }
             if (gl == 0) o[0] = f0 | (f1 << 8);
             if (gl == 1) o[0] = f1 | (h << 8);
             if (gl == 2) o[0] = h | (f0 << 8);
         }
-        unsigned live = 7u;
+        Live live = 7u;
         __syncwarp();
         bool run = ok;
 #pragma unroll 1
@@ -388,25 +469,35 @@ struct Tracer {
             // the lowest slot: new ends take the lowest free ones, so the newest go
             // first (oldest first leaves more ends open: 1.7% of the cells of
             // uniform points ran out of 16 slots, against 0.4%)
-            const int slot = __ffs(live) - 1;
-            const int got = G.bcast(SR == 1 || slot < TT ? o[0] : o[SR - 1], slot & (TT - 1));
+            const int slot = lowest(live);
+            const int got = G.bcast(slot < TT ? o[0] : o[1], slot & (TT - 1));
 #pragma unroll
             for (int i = 0; i < SR; ++i) o[i] = gl + i * TT == slot ? -1 : o[i];
             const int ent = run ? got : 0;
             const int a = ent & 0xff, b = (ent >> 8) & 0xff, w = ent >> 16;
-            const float4 v = sm.vp[w], na = sm.pl[a], nbp = sm.pl[b];
+            W vx, vy, vz, ax, ay, az, bx, by, bz, unused;
+            {
+                const float4 v = sm.vp[w];
+                vx = v.x;
+                vy = v.y;
+                vz = v.z;
+                if constexpr (DBL) {
+                    vx += (double)lo[w].x;
+                    vy += (double)lo[w].y;
+                    vz += (double)lo[w].z;
+                }
+            }
+            plane(a, ax, ay, az, unused);
+            plane(b, bx, by, bz, unused);
             // the edge on a and b leaves (a, b, c) along n_b x n_a
-            const float dx = nbp.y * na.z - nbp.z * na.y, dy = nbp.z * na.x - nbp.x * na.z,
-                        dz = nbp.x * na.y - nbp.y * na.x;
-            const int hit = first_hit(G, v.x, v.y, v.z, dx, dy, dz, UNIT_MIN * sm.u.nl[a] * sm.u.nl[b]);
+            const W dx = by * az - bz * ay, dy = bz * ax - bx * az, dz = bx * ay - by * ax;
+            const int hit = hit_of(vx, vy, vz, dx, dy, dz, LEAST * sm.u.nl[a] * sm.u.nl[b]);
             if (hit < 0 || V >= NV || E > NE - 3) {
                 ok = ok && !run;
                 run = false;
             }
             const int h = run ? hit : 0;
-            const float4 nh = sm.pl[h];
-            const float t = fmaf(-nh.x, v.x, fmaf(-nh.y, v.y, fmaf(-nh.z, v.z, nh.w))) *
-                            rcp_fast(fmaf(nh.x, dx, fmaf(nh.y, dy, nh.z * dz)));
+            advance(vx, vy, vz, dx, dy, dz, h);
             // the vertex (b, a, h): its other two edges, (a, h) and (h, b), close
             // against an open end of the same edge, (h, a) or (b, h), or stay open
             const int k1 = run ? h | (a << 8) : 0xfffe, k2 = run ? b | (h << 8) : 0xfffe;
@@ -425,24 +516,23 @@ struct Tracer {
                     o[i] = -1;
                 }
             }
-            if (SR == 1) live = G.ballot(o[0] >= 0);
-            else live = G.ballot(o[0] >= 0) | (G.ballot(o[SR - 1] >= 0) << (TT & 31));
+            live = (Live)G.ballot(o[0] >= 0) | ((Live)G.ballot(o[1] >= 0) << TT);
             if (run) {
                 if (gl == 0) {
-                    sm.vp[V] = make_float4(fmaf(t, dx, v.x), fmaf(t, dy, v.y), fmaf(t, dz, v.z), 0.0f);
+                    put(V, vx, vy, vz);
                     *reinterpret_cast<uint32_t*>(sm.vid[V]) = (uint32_t)b | ((uint32_t)a << 8) | ((uint32_t)h << 16);
                     sm.ed[E] = (uint32_t)ent | ((uint32_t)V << 24);
                 }
                 // the lowest free slots take what stays open
-                const unsigned free1 = ~live, free2 = c1 ? free1 : free1 & (free1 - 1u);
-                const int s1 = c1 ? 31 : __ffs(free1) - 1, s2 = c2 ? 31 : __ffs(free2) - 1;
+                const Live free1 = ~live, free2 = c1 ? free1 : free1 & (free1 - 1u);
+                const int s1 = c1 ? CLOSED : lowest(free1), s2 = c2 ? CLOSED : lowest(free2);
 #pragma unroll
                 for (int i = 0; i < SR; ++i) {
                     const int at = gl + i * TT;
                     o[i] = at == s1 ? a | (h << 8) | (V << 16) : (at == s2 ? h | (b << 8) | (V << 16) : o[i]);
                 }
                 if ((!c1 && s1 >= SLOTS) || (!c2 && (unsigned)s2 >= (unsigned)SLOTS)) ok = run = false;
-                live = (live | (1u << s1) | (1u << (s2 & 31))) & ((1u << SLOTS) - 1u);
+                live = (live | ((Live)1 << s1) | ((Live)1 << (s2 & CLOSED))) & (((Live)1 << SLOTS) - 1u);
                 E += 1 + c1 + c2;
                 ++V;
                 run = run && live != 0;
@@ -453,10 +543,11 @@ struct Tracer {
 
     // the vertices from their planes (in the arithmetic of the form), R, the faces
     __device__ __forceinline__ void solve(const Sub<TT>& G, S& sm, float4 pi, const GridDesc& grid,
-                                          const float4* __restrict__ sorted, float unit_f64)
+                                          const float4* __restrict__ sorted, float unit_f64, float unit_min,
+                                          float4* lo = nullptr)
     {
         R2d = 0.0;
-        R2 = emax = 0.0f;
+        R2 = 0.0f;
         faces.clear();
 #pragma unroll 1
         for (int s = G.gl; s < V; s += TT) {
@@ -470,7 +561,7 @@ struct Tracer {
             const float det = p.x * bcx + p.y * bcy + p.z * bcz;
             // |det| of the unit normals: the vertex moves by (rounding) / this
             const float unit = fabsf(det) * rcp_fast(sm.u.nl[a] * sm.u.nl[b] * sm.u.nl[c]);
-            if (!(unit > UNIT_MIN)) ok = false;
+            if (!(unit > unit_min)) ok = false;
             float x, y, z, err;
             if constexpr (F64) {
                 const double ax = sm.pn[a][0], ay = sm.pn[a][1], az = sm.pn[a][2];
@@ -499,24 +590,26 @@ struct Tracer {
                 z = (p.w * bcz + o.w * caz + h.w * abz) * inv;
                 err = 1e-6f + 1.5e-6f * rcp_fast(unit);
                 if (unit < unit_f64) {  // ill-conditioned: float32 would lose digits
-                    if (!solve_vertex64<PER>(sm.src[a], sm.src[b], sm.src[c], sorted, pi, grid, x, y, z)) ok = false;
+                    double dx, dy, dz;
+                    if (!solve_vertex64<PER>(sm.src[a], sm.src[b], sm.src[c], sorted, pi, grid, dx, dy, dz)) ok = false;
+                    x = (float)dx;
+                    y = (float)dy;
+                    z = (float)dz;
+                    if (lo) lo[s] = low_half(dx, dy, dz);
                     err = 1e-6f;
                 }
             }
             const float d = x * x + y * y + z * z;
             if (!isfinite(d)) ok = false;
             R2 = fmaxf(R2, d);
-            emax = fmaxf(emax, err);
-            sm.vp[s] = make_float4(x, y, z, err);
+            sm.vp[s] = make_float4(x, y, z, err * sqrt_fast(d));
         }
         R2 = G.max(R2);
-        emax = G.max(emax);
         if (F64) R2d = G.maxd(R2d);
 #pragma unroll
         for (int i = 0; i < (NP + 31) / 32; ++i)
 #pragma unroll
             for (int o = TT / 2; o >= 1; o >>= 1) faces.w[i] |= __shfl_xor_sync(TFULL, faces.w[i], o);
-        R = sqrtf(R2);
         __syncwarp();
     }
 
@@ -538,7 +631,7 @@ struct Tracer {
 #pragma unroll 2
         for (int s = 0; s < vmax; ++s) {
             const float4 v = sm.vp[s];
-            const float thr = s < V ? v.w * R : -INFINITY;  // (other slots hold anything)
+            const float thr = s < V ? v.w : -INFINITY;  // (other slots hold anything)
             if (NR > 3 && rows <= 3) near += near_rows<(NR > 3 ? 3 : NR)>(v, thr);
             else near += near_rows<NR>(v, thr);
         }
@@ -546,10 +639,9 @@ struct Tracer {
         ok = !G.any(!ok) && near == 3 * V && 2 * E == 3 * V;
     }
     // the same with FP64 where float32 does not decide: a plane too close to a
-    // vertex passes when the vertex, solved in FP64, is inside it by 1e-10 |n| R
-    // (a warp per cell only)
-    __device__ __forceinline__ void certify64(const Sub<TT>& G, const S& sm, float4 pi, const GridDesc& grid,
-                                              const float4* __restrict__ sorted)
+    // vertex passes when the vertex, solved in FP64, is inside it by 1e-8 |n| |v|,
+    // ten times what FP64 leaves at UNIT_MIN64 (a warp per cell only)
+    __device__ __forceinline__ void certify64(const Sub<TT>& G, const S& sm, const double (*pd)[4], const float4* lo)
     {
         bool fine = ok && 2 * E == 3 * V;
         const int vmax = __any_sync(TFULL, !ok) ? 0 : V;
@@ -557,20 +649,26 @@ struct Tracer {
         for (int s = 0; s < vmax; ++s) {
             const float4 v = sm.vp[s];
             const uint32_t ids = *reinterpret_cast<const uint32_t*>(sm.vid[s]);
-#pragma unroll 1
+#pragma unroll
             for (int r = 0; r < NR; ++r) {
                 const int p = r * TT + G.gl;
-                const float4 n = sm.pl[p];
-                const float len = sqrt_fast(n.x * n.x + n.y * n.y + n.z * n.z);
-                const float d = fmaf(-n.x, v.x, fmaf(-n.y, v.y, fmaf(-n.z, v.z, n.w)));
                 const bool own = p == (int)(ids & 0xff) || p == (int)((ids >> 8) & 0xff) || p == (int)((ids >> 16) & 0xff);
-                if (own || !(d < v.w * R * len)) continue;
+                const float d = fmaf(-nx[r], v.x, fmaf(-ny[r], v.y, fmaf(-nz[r], v.z, nb[r])));
+                if (own || !(d < v.w)) continue;
                 double x, y, z;
-                const P64 h = plane64<PER>(sm.src[p], sorted, pi, grid);
-                const bool solved = vertex64(plane64<PER>(sm.src[ids & 0xff], sorted, pi, grid),
-                                             plane64<PER>(sm.src[(ids >> 8) & 0xff], sorted, pi, grid),
-                                             plane64<PER>(sm.src[(ids >> 16) & 0xff], sorted, pi, grid), x, y, z);
-                if (!solved || !(h.b - ((h.x * x + h.y * y) + h.z * z) > 1e-10 * (double)len * (double)R)) fine = false;
+                if constexpr (F64) {
+                    x = sm.v[s][0];
+                    y = sm.v[s][1];
+                    z = sm.v[s][2];
+                } else {
+                    x = (double)v.x + (double)lo[s].x;
+                    y = (double)v.y + (double)lo[s].y;
+                    z = (double)v.z + (double)lo[s].z;
+                }
+                const double* h = pd[p];
+                const double in = h[3] - ((h[0] * x + h[1] * y) + h[2] * z);
+                const float4 n = sm.pl[p];
+                if (!(in > 1e-2 * (double)(v.w * sqrt_fast(n.x * n.x + n.y * n.y + n.z * n.z)))) fine = false;
             }
         }
         ok = !__any_sync(TFULL, !fine);
@@ -854,13 +952,18 @@ struct alignas(16) OpenCell {
     int32_t np, nf;
     float reach;              // generators with a float key below this are behind it
     float all2;               // (2R)^2
-    float band;               // error bound of the vertex positions
+    int32_t turns;            // times it was built
     int32_t pad[3];
     int32_t src[40];          // its planes: the faces, then what cuts it
-    float4 far[48];           // vertices a generator at `reach` or beyond can cut
+    float4 far[48];           // vertices a generator at `reach` or beyond can cut (see far_vertices)
 };
 static_assert(sizeof(OpenCell) <= StateLayout<float, 64, 64>::BYTES, "an open cell fits the state slot");
 
+// a walk that met a cutting generator goes on for this many limits, or until
+// it has this many: one annulus of a sparse side rarely closes a cell (0, 1 and
+// 2 limits: 139, 85 and 74 thousand turns of the warp-per-cell kernel on 1M
+// points half in clumps)
+constexpr int WALK_ENOUGH = 8, WALK_PAST = 2;
 // a warp's list of cutting generators: the ones kept, and a batch
 constexpr int CUT_LIST = 64;
 
@@ -892,18 +995,22 @@ __device__ __forceinline__ int keep_nearest(float* key, int32_t* id, int ns, int
 }
 
 // The walk of a cell, by a warp: the generators with keys of at least `reach`
-// and within 2R (all2) that cut one of the nf far vertices (x, y, z, |v|^2;
-// shared memory, as the lists key and id), the nearest `keep` of them in order;
+// and within 2R (all2) that cut one of the nf far vertices (position and
+// error bound; shared memory, as the lists key and id), the nearest `keep` of them in order;
 // returns their count. own[0, np): the cell's planes. It takes the rows of the
 // grid that meet the box of the far vertices' balls and the ball of the current
 // limit, less the grid cells that are behind; the limit grows from the reach by
-// half its radius at a time, and the walk ends at the first limit that met a
-// cutting generator (the cell it leaves is smaller). A lane per row finds the
+// half its radius at a time, and the walk ends soon after the first limit that
+// met a cutting generator (the cell it leaves is smaller). A lane per row finds the
 // row's runs, then the lanes share the rows' generators. reach becomes what a
 // later walk of the cell need not look at again.
-template <bool PER>
+// SPREAD: no far vertices; the nearest two generators at `reach` or beyond of
+// each octant around the generator, as far out as the emptiest octants but one
+// need (an octant also ends at a wall): planes that close a cell whose list
+// lies to one side of it.
+template <bool PER, bool SPREAD>
 __device__ __forceinline__ int walk(const TraceArgs& A, const GridDesc& grid, int q, float4 pi, const float4* far, int nf,
-                                    const int32_t* own, int np, float all2, float band, int keep, float& reach,
+                                    const int32_t* own, int np, float all2, int keep, float& reach,
                                     float* key, int32_t* id, unsigned& cands)
 {
     const int lane = threadIdx.x & 31;
@@ -911,7 +1018,7 @@ __device__ __forceinline__ int walk(const TraceArgs& A, const GridDesc& grid, in
     float l0 = 0, l1 = 0, l2 = 0, h0 = 0, h1 = 0, h2 = 0;
     for (int s = lane; s < nf; s += 32) {
         const float4 v = far[s];
-        const float r = sqrt_fast(v.w) * (1.0f + 1e-4f);
+        const float r = sqrt_fast(v.x * v.x + v.y * v.y + v.z * v.z) * (1.0f + 1e-4f);
         l0 = fminf(l0, v.x - r); h0 = fmaxf(h0, v.x + r);
         l1 = fminf(l1, v.y - r); h1 = fmaxf(h1, v.y + r);
         l2 = fminf(l2, v.z - r); h2 = fmaxf(h2, v.z + r);
@@ -931,11 +1038,20 @@ __device__ __forceinline__ int walk(const TraceArgs& A, const GridDesc& grid, in
                 lim_hi = PER ? 3.0f * (float)Gr - 1.0f : (float)Gr - 1.0f;
     auto clamp = [&](float t) { return (int)floorf(fminf(fmaxf(t, lim_lo), lim_hi)); };
     int ns = 0;
-    bool more = false, end = nf == 0;
+    bool more = false, end = !SPREAD && nf == 0;
+    if (SPREAD) {
+        l0 = l1 = l2 = -FLT_MAX;
+        h0 = h1 = h2 = FLT_MAX;
+        if (lane < 16) {
+            key[lane] = FLT_MAX;
+            id[lane] = -1;
+        }
+        __syncwarp();
+    }
     // (40 steps of 2.25 cover every ratio of float32 keys that differ; the
     // last one takes the whole ball)
 #pragma unroll 1
-    for (int it = 0; !end && ns == 0; ++it) {
+    for (int it = 0, past = 0; !end && (ns == 0 || (ns < WALK_ENOUGH && past++ < WALK_PAST)); ++it) {
         const float lim2 = it < 40 ? fminf(all2, 2.25f * reach) : all2;
         const float r_out2 = lim2 * (1.0f + 1e-4f), r_in2 = reach * (1.0f - 1e-4f);
         const float rr = sqrt_fast(r_out2) * (1.0f + 1e-5f);
@@ -966,9 +1082,26 @@ __device__ __forceinline__ int walk(const TraceArgs& A, const GridDesc& grid, in
                 const float dxf = fmaxf(pi.x - gx0, gx1 - pi.x), dyf = fmaxf(pi.y - gy0, gy1 - pi.y);
                 const float dn2 = dxn * dxn + dyn * dyn, df2 = dxf * dxf + dyf * dyf;
                 if (dn2 <= r_out2) {
-                    const float zr = sqrtf(r_out2 - dn2) + m;
-                    int za = clamp((fmaxf(pi.z - zr, z_lo) - grid.lo[2]) * grid.scale[2] - 1e-3f);
-                    int zb = clamp((fminf(pi.z + zr, z_hi) - grid.lo[2]) * grid.scale[2] + 1e-3f);
+                    const float zr = sqrtf(r_out2 - dn2);
+                    // the part of the row inside the balls: the hull of their spans
+                    float s0 = SPREAD ? -FLT_MAX : FLT_MAX, s1 = -s0;
+#pragma unroll 2
+                    for (int k = 0; !SPREAD && k < nf; ++k) {
+                        const float4 v = far[k];
+                        const float bx = fmaxf(fmaxf(gx0 - pi.x - v.x, v.x - (gx1 - pi.x)), 0.0f);
+                        const float by = fmaxf(fmaxf(gy0 - pi.y - v.y, v.y - (gy1 - pi.y)), 0.0f);
+                        const float left = (v.x * v.x + v.y * v.y + v.z * v.z) * (1.0f + 2e-4f) - (bx * bx + by * by);
+                        const float half = sqrt_fast(fmaxf(left, 0.0f));
+                        if (left >= 0.0f) {
+                            s0 = fminf(s0, v.z - half);
+                            s1 = fmaxf(s1, v.z + half);
+                        }
+                    }
+                    s0 = pi.z + fmaxf(s0, -zr) - m;
+                    s1 = pi.z + fminf(s1, zr) + m;
+                    int za = clamp((s0 - grid.lo[2]) * grid.scale[2] - 1e-3f);
+                    int zb = clamp((s1 - grid.lo[2]) * grid.scale[2] + 1e-3f);
+                    if (s0 > s1) zb = za - 1;
                     if (PER) {
                         za = za > tz * Gr ? za : tz * Gr;
                         zb = zb < tz * Gr + Gr - 1 ? zb : tz * Gr + Gr - 1;
@@ -1025,15 +1158,45 @@ __device__ __forceinline__ int walk(const TraceArgs& A, const GridDesc& grid, in
                 const bool in = i < total && j != q;
                 if (in) o = img_off_t<PER>(pi, A.sorted[j], cd, grid);
                 const float d2 = fmaf(o.z, o.z, fmaf(o.y, o.y, o.x * o.x));
-                bool cuts = in && d2 >= reach && d2 <= r_out2;
+                bool cuts = in && d2 >= reach && d2 < lim2;
                 if (!__any_sync(TFULL, cuts)) continue;
+                if (SPREAD) {
+                    if (cuts)
+                        for (int p = 0; p < np; ++p)
+                            if (own[p] == jj) cuts = false;
+                    const int oct = (o.x < 0.0f ? 1 : 0) | (o.y < 0.0f ? 2 : 0) | (o.z < 0.0f ? 4 : 0);
+#pragma unroll 1
+                    for (int e = 0; e < 16; ++e) {  // an octant's nearest, then its next
+                        const bool mine = cuts && oct == e >> 1 && d2 < key[e | 1];
+                        const unsigned near = __reduce_min_sync(TFULL, mine ? __float_as_uint(d2) : 0x7fffffffu);
+                        if (near == 0x7fffffffu) continue;
+                        const unsigned who = __ballot_sync(TFULL, mine && __float_as_uint(d2) == near);
+                        const bool me = lane == __ffs(who) - 1;
+                        if (me) {
+                            const int f = e & ~1;
+                            if (d2 < key[f]) {
+                                key[f + 1] = key[f];
+                                id[f + 1] = id[f];
+                                key[f] = d2;
+                                id[f] = jj;
+                            } else {
+                                key[f + 1] = d2;
+                                id[f + 1] = jj;
+                            }
+                            cuts = false;
+                        }
+                        __syncwarp();
+                    }
+                    continue;
+                }
+                const float len = sqrt_fast(d2);
                 float top = -FLT_MAX;
 #pragma unroll 2
                 for (int k = 0; k < nf; ++k) {
                     const float4 v = far[k];
-                    top = fmaxf(top, fmaf(o.x, v.x, fmaf(o.y, v.y, o.z * v.z)));
+                    top = fmaxf(top, fmaf(o.x, v.x, fmaf(o.y, v.y, fmaf(o.z, v.z, len * v.w))));
                 }
-                cuts = cuts && 0.5f * d2 - top <= band * sqrt_fast(d2);
+                cuts = cuts && 0.5f * d2 <= top;
                 if (cuts)  // (the cell's own faces touch their vertices)
                     for (int p = 0; p < np; ++p)
                         if (own[p] == jj) cuts = false;
@@ -1052,6 +1215,28 @@ __device__ __forceinline__ int walk(const TraceArgs& A, const GridDesc& grid, in
         }
         end = lim2 >= all2;
         if (!more) reach = lim2;  // (all of it is behind)
+        if (SPREAD) {
+            bool full = true;
+            if (lane < 8) {
+                full = key[2 * lane] < FLT_MAX;
+                if (!PER) {
+                    const float wx = lane & 1 ? pi.x - grid.lo[0] : grid.hi[0] - pi.x;
+                    const float wy = lane & 2 ? pi.y - grid.lo[1] : grid.hi[1] - pi.y;
+                    const float wz = lane & 4 ? pi.z - grid.lo[2] : grid.hi[2] - pi.z;
+                    const float wall = fminf(wx, fminf(wy, wz));
+                    full = full || wall * wall < lim2;
+                }
+            }
+            end = end || __popc(__ballot_sync(TFULL, full)) >= 31;
+        }
+    }
+    if (SPREAD) {
+        const int j = lane < 16 ? id[lane] : -1;
+        const unsigned m = __ballot_sync(TFULL, j >= 0);
+        __syncwarp();
+        if (j >= 0) id[__popc(m & ((1u << lane) - 1u))] = j;
+        __syncwarp();
+        return __popc(m);
     }
     if (ns > 0) {
         ns = keep_nearest(key, id, ns, keep, lane);
@@ -1060,7 +1245,7 @@ __device__ __forceinline__ int walk(const TraceArgs& A, const GridDesc& grid, in
     return ns;
 }
 
-// vertices beyond half the reach into far (x, y, z, |v|^2): a generator cuts a
+// vertices beyond half the reach into far (position, error bound): a generator cuts a
 // vertex v only from inside the ball of radius |v| around v
 template <int TT, typename S>
 __device__ __forceinline__ int far_vertices(const Sub<TT>& G, const S& sm, bool on, int V, float reach, float4* far)
@@ -1075,7 +1260,7 @@ __device__ __forceinline__ int far_vertices(const Sub<TT>& G, const S& sm, bool 
         const float d = v.x * v.x + v.y * v.y + v.z * v.z;
         const bool is = on && s < V && d >= half;
         const unsigned m = G.ballot(is);
-        if (is) far[nf + __popc(m & ((1u << G.gl) - 1u))] = make_float4(v.x, v.y, v.z, d);
+        if (is) far[nf + __popc(m & ((1u << G.gl) - 1u))] = v;
         nf += __popc(m);
     }
     return nf;
@@ -1107,7 +1292,7 @@ __global__ void __launch_bounds__(CUT_BLOCK) k_cutters(const __grid_constant__ T
         float reach = h->reach;
         for (int s = lane; s < nf; s += 32) s_far[warp][s] = h->far[s];
         __syncwarp();
-        const int ns = walk<PER>(A, grid, q, pi, s_far[warp], nf, h->src, np, h->all2, h->band, TRACE_KEEP, reach,
+        const int ns = walk<PER, false>(A, grid, q, pi, s_far[warp], nf, h->src, np, h->all2, TRACE_KEEP, reach,
                                  s_key[warp], s_id[warp], cands);
         ++cells;
         if (ns > 0) {
@@ -1207,9 +1392,9 @@ __global__ void __launch_bounds__(TRACE_BLOCK, (sizeof(Real) == 4 ? TRACE_MINB :
         __syncwarp();
         const bool all = G.any(end);
         const unsigned gen0 = G.ballot(sm.src[gl] >= 0);  // the nearest generator's plane follows the walls
-        t.trace(G, sm, gen0 != 0, gen0 ? __ffs(gen0) - 1 : 0);
+        t.template trace<float>(G, sm, gen0 != 0, gen0 ? __ffs(gen0) - 1 : 0, nullptr, nullptr);
         __syncthreads();
-        t.solve(G, sm, pi, grid, A.sorted, T::UNIT_F64);
+        t.solve(G, sm, pi, grid, A.sorted, T::UNIT_F64, T::UNIT_MIN);
         t.certify(G, sm);
         // security radius
         bool valid = all;
@@ -1239,10 +1424,10 @@ __global__ void __launch_bounds__(TRACE_BLOCK, (sizeof(Real) == 4 ? TRACE_MINB :
         if ((open || failed) && gl == 0) {
             h->np = open ? F : P;
             h->nf = nf;
+            h->turns = A.round + (open ? 1 : 0);
             // (a failed list that holds every other generator has no beyond)
             h->reach = failed && all ? FLT_MAX : reach;
             h->all2 = 4.0f * t.R2 * (1.0f + 2e-5f);
-            h->band = t.emax * t.R;
         }
         __syncwarp();
     }
@@ -1257,10 +1442,12 @@ __global__ void __launch_bounds__(TRACE_BLOCK, (sizeof(Real) == 4 ? TRACE_MINB :
 // of 32 planes instead of five of 8. A cell comes out the same bit for bit from
 // either kernel.
 constexpr int TAIL_BLOCK = 128;
+constexpr int TAIL_KEEP = 32;  // cutting generators taken at once from the third turn on
 template <typename Real, bool PER>
 struct TailSmem {
-    typename Tracer<Real, 32, 3, 96, PER>::S t;
-    float4 far[96];
+    typename Tracer<Real, 32, 3, 128, PER>::S t;
+    double pd[96][4];  // planes in FP64, when float32 does not settle a cell
+    float4 far[128];   // far vertices; before that the low halves of FP64 positions
     int32_t src[96];
     float key[CUT_LIST];
     int32_t id[CUT_LIST];
@@ -1268,10 +1455,10 @@ struct TailSmem {
 template <typename Real, bool PER>
 __global__ void __launch_bounds__(TAIL_BLOCK, 4) k_trace_tail(const __grid_constant__ TraceArgs A)
 {
-    constexpr int TT = 32, NR = 3, NV = 96;
+    constexpr int TT = 32, NR = 3, NV = 128;
     using T = Tracer<Real, TT, NR, NV, PER>;
     constexpr bool F64 = T::F64;
-    static_assert(NV / 2 + 2 + TRACE_KEEP <= T::NP && NV / 2 + 2 <= REC_FACES && NV <= REC_VERTS, "capacities");
+    static_assert(REC_FACES + TAIL_KEEP <= T::NP && NV <= REC_VERTS && TAIL_KEEP + 32 <= CUT_LIST, "capacities");
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const Sub<TT> G;
     const int lane = G.lane;
@@ -1294,10 +1481,9 @@ __global__ void __launch_bounds__(TAIL_BLOCK, 4) k_trace_tail(const __grid_const
         int P;
         float reach;
         bool all = false;
-        const Real* keys = nullptr;
+        const int64_t li = (int64_t)q * A.kstride;  // (lists of all cells, in order)
+        const Real* keys = reinterpret_cast<const Real*>(A.d2) + li;
         if (A.round == 0) {
-            const int64_t li = (int64_t)c * A.kstride;
-            keys = reinterpret_cast<const Real*>(A.d2) + li;
             P = 6 + A.kc;
             reach = (float)keys[A.kc - 1] * (F64 ? 1.0f - 1e-6f : 1.0f);
             bool end = false;
@@ -1319,11 +1505,11 @@ __global__ void __launch_bounds__(TAIL_BLOCK, 4) k_trace_tail(const __grid_const
         __syncwarp();
         T t;
         t.rows = NR;
-        bool done = false;
+        bool done = false, spread = false;
         // (every turn adds a generator that cuts; the bound only ends what float
         // round-off could keep turning)
 #pragma unroll 1
-        for (int turn = 0; turn < 200 && !done; ++turn) {
+        for (int turn = A.round == 0 ? 0 : h->turns; turn < 200 && !done; ++turn) {
 #pragma unroll
             for (int r = 0; r < NR; ++r) {
                 const int p = r * TT + lane;
@@ -1331,31 +1517,60 @@ __global__ void __launch_bounds__(TAIL_BLOCK, 4) k_trace_tail(const __grid_const
             }
             __syncwarp();
             const unsigned gen0 = G.ballot(m.t.src[lane] >= 0);
-            t.trace(G, m.t, gen0 != 0, gen0 ? __ffs(gen0) - 1 : 0);
+            const int f0 = gen0 ? __ffs(gen0) - 1 : 0;
+            t.template trace<float>(G, m.t, gen0 != 0, f0, nullptr, nullptr);
             const bool traced = t.ok;
-            t.solve(G, m.t, pi, grid, A.sorted, T::UNIT_F64);
+            t.solve(G, m.t, pi, grid, A.sorted, T::UNIT_F64, T::UNIT_MIN);
             t.certify(G, m.t);
-            if (!t.ok && traced) {
-                t.ok = true;
-                t.solve(G, m.t, pi, grid, A.sorted, T::UNIT_F64_AGAIN);
-                t.certify64(G, m.t, pi, grid, A.sorted);
+            if (turn == 0 && !t.ok && !all && !spread) {
+                // most often a list to one side of its generator
+                spread = true;
+                float r = reach;
+                const float lx = grid.hi[0] - grid.lo[0], ly = grid.hi[1] - grid.lo[1], lz = grid.hi[2] - grid.lo[2];
+                const int ns = walk<PER, true>(A, grid, q, pi, nullptr, 0, m.t.src, P, 1.01f * (lx * lx + ly * ly + lz * lz),
+                                               0, r, m.key, m.id, cands);
+                if (lane < ns) m.src[P + lane] = m.id[lane];
+                P += ns;
+                --turn;
+                __syncwarp();
+                continue;
             }
-            if (!t.ok) break;
+            if (!t.ok) {
+                // what float32 does not settle: every vertex and every close
+                // decision in FP64, then the rays as well
+                for (int p = lane; p < T::NP; p += TT) {
+                    P64 d = {0.0, 0.0, 0.0, 1.0};
+                    if (m.t.src[p] != PAD_PLANE) d = plane64<PER>(m.t.src[p], A.sorted, pi, grid);
+                    m.pd[p][0] = d.x;
+                    m.pd[p][1] = d.y;
+                    m.pd[p][2] = d.z;
+                    m.pd[p][3] = d.b;
+                }
+                __syncwarp();
+            }
+#pragma unroll 1
+            for (int again = traced ? 0 : 1; again < 2 && !t.ok; ++again) {
+                if (again == 1) t.template trace<double>(G, m.t, gen0 != 0, f0, m.pd, m.far);
+                else t.ok = true;
+                t.solve(G, m.t, pi, grid, A.sorted, 2.0f, again == 0 ? T::UNIT_MIN : -1.0f, m.far);
+                t.certify64(G, m.t, m.pd, m.far);
+            }
+            if (!t.ok || t.faces.count() > REC_FACES) break;
             bool valid = all;
-            if (A.round == 0 && turn == 0) {
+            if (turn == 0) {
                 if (!all) valid = F64 ? 4.0 * t.R2d <= (double)keys[A.kc - 1] : 4.0f * t.R2 <= reach * (1.0f - 1e-5f);
                 n_open += !valid;
-                if (A.k_first > 0 && m.t.src[6 + A.k_first] >= 0)
+                if (A.k_first > 0 && keys[A.k_first] < (Real)FLT_MAX)
                     n_second += F64 ? 4.0 * t.R2d > (double)keys[A.k_first] : 4.0f * t.R2 > (float)keys[A.k_first];
+                walks += !valid;
             }
             const float all2 = 4.0f * t.R2 * (1.0f + 2e-5f);
             if (!valid && all2 > reach) {
                 const int F = t.faces.count();
                 const int nf = far_vertices<TT>(G, m.t, true, t.V, reach, m.far);
                 __syncwarp();
-                if (turn == 0 && A.round == 0) ++walks;
-                const int ns = walk<PER>(A, grid, q, pi, m.far, nf, m.t.src, P, all2, t.emax * t.R, TRACE_KEEP, reach,
-                                         m.key, m.id, cands);
+                const int ns = walk<PER, false>(A, grid, q, pi, m.far, nf, m.t.src, P, all2,
+                                         turn < TRACE_ROUNDS ? TRACE_KEEP : TAIL_KEEP, reach, m.key, m.id, cands);
                 if (ns > 0) {
                     __syncwarp();
                     for (int i = lane; i < F; i += TT) m.src[i] = m.t.src[t.faces.nth(i)];
