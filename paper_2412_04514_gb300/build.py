@@ -21,7 +21,7 @@ INCLUDE = os.path.join(ROOT, "include")
 # VT_BUILD_DIR: another build directory (a debug build beside the regular one)
 BUILD = os.environ.get("VT_BUILD_DIR") or os.path.join(HERE, "_build")
 LIB = os.path.join(BUILD, "libvt.so")
-SOURCES = ["scan.cu", "grid.cu", "knn.cu", "clip_f32.cu", "clip_f64.cu", "clip_robust.cu", "emit.cu", "vt_api.cu", "grid_static.cu", "adjoint.cu", "tune.cu", "range.cu", "clip_big.cu", "probe.cu", "trace_f32.cu", "trace_f64.cu"]
+SOURCES = ["scan.cu", "grid.cu", "knn.cu", "clip_f32.cu", "clip_f64.cu", "clip_robust.cu", "emit.cu", "vt_api.cu", "grid_static.cu", "adjoint.cu", "tune.cu", "range.cu", "clip_big.cu", "probe.cu", "trace_f32.cu", "trace_f64.cu", "near.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-Xcompiler", "-fvisibility=hidden",
          "--expt-relaxed-constexpr", "-I", INCLUDE, "-I", CSRC]

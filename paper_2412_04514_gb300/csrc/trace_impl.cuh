@@ -613,6 +613,17 @@ struct Tracer {
         __syncwarp();
     }
 
+    // the cell's listed generators within 2R
+    __device__ __forceinline__ int listed_within(const Sub<TT>& G, const S& sm) const
+    {
+        int c = 0;
+#pragma unroll
+        for (int r = 0; r < NR; ++r) {
+            const int p = r * TT + G.gl;
+            c += sm.src[p] >= 0 && sm.pl[p].w < 2.0f * R2 ? 1 : 0;
+        }
+        return G.bcast(G.incl_scan(c), TT - 1);
+    }
     // planes of the lane's first N rows closer than thr to v (or behind it)
     template <int N>
     __device__ __forceinline__ int near_rows(float4 v, float thr) const
@@ -1357,15 +1368,11 @@ __global__ void __launch_bounds__(TRACE_BLOCK, (sizeof(Real) == 4 ? TRACE_MINB :
         T t;
         int P;
         float reach;  // every generator with a float key below this was in the lists so far
-        bool end = false;
         const int32_t* srcs;
-        const Real* keys = nullptr;
         if (A.round == 0) {
-            const int64_t li = (int64_t)c * A.kstride;
-            srcs = A.nbr + li - 6;
-            keys = reinterpret_cast<const Real*>(A.d2) + li;
+            srcs = A.nbr + (int64_t)c * A.kstride - 6;
             P = 6 + A.kc;
-            reach = (float)keys[A.kc - 1] * (F64 ? 1.0f - 1e-6f : 1.0f);  // (FP64 keys round)
+            reach = A.reach[c];
         } else {
             srcs = h->src;
             P = h->np;
@@ -1377,34 +1384,27 @@ __global__ void __launch_bounds__(TRACE_BLOCK, (sizeof(Real) == 4 ? TRACE_MINB :
             const int p = r * TT + gl;
             int src = PAD_PLANE;
             if (p < P) {
-                if (A.round == 0 && p < 6) {
-                    src = -(p + 1);
-                } else {
-                    src = srcs[p];
-                    if (A.round == 0 && src < 0) {  // the list holds every other generator
-                        src = PAD_PLANE;
-                        end = true;
-                    }
-                }
+                src = A.round == 0 && p < 6 ? -(p + 1) : srcs[p];
+                if (A.round == 0 && p >= 6 && src < 0) src = PAD_PLANE;  // the list is shorter
             }
             t.set_plane(sm, r, p, src, pi, grid, A.sorted);
         }
         __syncwarp();
-        const bool all = G.any(end);
+        const bool all = reach == FLT_MAX;  // the list holds every other generator
         const unsigned gen0 = G.ballot(sm.src[gl] >= 0);  // the nearest generator's plane follows the walls
         t.template trace<float>(G, sm, gen0 != 0, gen0 ? __ffs(gen0) - 1 : 0, nullptr, nullptr);
         __syncthreads();
         t.solve(G, sm, pi, grid, A.sorted, T::UNIT_F64, T::UNIT_MIN);
         t.certify(G, sm);
         // security radius
-        bool valid = all;
-        if (A.round == 0 && !all)
-            valid = F64 ? 4.0 * t.R2d <= (double)keys[A.kc - 1] : 4.0f * t.R2 <= reach * (1.0f - 1e-5f);
+        const bool valid = all || (A.round == 0 && 4.0f * t.R2 <= reach * (1.0f - 1e-5f));
         const bool open = act && t.ok && !valid;
-        if (A.round == 0 && act && t.ok && gl == 0) {
-            n_open += open;
-            if (A.k_first > 0 && srcs[6 + A.k_first] >= 0)
-                n_second += F64 ? 4.0 * t.R2d > (double)keys[A.k_first] : 4.0f * t.R2 > (float)keys[A.k_first];
+        if (A.round == 0) {
+            const int within = t.listed_within(G, sm);
+            if (act && t.ok && gl == 0) {
+                n_open += open;
+                n_second += A.k_first > 0 && within > A.k_first;
+            }
         }
         // the results of an open cell stand unless a generator beyond the list
         // turns out to cut it
@@ -1425,8 +1425,7 @@ __global__ void __launch_bounds__(TRACE_BLOCK, (sizeof(Real) == 4 ? TRACE_MINB :
             h->np = open ? F : P;
             h->nf = nf;
             h->turns = A.round + (open ? 1 : 0);
-            // (a failed list that holds every other generator has no beyond)
-            h->reach = failed && all ? FLT_MAX : reach;
+            h->reach = reach;
             h->all2 = 4.0f * t.R2 * (1.0f + 2e-5f);
         }
         __syncwarp();
@@ -1480,28 +1479,19 @@ __global__ void __launch_bounds__(TAIL_BLOCK, 4) k_trace_tail(const __grid_const
         const OpenCell* h = reinterpret_cast<const OpenCell*>(A.state + (size_t)q * A.state_stride);
         int P;
         float reach;
-        bool all = false;
-        const int64_t li = (int64_t)q * A.kstride;  // (lists of all cells, in order)
-        const Real* keys = reinterpret_cast<const Real*>(A.d2) + li;
         if (A.round == 0) {
             P = 6 + A.kc;
-            reach = (float)keys[A.kc - 1] * (F64 ? 1.0f - 1e-6f : 1.0f);
-            bool end = false;
+            reach = A.reach[c];
             for (int p = lane; p < P; p += TT) {
-                int src = p < 6 ? -(p + 1) : A.nbr[li + p - 6];
-                if (p >= 6 && src < 0) {
-                    src = PAD_PLANE;
-                    end = true;
-                }
-                m.src[p] = src;
+                const int src = p < 6 ? -(p + 1) : A.nbr[(int64_t)c * A.kstride + p - 6];
+                m.src[p] = p >= 6 && src < 0 ? PAD_PLANE : src;
             }
-            all = __any_sync(TFULL, end);
         } else {
             P = h->np;
             reach = h->reach;
-            all = reach == FLT_MAX;
             for (int p = lane; p < P; p += TT) m.src[p] = h->src[p];
         }
+        const bool all = reach == FLT_MAX;
         __syncwarp();
         T t;
         t.rows = NR;
@@ -1558,10 +1548,9 @@ __global__ void __launch_bounds__(TAIL_BLOCK, 4) k_trace_tail(const __grid_const
             if (!t.ok || t.faces.count() > REC_FACES) break;
             bool valid = all;
             if (turn == 0) {
-                if (!all) valid = F64 ? 4.0 * t.R2d <= (double)keys[A.kc - 1] : 4.0f * t.R2 <= reach * (1.0f - 1e-5f);
+                valid = all || 4.0f * t.R2 <= reach * (1.0f - 1e-5f);
                 n_open += !valid;
-                if (A.k_first > 0 && keys[A.k_first] < (Real)FLT_MAX)
-                    n_second += F64 ? 4.0 * t.R2d > (double)keys[A.k_first] : 4.0f * t.R2 > (float)keys[A.k_first];
+                n_second += A.k_first > 0 && t.listed_within(G, m.t) > A.k_first;
                 walks += !valid;
             }
             const float all2 = 4.0f * t.R2 * (1.0f + 2e-5f);

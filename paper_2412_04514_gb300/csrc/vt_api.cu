@@ -494,10 +494,10 @@ bool traced_pass(const vt_params* p, const Layout& L, int kl)
 // 65,536 uniform points 5.4 against 4.3 ms for two Lloyd iterations)
 constexpr int64_t TRACE_SMALL = 16384;
 
-// The list pass over all n cells by edge tracing: kNN with k_list entries,
+// The list pass over all n cells by edge tracing: unordered lists of k_list,
 // two rounds of groups of 8 lanes and the walk, a warp per cell for what they
 // leave, and the plane-by-plane clipper for the cells whose certificate failed
-// there too. Every count stays on the device. slow, open, next, tail: lists of n
+// there too (with sorted lists of their own). Every count stays on the device. slow, open, next, tail: lists of n
 // cells, scratch of the pass (slow until its clipper launch).
 int trace_pass(const Ctx& c, const vt_params* p, int64_t n, int k, int k_list, int variant, vt_cells_out* out,
                int32_t* slow, int32_t* open, int32_t* next, int32_t* tail, int32_t* fail_next, int32_t* ctr_next,
@@ -508,9 +508,10 @@ int trace_pass(const Ctx& c, const vt_params* p, int64_t n, int k, int k_list, i
     StageTimer& T = c.timer ? *c.timer : dummy;
     int32_t* ctr = c.at<int32_t>(L.ctr);
     T.begin(StageTimer::KNNL);
-    cudaError_t e = launch_knn(c.at<float4>(L.sorted), c.at<int32_t>(L.cell_off), c.g, n, nullptr, n, k_list,
-                               p->precision, c.at<int32_t>(L.knn_nbr), c.at<void>(L.knn_d2), c.st, c.s, c.sets,
-                               c.set_of(), nullptr, 0, c.at<int32_t>(L.ctr) + CTR_QUEUE);
+    const int kc = k_list < TRACE_LIST ? k_list : TRACE_LIST;
+    cudaError_t e = launch_near(c.at<float4>(L.sorted), c.at<int32_t>(L.cell_off), c.g, c.sets, c.set_of(), n, kc, kc,
+                                c.at<int32_t>(L.knn_nbr), c.at<float>(L.knn_d2), c.st,
+                                c.at<int32_t>(L.ctr) + CTR_QUEUE, c.s);
     T.end();
     if (c.knn_launches) ++*c.knn_launches;
     if (e != cudaSuccess) return cuda_fail(e, "knn launch");
@@ -522,10 +523,9 @@ int trace_pass(const Ctx& c, const vt_params* p, int64_t n, int k, int k_list, i
     a.set_of = c.set_of();
     a.nq = n;
     a.nbr = c.at<int32_t>(L.knn_nbr);
-    a.d2 = c.at<void>(L.knn_d2);
-    a.kstride = k_list;
-    a.kc = k_list < TRACE_LIST ? k_list : TRACE_LIST;
-    a.k_first = k < a.kc ? k : 0;
+    a.reach = c.at<float>(L.knn_d2);
+    a.kstride = a.kc = kc;
+    a.k_first = k < kc ? k : 0;
     a.emit = p->emit;
     a.index_space = p->index_space;
     a.rec_f32 = p->precision != VT_FP64 ? 1 : 0;
@@ -579,7 +579,7 @@ int trace_pass(const Ctx& c, const vt_params* p, int64_t n, int k, int k_list, i
     if (c.clip_launches) ++*c.clip_launches;
     if (e != cudaSuccess) return cuda_fail(e, "trace launch");
     return clip_pass(c, p, slow, n, ctr + CTR_SLOW, k, false, 0, variant, p->precision, out, fail_next, ctr_next, fail_robust,
-                     ctr_robust, k_list, true, k_list > k ? k_list : 0);
+                     ctr_robust, k_list, false, k_list > k ? k_list : 0);
 }
 
 // the last pass for resumed regular cells (`list`, m cells or *m_dev): range

@@ -616,6 +616,12 @@ cudaError_t launch_knn(const float4* sorted, const int32_t* cell_off, const Grid
                        DevStatus* st, cudaStream_t s, const GridDesc* sets = nullptr, const int32_t* set_of = nullptr,
                        const int32_t* nq_dev = nullptr, int64_t nq_off = 0, int32_t* queue = nullptr);
 
+// lists of the traced pass (near.cu): at most k generators, unordered but for the
+// nearest, kstride apart (-1 past the end), and each list's reach; all n cells
+cudaError_t launch_near(const float4* sorted, const int32_t* cell_off, const GridDesc& g, const GridDesc* sets,
+                        const int32_t* set_of, int64_t n, int k, int kstride, int32_t* nbr, float* reach, DevStatus* st,
+                        int32_t* queue, cudaStream_t s);
+
 struct ClipArgs {
     const float4* sorted;
     const int32_t* cell_off;
@@ -672,8 +678,8 @@ struct TraceArgs {
     int64_t nq;               // cells (the bound when nq_dev is set)
     const int32_t* nq_dev;
     const int32_t* queries;   // sorted indices (NULL = 0..nq-1, with lists)
-    const int32_t* nbr;       // round 0: lists, kstride entries per cell, the first kc used
-    const void* d2;
+    const int32_t* nbr;       // round 0: lists of at most kc (-1: shorter), kstride apart, the nearest first
+    const float* reach;       // round 0: float keys below this are in the list (FLT_MAX: every generator is)
     int kstride, kc;
     int k_first;              // > 0: count the cells still open at this entry (statistics)
     int round;                // 0: lists; > 0: the planes in the cells' state slots

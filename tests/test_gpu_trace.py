@@ -6,6 +6,8 @@ counts that leave groups and blocks partly empty, and small sets in a batch.
 Both forms against the FP64 oracle, to the tolerances of the other parity tests
 (FP32: 1e-5 relative, about 150 roundings of the volume's terms; FP64: 1e-12,
 the oracle's own bound on cells of clumps)."""
+import itertools
+
 import numpy as np
 import pytest
 
@@ -84,6 +86,22 @@ def test_lattices(make, prec):
     # every vertex of the cubic lattice and the walls' of the BCC lattice have
     # more than three planes: the certificate sends the cells to the clipper
     pts = make()
+    want = oracle.tessellate(pts)
+    cells = vt.tessellate(torch.from_numpy(pts).cuda(), vt.Params(precision=prec, emit=("nbr", "vol", "cen")))
+    np.testing.assert_allclose(cells.vol.cpu().numpy(), want["vol"], rtol=TOL[prec])
+    np.testing.assert_allclose(cells.cen.cpu().numpy(), want["cen"], rtol=TOL[prec])
+
+
+@pytest.mark.parametrize("prec", ["fp32", "fp64"])
+def test_more_equal_distances_than_a_list_holds(prec):
+    # 48 generators at one exact distance around the middle one: no limit keeps
+    # between a list's length less one and a list's length of them. (Nothing
+    # else: the middle cell's vertices have up to eight planes, and beside
+    # generic points no schedule validates such a cell.)
+    d = np.array([1.0, 2.0, 4.0]) / 32
+    ring = [0.5 + np.array(s) * d[list(o)] for o in itertools.permutations(range(3))
+            for s in itertools.product([-1, 1], repeat=3)]
+    pts = np.concatenate([[[0.5, 0.5, 0.5]], ring]).astype(np.float32)
     want = oracle.tessellate(pts)
     cells = vt.tessellate(torch.from_numpy(pts).cuda(), vt.Params(precision=prec, emit=("nbr", "vol", "cen")))
     np.testing.assert_allclose(cells.vol.cpu().numpy(), want["vol"], rtol=TOL[prec])
