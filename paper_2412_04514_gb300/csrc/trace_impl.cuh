@@ -233,8 +233,12 @@ struct Tracer {
     static constexpr int NE = 3 * NV / 2;
     using S = TraceSmem<Real, NP, NV>;
     // smallest |det| of a vertex's three unit normals, above the rounding of the
-    // rates of approach in float32, and in FP64
-    static constexpr float UNIT_MIN = F64 ? 2e-5f : 2e-4f, UNIT_MIN64 = 1e-7f;
+    // rates of approach in float32, and in FP64. Both forms take the same for the
+    // rays: the FP32 form solves such vertices in FP64 (UNIT_F64), and at 2e-4 the
+    // sliver-cornered cells beside clumps, traced again with FP64 rays a warp each,
+    // were the last to finish (500 points in clumps 0.63 -> 0.33 ms, 15,000 1.32 ->
+    // 0.90 ms, periodic 2.80 -> 1.72 ms)
+    static constexpr float UNIT_MIN = 2e-5f, UNIT_MIN64 = 1e-7f;
     // below this |det| the FP32 form solves a vertex in FP64 (about 1 in 3,000)
     static constexpr float UNIT_F64 = 1e-2f;
     static constexpr int SR = 2;                     // registers of open edge ends per lane

@@ -490,9 +490,10 @@ bool traced_pass(const vt_params* p, const Layout& L, int kl)
 
 // point counts up to which every cell goes to the warp-per-cell kernel at once
 // (the latency of a few launches less; above it the 8-lane groups' throughput
-// counts: 1,000 points 374 against 463 us, 4,096 in FP64 500 against 657 us, but
-// 65,536 uniform points 5.4 against 4.3 ms for two Lloyd iterations)
-constexpr int64_t TRACE_SMALL = 16384;
+// counts). With neighbours, ms: 3,000 uniform points 0.34 against 0.43 (half in
+// clumps 0.56 against 0.68), 8,000 0.44 against 0.48 (0.68 and 0.81), 11,000 0.48
+// and 0.48 (0.81 and 1.02), 15,000 0.59 and 0.54 (0.89 and 0.85)
+constexpr int64_t TRACE_SMALL = 12288;
 
 // The list pass over all n cells by edge tracing: unordered lists of k_list,
 // two rounds of groups of 8 lanes and the walk, a warp per cell for what they
