@@ -124,14 +124,15 @@ enum {
                                Requires |L|^2 <= 4 min_a L_a^2 (images shifted by more than two
                                periods cannot then cut) and fewer than 2^24 points in the call
                                (a batch counts all its sets); otherwise VT_ERR_INVALID_ARG. */
-    VT_FLAG_FUSED = 8        /* kNN and clipping in one kernel: no neighbour lists. Every cell
-                               starts from the box and walks the grid shells around its generator,
-                               clipping the candidates of each batch of grid cells nearest first,
-                               until the security radius (no unvisited generator within 2R)
-                               concludes it. The n x k list buffer and the saved polyhedra are
-                               not allocated (vt_workspace_size is smaller); k0 and k_max are
-                               still validated and size only the robust variant's lists. Cells
-                               and outputs are those of the list schedules. Combines with
+    VT_FLAG_FUSED = 8        /* The schedule that needs little memory: no n x k neighbour lists and
+                               no saved polyhedra (vt_workspace_size is smaller). The cells are
+                               built in parts whose lists live in the workspace of the robust
+                               variant; a cell that its certificate refuses starts from the box
+                               and walks the grid shells around its generator until the security
+                               radius (no unvisited generator within 2R) concludes it. k0 and
+                               k_max are still validated and size only the robust variant's
+                               lists. Cells and outputs are those of the list schedules. Combines
+                               with
                                VT_FLAG_NO_SYNC and VT_FLAG_PERIODIC. */
 };
 

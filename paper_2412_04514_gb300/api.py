@@ -27,8 +27,8 @@ class Params:
     """Run-time parameters (vt_params). ``precision`` is ``"fp32"`` (float32
     clipping with FP64 rechecks) or ``"fp64"`` (plain FP64). ``periodic``:
     the box [box_lo, box_hi) is periodic (VT_FLAG_PERIODIC). ``fused``: no
-    neighbour lists, every cell clips straight from its grid-shell walk
-    (VT_FLAG_FUSED)."""
+    neighbour lists or saved cells for all points, a quarter of the workspace:
+    the cells are built in parts (VT_FLAG_FUSED)."""
 
     k0: int = 16
     k_max: int = 32

@@ -85,7 +85,8 @@ __global__ void __launch_bounds__(NEAR_BLOCK) k_near(const float4* __restrict__ 
                                                      const int32_t* __restrict__ cell_off0,
                                                      const __grid_constant__ GridDesc g0,
                                                      const GridDesc* __restrict__ sets,
-                                                     const int32_t* __restrict__ set_of, int n, int k, int kstride,
+                                                     const int32_t* __restrict__ set_of, int first, int n, int k,
+                                                     int kstride,
                                                      int32_t* __restrict__ nbr, float* __restrict__ reach_out,
                                                      DevStatus* st, int32_t* __restrict__ queue)
 {
@@ -96,10 +97,11 @@ __global__ void __launch_bounds__(NEAR_BLOCK) k_near(const float4* __restrict__ 
     int32_t* id = s_id[threadIdx.x >> 5];
     unsigned long long evals = 0, answered = 0;
     for (;;) {
-        int q = 0;
-        if (lane == 0) q = atomicAdd(queue, 1);
-        q = __shfl_sync(FULL, q, 0);
-        if (q >= n) break;
+        int c = 0;
+        if (lane == 0) c = atomicAdd(queue, 1);
+        c = __shfl_sync(FULL, c, 0);
+        if (c >= n) break;
+        const int q = first + c;
         ++answered;
         const float4 pq = sorted[q];
         const GridDesc& g = grid_of(g0, sets, set_of, q);
@@ -239,12 +241,12 @@ __global__ void __launch_bounds__(NEAR_BLOCK) k_near(const float4* __restrict__ 
         const unsigned best = __reduce_min_sync(FULL, ::min(ka, kb));
         const unsigned ma = __ballot_sync(FULL, ka == best), mb = __ballot_sync(FULL, kb == best);
         const int at = ma ? __ffs(ma) - 1 : 32 + __ffs(mb) - 1;
-        int32_t* out = nbr + (int64_t)q * kstride;
+        int32_t* out = nbr + (int64_t)c * kstride;
         for (int i = lane; i < k; i += 32) {
             const int from = i == 0 ? at : (i == at ? 0 : i);
             out[i] = i < cnt ? id[from] : -1;
         }
-        if (lane == 0) reach_out[q] = all ? FLT_MAX : lim;
+        if (lane == 0) reach_out[c] = all ? FLT_MAX : lim;
         __syncwarp();
     }
     if (lane == 0 && answered) {
@@ -256,8 +258,8 @@ __global__ void __launch_bounds__(NEAR_BLOCK) k_near(const float4* __restrict__ 
 }  // namespace
 
 cudaError_t launch_near(const float4* sorted, const int32_t* cell_off, const GridDesc& g, const GridDesc* sets,
-                        const int32_t* set_of, int64_t n, int k, int kstride, int32_t* nbr, float* reach, DevStatus* st,
-                        int32_t* queue, cudaStream_t s)
+                        const int32_t* set_of, int64_t first, int64_t n, int k, int kstride, int32_t* nbr, float* reach,
+                        DevStatus* st, int32_t* queue, cudaStream_t s)
 {
     if (n <= 0) return cudaSuccess;
     if (k < 1 || k > 64) return cudaErrorInvalidValue;
@@ -272,8 +274,8 @@ cudaError_t launch_near(const float4* sorted, const int32_t* cell_off, const Gri
     int64_t blocks = (n + NEAR_BLOCK / 32 - 1) / (NEAR_BLOCK / 32);
     const int64_t resident = (int64_t)sms * (per_sm > 0 ? per_sm : 1);
     if (blocks > resident) blocks = resident;
-    kern<<<(unsigned)blocks, NEAR_BLOCK, 0, s>>>(sorted, cell_off, g, sets, set_of, (int)n, k, kstride, nbr, reach, st,
-                                                 queue);
+    kern<<<(unsigned)blocks, NEAR_BLOCK, 0, s>>>(sorted, cell_off, g, sets, set_of, (int)first, (int)n, k, kstride, nbr,
+                                                 reach, st, queue);
     count_launch();
     return cudaGetLastError();
 }

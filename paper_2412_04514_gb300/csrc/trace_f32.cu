@@ -5,6 +5,15 @@ namespace vt {
 
 cudaError_t launch_trace_f32(const TraceArgs& a, cudaStream_t s) { return launch_trace_t<float>(a, s); }
 
+size_t trace_state_bytes() { return (sizeof(OpenCell) + 15) / 16 * 16; }
+
+cudaError_t launch_keep_tail(const TraceArgs& a, const int32_t* before, uint8_t* kept, int64_t cap, cudaStream_t s)
+{
+    k_keep_tail<<<304, 256, 0, s>>>(a, before, kept, (int)cap);
+    count_launch();
+    return cudaGetLastError();
+}
+
 cudaError_t launch_cutters(const TraceArgs& a, cudaStream_t s)
 {
     if (a.nq <= 0) return cudaSuccess;

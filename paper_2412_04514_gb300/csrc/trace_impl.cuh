@@ -1340,7 +1340,7 @@ __global__ void __launch_bounds__(CUT_BLOCK) k_cutters(const __grid_constant__ T
         const int q = A.queries[c];
         const GridDesc& grid = grid_of(A.g, A.sets, A.set_of, q);
         const float4 pi = A.sorted[q];
-        OpenCell* h = reinterpret_cast<OpenCell*>(A.state + (size_t)q * A.state_stride);
+        OpenCell* h = reinterpret_cast<OpenCell*>(A.state + (size_t)(q - A.first) * A.state_stride);
         const int np = h->np, nf = h->nf;
         float reach = h->reach;
         for (int s = lane; s < nf; s += 32) s_far[warp][s] = h->far[s];
@@ -1403,10 +1403,10 @@ __global__ void __launch_bounds__(TRACE_BLOCK, (sizeof(Real) == 4 ? TRACE_MINB :
         const int c0 = c_block + threadIdx.x / TT;
         const bool act = c0 < nq;  // a group past the end repeats the last cell and writes nothing
         const int c = act ? c0 : nq - 1;
-        const int q = A.queries ? A.queries[c] : c;
+        const int q = A.queries ? A.queries[c] : (int)A.first + c;
         const GridDesc& grid = grid_of(A.g, A.sets, A.set_of, q);
         const float4 pi = A.sorted[q];
-        OpenCell* h = reinterpret_cast<OpenCell*>(A.state + (size_t)q * A.state_stride);
+        OpenCell* h = reinterpret_cast<OpenCell*>(A.state + (size_t)(q - A.first) * A.state_stride);
         T t;
         int P;
         float reach;  // every generator with a float key below this was in the lists so far
@@ -1509,16 +1509,18 @@ __global__ void __launch_bounds__(TAIL_BLOCK, 4) k_trace_tail(const __grid_const
         const int have = *A.nq_dev;
         nq = have < nq ? have : nq;
     }
+    int begin = 0;
+    if (A.from_dev) begin = ::max(*A.from_dev, A.from);
     unsigned walks = 0, cands = 0, n_open = 0, n_second = 0;
     for (;;) {
         int c = 0;
-        if (lane == 0) c = atomicAdd(A.queue, 1);
+        if (lane == 0) c = begin + atomicAdd(A.queue, 1);
         c = __shfl_sync(TFULL, c, 0);
         if (c >= nq) break;
-        const int q = A.queries ? A.queries[c] : c;
+        const int q = A.queries ? A.queries[c] : (int)A.first + c;
         const GridDesc& grid = grid_of(A.g, A.sets, A.set_of, q);
         const float4 pi = A.sorted[q];
-        const OpenCell* h = reinterpret_cast<const OpenCell*>(A.state + (size_t)q * A.state_stride);
+        const OpenCell* h = reinterpret_cast<const OpenCell*>(A.state + (size_t)(A.kept ? c : q - A.first) * A.state_stride);
         int P;
         float reach;
         if (A.round == 0) {
@@ -1627,6 +1629,22 @@ __global__ void __launch_bounds__(TAIL_BLOCK, 4) k_trace_tail(const __grid_const
         if (cands) atomicAdd(&A.st->walk_cands, (unsigned long long)cands);
         if (n_open) atomicAdd(&A.st->n_open, (int)n_open);
         if (n_second) atomicAdd(&A.st->n_second, (int)n_second);
+    }
+}
+
+// the state slots of the tail cells a part added, from its slots (A.state) to
+// the kept ones (by place in the tail list, the first cap)
+__global__ void __launch_bounds__(256) k_keep_tail(const __grid_constant__ TraceArgs A, const int32_t* __restrict__ before,
+                                                   uint8_t* __restrict__ kept, int cap)
+{
+    constexpr int W = (int)(sizeof(OpenCell) + 15) / 16;
+    const int i0 = *before, have = *A.tail_ctr, i1 = have < cap ? have : cap;
+    for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < (int64_t)(i1 - i0) * W;
+         t += (int64_t)gridDim.x * blockDim.x) {
+        const int i = i0 + (int)(t / W), w = (int)(t % W);
+        const int q = A.tail_list[i];
+        reinterpret_cast<uint4*>(kept + (size_t)i * A.state_stride)[w] =
+            reinterpret_cast<const uint4*>(A.state + (size_t)(q - A.first) * A.state_stride)[w];
     }
 }
 

@@ -193,8 +193,9 @@ Layout make_layout(const vt_params* p, int64_t n, int64_t cells, bool batch)
     // within k_max (2 k0 entries per cell, all cells at once)
     const int kmx = p->k_max > RANGE_CAP ? p->k_max : RANGE_CAP;
     const int kpre = 2 * p->k0 <= p->k_max ? 2 * p->k0 : p->k0;
-    // the fused schedule clips from the grid walk: no list buffer (one small
-    // block keeps the layout uniform) and no saved polyhedra
+    // the fused schedule's lists and state slots are in the robust variant's
+    // buffers: no list buffer (one small block keeps the layout uniform) and no
+    // saved polyhedra
     const bool fused = (p->flags & VT_FLAG_FUSED) != 0;
     int64_t cap = fused ? 64 : nn * (int64_t)(nosync ? (kmx > kpre ? kmx : kpre) : kpre);
     if (!fused && cap < (int64_t)p->k_max * 64) cap = (int64_t)p->k_max * 64;
@@ -483,10 +484,7 @@ int clip_pass(const Ctx& c, const vt_params* p, const int32_t* list, int64_t m, 
 // tracing finishes every open cell by its own walk, so a caller's further
 // doubling passes stay as they are), and the list is long enough that what it
 // leaves to the walk is small.
-bool traced_pass(const vt_params* p, const Layout& L, int kl)
-{
-    return L.state_stride > 0 && kl >= 12 && 2 * kl > p->k_max;
-}
+bool traced_pass(const vt_params* p, int kl) { return kl >= 12 && 2 * kl > p->k_max; }
 
 // point counts up to which every cell goes to the warp-per-cell kernel at once
 // (the latency of a few launches less; above it the 8-lane groups' throughput
@@ -495,11 +493,22 @@ bool traced_pass(const vt_params* p, const Layout& L, int kl)
 // and 0.48 (0.81 and 1.02), 15,000 0.59 and 0.54 (0.89 and 0.85)
 constexpr int64_t TRACE_SMALL = 12288;
 
-// The list pass over all n cells by edge tracing: unordered lists of k_list,
-// two rounds of groups of 8 lanes and the walk, a warp per cell for what they
-// leave, and the plane-by-plane clipper for the cells whose certificate failed
-// there too (with sorted lists of their own). Every count stays on the device. slow, open, next, tail: lists of n
-// cells, scratch of the pass (slow until its clipper launch).
+// The cells by edge tracing: unordered lists, two rounds of groups of 8 lanes
+// and the walk, a warp per cell for what they leave, and the plane-by-plane
+// clipper for the cells whose certificate failed there too. Every count stays
+// on the device. slow, open, next, tail: lists of n cells, scratch of the pass
+// (slow until its clipper launch).
+//
+// The list schedule has lists of k_list for all cells and a state slot for
+// each; its slow cells get sorted lists. The fused schedule (k_list = 0) has
+// neither: it takes the cells in parts whose lists and state fit the robust
+// variant's list buffers, idle until later and of at least 1536 bytes for every
+// eighth cell. The parts' tail cells keep their slots behind the lists for one
+// launch over all of them (a tail per part: each leaves the device to its last
+// few cells, 10.3 against 8.4 ms at 500,000 points half in clumps), and the slow
+// cells walk from the box. Against every cell walked from the box, at 1M points:
+// uniform 19.5 -> 8.2 ms, clumps 28.1 -> 13.5, FP64 154 -> 20.4 and 229 -> 26.9;
+// the list schedule takes 7.8, 12.0, 19.8 and 25.5 ms.
 int trace_pass(const Ctx& c, const vt_params* p, int64_t n, int k, int k_list, int variant, vt_cells_out* out,
                int32_t* slow, int32_t* open, int32_t* next, int32_t* tail, int32_t* fail_next, int32_t* ctr_next,
                int32_t* fail_robust, int32_t* ctr_robust)
@@ -508,25 +517,16 @@ int trace_pass(const Ctx& c, const vt_params* p, int64_t n, int k, int k_list, i
     StageTimer dummy;
     StageTimer& T = c.timer ? *c.timer : dummy;
     int32_t* ctr = c.at<int32_t>(L.ctr);
-    T.begin(StageTimer::KNNL);
-    const int kc = k_list < TRACE_LIST ? k_list : TRACE_LIST;
-    cudaError_t e = launch_near(c.at<float4>(L.sorted), c.at<int32_t>(L.cell_off), c.g, c.sets, c.set_of(), n, kc, kc,
-                                c.at<int32_t>(L.knn_nbr), c.at<float>(L.knn_d2), c.st,
-                                c.at<int32_t>(L.ctr) + CTR_QUEUE, c.s);
-    T.end();
-    if (c.knn_launches) ++*c.knn_launches;
-    if (e != cudaSuccess) return cuda_fail(e, "knn launch");
+    const bool fused = k_list == 0;
+    const int kc = !fused && k_list < TRACE_LIST ? k_list : TRACE_LIST;
     TraceArgs a{};
     a.sorted = c.at<float4>(L.sorted);
     a.cell_off = c.at<int32_t>(L.cell_off);
     a.g = c.g;
     a.sets = c.sets;
     a.set_of = c.set_of();
-    a.nq = n;
-    a.nbr = c.at<int32_t>(L.knn_nbr);
-    a.reach = c.at<float>(L.knn_d2);
     a.kstride = a.kc = kc;
-    a.k_first = k < kc ? k : 0;
+    a.k_first = !fused && k < kc ? k : 0;
     a.emit = p->emit;
     a.index_space = p->index_space;
     a.rec_f32 = p->precision != VT_FP64 ? 1 : 0;
@@ -535,52 +535,110 @@ int trace_pass(const Ctx& c, const vt_params* p, int64_t n, int k, int k_list, i
     a.m2 = (p->emit & VT_EMIT_M2) ? out->m2 : nullptr;
     a.rec = L.rec_stride ? c.at<uint8_t>(L.rec) : nullptr;
     a.rec_stride = L.rec_stride;
-    a.state = c.at<uint8_t>(L.state);
-    a.state_stride = L.state_stride;
     a.slow_list = slow;
     a.slow_ctr = ctr + CTR_SLOW;
+    a.open_list = open;
+    a.tail_list = tail;
+    a.tail_ctr = &ctr[CTR_TAIL];
     a.st = c.st;
+    int32_t* nbr = c.at<int32_t>(fused ? L.rob_nbr : L.knn_nbr);
+    float* reach;
+    int64_t part = n, cap = n;
+    uint8_t* kept = nullptr;
+    if (fused) {
+        a.state_stride = trace_state_bytes();
+        a.state = c.at<uint8_t>(L.rob_d2);
+        // the lists, the reaches behind them, then the kept slots (a 32nd of the room at least)
+        const int64_t lists = L.rob_cap / 32 * 31 / (kc + 1);
+        const int64_t slots = (int64_t)(sizeof(double) * L.rob_cap / a.state_stride);
+        part = lists < slots ? lists : slots;
+        const int64_t parts = (n + part - 1) / part;
+        part = (n + parts - 1) / parts;
+        reach = reinterpret_cast<float*>(nbr + part * kc);
+        const size_t used = align256(sizeof(int32_t) * part * (kc + 1));
+        kept = reinterpret_cast<uint8_t*>(nbr) + used;
+        cap = (int64_t)((sizeof(int32_t) * L.rob_cap - used) / a.state_stride);
+    } else {
+        reach = c.at<float>(L.knn_d2);
+        a.state = c.at<uint8_t>(L.state);
+        a.state_stride = L.state_stride;
+    }
+    a.nbr = nbr;
+    a.reach = reach;
     const bool small = n <= TRACE_SMALL;
-    for (int round = 0; !small && round < TRACE_ROUNDS; ++round) {
-        // the cells (all, or those the walk before sent back), then the walk over
-        // the open ones among them
-        const bool last = round == TRACE_ROUNDS - 1;
-        a.round = round;
-        a.queries = round == 0 ? nullptr : next;
-        a.nq_dev = round == 0 ? nullptr : &ctr[CTR_TRACE + 2 * round - 1];
-        a.open_list = open;
-        a.open_ctr = &ctr[CTR_TRACE + 2 * round];
-        a.tail_list = tail;
-        a.tail_ctr = &ctr[CTR_TAIL];
-        a.queue = &ctr[CTR_TQUEUE + 2 * round];
-        T.begin(StageTimer::CLIP);
-        e = launch_trace(a, p->precision, c.s);
-        T.end();
-        if (c.clip_launches) ++*c.clip_launches;
-        if (e != cudaSuccess) return cuda_fail(e, "trace launch");
-        a.queries = open;
-        a.nq_dev = a.open_ctr;
-        a.next_list = last ? tail : next;
-        a.next_ctr = last ? &ctr[CTR_TAIL] : &ctr[CTR_TRACE + 2 * round + 1];
-        a.queue = &ctr[CTR_TQUEUE + 2 * round + 1];
-        T.begin(StageTimer::KNN);
-        e = launch_cutters(a, c.s);
+    for (int64_t first = 0; first < n; first += part) {
+        const int64_t m = n - first < part ? n - first : part;
+        cudaError_t e = cudaSuccess;
+        if (first > 0) {  // the part's own counters (the tail and slow lists go on)
+            e = cudaMemcpyAsync(&ctr[CTR_KEPT], &ctr[CTR_TAIL], sizeof(int32_t), cudaMemcpyDeviceToDevice, c.s);
+            if (e == cudaSuccess)
+                e = cudaMemsetAsync(&ctr[CTR_TRACE], 0, sizeof(int32_t) * (CTR_TAIL - CTR_TRACE), c.s);
+            if (e == cudaSuccess)
+                e = cudaMemsetAsync(&ctr[CTR_TQUEUE], 0, sizeof(int32_t) * (CTR_COUNT - CTR_TQUEUE), c.s);
+            if (e != cudaSuccess) return cuda_fail(e, "counter reset");
+        }
+        a.first = first;
+        a.nq = m;
+        T.begin(StageTimer::KNNL);
+        e = launch_near(a.sorted, a.cell_off, c.g, c.sets, c.set_of(), first, m, kc, kc, nbr, reach, c.st,
+                        ctr + CTR_QUEUE, c.s);
         T.end();
         if (c.knn_launches) ++*c.knn_launches;
-        if (e != cudaSuccess) return cuda_fail(e, "walk launch");
+        if (e != cudaSuccess) return cuda_fail(e, "near launch");
+        for (int round = 0; !small && round < TRACE_ROUNDS; ++round) {
+            // the cells (all, or those the walk before sent back), then the walk over
+            // the open ones among them
+            const bool last = round == TRACE_ROUNDS - 1;
+            a.round = round;
+            a.queries = round == 0 ? nullptr : next;
+            a.nq_dev = round == 0 ? nullptr : &ctr[CTR_TRACE + 2 * round - 1];
+            a.open_ctr = &ctr[CTR_TRACE + 2 * round];
+            a.queue = &ctr[CTR_TQUEUE + 2 * round];
+            T.begin(StageTimer::CLIP);
+            e = launch_trace(a, p->precision, c.s);
+            T.end();
+            if (c.clip_launches) ++*c.clip_launches;
+            if (e != cudaSuccess) return cuda_fail(e, "trace launch");
+            a.queries = open;
+            a.nq_dev = a.open_ctr;
+            a.next_list = last ? tail : next;
+            a.next_ctr = last ? &ctr[CTR_TAIL] : &ctr[CTR_TRACE + 2 * round + 1];
+            a.queue = &ctr[CTR_TQUEUE + 2 * round + 1];
+            T.begin(StageTimer::KNN);
+            e = launch_cutters(a, c.s);
+            T.end();
+            if (c.knn_launches) ++*c.knn_launches;
+            if (e != cudaSuccess) return cuda_fail(e, "walk launch");
+        }
+        if (part < n) e = launch_keep_tail(a, &ctr[CTR_KEPT], kept, cap, c.s);
+        if (e != cudaSuccess) return cuda_fail(e, "tail slots");
+        // the tail: of the last part all cells that have a kept slot, of each part those
+        // that have none
+        for (int all = part < n ? 0 : 1; all < (first + m < n ? 1 : 2); ++all) {
+            TraceArgs t = a;
+            t.round = small ? 0 : TRACE_ROUNDS;
+            t.tail = 1;
+            t.queries = small ? nullptr : tail;
+            t.nq_dev = small ? nullptr : &ctr[CTR_TAIL];
+            t.queue = &ctr[CTR_TQUEUE + 2 * TRACE_ROUNDS + all];
+            if (all == 0) {
+                t.nq = n;
+                t.from_dev = &ctr[CTR_KEPT];
+                t.from = (int)(cap < n ? cap : n);
+            } else if (part < n) {
+                t.nq = cap < n ? cap : n;
+                t.kept = 1;
+                t.state = kept;
+            }
+            T.begin(StageTimer::CLIP);
+            e = launch_trace(t, p->precision, c.s);
+            T.end();
+            if (c.clip_launches) ++*c.clip_launches;
+            if (e != cudaSuccess) return cuda_fail(e, "trace launch");
+        }
     }
-    a.round = small ? 0 : TRACE_ROUNDS;
-    a.tail = 1;
-    a.queries = small ? nullptr : tail;
-    a.nq_dev = small ? nullptr : &ctr[CTR_TAIL];
-    a.queue = &ctr[CTR_TQUEUE + 2 * TRACE_ROUNDS];
-    T.begin(StageTimer::CLIP);
-    e = launch_trace(a, p->precision, c.s);
-    T.end();
-    if (c.clip_launches) ++*c.clip_launches;
-    if (e != cudaSuccess) return cuda_fail(e, "trace launch");
-    return clip_pass(c, p, slow, n, ctr + CTR_SLOW, k, false, 0, variant, p->precision, out, fail_next, ctr_next, fail_robust,
-                     ctr_robust, k_list, false, k_list > k ? k_list : 0);
+    return clip_pass(c, p, slow, n, ctr + CTR_SLOW, fused ? 0 : k, fused, 0, variant, p->precision, out, fail_next,
+                     ctr_next, fail_robust, ctr_robust, k_list, false, k_list > k ? k_list : 0);
 }
 
 // the last pass for resumed regular cells (`list`, m cells or *m_dev): range
@@ -760,7 +818,7 @@ int tessellate_run(Ctx& c, const float* pts, int64_t n, const vt_params* p, vt_c
     if ((p->emit & VT_EMIT_CEN) && n > 0 && !out->cen) return fail(VT_ERR_INVALID_ARG, "VT_EMIT_CEN needs cen");
     if ((p->emit & VT_EMIT_M2) && n > 0 && !out->m2) return fail(VT_ERR_INVALID_ARG, "VT_EMIT_M2 needs m2");
     const bool nosync = (p->flags & VT_FLAG_NO_SYNC) != 0;
-    const bool fused = (p->flags & VT_FLAG_FUSED) != 0;  // one walk pass from the box, no lists
+    const bool fused = (p->flags & VT_FLAG_FUSED) != 0;  // one pass in parts, no lists for all cells
     if (nosync && (p->flags & VT_FLAG_STAGE_TIMES))
         return fail(VT_ERR_INVALID_ARG, "VT_FLAG_STAGE_TIMES needs the synchronising schedule");
     const int64_t l0 = launches();
@@ -848,7 +906,7 @@ int tessellate_run(Ctx& c, const float* pts, int64_t n, const vt_params* p, vt_c
             if (last && pi > 0)
                 r = range_pass(c, p, q, n, qn, k_prev, variant_reg, out, regl[(pi + 1) % 2], &ctr_reg[pi], rob_new,
                                &ctr_new[pi], unval, &c.st->n_unval);
-            else if (pi == 0 && !last && traced_pass(p, L, kk))
+            else if (pi == 0 && (fused || traced_pass(p, kk)))
                 r = trace_pass(c, p, n, merged ? p->k0 : kk, kk, variant_reg, out, regl[0], robl[0], robl[1], rob64, rn,
                                rc, rob_new, &ctr_new[pi]);
             else
@@ -886,7 +944,7 @@ int tessellate_run(Ctx& c, const float* pts, int64_t n, const vt_params* p, vt_c
 
     int64_t m_reg = n, m_rob = 0, n_unval = 0;
     bool implicit = true;  // the first pass runs over all cells without a list
-    int k = fused ? p->k_max + 1 : p->k0;  // fused: the exhaustive walk is the first pass
+    int k = fused ? p->k_max + 1 : p->k0;  // fused: the last pass is the first one
     int k_prev = 0;  // regular cells resume from their saved state after list entry k_prev
     int64_t n_open = 0;  // cells that a traced list pass left open and finished itself
 
@@ -914,7 +972,7 @@ int tessellate_run(Ctx& c, const float* pts, int64_t n, const vt_params* p, vt_c
             if (by_range)
                 r = range_pass(c, p, reg_cur, m_reg, nullptr, k_prev, variant_reg, out, reg_nxt, &c.st->n_range_over,
                                rob_new, &c.st->n_fail_robust, unval + n_unval, &c.st->n_fail_next);
-            else if (implicit && !exhaustive && traced_pass(p, L, merged ? 2 * kk : kk))
+            else if (implicit && (fused || (!exhaustive && traced_pass(p, merged ? 2 * kk : kk))))
                 r = trace_pass(c, p, m_reg, kk, merged ? 2 * kk : kk, variant_reg, out, reg_cur, rob_cur, rob_nxt,
                                rob64, reg_nxt, &c.st->n_fail_next, rob_new, &c.st->n_fail_robust);
             else

@@ -556,8 +556,9 @@ constexpr int TRACE_ROUNDS = 2;
 constexpr int CTR_TRACE = CTR_QUEUE + 1;            // open and next list of each round
 constexpr int CTR_TAIL = CTR_TRACE + 2 * TRACE_ROUNDS - 1;  // (the last next list)
 constexpr int CTR_SLOW = CTR_TAIL + 1;
-constexpr int CTR_TQUEUE = CTR_SLOW + 1;            // a cell counter per launch of the pass
-constexpr int CTR_COUNT = CTR_TQUEUE + 2 * TRACE_ROUNDS + 1;
+constexpr int CTR_KEPT = CTR_SLOW + 1;              // tail cells of the parts before
+constexpr int CTR_TQUEUE = CTR_KEPT + 1;            // a cell counter per launch of the pass
+constexpr int CTR_COUNT = CTR_TQUEUE + 2 * TRACE_ROUNDS + 2;
 
 struct Layout {
     int G;
@@ -617,10 +618,11 @@ cudaError_t launch_knn(const float4* sorted, const int32_t* cell_off, const Grid
                        const int32_t* nq_dev = nullptr, int64_t nq_off = 0, int32_t* queue = nullptr);
 
 // lists of the traced pass (near.cu): at most k generators, unordered but for the
-// nearest, kstride apart (-1 past the end), and each list's reach; all n cells
+// nearest, kstride apart (-1 past the end), and each list's reach; cells first to
+// first + n - 1
 cudaError_t launch_near(const float4* sorted, const int32_t* cell_off, const GridDesc& g, const GridDesc* sets,
-                        const int32_t* set_of, int64_t n, int k, int kstride, int32_t* nbr, float* reach, DevStatus* st,
-                        int32_t* queue, cudaStream_t s);
+                        const int32_t* set_of, int64_t first, int64_t n, int k, int kstride, int32_t* nbr, float* reach,
+                        DevStatus* st, int32_t* queue, cudaStream_t s);
 
 struct ClipArgs {
     const float4* sorted;
@@ -677,13 +679,17 @@ struct TraceArgs {
     const int32_t* set_of;
     int64_t nq;               // cells (the bound when nq_dev is set)
     const int32_t* nq_dev;
-    const int32_t* queries;   // sorted indices (NULL = 0..nq-1, with lists)
+    const int32_t* queries;   // sorted indices (NULL = first..first+nq-1, with lists)
+    int64_t first;            // the first cell of the lists and of the state slots
     const int32_t* nbr;       // round 0: lists of at most kc (-1: shorter), kstride apart, the nearest first
     const float* reach;       // round 0: float keys below this are in the list (FLT_MAX: every generator is)
     int kstride, kc;
     int k_first;              // > 0: count the cells still open at this entry (statistics)
     int round;                // 0: lists; > 0: the planes in the cells' state slots
     int tail;                 // 1: a warp per cell, until nothing cuts it
+    int kept;                 // 1: the state slots are in the order of the list
+    const int32_t* from_dev;  // tail: list places before *from_dev or from are left out
+    int from;
     int emit, index_space, rec_f32;
     double *vol, *cen, *m2;
     uint8_t* rec;
@@ -697,6 +703,9 @@ struct TraceArgs {
     DevStatus* st;
     int32_t* queue;           // the launch's cell counter (zero)
 };
+size_t trace_state_bytes();  // an open cell's state slot
+// the slots of the tail cells from list place *before on to kept slots, cap at most
+cudaError_t launch_keep_tail(const TraceArgs& a, const int32_t* before, uint8_t* kept, int64_t cap, cudaStream_t s);
 // lists used per cell at most: with the six walls they fill the planes of a group
 constexpr int TRACE_LIST = 34;
 cudaError_t launch_trace(const TraceArgs& a, int precision, cudaStream_t s);

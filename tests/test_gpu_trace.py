@@ -132,3 +132,21 @@ def test_repeats_bit_for_bit():
             b = vt.tessellate(pts, p)
             for name in ("vol", "cen", "m2", "nbr", "vtx", "face_nbr", "face_vtx"):
                 assert torch.equal(getattr(a, name), getattr(b, name)), (prec, name)
+
+
+@pytest.mark.parametrize("prec", ["fp32", "fp64"])
+@pytest.mark.parametrize("lattice", [False, True])
+def test_fused_schedule_in_parts(lattice, prec):
+    # two parts; of the lattice every cell fails its certificate, more than the
+    # slots that outlive a part. The list schedule builds the same cells at once
+    # (but which of the lattice's faces without area it lists is round-off)
+    x = torch.from_numpy(W.cubic_lattice(60) if lattice else W.mixed(200_000, 2, n_clumps=100)).cuda()
+    emit = ("nbr", "vol", "cen")
+    a = vt.tessellate(x, vt.Params(precision=prec, emit=emit))
+    b = vt.tessellate(x, vt.Params(precision=prec, emit=emit, fused=True))
+    torch.testing.assert_close(b.vol, a.vol, rtol=TOL[prec], atol=0)
+    torch.testing.assert_close(b.cen, a.cen, rtol=0, atol=TOL[prec] * float(a.vol.max()) ** (1 / 3))
+    if prec == "fp64" and not lattice:
+        assert torch.equal(b.nbr_off, a.nbr_off) and torch.equal(b.nbr, a.nbr)
+    again = vt.tessellate(x, vt.Params(precision=prec, emit=emit, fused=True, no_sync=True))
+    assert torch.equal(again.vol, b.vol) and torch.equal(again.nbr[:int(b.nbr_off[-1])], b.nbr[:int(b.nbr_off[-1])])
