@@ -150,3 +150,18 @@ def test_fused_schedule_in_parts(lattice, prec):
         assert torch.equal(b.nbr_off, a.nbr_off) and torch.equal(b.nbr, a.nbr)
     again = vt.tessellate(x, vt.Params(precision=prec, emit=emit, fused=True, no_sync=True))
     assert torch.equal(again.vol, b.vol) and torch.equal(again.nbr[:int(b.nbr_off[-1])], b.nbr[:int(b.nbr_off[-1])])
+
+
+def test_differentiable_moments_free_their_cells():
+    # after a step only its gradient is left: the cells are not kept by a cycle
+    # between the outputs and their node
+    x = torch.from_numpy(W.uniform(20_000, 5)).cuda().requires_grad_(True)
+    held = []
+    for _ in range(4):
+        x.grad = None
+        vol, cen, m2 = vt.voronoi_moments(x, vt.Params())
+        (m2.sum() + (vol * vol).sum() + cen.sum()).backward()
+        del vol, cen, m2
+        torch.cuda.synchronize()
+        held.append(torch.cuda.memory_allocated())
+    assert held[-1] == held[0], held
