@@ -383,7 +383,7 @@ def run_gpu(args, rank: int, world: int, local: int):
         tot64 = dist_max(sum(ms64), world)
         value64 = n * world * len(ms64) / (tot64 / 1e3)
 
-    # the fused schedule (VT_FLAG_FUSED): kNN and clip in one walk, no lists
+    # the fused schedule (VT_FLAG_FUSED): cells traced in parts, no lists for all points
     cellsF = None
     if args.steps_fused > 0:
         pF = vt.Params(**{**p32.__dict__, "fused": True})
@@ -538,7 +538,7 @@ def run_gpu(args, rank: int, world: int, local: int):
         "fused_value": None if cellsF is None else valueF,
         "fused_form": None if cellsF is None else {
             "value": valueF, "unit": "cells/s", "ms_per_step": totF / len(msF), "steps": len(msF),
-            "schedule": "VT_FLAG_FUSED: every cell clips straight from its grid-shell walk (no neighbour lists)",
+            "schedule": "VT_FLAG_FUSED: cells traced in parts (no neighbour lists for all points)",
             "stage_ms": {k: statistics.mean(s[k] for s in stF) for k in ("ms_grid", "ms_knn", "ms_clip", "ms_emit")},
             "workspace_bytes_per_point": wsF / n, "list_schedule_workspace_bytes_per_point": ws32 / n},
         "fp64_form": None if args.steps_fp64 <= 0 else {
