@@ -673,7 +673,8 @@ struct Tracer {
             for (int r = 0; r < NR; ++r) {
                 const int p = r * TT + G.gl;
                 const float d = fmaf(-nx[r], v.x, fmaf(-ny[r], v.y, fmaf(-nz[r], v.z, nb[r])));
-                if (p != a && p != b && p != c && fabsf(d) < v.w) at = p;
+                // (v.w is infinite where |v|^2 overflows: no finite distance keeps a padding plane out)
+                if (p != a && p != b && p != c && sm.src[p] != PAD_PLANE && fabsf(d) < v.w) at = p;
             }
             if (!__any_sync(TFULL, at >= 0)) continue;
             bool tie = false;

@@ -109,6 +109,22 @@ def test_more_equal_distances_than_a_list_holds(prec):
 
 
 @pytest.mark.parametrize("prec", ["fp32", "fp64"])
+@pytest.mark.parametrize("n", [3, 20, 300])
+def test_box_whose_plane_products_overflow(n, prec):
+    # a box of 2^40: the float32 products of a vertex's three planes overflow,
+    # its error bound can become infinite, and short lists have padding planes.
+    # The cells are those of the unit box, scaled by a power of two.
+    pts = W.uniform(n, 60 + n)
+    want = oracle.tessellate(pts)
+    scale = 2.0 ** 40
+    cells = vt.tessellate(torch.from_numpy(pts * np.float32(scale)).cuda(),
+                          vt.Params(precision=prec, emit=("nbr", "vol", "cen"), box_hi=(scale,) * 3))
+    np.testing.assert_allclose(cells.vol.cpu().numpy() / scale ** 3, want["vol"], rtol=TOL[prec])
+    if prec == "fp64":  # (first moments, fourth powers of a length, overflow float32 here)
+        np.testing.assert_allclose(cells.cen.cpu().numpy() / scale, want["cen"], rtol=1e-12)
+
+
+@pytest.mark.parametrize("prec", ["fp32", "fp64"])
 def test_batch_of_small_sets(prec):
     sizes = [1, 2, 0, 7, 33, 34, 35, 200, 1, 1500]
     parts = [W.uniform(n, 40 + i) for i, n in enumerate(sizes)]
