@@ -32,7 +32,10 @@
 // them, so an accepted topology is the exact one. A cell that fails (vertices
 // within round-off of a further plane, ill-conditioned or too many of them) is
 // built again by other means, in the end by the plane-by-plane clipper with its
-// FP64 rechecks.
+// FP64 rechecks. The bounds hold while squares of lengths are normal float32
+// numbers: a cell with a generator or a vertex closer than 1e-18 to its own
+// generator fails too, and one with a vertex whose products of three normals
+// leave 1e-25..1e25 goes to the warp per cell, which solves it in FP64.
 //
 // Security radius. A cell whose 4 R^2 is within the list's reach is final.
 // Otherwise its results are written all the same and a second kernel (a warp
@@ -166,6 +169,16 @@ __device__ VT_RARE bool solve_vertex64(int a, int b, int c, const float4* __rest
     return vertex64(plane64<PER>(a, sorted, pi, grid), plane64<PER>(b, sorted, pi, grid),
                     plane64<PER>(c, sorted, pi, grid), x, y, z);
 }
+// |det| of the unit normals of three planes of any scale
+__device__ VT_RARE float unit_det(float4 p, float4 o, float4 h)
+{
+    const double bcx = (double)o.y * h.z - (double)o.z * h.y, bcy = (double)o.z * h.x - (double)o.x * h.z,
+                 bcz = (double)o.x * h.y - (double)o.y * h.x;
+    const double pp = (double)p.x * p.x + (double)p.y * p.y + (double)p.z * p.z,
+                 oo = (double)o.x * o.x + (double)o.y * o.y + (double)o.z * o.z,
+                 hh = (double)h.x * h.x + (double)h.y * h.y + (double)h.z * h.z;
+    return (float)(fabs(p.x * bcx + p.y * bcy + p.z * bcz) / (sqrt(pp) * sqrt(oo) * sqrt(hh)));
+}
 // the low halves of a position in FP64 beside its float32 value
 __device__ __forceinline__ float4 low_half(double x, double y, double z)
 {
@@ -253,6 +266,11 @@ struct Tracer {
     float R2;               // max |v|^2
     double R2d;
     Faces<(NP + 31) / 32> faces;  // the planes that are faces
+
+    // squares below this lose digits in float32: a cell with such a vertex, or
+    // whose first generator, the nearest of its lists, is so close, fails
+    static constexpr float SQUARE_MIN = 1e-36f;
+    static __device__ __forceinline__ bool in_range(const S& sm, int f0) { return sm.pl[f0].w >= 0.5f * SQUARE_MIN; }
 
     // plane row r of the lane from its source
     __device__ __forceinline__ void set_plane(S& sm, int r, int p, int src, float4 pi, const GridDesc& grid,
@@ -564,8 +582,14 @@ struct Tracer {
             const float bcx = o.y * h.z - o.z * h.y, bcy = o.z * h.x - o.x * h.z, bcz = o.x * h.y - o.y * h.x;
             const float det = p.x * bcx + p.y * bcy + p.z * bcz;
             // |det| of the unit normals: the vertex moves by (rounding) / this
-            const float unit = fabsf(det) * rcp_fast(sm.u.nl[a] * sm.u.nl[b] * sm.u.nl[c]);
-            if (!(unit > unit_min)) ok = false;
+            const float len = sm.u.nl[a] * sm.u.nl[b] * sm.u.nl[c];
+            float unit = fabsf(det) * rcp_fast(len);
+            // terms of the determinant or of the position leave float32's range (at
+            // unit >= UNIT_F64): for the warp per cell, which solves them in FP64
+            const bool far_scale = __float_as_uint(len) - __float_as_uint(1e-25f) >
+                                   __float_as_uint(1e25f) - __float_as_uint(1e-25f);
+            if (TT == 32 && far_scale) unit = unit_det(p, o, h);
+            if (!(unit > unit_min) || (TT < 32 && far_scale)) ok = false;
             float x, y, z, err;
             if constexpr (F64) {
                 const double ax = sm.pn[a][0], ay = sm.pn[a][1], az = sm.pn[a][2];
@@ -593,7 +617,7 @@ struct Tracer {
                 y = (p.w * bcy + o.w * cay + h.w * aby) * inv;
                 z = (p.w * bcz + o.w * caz + h.w * abz) * inv;
                 err = 1e-6f + 1.5e-6f * rcp_fast(unit);
-                if (unit < unit_f64) {  // ill-conditioned: float32 would lose digits
+                if (unit < unit_f64 || (TT == 32 && far_scale)) {  // ill-conditioned: float32 would lose digits
                     double dx, dy, dz;
                     if (!solve_vertex64<PER>(sm.src[a], sm.src[b], sm.src[c], sorted, pi, grid, dx, dy, dz)) ok = false;
                     x = (float)dx;
@@ -604,7 +628,7 @@ struct Tracer {
                 }
             }
             const float d = x * x + y * y + z * z;
-            if (!isfinite(d)) ok = false;
+            if (__float_as_uint(d) - __float_as_uint(SQUARE_MIN) >= 0x7f800000u - __float_as_uint(SQUARE_MIN)) ok = false;
             R2 = fmaxf(R2, d);
             sm.vp[s] = make_float4(x, y, z, err * sqrt_fast(d));
         }
@@ -708,7 +732,7 @@ struct Tracer {
                 const int p = r * TT + G.gl;
                 const bool own = p == (int)(ids & 0xff) || p == (int)((ids >> 8) & 0xff) || p == (int)((ids >> 16) & 0xff);
                 const float d = fmaf(-nx[r], v.x, fmaf(-ny[r], v.y, fmaf(-nz[r], v.z, nb[r])));
-                if (own || !(d < v.w)) continue;
+                if (own || d >= v.w) continue;
                 double x, y, z;
                 if constexpr (F64) {
                     x = sm.v[s][0];
@@ -722,7 +746,7 @@ struct Tracer {
                 const double* h = pd[p];
                 const double in = h[3] - ((h[0] * x + h[1] * y) + h[2] * z);
                 const float4 n = sm.pl[p];
-                if (!(in > 1e-2 * (double)(v.w * sqrt_fast(n.x * n.x + n.y * n.y + n.z * n.z)))) fine = false;
+                if (!(in > 1e-2 * (double)v.w * (double)sqrt_fast(n.x * n.x + n.y * n.y + n.z * n.z))) fine = false;
             }
         }
         ok = !__any_sync(TFULL, !fine);
@@ -1435,7 +1459,8 @@ __global__ void __launch_bounds__(TRACE_BLOCK, (sizeof(Real) == 4 ? TRACE_MINB :
         __syncwarp();
         const bool all = reach == FLT_MAX;  // the list holds every other generator
         const unsigned gen0 = G.ballot(sm.src[gl] >= 0);  // the nearest generator's plane follows the walls
-        t.template trace<float>(G, sm, gen0 != 0, gen0 ? __ffs(gen0) - 1 : 0, nullptr, nullptr);
+        const int f0 = gen0 ? __ffs(gen0) - 1 : 0;
+        t.template trace<float>(G, sm, gen0 != 0 && T::in_range(sm, f0), f0, nullptr, nullptr);
         __syncthreads();
         t.solve(G, sm, pi, grid, A.sorted, T::UNIT_F64, T::UNIT_MIN);
         t.certify(G, sm);
@@ -1553,6 +1578,7 @@ __global__ void __launch_bounds__(TAIL_BLOCK, 4) k_trace_tail(const __grid_const
             __syncwarp();
             const unsigned gen0 = G.ballot(m.t.src[lane] >= 0);
             const int f0 = gen0 ? __ffs(gen0) - 1 : 0;
+            if (!T::in_range(m.t, f0)) break;
             t.template trace<float>(G, m.t, gen0 != 0, f0, nullptr, nullptr);
             const bool traced = t.ok;
             t.solve(G, m.t, pi, grid, A.sorted, T::UNIT_F64, T::UNIT_MIN);

@@ -486,6 +486,17 @@ int clip_pass(const Ctx& c, const vt_params* p, const int32_t* list, int64_t m, 
 // leaves to the walk is small.
 bool traced_pass(const vt_params* p, int kl) { return kl >= 12 && 2 * kl > p->k_max; }
 
+// Whether the box is one the traced pass may run in: it compares float32 squares
+// (list keys, reaches, 4 R^2), which of boxes beyond 2^58 can become infinite and
+// then compare as equal. (Small scales have no such bound: a cell whose squares
+// are too small is refused by its certificate.)
+bool traced_box(const vt_params* p)
+{
+    for (int a = 0; a < 3; ++a)
+        if ((double)p->box_hi[a] - (double)p->box_lo[a] > std::ldexp(1.0, 58)) return false;
+    return true;
+}
+
 // point counts up to which every cell goes to the warp-per-cell kernel at once
 // (the latency of a few launches less; above it the 8-lane groups' throughput
 // counts). With neighbours, ms: 3,000 uniform points 0.34 against 0.43 (half in
@@ -906,7 +917,7 @@ int tessellate_run(Ctx& c, const float* pts, int64_t n, const vt_params* p, vt_c
             if (last && pi > 0)
                 r = range_pass(c, p, q, n, qn, k_prev, variant_reg, out, regl[(pi + 1) % 2], &ctr_reg[pi], rob_new,
                                &ctr_new[pi], unval, &c.st->n_unval);
-            else if (pi == 0 && (fused || traced_pass(p, kk)))
+            else if (pi == 0 && traced_box(p) && (fused || traced_pass(p, kk)))
                 r = trace_pass(c, p, n, merged ? p->k0 : kk, kk, variant_reg, out, regl[0], robl[0], robl[1], rob64, rn,
                                rc, rob_new, &ctr_new[pi]);
             else
@@ -972,7 +983,7 @@ int tessellate_run(Ctx& c, const float* pts, int64_t n, const vt_params* p, vt_c
             if (by_range)
                 r = range_pass(c, p, reg_cur, m_reg, nullptr, k_prev, variant_reg, out, reg_nxt, &c.st->n_range_over,
                                rob_new, &c.st->n_fail_robust, unval + n_unval, &c.st->n_fail_next);
-            else if (implicit && (fused || (!exhaustive && traced_pass(p, merged ? 2 * kk : kk))))
+            else if (implicit && traced_box(p) && (fused || (!exhaustive && traced_pass(p, merged ? 2 * kk : kk))))
                 r = trace_pass(c, p, m_reg, kk, merged ? 2 * kk : kk, variant_reg, out, reg_cur, rob_cur, rob_nxt,
                                rob64, reg_nxt, &c.st->n_fail_next, rob_new, &c.st->n_fail_robust);
             else

@@ -124,6 +124,48 @@ def test_box_whose_plane_products_overflow(n, prec):
         np.testing.assert_allclose(cells.cen.cpu().numpy() / scale, want["cen"], rtol=1e-12)
 
 
+@pytest.mark.parametrize("n,clumps,k", [(300, 0, -33), (2000, 2, -26), (20_000, 10, -26)])
+def test_small_scales(n, clumps, k):
+    # the clouds' products of three normals (and of their squares) underflow float32
+    pts = W.mixed(n, 3, n_clumps=clumps) if clumps else W.uniform(n, 1)
+    want = oracle.tessellate(pts)
+    scale = 2.0 ** k
+    cells = vt.tessellate(torch.from_numpy(pts * np.float32(scale)).cuda(),
+                          vt.Params(precision="fp32", emit=("nbr", "vol"), box_hi=(scale,) * 3))
+    np.testing.assert_allclose(cells.vol.cpu().numpy() / scale ** 3, want["vol"], rtol=TOL["fp32"])
+
+
+@pytest.mark.parametrize("prec", ["fp32", "fp64"])
+@pytest.mark.parametrize("spacing", [1e-20, 1e-19, 1e-18, 1e-13])
+def test_generators_whose_squares_underflow(spacing, prec):
+    # three generators on a line: the cell between two others is a slab of the
+    # box as thick as their spacing. Beyond the range of the certificate's bounds
+    # the cells are the clipper's (k_max = 4 k0 is not traced), whose FP64 form
+    # takes a plane within 1e-14 R of the vertices it cuts as touching them.
+    x = np.array([1, 2, 3]) * spacing
+    pts = np.stack([x, np.full(3, 0.5), np.full(3, 0.5)], 1).astype(np.float32)
+    cells, clip = (vt.tessellate(torch.from_numpy(pts).cuda(), vt.Params(precision=prec, emit=("nbr", "vol"), **kw))
+                   for kw in ({}, {"k0": 6, "k_max": 24}))
+    torch.testing.assert_close(cells.vol, clip.vol, rtol=TOL[prec], atol=0)
+    assert torch.equal(cells.nbr_off, clip.nbr_off) and torch.equal(cells.nbr, clip.nbr)
+    if prec == "fp32" or spacing > 1e-14:
+        x = pts[:, 0].astype(np.float64)
+        cut = [0.0, (x[0] + x[1]) / 2, (x[1] + x[2]) / 2, 1.0]
+        np.testing.assert_allclose(cells.vol.cpu().numpy(), np.diff(cut), rtol=TOL[prec])
+        assert cells.nbr_off.tolist() == [0, 1, 3, 4] and cells.nbr.tolist() == [1, 0, 2, 1]
+
+
+def test_box_beyond_float_squares():
+    # 2^60: not traced, the clipper's FP64 form builds the unit box's cells scaled
+    pts = W.uniform(300, 8)
+    want = oracle.tessellate(pts)
+    for fused in (False, True):
+        cells = vt.tessellate(torch.from_numpy(pts * np.float32(2.0 ** 60)).cuda(),
+                              vt.Params(precision="fp64", emit=("nbr", "vol"), box_hi=(2.0 ** 60,) * 3, fused=fused))
+        np.testing.assert_allclose(cells.vol.cpu().numpy() / 2.0 ** 180, want["vol"], rtol=1e-12)
+        assert np.array_equal(cells.nbr.cpu().numpy(), want["nbr"])
+
+
 @pytest.mark.parametrize("prec", ["fp32", "fp64"])
 def test_batch_of_small_sets(prec):
     sizes = [1, 2, 0, 7, 33, 34, 35, 200, 1, 1500]
