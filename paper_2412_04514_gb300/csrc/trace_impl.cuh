@@ -255,9 +255,9 @@ struct Tracer {
     // below this |det| the FP32 form solves a vertex in FP64 (about 1 in 3,000)
     static constexpr float UNIT_F64 = 1e-2f;
     static constexpr int SR = 2;                     // registers of open edge ends per lane
-    using Live = typename LiveMask<TT>::T;           // a bit per slot; the top bit marks a closed edge
-    static constexpr int CLOSED = 8 * sizeof(Live) - 1;
-    static constexpr int SLOTS = SR * TT < CLOSED ? SR * TT : CLOSED;
+    using Live = typename LiveMask<TT>::T;           // a bit per slot; the top bit takes the edges that closed
+    static constexpr int TOP = 8 * sizeof(Live) - 1;
+    static constexpr int SLOTS = SR * TT < TOP ? SR * TT : TOP;
 
     float nx[NR], ny[NR], nz[NR], nb[NR];
     int rows;               // rows of planes in use over the warp
@@ -545,16 +545,16 @@ struct Tracer {
                     *reinterpret_cast<uint32_t*>(sm.vid[V]) = (uint32_t)b | ((uint32_t)a << 8) | ((uint32_t)h << 16);
                     sm.ed[E] = (uint32_t)ent | ((uint32_t)V << 24);
                 }
-                // the lowest free slots take what stays open
+                // the lowest free slots take what stays open (an edge that closed: no slot)
                 const Live free1 = ~live, free2 = c1 ? free1 : free1 & (free1 - 1u);
-                const int s1 = c1 ? CLOSED : lowest(free1), s2 = c2 ? CLOSED : lowest(free2);
+                const int s1 = c1 ? -1 : lowest(free1), s2 = c2 ? -1 : lowest(free2);
 #pragma unroll
                 for (int i = 0; i < SR; ++i) {
                     const int at = gl + i * TT;
                     o[i] = at == s1 ? a | (h << 8) | (V << 16) : (at == s2 ? h | (b << 8) | (V << 16) : o[i]);
                 }
                 if ((!c1 && s1 >= SLOTS) || (!c2 && (unsigned)s2 >= (unsigned)SLOTS)) ok = run = false;
-                live = (live | ((Live)1 << s1) | ((Live)1 << (s2 & CLOSED))) & (((Live)1 << SLOTS) - 1u);
+                live = (live | ((Live)1 << (s1 & TOP)) | ((Live)1 << (s2 & TOP))) & (((Live)1 << SLOTS) - 1u);
                 E += 1 + c1 + c2;
                 ++V;
                 run = run && live != 0;
