@@ -58,6 +58,18 @@ constexpr unsigned TFULL = 0xffffffffu;
 constexpr int TRACE_KEEP = 12;     // cutting generators handed to the next round
 constexpr int PAD_PLANE = INT_MIN;
 
+// A vertex is known to VERT_ERR |v|: float32 at the smallest |det| that the FP32
+// form solves in float32 (UNIT_F64), rounding included. Whatever decides which
+// generators can still cut a vertex allows for it: the true vertex v' has
+// |v'| <= (1 + VERT_ERR) |v|, and the ball of its cutting generators, of radius
+// |v'| around v', lies in the ball of (1 + 2 VERT_ERR) |v| around v. (Factors on
+// squares; 1e-5 more covers the rounding of the comparisons.)
+constexpr float UNIT_F64 = 1e-2f;
+constexpr float VERT_ERR0 = 1e-6f, VERT_ERR1 = 1.5e-6f;  // VERT_ERR0 + VERT_ERR1 / |det|
+constexpr float VERT_ERR = VERT_ERR0 + VERT_ERR1 / UNIT_F64;
+constexpr float FAR_R2 = (1.0f + VERT_ERR) * (1.0f + VERT_ERR) + 1e-5f;
+constexpr float FAR_BALL = 1.0f + 2.0f * VERT_ERR + 5e-6f;
+
 // groups of TT lanes of a warp in lockstep
 template <int TT>
 struct Sub {
@@ -81,15 +93,6 @@ struct Sub {
     {
 #pragma unroll
         for (int o = TT / 2; o >= 1; o >>= 1) v = fmaxf(v, __shfl_xor_sync(TFULL, v, o));
-        return v;
-    }
-    __device__ __forceinline__ double maxd(double v) const
-    {
-#pragma unroll
-        for (int o = TT / 2; o >= 1; o >>= 1) {
-            const double u = __shfl_xor_sync(TFULL, v, o);
-            v = u > v ? u : v;
-        }
         return v;
     }
     __device__ __forceinline__ int incl_scan(int v) const
@@ -252,8 +255,8 @@ struct Tracer {
     // were the last to finish (500 points in clumps 0.63 -> 0.33 ms, 15,000 1.32 ->
     // 0.90 ms, periodic 2.80 -> 1.72 ms)
     static constexpr float UNIT_MIN = 2e-5f, UNIT_MIN64 = 1e-7f;
-    // below this |det| the FP32 form solves a vertex in FP64 (about 1 in 3,000)
-    static constexpr float UNIT_F64 = 1e-2f;
+    // (below UNIT_F64 the FP32 form solves a vertex in FP64, about 1 in 3,000)
+    static constexpr float UNIT_F64 = vt::UNIT_F64;
     static constexpr int SR = 2;                     // registers of open edge ends per lane
     using Live = typename LiveMask<TT>::T;           // a bit per slot; the top bit takes the edges that closed
     static constexpr int TOP = 8 * sizeof(Live) - 1;
@@ -264,7 +267,6 @@ struct Tracer {
     bool ok;
     int V, E;
     float R2;               // max |v|^2
-    double R2d;
     Faces<(NP + 31) / 32> faces;  // the planes that are faces
 
     // squares below this lose digits in float32: a cell with such a vertex, or
@@ -568,7 +570,6 @@ struct Tracer {
                                           const float4* __restrict__ sorted, float unit_f64, float unit_min,
                                           float4* lo = nullptr)
     {
-        R2d = 0.0;
         R2 = 0.0f;
         faces.clear();
 #pragma unroll 1
@@ -603,12 +604,10 @@ struct Tracer {
                 sm.v[s][0] = dx;
                 sm.v[s][1] = dy;
                 sm.v[s][2] = dz;
-                const double d = (dx * dx + dy * dy) + dz * dz;
-                R2d = d > R2d ? d : R2d;
                 x = (float)dx;
                 y = (float)dy;
                 z = (float)dz;
-                err = 1e-6f;  // float rounding of the position, of the plane and of the test
+                err = VERT_ERR0;  // float rounding of the position, of the plane and of the test
             } else {
                 const float cax = h.y * p.z - h.z * p.y, cay = h.z * p.x - h.x * p.z, caz = h.x * p.y - h.y * p.x;
                 const float abx = p.y * o.z - p.z * o.y, aby = p.z * o.x - p.x * o.z, abz = p.x * o.y - p.y * o.x;
@@ -616,7 +615,7 @@ struct Tracer {
                 x = (p.w * bcx + o.w * cax + h.w * abx) * inv;
                 y = (p.w * bcy + o.w * cay + h.w * aby) * inv;
                 z = (p.w * bcz + o.w * caz + h.w * abz) * inv;
-                err = 1e-6f + 1.5e-6f * rcp_fast(unit);
+                err = VERT_ERR0 + VERT_ERR1 * rcp_fast(unit);
                 if (unit < unit_f64 || (TT == 32 && far_scale)) {  // ill-conditioned: float32 would lose digits
                     double dx, dy, dz;
                     if (!solve_vertex64<PER>(sm.src[a], sm.src[b], sm.src[c], sorted, pi, grid, dx, dy, dz)) ok = false;
@@ -624,7 +623,7 @@ struct Tracer {
                     y = (float)dy;
                     z = (float)dz;
                     if (lo) lo[s] = low_half(dx, dy, dz);
-                    err = 1e-6f;
+                    err = VERT_ERR0;
                 }
             }
             const float d = x * x + y * y + z * z;
@@ -633,7 +632,6 @@ struct Tracer {
             sm.vp[s] = make_float4(x, y, z, err * sqrt_fast(d));
         }
         R2 = G.max(R2);
-        if (F64) R2d = G.maxd(R2d);
 #pragma unroll
         for (int i = 0; i < (NP + 31) / 32; ++i)
 #pragma unroll
@@ -1096,7 +1094,7 @@ __device__ __forceinline__ int walk(const TraceArgs& A, const GridDesc& grid, in
     float l0 = 0, l1 = 0, l2 = 0, h0 = 0, h1 = 0, h2 = 0;
     for (int s = lane; s < nf; s += 32) {
         const float4 v = far[s];
-        const float r = sqrt_fast(v.x * v.x + v.y * v.y + v.z * v.z) * (1.0f + 1e-4f);
+        const float r = sqrt_fast(v.x * v.x + v.y * v.y + v.z * v.z) * FAR_BALL;
         l0 = fminf(l0, v.x - r); h0 = fmaxf(h0, v.x + r);
         l1 = fminf(l1, v.y - r); h1 = fmaxf(h1, v.y + r);
         l2 = fminf(l2, v.z - r); h2 = fmaxf(h2, v.z + r);
@@ -1168,7 +1166,7 @@ __device__ __forceinline__ int walk(const TraceArgs& A, const GridDesc& grid, in
                         const float4 v = far[k];
                         const float bx = fmaxf(fmaxf(gx0 - pi.x - v.x, v.x - (gx1 - pi.x)), 0.0f);
                         const float by = fmaxf(fmaxf(gy0 - pi.y - v.y, v.y - (gy1 - pi.y)), 0.0f);
-                        const float left = (v.x * v.x + v.y * v.y + v.z * v.z) * (1.0f + 2e-4f) - (bx * bx + by * by);
+                        const float left = (v.x * v.x + v.y * v.y + v.z * v.z) * (FAR_BALL * FAR_BALL) - (bx * bx + by * by);
                         const float half = sqrt_fast(fmaxf(left, 0.0f));
                         if (left >= 0.0f) {
                             s0 = fminf(s0, v.z - half);
@@ -1330,7 +1328,7 @@ __device__ __forceinline__ int far_vertices(const Sub<TT>& G, const S& sm, bool 
 {
     int nf = 0;
     const int vmax = __reduce_max_sync(TFULL, on ? V : 0);
-    const float half = 0.25f * reach * (1.0f - 1e-4f);
+    const float half = 0.25f * reach * (1.0f / FAR_R2);
 #pragma unroll 1
     for (int s0 = 0; s0 < vmax; s0 += TT) {
         const int s = s0 + G.gl;  // (the slots are a multiple of TT)
@@ -1465,7 +1463,7 @@ __global__ void __launch_bounds__(TRACE_BLOCK, (sizeof(Real) == 4 ? TRACE_MINB :
         t.solve(G, sm, pi, grid, A.sorted, T::UNIT_F64, T::UNIT_MIN);
         t.certify(G, sm);
         // security radius
-        const bool valid = all || (A.round == 0 && 4.0f * t.R2 <= reach * (1.0f - 1e-5f));
+        const bool valid = all || (A.round == 0 && 4.0f * FAR_R2 * t.R2 <= reach);
         const bool open = act && t.ok && !valid;
         if (A.round == 0) {
             const int within = t.listed_within(G, sm);
@@ -1494,7 +1492,7 @@ __global__ void __launch_bounds__(TRACE_BLOCK, (sizeof(Real) == 4 ? TRACE_MINB :
             h->nf = nf;
             h->turns = A.round + (open ? 1 : 0);
             h->reach = reach;
-            h->all2 = 4.0f * t.R2 * (1.0f + 2e-5f);
+            h->all2 = 4.0f * FAR_R2 * t.R2;
         }
         __syncwarp();
     }
@@ -1621,12 +1619,12 @@ __global__ void __launch_bounds__(TAIL_BLOCK, 4) k_trace_tail(const __grid_const
             if (!t.ok || t.faces.count() > REC_FACES) break;
             bool valid = all;
             if (turn == 0) {
-                valid = all || 4.0f * t.R2 <= reach * (1.0f - 1e-5f);
+                valid = all || 4.0f * FAR_R2 * t.R2 <= reach;
                 n_open += !valid;
                 n_second += A.k_first > 0 && t.listed_within(G, m.t) > A.k_first;
                 walks += !valid;
             }
-            const float all2 = 4.0f * t.R2 * (1.0f + 2e-5f);
+            const float all2 = 4.0f * FAR_R2 * t.R2;
             if (!valid && all2 > reach) {
                 const int F = t.faces.count();
                 const int nf = far_vertices<TT>(G, m.t, true, t.V, reach, m.far);
