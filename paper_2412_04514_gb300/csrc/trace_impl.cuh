@@ -799,49 +799,58 @@ __device__ __forceinline__ void trace_finish(TraceSmem<Real, NP, NV>& sm, const 
             z = p.z;
         }
     };
-    // tetrahedra (0, foot of face, v, next(v around the face))
-    Real vol = 0, mx = 0, my = 0, mz = 0, m2 = 0;
+    // tetrahedra (0, foot of face, v, next(v around the face)); float sums of three
+    // edges' six, FP64 between them
+    double s0[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
     const float fix = 1048576.0f * rcp_fast(R2);
 #pragma unroll 1
-    for (int e = gl < 8 ? gl : E; e < E; e += 8) {
-        const uint32_t ed = sm.ed[e];
-        Real ax, ay, az, bx, by, bz;
-        vert((ed >> 16) & 0xff, ax, ay, az);
-        vert(ed >> 24, bx, by, bz);
-        const Real cx = ay * bz - az * by, cy = az * bx - ax * bz, cz = ax * by - ay * bx;
-        const Real ab2 = ax * ax + ay * ay + az * az + bx * bx + by * by + bz * bz;
-        const Real tx = ax + bx, ty = ay + by, tz = az + bz;
+    for (int e0 = gl < 8 ? gl : E; e0 < E; e0 += 24) {
+        Real vol = 0, mx = 0, my = 0, mz = 0, m2 = 0;
+#pragma unroll 1
+        for (int e = e0; e < E && e < e0 + 24; e += 8) {
+            const uint32_t ed = sm.ed[e];
+            Real ax, ay, az, bx, by, bz;
+            vert((ed >> 16) & 0xff, ax, ay, az);
+            vert(ed >> 24, bx, by, bz);
+            const Real cx = ay * bz - az * by, cy = az * bx - ax * bz, cz = ax * by - ay * bx;
+            const Real ab2 = ax * ax + ay * ay + az * az + bx * bx + by * by + bz * bz;
+            const Real tx = ax + bx, ty = ay + by, tz = az + bz;
 #pragma unroll
-        for (int t = 0; t < 2; ++t) {
-            const int f = vt_ck((ed >> (8 * t)) & 0xff, NP, CK_PLANE, A.st);
-            Real px, py, pz, sc;
-            plane(f, px, py, pz, sc);
-            const Real qx = px * sc, qy = py * sc, qz = pz * sc;
-            const Real qc = qx * cx + qy * cy + qz * cz;
-            const Real dv = qc * (Real)(t ? 1.0 / 6.0 : -1.0 / 6.0);
-            const Real sx = qx + tx, sy = qy + ty, sz = qz + tz;
-            const Real q2 = qx * qx + qy * qy + qz * qz;
-            vol += dv;
-            mx += dv * sx;
-            my += dv * sy;
-            mz += dv * sz;
-            m2 += dv * (q2 + ab2 + sx * sx + sy * sy + sz * sz);
-            if (A.rec) {  // twice the triangle's signed area is q.c / |q|
-                const float a2 = (float)qc * rsqrt_fast((float)q2) * fix;
-                atomicAdd(&sm.u.f[f], __float2int_rn(t ? a2 : -a2));
+            for (int t = 0; t < 2; ++t) {
+                const int f = vt_ck((ed >> (8 * t)) & 0xff, NP, CK_PLANE, A.st);
+                Real px, py, pz, sc;
+                plane(f, px, py, pz, sc);
+                const Real qx = px * sc, qy = py * sc, qz = pz * sc;
+                const Real qc = qx * cx + qy * cy + qz * cz;
+                const Real dv = qc * (Real)(t ? 1.0 / 6.0 : -1.0 / 6.0);
+                const Real sx = qx + tx, sy = qy + ty, sz = qz + tz;
+                const Real q2 = qx * qx + qy * qy + qz * qz;
+                vol += dv;
+                mx += dv * sx;
+                my += dv * sy;
+                mz += dv * sz;
+                m2 += dv * (q2 + ab2 + sx * sx + sy * sy + sz * sz);
+                if (A.rec) {  // twice the triangle's signed area is q.c / |q|
+                    const float a2 = (float)qc * rsqrt_fast((float)q2) * fix;
+                    atomicAdd(&sm.u.f[f], __float2int_rn(t ? a2 : -a2));
+                }
             }
         }
+        s0[0] += (double)vol;
+        s0[1] += (double)mx;
+        s0[2] += (double)my;
+        s0[3] += (double)mz;
+        s0[4] += (double)m2;
     }
     // FP64 sums over the 8 lanes by reduce-scatter: 7 additions instead of 15
     double w;
     {
-        const double s0[8] = {(double)vol, (double)mx, (double)my, (double)mz, (double)m2, 0.0, 0.0, 0.0};
         double t4[4], t2[2];
         const bool hi1 = (gl & 4) != 0, hi2 = (gl & 2) != 0, hi3 = (gl & 1) != 0;
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
-            const double send = hi1 ? s0[i] : s0[4 + i];
-            t4[i] = (hi1 ? s0[4 + i] : s0[i]) + __shfl_xor_sync(TFULL, send, 4);
+            const double up = i == 0 ? s0[4] : 0.0, send = hi1 ? s0[i] : up;
+            t4[i] = (hi1 ? up : s0[i]) + __shfl_xor_sync(TFULL, send, 4);
         }
 #pragma unroll
         for (int i = 0; i < 2; ++i) {
