@@ -143,3 +143,31 @@ def test_lloyd_step_kernel_moves_wraps_and_clamps():
     assert np.array_equal(per[0], want[0])
     assert np.array_equal(per[1], np.array([0.25, 0.5, 0.2], np.float32))
     assert per[2, 0] == 0.0  # rounds onto hi: belongs at lo
+
+
+def one_cell_of_triangles(faces):
+    """Points and cells of one cell whose `faces` faces are one and the same triangle, each across to a
+    neighbour of its own at one and the same place (for the kernel's sums, not a tessellation)."""
+    n = faces + 1
+    pts = torch.tensor([[0.5, 0.5, 0.5]] + [[0.75, 0.5, 0.5]] * faces, device="cuda")
+    i64 = dict(dtype=torch.int64, device="cuda")
+    vtx = torch.tensor([[0.625, 0.5, 0.5], [0.625, 0.75, 0.5], [0.625, 0.5, 0.75]], dtype=torch.float64, device="cuda")
+    one = [0] + [1] * n
+    cells = vt.Cells(vol=torch.ones(n, dtype=torch.float64, device="cuda"), cen=pts.double(),
+                     vtx_off=torch.tensor([3 * e for e in one], **i64), vtx=vtx,
+                     face_off=torch.tensor([faces * e for e in one], **i64),
+                     face_nbr=torch.arange(1, n, dtype=torch.int32, device="cuda"),
+                     face_vtx_off=torch.arange(0, 3 * faces + 1, 3, **i64),
+                     face_vtx=torch.tensor([0, 1, 2] * faces, dtype=torch.int32, device="cuda"))
+    return pts, cells
+
+
+def test_fp32_face_sums_keep_the_rounding_of_their_additions():
+    # 24 equal faces, three to a lane, of weights 2^26, 1 and -2^26: the large ones
+    # cancel exactly, and adding 1 to 2^26 in float32 alone would lose it
+    pts, cells = one_cell_of_triangles(24)
+    gV = torch.zeros(25, dtype=torch.float64, device="cuda")
+    gV[1:9], gV[9:17], gV[17:25] = 2.0 ** 26, 1.0, -2.0 ** 26
+    got, want = (vt.moments_adjoint(pts, cells, gV=gV, precision=p)[0] for p in ("fp32", "fp64"))
+    assert float(want.abs().min()) > 1e-3
+    torch.testing.assert_close(got, want, rtol=1e-6, atol=0)
