@@ -60,10 +60,10 @@ __device__ __forceinline__ Dens<Real> density(int i, double px, double py, doubl
     d.bx = d.by = d.bz = (Real)0;
     d.a = gV ? (Real)gV[i] : (Real)0;
     if (gC) {  // gV + b.(x - c) with x = y + p, b = gC / V
-        const Real iv = (Real)1 / (Real)vol[i];
-        d.bx = (Real)gC[3 * i] * iv;
-        d.by = (Real)gC[3 * i + 1] * iv;
-        d.bz = (Real)gC[3 * i + 2] * iv;
+        const Real V = (Real)vol[i];  // (divided, not times a reciprocal: one rounding; 1M cells, FP64: 30.1 -> 30.8 ms)
+        d.bx = (Real)gC[3 * i] / V;
+        d.by = (Real)gC[3 * i + 1] / V;
+        d.bz = (Real)gC[3 * i + 2] / V;
         d.a += d.bx * (Real)(px - cen[3 * i]) + d.by * (Real)(py - cen[3 * i + 1]) +
                d.bz * (Real)(pz - cen[3 * i + 2]);
     }

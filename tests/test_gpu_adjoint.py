@@ -171,3 +171,18 @@ def test_fp32_face_sums_keep_the_rounding_of_their_additions():
     got, want = (vt.moments_adjoint(pts, cells, gV=gV, precision=p)[0] for p in ("fp32", "fp64"))
     assert float(want.abs().min()) > 1e-3
     torch.testing.assert_close(got, want, rtol=1e-6, atol=0)
+
+
+def test_centroid_weights_are_quotients():
+    # gC / V of a cell enters as one correctly rounded quotient: the gradient for
+    # (gC, V) is that for (gC / V, 1), bit for bit, whatever V
+    rng = np.random.default_rng(3)
+    pts, cells = one_cell_of_triangles(24)
+    cells.cen = cells.cen + dev(0.01 * rng.standard_normal((25, 3)))
+    for prec, dt in (("fp64", np.float64), ("fp32", np.float32)):
+        gC, V = rng.standard_normal((25, 3)).astype(dt), (0.1 + rng.random(25)).astype(dt)
+        cells.vol = dev(V.astype(np.float64))
+        a = vt.moments_adjoint(pts, cells, gC=dev(gC.astype(np.float64)), precision=prec)
+        cells.vol = torch.ones(25, dtype=torch.float64, device="cuda")
+        b = vt.moments_adjoint(pts, cells, gC=dev((gC / V[:, None]).astype(np.float64)), precision=prec)
+        assert torch.equal(a, b), prec
