@@ -190,13 +190,20 @@ typedef struct vt_set_desc {
 #define VT_MAX_PASSES 16
 
 typedef struct vt_stats {
-    int passes;                          /* clip passes run (1 + doubling passes + exhaustive) */
+    int passes;                          /* clip passes run (1 + doubling passes + exhaustive). A call whose
+                                            cells are traced builds them from their whole lists at once; its
+                                            entries are the passes that the lists stand for */
     int k_of_pass[VT_MAX_PASSES];        /* k of each pass (0 = exhaustive pass) */
-    int64_t cells_of_pass[VT_MAX_PASSES];/* cells entering each pass */
-    int64_t exhaustive_cells;            /* cells finished by the exhaustive pass */
-    int64_t capacity_retries;            /* cells re-run because a polyhedron outgrew its slots */
-    int64_t precision_retries;           /* FP32 cells re-run in FP64 after an inconsistency */
-    int64_t fp64_rechecks;               /* FP32 sign / radius tests re-decided in FP64 */
+    int64_t cells_of_pass[VT_MAX_PASSES];/* cells entering each pass (traced: cells that the nearest k of the
+                                            pass before leave open) */
+    int64_t exhaustive_cells;            /* cells finished by the exhaustive pass (traced: cells that looked
+                                            at generators beyond their lists, and those the clipper finished) */
+    int64_t capacity_retries;            /* cells re-run because a polyhedron outgrew its slots (traced: its
+                                            vertices or open edges) */
+    int64_t precision_retries;           /* FP32 cells re-run in FP64 after an inconsistency (traced: built
+                                            again along FP64 rays) */
+    int64_t fp64_rechecks;               /* FP32 sign / radius tests re-decided in FP64 (traced: tests of a
+                                            vertex against a plane too close for float32) */
     int64_t unvalidated;                 /* cells left without a validated cell */
     int grid_res;                        /* G used */
     int launches;                        /* kernels launched by the call */
@@ -214,8 +221,9 @@ typedef struct vt_stats {
     int64_t knn_queries;                 /* queries they answered */
     int64_t walk_cells;                  /* walks over the grid shells within 2R of a cell in the last
                                             pass (range lists and the exhaustive walk; a cell whose
-                                            range list overflows walks twice) */
-    int64_t walk_candidates;             /* generators those walks examined. Most cells walking with
+                                            range list overflows walks twice; a traced cell counts once) */
+    int64_t walk_candidates;             /* generators those walks examined (traced: by all the walks of a
+                                            cell, so more than n per cell can be). Most cells walking with
                                             about n each means near-degenerate input (coplanar or
                                             collinear generators: every cell reaches the walls), whose
                                             cost grows as n^2 */

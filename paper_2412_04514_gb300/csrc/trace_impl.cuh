@@ -555,7 +555,10 @@ struct Tracer {
                     const int at = gl + i * TT;
                     o[i] = at == s1 ? a | (h << 8) | (V << 16) : (at == s2 ? h | (b << 8) | (V << 16) : o[i]);
                 }
-                if ((!c1 && s1 >= SLOTS) || (!c2 && (unsigned)s2 >= (unsigned)SLOTS)) ok = run = false;
+                if ((!c1 && s1 >= SLOTS) || (!c2 && (unsigned)s2 >= (unsigned)SLOTS)) {
+                    ok = run = false;
+                    E = NE;  // (see outgrown)
+                }
                 live = (live | ((Live)1 << (s1 & TOP)) | ((Live)1 << (s2 & TOP))) & (((Live)1 << SLOTS) - 1u);
                 E += 1 + c1 + c2;
                 ++V;
@@ -564,6 +567,9 @@ struct Tracer {
             __syncwarp();
         }
     }
+
+    // whether the polyhedron that failed had more vertices or open edges than there are places
+    __device__ __forceinline__ bool outgrown() const { return V >= NV || E > NE - 3; }
 
     // the vertices from their planes (in the arithmetic of the form), R, the faces
     __device__ __forceinline__ void solve(const Sub<TT>& G, S& sm, float4 pi, const GridDesc& grid,
@@ -717,7 +723,8 @@ struct Tracer {
     // the same with FP64 where float32 does not decide: a plane too close to a
     // vertex passes when the vertex, solved in FP64, is inside it by 1e-8 |n| |v|,
     // ten times what FP64 leaves at UNIT_MIN64 (a warp per cell only)
-    __device__ __forceinline__ void certify64(const Sub<TT>& G, const S& sm, const double (*pd)[4], const float4* lo)
+    __device__ __forceinline__ void certify64(const Sub<TT>& G, const S& sm, const double (*pd)[4], const float4* lo,
+                                              unsigned& decided)
     {
         bool fine = ok && 2 * E == 3 * V;
         const int vmax = __any_sync(TFULL, !ok) ? 0 : V;
@@ -731,6 +738,7 @@ struct Tracer {
                 const bool own = p == (int)(ids & 0xff) || p == (int)((ids >> 8) & 0xff) || p == (int)((ids >> 16) & 0xff);
                 const float d = fmaf(-nx[r], v.x, fmaf(-ny[r], v.y, fmaf(-nz[r], v.z, nb[r])));
                 if (own || d >= v.w) continue;
+                ++decided;
                 double x, y, z;
                 if constexpr (F64) {
                     x = sm.v[s][0];
@@ -1487,6 +1495,7 @@ __global__ void __launch_bounds__(TRACE_BLOCK, (sizeof(Real) == 4 ? TRACE_MINB :
         trace_finish<Real, TT, T::NP, NV, PER>(sm, G, act && t.ok ? t.V : 0, t.faces, t.R2, pi, out_idx, A);
         const bool failed = act && !t.ok;
         if (!__any_sync(TFULL, open || failed)) continue;
+        if (failed && gl == 0 && t.outgrown()) atomicAdd(&A.st->capacity_events, 1ull);
         append(A.open_list, A.open_ctr, open && gl == 0, q, G.lane);
         append(A.tail_list, A.tail_ctr, failed && gl == 0, q, G.lane);
         // its faces, or all planes of a failed one
@@ -1544,7 +1553,7 @@ __global__ void __launch_bounds__(TAIL_BLOCK, 4) k_trace_tail(const __grid_const
     }
     int begin = 0;
     if (A.from_dev) begin = ::max(*A.from_dev, A.from);
-    unsigned walks = 0, cands = 0, n_open = 0, n_second = 0;
+    unsigned walks = 0, cands = 0, n_open = 0, n_second = 0, rechecks = 0;
     for (;;) {
         int c = 0;
         if (lane == 0) c = begin + atomicAdd(A.queue, 1);
@@ -1620,10 +1629,14 @@ __global__ void __launch_bounds__(TAIL_BLOCK, 4) k_trace_tail(const __grid_const
             }
 #pragma unroll 1
             for (int again = traced ? 0 : 1; again < 2 && !t.ok; ++again) {
-                if (again == 1) t.template trace<double>(G, m.t, gen0 != 0, f0, m.pd, m.far);
-                else t.ok = true;
+                if (again == 1) {
+                    if (!F64 && lane == 0) atomicAdd(&A.st->precision_events, 1ull);
+                    t.template trace<double>(G, m.t, gen0 != 0, f0, m.pd, m.far);
+                } else {
+                    t.ok = true;
+                }
                 t.solve(G, m.t, pi, grid, A.sorted, 2.0f, again == 0 ? T::UNIT_MIN : -1.0f, m.far);
-                t.certify64(G, m.t, m.pd, m.far);
+                t.certify64(G, m.t, m.pd, m.far, rechecks);
             }
             if (!t.ok || t.faces.count() > REC_FACES) break;
             bool valid = all;
@@ -1654,11 +1667,15 @@ __global__ void __launch_bounds__(TAIL_BLOCK, 4) k_trace_tail(const __grid_const
         const int64_t out_idx = A.index_space == VT_INDEX_ORIGINAL ? (int64_t)__float_as_int(pi.w) : (int64_t)q;
         if (done)
             trace_finish<Real, TT, T::NP, NV, PER>(m.t, G, t.V, t.faces, t.R2, pi, out_idx, A);
-        else if (lane == 0)
+        else if (lane == 0) {
             A.slow_list[atomicAdd(A.slow_ctr, 1)] = q;
+            if (!t.ok && t.outgrown()) atomicAdd(&A.st->capacity_events, 1ull);
+        }
         __syncwarp();
     }
+    if (!F64) rechecks = __reduce_add_sync(TFULL, rechecks);
     if (lane == 0) {
+        if (!F64 && rechecks) atomicAdd(&A.st->fp64_rechecks, (unsigned long long)rechecks);
         if (walks) atomicAdd(&A.st->walk_cells, (unsigned long long)walks);
         if (cands) atomicAdd(&A.st->walk_cands, (unsigned long long)cands);
         if (n_open) atomicAdd(&A.st->n_open, (int)n_open);

@@ -232,6 +232,26 @@ def test_fused_schedule_in_parts(lattice, prec):
     assert torch.equal(again.vol, b.vol) and torch.equal(again.nbr[:int(b.nbr_off[-1])], b.nbr[:int(b.nbr_off[-1])])
 
 
+def test_retries_and_rechecks_are_counted():
+    # a lattice moved by 1e-4 of its spacing has planes within float32 round-off of
+    # most cells' vertices, and a shell of 60 generators gives a cell of more than
+    # the 48 vertices of a group (beside enough points that groups run)
+    rng = np.random.default_rng(2)
+    x = W.cubic_lattice(20)
+    x = (x + rng.uniform(-1e-4 / 20, 1e-4 / 20, x.shape)).astype(np.float32)
+    s = vt.tessellate(torch.from_numpy(x).cuda(), vt.Params(emit=("vol",))).stats
+    assert s["fp64_rechecks"] > len(x) // 4 and s["precision_retries"] > len(x) // 100, s
+    d = rng.standard_normal((60, 3))
+    shell = 0.5 + (0.2 + 1e-3 * rng.random((60, 1))) * d / np.linalg.norm(d, axis=1, keepdims=True)
+    far = rng.random((20_000, 3))
+    far = far[np.linalg.norm(far - 0.5, axis=1) > 0.42]
+    x = torch.from_numpy(np.concatenate([[[0.5, 0.5, 0.5]], shell, far]).astype(np.float32)).cuda()
+    for prec in ("fp32", "fp64"):
+        s = vt.tessellate(x, vt.Params(precision=prec, emit=("vol",))).stats
+        assert s["capacity_retries"] >= 1 and s["unvalidated"] == 0, s
+    assert s["fp64_rechecks"] == 0  # (of the FP32 form)
+
+
 def test_differentiable_moments_free_their_cells():
     # after a step only its gradient is left: the cells are not kept by a cycle
     # between the outputs and their node
