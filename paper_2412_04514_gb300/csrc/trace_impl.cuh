@@ -257,6 +257,8 @@ struct Tracer {
     static constexpr float UNIT_MIN = 2e-5f, UNIT_MIN64 = 1e-7f;
     // (below UNIT_F64 the FP32 form solves a vertex in FP64, about 1 in 3,000)
     static constexpr float UNIT_F64 = vt::UNIT_F64;
+    static constexpr float REGULAR = 2e-6f;
+    static constexpr double TIE = 1e-13;             // of |n| |v|: FP64 does not tell the plane from the vertex
     static constexpr int SR = 2;                     // registers of open edge ends per lane
     using Live = typename LiveMask<TT>::T;           // a bit per slot; the top bit takes the edges that closed
     static constexpr int TOP = 8 * sizeof(Live) - 1;
@@ -635,7 +637,7 @@ struct Tracer {
             const float d = x * x + y * y + z * z;
             if (__float_as_uint(d) - __float_as_uint(SQUARE_MIN) >= 0x7f800000u - __float_as_uint(SQUARE_MIN)) ok = false;
             R2 = fmaxf(R2, d);
-            sm.vp[s] = make_float4(x, y, z, err * sqrt_fast(d));
+            sm.vp[s] = make_float4(x, y, z, TT < 32 && far_scale ? -INFINITY : err * sqrt_fast(d));
         }
         R2 = G.max(R2);
 #pragma unroll
@@ -681,48 +683,80 @@ struct Tracer {
         near = G.bcast(G.incl_scan(near), TT - 1);
         ok = !G.any(!ok) && near == 3 * V && 2 * E == 3 * V;
     }
+    // whether a vertex found so far that no generator beyond `reach` cuts has a
+    // fourth plane within its error bound or behind it
+    __device__ __forceinline__ bool close_vertex(const Sub<TT>& G, const S& sm, bool on, float reach) const
+    {
+        bool found = false;
+        const int vmax = __reduce_max_sync(TFULL, on ? V : 0);
+#pragma unroll 1
+        for (int s = 0; s < vmax; ++s) {
+            const float4 v = sm.vp[s];
+            const bool is = on && !found && s < V && 4.0f * (v.x * v.x + v.y * v.y + v.z * v.z) <= reach;
+            if (!__any_sync(TFULL, is)) continue;
+            int near = near_rows<NR>(v, v.w);
+#pragma unroll
+            for (int o = TT / 2; o >= 1; o >>= 1) near += __shfl_xor_sync(TFULL, near, o);
+            found = found || (is && near > 3);
+        }
+        return found;
+    }
     // a fourth plane at a vertex found so far (a warp per cell only): 2 when one
-    // passes through it to what FP64 resolves, as certify64 would find at length,
-    // 1 when one is close, 0 when neither. The first two such vertices tell.
+    // passes through it to what FP64 resolves, as certify64 would find at length
+    // (the first two such vertices tell), or when so `many` vertices within half the
+    // reach have one within REGULAR |v|, 1 when one is close, 0 when none is.
     // (343,000 points of a cubic lattice, every cell tied: 169 ms when each ran
     // through the walk and the FP64 rays first, now 60 ms, against 51 ms with the
     // clipper alone; 512,000 of a BCC lattice 19.0 -> 5.0 ms)
     __device__ __forceinline__ int tied(const Sub<TT>& G, const S& sm, const float4* __restrict__ sorted, float4 pi,
-                                        const GridDesc& grid) const
+                                        const GridDesc& grid, float reach, int many) const
     {
-        int close = 0;
+        int close = 0, tights = 0;
 #pragma unroll 1
-        for (int s = 0; s < V && close < 2; ++s) {
+        for (int s = 0; s < V; ++s) {
             const float4 v = sm.vp[s];
             const uint32_t ids = *reinterpret_cast<const uint32_t*>(sm.vid[s]);
             const int a = ids & 0xff, b = (ids >> 8) & 0xff, c = (ids >> 16) & 0xff;
+            const float v2 = v.x * v.x + v.y * v.y + v.z * v.z;
             int at = -1;
+            bool tight = false;
 #pragma unroll
             for (int r = 0; r < NR; ++r) {
                 const int p = r * TT + G.gl;
-                const float d = fmaf(-nx[r], v.x, fmaf(-ny[r], v.y, fmaf(-nz[r], v.z, nb[r])));
+                const float d = fabsf(fmaf(-nx[r], v.x, fmaf(-ny[r], v.y, fmaf(-nz[r], v.z, nb[r]))));
                 // (v.w is infinite where |v|^2 overflows: no finite distance keeps a padding plane out)
-                if (p != a && p != b && p != c && sm.src[p] != PAD_PLANE && fabsf(d) < v.w) at = p;
+                if (p != a && p != b && p != c && sm.src[p] != PAD_PLANE && d < v.w) {
+                    at = p;
+                    tight = tight || d * d < REGULAR * REGULAR * v2;
+                }
             }
             if (!__any_sync(TFULL, at >= 0)) continue;
+            tights += __any_sync(TFULL, tight) && 4.0f * v2 <= reach;
+            if (tights >= many) return 2;
+            if (++close > 2) {
+                if (tights == 0 || many == INT_MAX) break;
+                continue;
+            }
             bool tie = false;
             if (at >= 0) {
                 double x, y, z;
                 if (solve_vertex64<PER>(sm.src[a], sm.src[b], sm.src[c], sorted, pi, grid, x, y, z)) {
                     const P64 h = plane64<PER>(sm.src[at], sorted, pi, grid);
                     const double in = h.b - ((h.x * x + h.y * y) + h.z * z);
-                    const double n2 = (h.x * h.x + h.y * h.y) + h.z * h.z, v2 = (x * x + y * y) + z * z;
-                    tie = in * in < 1e-18 * (n2 * v2);
+                    const double n2 = (h.x * h.x + h.y * h.y) + h.z * h.z, w2 = (x * x + y * y) + z * z;
+                    tie = in * in < TIE * TIE * (n2 * w2);
                 }
             }
             if (__any_sync(TFULL, tie)) return 2;
-            ++close;
         }
         return close > 0 ? 1 : 0;
     }
     // the same with FP64 where float32 does not decide: a plane too close to a
-    // vertex passes when the vertex, solved in FP64, is inside it by 1e-8 |n| |v|,
-    // ten times what FP64 leaves at UNIT_MIN64 (a warp per cell only)
+    // vertex passes when the vertex, solved in FP64, is inside it by more than the
+    // error of that test (a warp per cell only). With e = 2^-53 a vertex of three
+    // planes is known to 32 e / |det| of its length (22 e for the three terms of
+    // Cramer's rule, 10 e for the determinant, both over |det| of the unit
+    // normals), its two float halves to 2^-48, and the test adds 6 e.
     __device__ __forceinline__ void certify64(const Sub<TT>& G, const S& sm, const double (*pd)[4], const float4* lo,
                                               unsigned& decided)
     {
@@ -732,27 +766,38 @@ struct Tracer {
         for (int s = 0; s < vmax; ++s) {
             const float4 v = sm.vp[s];
             const uint32_t ids = *reinterpret_cast<const uint32_t*>(sm.vid[s]);
+            const int a = ids & 0xff, b = (ids >> 8) & 0xff, c = (ids >> 16) & 0xff;
+            uint32_t close = 0;  // rows of the lane's planes too close (PAD_PLANE never is: its distance is FLT_MAX)
 #pragma unroll
             for (int r = 0; r < NR; ++r) {
                 const int p = r * TT + G.gl;
-                const bool own = p == (int)(ids & 0xff) || p == (int)((ids >> 8) & 0xff) || p == (int)((ids >> 16) & 0xff);
                 const float d = fmaf(-nx[r], v.x, fmaf(-ny[r], v.y, fmaf(-nz[r], v.z, nb[r])));
-                if (own || d >= v.w) continue;
-                ++decided;
-                double x, y, z;
-                if constexpr (F64) {
-                    x = sm.v[s][0];
-                    y = sm.v[s][1];
-                    z = sm.v[s][2];
-                } else {
-                    x = (double)v.x + (double)lo[s].x;
-                    y = (double)v.y + (double)lo[s].y;
-                    z = (double)v.z + (double)lo[s].z;
-                }
-                const double* h = pd[p];
+                close |= p != a && p != b && p != c && !(d >= v.w) ? 1u << r : 0u;
+            }
+            if (!__any_sync(TFULL, close != 0)) continue;
+            double x, y, z;
+            if constexpr (F64) {
+                x = sm.v[s][0];
+                y = sm.v[s][1];
+                z = sm.v[s][2];
+            } else {
+                x = (double)v.x + (double)lo[s].x;
+                y = (double)v.y + (double)lo[s].y;
+                z = (double)v.z + (double)lo[s].z;
+            }
+            const double *A = pd[a], *B = pd[b], *C = pd[c];
+            const double det = A[0] * (B[1] * C[2] - B[2] * C[1]) + A[1] * (B[2] * C[0] - B[0] * C[2]) +
+                               A[2] * (B[0] * C[1] - B[1] * C[0]);
+            const double aa = A[0] * A[0] + A[1] * A[1] + A[2] * A[2], bb = B[0] * B[0] + B[1] * B[1] + B[2] * B[2],
+                         cc = C[0] * C[0] + C[1] * C[1] + C[2] * C[2];
+            // (squared: the test's margin is (4.3e-15 + 3.6e-15 / |det|) |n| |v|)
+            const double m = 4.3e-15 + 3.6e-15 * sqrt(aa) * sqrt(bb) * sqrt(cc) / fabs(det);
+            const double lim = m * m * ((x * x + y * y) + z * z);
+            for (; close; close &= close - 1) {
+                const double* h = pd[(__ffs(close) - 1) * TT + G.gl];
                 const double in = h[3] - ((h[0] * x + h[1] * y) + h[2] * z);
-                const float4 n = sm.pl[p];
-                if (!(in > 1e-2 * (double)v.w * (double)sqrt_fast(n.x * n.x + n.y * n.y + n.z * n.z))) fine = false;
+                if (!(in > 0.0 && in * in > lim * ((h[0] * h[0] + h[1] * h[1]) + h[2] * h[2]))) fine = false;
+                ++decided;
             }
         }
         ok = !__any_sync(TFULL, !fine);
@@ -1046,7 +1091,8 @@ struct alignas(16) OpenCell {
     float reach;              // generators with a float key below this are behind it
     float all2;               // (2R)^2
     int32_t turns;            // times it was built
-    int32_t pad[3];
+    int32_t close;            // 1: failed with a fourth plane at a vertex (see close_vertex)
+    int32_t pad[2];
     int32_t src[40];          // its planes: the faces, then what cuts it
     float4 far[48];           // vertices a generator at `reach` or beyond can cut (see far_vertices)
 };
@@ -1479,6 +1525,7 @@ __global__ void __launch_bounds__(TRACE_BLOCK, (sizeof(Real) == 4 ? TRACE_MINB :
         __syncthreads();
         t.solve(G, sm, pi, grid, A.sorted, T::UNIT_F64, T::UNIT_MIN);
         t.certify(G, sm);
+        const bool close = A.round == 0 && __any_sync(TFULL, act && !t.ok) && t.close_vertex(G, sm, act && !t.ok, reach);
         // security radius
         const bool valid = all || (A.round == 0 && 4.0f * FAR_R2 * t.R2 <= reach);
         const bool open = act && t.ok && !valid;
@@ -1498,6 +1545,8 @@ __global__ void __launch_bounds__(TRACE_BLOCK, (sizeof(Real) == 4 ? TRACE_MINB :
         if (failed && gl == 0 && t.outgrown()) atomicAdd(&A.st->capacity_events, 1ull);
         append(A.open_list, A.open_ctr, open && gl == 0, q, G.lane);
         append(A.tail_list, A.tail_ctr, failed && gl == 0, q, G.lane);
+        const unsigned closes = __ballot_sync(TFULL, gl == 0 && close);
+        if (closes && G.lane == 0) atomicAdd(A.close_ctr, __popc(closes));
         // its faces, or all planes of a failed one
         const int F = t.faces.count();
         if (open)
@@ -1509,6 +1558,7 @@ __global__ void __launch_bounds__(TRACE_BLOCK, (sizeof(Real) == 4 ? TRACE_MINB :
             h->np = open ? F : P;
             h->nf = nf;
             h->turns = A.round + (open ? 1 : 0);
+            h->close = close;
             h->reach = reach;
             h->all2 = 4.0f * FAR_R2 * t.R2;
         }
@@ -1525,6 +1575,11 @@ __global__ void __launch_bounds__(TRACE_BLOCK, (sizeof(Real) == 4 ? TRACE_MINB :
 // of 32 planes instead of five of 8. A cell comes out the same bit for bit from
 // either kernel.
 constexpr int TAIL_BLOCK = 128;
+constexpr int TAIL_TURNS = 16, HARD_TURNS = 2;
+// close vertices of a cell in a call whose cells all run here, with no count to
+// go by, from which it is taken as one of a lattice (one degenerate vertex of a generic
+// cloud gives at most three): 8,000 points moved by 1e-5, 2.2 -> 1.4 ms
+constexpr int MANY_CLOSE = 6;
 constexpr int TAIL_KEEP = 32;  // cutting generators taken at once from the third turn on
 template <typename Real, bool PER>
 struct TailSmem {
@@ -1554,6 +1609,14 @@ __global__ void __launch_bounds__(TAIL_BLOCK, 4) k_trace_tail(const __grid_const
     int begin = 0;
     if (A.from_dev) begin = ::max(*A.from_dev, A.from);
     unsigned walks = 0, cands = 0, n_open = 0, n_second = 0, rechecks = 0;
+    // so many cells of the call have close vertices (a lattice whose points moved
+    // little): the clipper is faster than FP64 rays. 125,000 points of a cubic lattice
+    // moved by 1e-5 of the spacing: 24.6 -> 8.5 ms (clipper alone 7.8), FP64 form 30.9 ->
+    // 17.8 (16.7); by 1e-4 9.0 -> 3.8 (3.0), 11.6 -> 9.9 (14.0). Such cells are 0.02 to
+    // 0.1% of uniform and clumped clouds, 1.4% and 0.4% (FP64) of that lattice moved by
+    // 1e-2, 12 and 4% by 1e-3, 75 and 44% by 1e-4: the line lies at 1/16 in the FP32
+    // form and at 1/4 in the FP64 form, whose clipper takes five times as long.
+    const bool regular = A.round > 0 && *A.close_ctr > A.close_max;
     for (;;) {
         int c = 0;
         if (lane == 0) c = begin + atomicAdd(A.queue, 1);
@@ -1563,6 +1626,10 @@ __global__ void __launch_bounds__(TAIL_BLOCK, 4) k_trace_tail(const __grid_const
         const GridDesc& grid = grid_of(A.g, A.sets, A.set_of, q);
         const float4 pi = A.sorted[q];
         const OpenCell* h = reinterpret_cast<const OpenCell*>(A.state + (size_t)(A.kept ? c : q - A.first) * A.state_stride);
+        if (regular && h->close) {
+            if (lane == 0) A.slow_list[atomicAdd(A.slow_ctr, 1)] = q;
+            continue;
+        }
         int P;
         float reach;
         if (A.round == 0) {
@@ -1582,10 +1649,13 @@ __global__ void __launch_bounds__(TAIL_BLOCK, 4) k_trace_tail(const __grid_const
         T t;
         t.rows = NR;
         bool done = false, spread = false;
-        // (every turn adds a generator that cuts; the bound only ends what float
-        // round-off could keep turning)
+        int hard = 0;  // turns that took FP64 rays
+        // (every turn adds a generator that cuts; generic cells take fewer than
+        // TAIL_TURNS, and HARD_TURNS is what FP64 rays are worth: the 5,000 cells of a
+        // sphere's points, whose planes all pass within round-off of its centre, took 176 ms
+        // FP32 and 85 FP64 with 200 turns, with the clipper alone 123 and 34, now 123 and 30)
 #pragma unroll 1
-        for (int turn = A.round == 0 ? 0 : h->turns; turn < 200 && !done; ++turn) {
+        for (int turn = A.round == 0 ? 0 : h->turns; turn < TAIL_TURNS && !done; ++turn) {
 #pragma unroll
             for (int r = 0; r < NR; ++r) {
                 const int p = r * TT + lane;
@@ -1599,7 +1669,7 @@ __global__ void __launch_bounds__(TAIL_BLOCK, 4) k_trace_tail(const __grid_const
             const bool traced = t.ok;
             t.solve(G, m.t, pi, grid, A.sorted, T::UNIT_F64, T::UNIT_MIN);
             t.certify(G, m.t);
-            const int tied = t.ok ? 0 : t.tied(G, m.t, A.sorted, pi, grid);
+            const int tied = t.ok ? 0 : t.tied(G, m.t, A.sorted, pi, grid, reach, A.round == 0 ? MANY_CLOSE : INT_MAX);
             if (tied == 2) break;  // degenerate: nothing the rest of the turn could certify
             if (turn == 0 && !t.ok && !all && !spread && !(traced && tied)) {
                 // most often a list to one side of its generator
@@ -1630,6 +1700,7 @@ __global__ void __launch_bounds__(TAIL_BLOCK, 4) k_trace_tail(const __grid_const
 #pragma unroll 1
             for (int again = traced ? 0 : 1; again < 2 && !t.ok; ++again) {
                 if (again == 1) {
+                    ++hard;
                     if (!F64 && lane == 0) atomicAdd(&A.st->precision_events, 1ull);
                     t.template trace<double>(G, m.t, gen0 != 0, f0, m.pd, m.far);
                 } else {
@@ -1638,7 +1709,7 @@ __global__ void __launch_bounds__(TAIL_BLOCK, 4) k_trace_tail(const __grid_const
                 t.solve(G, m.t, pi, grid, A.sorted, 2.0f, again == 0 ? T::UNIT_MIN : -1.0f, m.far);
                 t.certify64(G, m.t, m.pd, m.far, rechecks);
             }
-            if (!t.ok || t.faces.count() > REC_FACES) break;
+            if (!t.ok || t.faces.count() > REC_FACES || hard > HARD_TURNS) break;
             bool valid = all;
             if (turn == 0) {
                 valid = all || 4.0f * FAR_R2 * t.R2 <= reach;

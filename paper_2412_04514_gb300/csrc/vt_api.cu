@@ -551,6 +551,7 @@ int trace_pass(const Ctx& c, const vt_params* p, int64_t n, int k, int k_list, i
     a.open_list = open;
     a.tail_list = tail;
     a.tail_ctr = &ctr[CTR_TAIL];
+    a.close_ctr = &ctr[CTR_CLOSE];
     a.st = c.st;
     int32_t* nbr = c.at<int32_t>(fused ? L.rob_nbr : L.knn_nbr);
     float* reach;
@@ -629,6 +630,7 @@ int trace_pass(const Ctx& c, const vt_params* p, int64_t n, int k, int k_list, i
             TraceArgs t = a;
             t.round = small ? 0 : TRACE_ROUNDS;
             t.tail = 1;
+            t.close_max = (first + m) / (p->precision == VT_FP64 ? 4 : 16);
             t.queries = small ? nullptr : tail;
             t.nq_dev = small ? nullptr : &ctr[CTR_TAIL];
             t.queue = &ctr[CTR_TQUEUE + 2 * TRACE_ROUNDS + all];

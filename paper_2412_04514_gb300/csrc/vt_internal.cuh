@@ -557,7 +557,8 @@ constexpr int CTR_TRACE = CTR_QUEUE + 1;            // open and next list of eac
 constexpr int CTR_TAIL = CTR_TRACE + 2 * TRACE_ROUNDS - 1;  // (the last next list)
 constexpr int CTR_SLOW = CTR_TAIL + 1;
 constexpr int CTR_KEPT = CTR_SLOW + 1;              // tail cells of the parts before
-constexpr int CTR_TQUEUE = CTR_KEPT + 1;            // a cell counter per launch of the pass
+constexpr int CTR_CLOSE = CTR_KEPT + 1;             // failed cells with close vertices
+constexpr int CTR_TQUEUE = CTR_CLOSE + 1;           // a cell counter per launch of the pass
 constexpr int CTR_COUNT = CTR_TQUEUE + 2 * TRACE_ROUNDS + 2;
 
 struct Layout {
@@ -700,6 +701,8 @@ struct TraceArgs {
     int32_t *next_list, *next_ctr;  // cells to build again (the walk's output)
     int32_t *tail_list, *tail_ctr;  // cells that failed: for the warp per cell
     int32_t *slow_list, *slow_ctr;  // cells for the plane-by-plane clipper
+    int32_t* close_ctr;       // failed cells with a fourth plane at a vertex; when there are more
+    int64_t close_max;        // than close_max, the warp per cell leaves them to the clipper
     DevStatus* st;
     int32_t* queue;           // the launch's cell counter (zero)
 };

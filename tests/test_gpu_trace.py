@@ -71,6 +71,25 @@ def test_many_faced_cells(around, prec):
     check(np.concatenate([[[0.5, 0.5, 0.5]], shell, far]).astype(np.float32), prec)
 
 
+@pytest.mark.parametrize("prec", ["fp32", "fp64"])
+@pytest.mark.parametrize("m,move", [(25, 1e-3), (25, 1e-4), (25, 1e-5), (12, 1e-4)])
+def test_lattices_that_moved_little(m, move, prec):
+    # most cells have planes within float32 round-off of their vertices. Where
+    # they are many, the clipper builds them and not the FP64 rays
+    rng = np.random.default_rng(m)
+    x = (W.cubic_lattice(m) + rng.uniform(-move / m, move / m, (m ** 3, 3))).astype(np.float32)
+    want = oracle.tessellate(x)
+    for kw in ({}, {"fused": True}):
+        cells = vt.tessellate(torch.from_numpy(x).cuda(), vt.Params(precision=prec, emit=("nbr", "vol", "cen"), **kw))
+        np.testing.assert_allclose(cells.vol.cpu().numpy(), want["vol"], rtol=TOL[prec])
+        np.testing.assert_allclose(cells.cen.cpu().numpy(), want["cen"], rtol=TOL[prec])
+        if prec == "fp64":
+            assert np.array_equal(cells.nbr_off.cpu().numpy(), want["nbr_off"])
+            assert np.array_equal(cells.nbr.cpu().numpy(), want["nbr"])
+        elif m == 25:
+            assert cells.stats["precision_retries"] < len(x) // 16
+
+
 def test_sums_of_many_edges():
     # the FP32 form's moments of cells of up to 60 faces (22 edges to a lane) are
     # no further off than the clipper's (k_max = 4 k0 is not traced), whose lanes
