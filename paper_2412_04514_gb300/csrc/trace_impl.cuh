@@ -1177,6 +1177,11 @@ __device__ __forceinline__ int walk(const TraceArgs& A, const GridDesc& grid, in
                 lim_hi = PER ? 3.0f * (float)Gr - 1.0f : (float)Gr - 1.0f;
     auto clamp = [&](float t) { return (int)floorf(fminf(fmaxf(t, lim_lo), lim_hi)); };
     int ns = 0;
+    // the farthest kept key once the list is full: what lies beyond it would be sorted
+    // in and dropped again (thousands of a clump's generators cut the sparse cells beside
+    // it: 30,000 points in one clump and 60 around it 17.6 -> 16.6 ms, 500,000 half in
+    // clumps, fused, 7.82 -> 7.51, 120,000 2.53 -> 2.50 ms)
+    float nearest = FLT_MAX;
     bool more = false, end = !SPREAD && nf == 0;
     if (SPREAD) {
         l0 = l1 = l2 = -FLT_MAX;
@@ -1297,7 +1302,7 @@ __device__ __forceinline__ int walk(const TraceArgs& A, const GridDesc& grid, in
                 const bool in = i < total && j != q;
                 if (in) o = img_off_t<PER>(pi, A.sorted[j], cd, grid);
                 const float d2 = fmaf(o.z, o.z, fmaf(o.y, o.y, o.x * o.x));
-                bool cuts = in && d2 >= reach && d2 < lim2;
+                bool cuts = in && d2 >= reach && d2 < lim2 && (SPREAD || d2 <= nearest);
                 if (!__any_sync(TFULL, cuts)) continue;
                 if (SPREAD) {
                     if (cuts)
@@ -1349,6 +1354,7 @@ __device__ __forceinline__ int walk(const TraceArgs& A, const GridDesc& grid, in
                 if (ns > keep) {
                     more = true;
                     ns = keep_nearest(key, id, ns, keep, lane);
+                    nearest = key[ns - 1];
                 }
             }
         }
