@@ -213,8 +213,8 @@ __global__ void __launch_bounds__(NEAR_BLOCK) k_near(const float4* __restrict__ 
                     if (!mask) continue;
                     if (in) {
                         const int at = cnt + __popc(mask & ((1u << lane) - 1u));
-                        key[at] = d2;
-                        id[at] = PER ? img_pack(j, cd) : j;
+                        key[vt_ck(at, NEAR_BUF, CK_RECORD, st)] = d2;
+                        id[vt_ck(at, NEAR_BUF, CK_RECORD, st)] = PER ? img_pack(j, cd) : j;
                     }
                     cnt += __popc(mask);
                     __syncwarp();
@@ -244,7 +244,7 @@ __global__ void __launch_bounds__(NEAR_BLOCK) k_near(const float4* __restrict__ 
         int32_t* out = nbr + (int64_t)c * kstride;
         for (int i = lane; i < k; i += 32) {
             const int from = i == 0 ? at : (i == at ? 0 : i);
-            out[i] = i < cnt ? id[from] : -1;
+            out[i] = i < cnt ? id[vt_ck(from, NEAR_BUF, CK_RECORD, st)] : -1;
         }
         if (lane == 0) reach_out[c] = all ? FLT_MAX : lim;
         __syncwarp();

@@ -268,6 +268,11 @@ struct Tracer {
     int rows;               // rows of planes in use over the warp
     bool ok;
     int V, E;
+    DevStatus* st;          // (the debug build's index checks)
+    // indices that come from data: a plane, a vertex, an edge
+    __device__ __forceinline__ int plane_ck(int p) const { return vt_ck(p, NP, CK_PLANE, st); }
+    __device__ __forceinline__ int vertex_ck(int s) const { return vt_ck(s, NV, CK_SLOT, st); }
+    __device__ __forceinline__ int edge_ck(int e) const { return vt_ck(e, NE, CK_EDGE, st); }
     float R2;               // max |v|^2
     Faces<(NP + 31) / 32> faces;  // the planes that are faces
 
@@ -468,7 +473,7 @@ struct Tracer {
                 const int hit = hit_of(vx, vy, vz, dx, dy, dz,
                                        e == 0 ? 1e-3f * sm.u.nl[f0] : LEAST * sm.u.nl[f0] * sm.u.nl[f1]);
                 ok = ok && hit >= 0;
-                h = ok ? hit : f0;
+                h = plane_ck(ok ? hit : f0);
                 advance(vx, vy, vz, dx, dy, dz, h);
                 if (e == 0) {
                     f1 = h;
@@ -500,7 +505,7 @@ struct Tracer {
 #pragma unroll
             for (int i = 0; i < SR; ++i) o[i] = gl + i * TT == slot ? -1 : o[i];
             const int ent = run ? got : 0;
-            const int a = ent & 0xff, b = (ent >> 8) & 0xff, w = ent >> 16;
+            const int a = plane_ck(ent & 0xff), b = plane_ck((ent >> 8) & 0xff), w = vertex_ck(ent >> 16);
             W vx, vy, vz, ax, ay, az, bx, by, bz, unused;
             {
                 const float4 v = sm.vp[w];
@@ -522,7 +527,7 @@ struct Tracer {
                 ok = ok && !run;
                 run = false;
             }
-            const int h = run ? hit : 0;
+            const int h = plane_ck(run ? hit : 0);
             advance(vx, vy, vz, dx, dy, dz, h);
             // the vertex (b, a, h): its other two edges, (a, h) and (h, b), close
             // against an open end of the same edge, (h, a) or (b, h), or stay open
@@ -538,16 +543,16 @@ struct Tracer {
             for (int i = 0; i < SR; ++i) {
                 const int k = o[i] & 0xffff;
                 if (k == k1 || k == k2) {
-                    sm.ed[E + (k == k1 ? 1 : 1 + c1)] = (uint32_t)o[i] | ((uint32_t)V << 24);
+                    sm.ed[edge_ck(E + (k == k1 ? 1 : 1 + c1))] = (uint32_t)o[i] | ((uint32_t)V << 24);
                     o[i] = -1;
                 }
             }
             live = (Live)G.ballot(o[0] >= 0) | ((Live)G.ballot(o[1] >= 0) << TT);
             if (run) {
                 if (gl == 0) {
-                    put(V, vx, vy, vz);
+                    put(vertex_ck(V), vx, vy, vz);
                     *reinterpret_cast<uint32_t*>(sm.vid[V]) = (uint32_t)b | ((uint32_t)a << 8) | ((uint32_t)h << 16);
-                    sm.ed[E] = (uint32_t)ent | ((uint32_t)V << 24);
+                    sm.ed[edge_ck(E)] = (uint32_t)ent | ((uint32_t)V << 24);
                 }
                 // the lowest free slots take what stays open (an edge that closed: no slot)
                 const Live free1 = ~live, free2 = c1 ? free1 : free1 & (free1 - 1u);
@@ -583,7 +588,7 @@ struct Tracer {
 #pragma unroll 1
         for (int s = G.gl; s < V; s += TT) {
             const uint32_t ids = *reinterpret_cast<const uint32_t*>(sm.vid[s]);
-            const int a = ids & 0xff, b = (ids >> 8) & 0xff, c = (ids >> 16) & 0xff;
+            const int a = plane_ck(ids & 0xff), b = plane_ck((ids >> 8) & 0xff), c = plane_ck((ids >> 16) & 0xff);
             faces.add(a);
             faces.add(b);
             faces.add(c);
@@ -716,7 +721,7 @@ struct Tracer {
         for (int s = 0; s < V; ++s) {
             const float4 v = sm.vp[s];
             const uint32_t ids = *reinterpret_cast<const uint32_t*>(sm.vid[s]);
-            const int a = ids & 0xff, b = (ids >> 8) & 0xff, c = (ids >> 16) & 0xff;
+            const int a = plane_ck(ids & 0xff), b = plane_ck((ids >> 8) & 0xff), c = plane_ck((ids >> 16) & 0xff);
             const float v2 = v.x * v.x + v.y * v.y + v.z * v.z;
             int at = -1;
             bool tight = false;
@@ -766,7 +771,7 @@ struct Tracer {
         for (int s = 0; s < vmax; ++s) {
             const float4 v = sm.vp[s];
             const uint32_t ids = *reinterpret_cast<const uint32_t*>(sm.vid[s]);
-            const int a = ids & 0xff, b = (ids >> 8) & 0xff, c = (ids >> 16) & 0xff;
+            const int a = plane_ck(ids & 0xff), b = plane_ck((ids >> 8) & 0xff), c = plane_ck((ids >> 16) & 0xff);
             uint32_t close = 0;  // rows of the lane's planes too close (PAD_PLANE never is: its distance is FLT_MAX)
 #pragma unroll
             for (int r = 0; r < NR; ++r) {
@@ -863,8 +868,8 @@ __device__ __forceinline__ void trace_finish(TraceSmem<Real, NP, NV>& sm, const 
         for (int e = e0; e < E && e < e0 + 24; e += 8) {
             const uint32_t ed = sm.ed[e];
             Real ax, ay, az, bx, by, bz;
-            vert((ed >> 16) & 0xff, ax, ay, az);
-            vert(ed >> 24, bx, by, bz);
+            vert(vt_ck((ed >> 16) & 0xff, NV, CK_SLOT, A.st), ax, ay, az);
+            vert(vt_ck(ed >> 24, NV, CK_SLOT, A.st), bx, by, bz);
             const Real cx = ay * bz - az * by, cy = az * bx - ax * bz, cz = ax * by - ay * bx;
             const Real ab2 = ax * ax + ay * ay + az * az + bx * bx + by * by + bz * bz;
             const Real tx = ax + bx, ty = ay + by, tz = az + bz;
@@ -934,7 +939,7 @@ __device__ __forceinline__ void trace_finish(TraceSmem<Real, NP, NV>& sm, const 
         const int i = i0 + gl;
         int key = INT_MAX;
         if (i < F) {
-            const int f = faces.nth(i);
+            const int f = vt_ck(faces.nth(i), NP, CK_PLANE, A.st);
             const int src = sm.src[f];
             int oid = src;  // wall ids stay
             if (PER) {
@@ -946,7 +951,7 @@ __device__ __forceinline__ void trace_finish(TraceSmem<Real, NP, NV>& sm, const 
             } else if (src >= 0 && A.index_space == VT_INDEX_ORIGINAL) {
                 oid = __float_as_int(A.sorted[src].w);
             }
-            if (geom) rfn[i] = oid;
+            if (geom) rfn[vt_ck(i, REC_FACES, CK_RECORD, A.st)] = oid;
             bool nb = true;
             if (sm.u.f[f] < 210) {  // 2e-4 R^2 of doubled area
                 Real fnx, fny, fnz, sc, area = 0, tau;
@@ -979,7 +984,7 @@ __device__ __forceinline__ void trace_finish(TraceSmem<Real, NP, NV>& sm, const 
             if (nb) key = PER ? oid * 128 + f : oid;
         }
         __syncwarp();  // (the i-th face is plane i or a later one: its area is read before this)
-        if (i < F) sm.u.f[i] = key;
+        if (i < F) sm.u.f[vt_ck(i, NP, CK_PLANE, A.st)] = key;
     }
     __syncwarp();
     int32_t* rnbr = reinterpret_cast<int32_t*>(rec + REC_NBR_OFF);
@@ -990,7 +995,7 @@ __device__ __forceinline__ void trace_finish(TraceSmem<Real, NP, NV>& sm, const 
         int rank = 0;
 #pragma unroll 4
         for (int k = 0; k < F; ++k) rank += sm.u.f[k] < key ? 1 : 0;
-        rnbr[rank] = PER ? key / 128 : key;
+        rnbr[vt_ck(rank, REC_FACES, CK_RECORD, A.st)] = PER ? key / 128 : key;
     }
     const int nn = G.bcast(G.incl_scan(kept), TT - 1);
     if (geom) {
@@ -1031,8 +1036,8 @@ __device__ __forceinline__ void trace_finish(TraceSmem<Real, NP, NV>& sm, const 
                 const int f = (ed >> (8 * k)) & 0xff, u = k ? s : t, v = k ? t : s;
                 const uint32_t ids = *reinterpret_cast<const uint32_t*>(sm.vid[u]);
                 const int at = (ids & 0xff) == (uint32_t)f ? 0 : (((ids >> 8) & 0xff) == (uint32_t)f ? 1 : 2);
-                next[4 * u + at] = (uint8_t)v;
-                atomicMin(&first[f], u);
+                next[vt_ck(4 * u + at, 4 * NV, CK_SLOT, A.st)] = (uint8_t)v;
+                atomicMin(&first[vt_ck(f, NP, CK_PLANE, A.st)], u);
                 atomicAdd(&degree[f], 1);
             }
         }
@@ -1050,13 +1055,13 @@ __device__ __forceinline__ void trace_finish(TraceSmem<Real, NP, NV>& sm, const 
             base += G.bcast(inc, TT - 1);
             if (i < F) {
                 rdeg[i] = (uint8_t)deg;
-                int cur = first[f];
+                int cur = vt_ck(first[f], NV, CK_SLOT, A.st);
 #pragma unroll 1
                 for (int k = 0; k < deg; ++k) {
                     const uint32_t ids = *reinterpret_cast<const uint32_t*>(sm.vid[cur]);
                     const int at = (ids & 0xff) == (uint32_t)f ? 0 : (((ids >> 8) & 0xff) == (uint32_t)f ? 1 : 2);
                     rfv[vt_ck(pos + k, 3 * REC_VERTS, CK_RECORD, A.st)] = (uint8_t)cur;
-                    cur = next[4 * cur + at];
+                    cur = vt_ck(next[4 * cur + at], NV, CK_SLOT, A.st);
                 }
             }
         }
@@ -1347,8 +1352,8 @@ __device__ __forceinline__ int walk(const TraceArgs& A, const GridDesc& grid, in
                 const unsigned cm = __ballot_sync(TFULL, cuts);
                 if (cuts) {
                     const int at = ns + __popc(cm & ((1u << lane) - 1u));
-                    key[at] = d2;
-                    id[at] = jj;
+                    key[vt_ck(at, CUT_LIST, CK_RECORD, A.st)] = d2;
+                    id[vt_ck(at, CUT_LIST, CK_RECORD, A.st)] = jj;
                 }
                 ns += __popc(cm);
                 if (ns > keep) {
@@ -1393,7 +1398,8 @@ __device__ __forceinline__ int walk(const TraceArgs& A, const GridDesc& grid, in
 // vertices beyond half the reach into far (position, error bound): a generator cuts a
 // vertex v only from inside the ball of radius |v| around v
 template <int TT, typename S>
-__device__ __forceinline__ int far_vertices(const Sub<TT>& G, const S& sm, bool on, int V, float reach, float4* far)
+__device__ __forceinline__ int far_vertices(const Sub<TT>& G, const S& sm, bool on, int V, float reach, float4* far, int cap,
+                                            DevStatus* st)
 {
     int nf = 0;
     const int vmax = __reduce_max_sync(TFULL, on ? V : 0);
@@ -1405,7 +1411,7 @@ __device__ __forceinline__ int far_vertices(const Sub<TT>& G, const S& sm, bool 
         const float d = v.x * v.x + v.y * v.y + v.z * v.z;
         const bool is = on && s < V && d >= half;
         const unsigned m = G.ballot(is);
-        if (is) far[nf + __popc(m & ((1u << G.gl) - 1u))] = v;
+        if (is) far[vt_ck(nf + __popc(m & ((1u << G.gl) - 1u)), cap, CK_SLOT, st)] = v;
         nf += __popc(m);
     }
     return nf;
@@ -1441,7 +1447,7 @@ __global__ void __launch_bounds__(CUT_BLOCK) k_cutters(const __grid_constant__ T
                                  s_key[warp], s_id[warp], cands);
         ++cells;
         if (ns > 0) {
-            if (lane < ns) h->src[np + lane] = s_id[warp][lane];
+            if (lane < ns) h->src[vt_ck(np + lane, 40, CK_PLANE, A.st)] = s_id[warp][lane];
             if (lane == 0) {
                 h->np = np + ns;
                 h->reach = reach;
@@ -1500,6 +1506,7 @@ __global__ void __launch_bounds__(TRACE_BLOCK, (sizeof(Real) == 4 ? TRACE_MINB :
         const float4 pi = A.sorted[q];
         OpenCell* h = reinterpret_cast<OpenCell*>(A.state + (size_t)(q - A.first) * A.state_stride);
         T t;
+        t.st = A.st;
         int P;
         float reach;  // every generator with a float key below this was in the lists so far
         const int32_t* srcs;
@@ -1556,10 +1563,10 @@ __global__ void __launch_bounds__(TRACE_BLOCK, (sizeof(Real) == 4 ? TRACE_MINB :
         // its faces, or all planes of a failed one
         const int F = t.faces.count();
         if (open)
-            for (int i = gl; i < F; i += TT) h->src[i] = sm.src[t.faces.nth(i)];
+            for (int i = gl; i < F; i += TT) h->src[vt_ck(i, 40, CK_PLANE, A.st)] = sm.src[t.plane_ck(t.faces.nth(i))];
         if (failed && A.round == 0)
             for (int p = gl; p < P; p += TT) h->src[p] = sm.src[p];
-        const int nf = far_vertices<TT>(G, sm, open, t.V, reach, h->far);
+        const int nf = far_vertices<TT>(G, sm, open, t.V, reach, h->far, NV, A.st);
         if ((open || failed) && gl == 0) {
             h->np = open ? F : P;
             h->nf = nf;
@@ -1653,6 +1660,7 @@ __global__ void __launch_bounds__(TAIL_BLOCK, 4) k_trace_tail(const __grid_const
         const bool all = reach == FLT_MAX;
         __syncwarp();
         T t;
+        t.st = A.st;
         t.rows = NR;
         bool done = false, spread = false;
         int hard = 0;  // turns that took FP64 rays
@@ -1684,7 +1692,7 @@ __global__ void __launch_bounds__(TAIL_BLOCK, 4) k_trace_tail(const __grid_const
                 const float lx = grid.hi[0] - grid.lo[0], ly = grid.hi[1] - grid.lo[1], lz = grid.hi[2] - grid.lo[2];
                 const int ns = walk<PER, true>(A, grid, q, pi, nullptr, 0, m.t.src, P, 1.01f * (lx * lx + ly * ly + lz * lz),
                                                0, r, m.key, m.id, cands);
-                if (lane < ns) m.src[P + lane] = m.id[lane];
+                if (lane < ns) m.src[t.plane_ck(P + lane)] = m.id[lane];
                 P += ns;
                 --turn;
                 __syncwarp();
@@ -1726,14 +1734,14 @@ __global__ void __launch_bounds__(TAIL_BLOCK, 4) k_trace_tail(const __grid_const
             const float all2 = 4.0f * FAR_R2 * t.R2;
             if (!valid && all2 > reach) {
                 const int F = t.faces.count();
-                const int nf = far_vertices<TT>(G, m.t, true, t.V, reach, m.far);
+                const int nf = far_vertices<TT>(G, m.t, true, t.V, reach, m.far, NV, A.st);
                 __syncwarp();
                 const int ns = walk<PER, false>(A, grid, q, pi, m.far, nf, m.t.src, P, all2,
                                          turn < TRACE_ROUNDS ? TRACE_KEEP : TAIL_KEEP, reach, m.key, m.id, cands);
                 if (ns > 0) {
                     __syncwarp();
-                    for (int i = lane; i < F; i += TT) m.src[i] = m.t.src[t.faces.nth(i)];
-                    if (lane < ns) m.src[F + lane] = m.id[lane];
+                    for (int i = lane; i < F; i += TT) m.src[i] = m.t.src[t.plane_ck(t.faces.nth(i))];
+                    if (lane < ns) m.src[t.plane_ck(F + lane)] = m.id[lane];
                     P = F + ns;
                     __syncwarp();
                     continue;
