@@ -92,7 +92,9 @@ typedef struct vt_params {
                                pass that follows finishes every remaining cell exactly) */
     float grid_density;     /* target generators per grid cell rho; G = ceil(cbrt(n / rho)) (default 2) */
     int grid_res;           /* G override per axis (0 = derive from grid_density) */
-    int threads_per_cell;   /* lanes cooperating on one cell: 8, 16 or 32 (0 = default 32) */
+    int threads_per_cell;   /* lanes of the plane-by-plane clipper on one cell: 8, 16 or 32 (0 = default
+                               32). Traced cells (the default k0 and k_max) have lanes of their own; the
+                               clipper builds those whose certificate fails */
     int precision;          /* VT_FP64 or VT_FP32_RECHECK */
     int emit;               /* VT_EMIT_* bitmask */
     int index_space;        /* VT_INDEX_ORIGINAL (default) or VT_INDEX_SORTED */

@@ -1,8 +1,9 @@
-"""The fused schedule (VT_FLAG_FUSED): kNN and clipping in one kernel, no
-neighbour lists. Every cell starts from the box and clips the generators its
+"""The fused schedule (VT_FLAG_FUSED): the one that needs little memory, with no
+neighbour lists and no saved cells for all points. The cells are traced in parts
+(paper, Summary: the kNN of a grid sort bounds what can cut a cell); those
+whose certificate fails start from the box and clip the generators their
 grid-shell walk meets, nearest first within each batch, until the security
-radius concludes it (paper, Summary: the kNN of a grid sort bounds what can
-cut a cell; the fused walk visits the same generators without storing them).
+radius concludes them.
 
 A validated cell is the exact cell whatever the order of its cuts, so the
 fused schedule must meet the oracle with the list schedules' tolerances:
@@ -90,14 +91,19 @@ def test_fused_clustered_matches_the_oracle(clustered, prec):
     cells = vt.tessellate(dev(pts), vt.Params(precision=prec, emit=EMIT, fused=True, stage_times=True))
     check(cells, want, prec)
     st = cells.stats
-    # one pass, no lists: the walk is the whole clip
+    # one pass, no lists for all points
     assert st["passes"] == 1 and st["k_of_pass"][0] == 0 and st["exhaustive_cells"] == len(pts)
     assert st["unvalidated"] == 0
 
 
+@pytest.mark.parametrize("cloud", ["uniform", "lattice"])
 @pytest.mark.parametrize("tpc", [8, 16])
-def test_fused_threads_per_cell(uniform, tpc):
+def test_fused_threads_per_cell(uniform, tpc, cloud):
+    # (every cell of the lattice is left to the clipper, whose lanes these are)
     pts, want = uniform
+    if cloud == "lattice":
+        pts = W.cubic_lattice(16)  # (exact coordinates: no faces at round-off size)
+        want = oracle.tessellate(pts)
     cells = vt.tessellate(dev(pts), vt.Params(precision="fp64", emit=EMIT, fused=True, threads_per_cell=tpc))
     check(cells, want, "fp64")
 
@@ -163,7 +169,7 @@ def test_fused_batch_matches_the_oracle_per_set(prec):
 
 
 def test_fused_no_sync_equals_sync_with_geometry():
-    # both schedules run the same single walk pass
+    # both schedules run the same pass
     pts = W.mixed(60000, 8, n_clumps=60)
     emit = EMIT + ("geom",)
     a = vt.tessellate(dev(pts), vt.Params(precision="fp32", emit=emit, fused=True))

@@ -179,17 +179,23 @@ def test_fp64_uniform_4096(cfg0):
     assert st["k_of_pass"][0] == 16 and st["unvalidated"] == 0
 
 
+# (k_max = 8 k0: every cell is clipped plane by plane, by these lanes; with the
+# default lists only the cells that the traced pass leaves)
+@pytest.mark.parametrize("k0,k_max", [(16, 32), (8, 64)])
 @pytest.mark.parametrize("tpc", [8, 16, 32])
-def test_fp32_uniform_4096(cfg0, tpc):
+def test_fp32_uniform_4096(cfg0, tpc, k0, k_max):
     pts, want = cfg0
-    cells = vt.tessellate(dev(pts), vt.Params(precision="fp32", threads_per_cell=tpc, emit=("nbr", "vol", "cen")))
+    cells = vt.tessellate(dev(pts), vt.Params(precision="fp32", threads_per_cell=tpc, k0=k0, k_max=k_max,
+                                              emit=("nbr", "vol", "cen")))
     check_fp32(np_(cells.vol), np_(cells.cen), csr_lists(np_(cells.nbr_off), np_(cells.nbr)), want)
 
 
+@pytest.mark.parametrize("k0,k_max", [(16, 32), (8, 64)])
 @pytest.mark.parametrize("tpc", [8, 32])
-def test_fp64_threads_per_cell(cfg0, tpc):
+def test_fp64_threads_per_cell(cfg0, tpc, k0, k_max):
     pts, want = cfg0
-    cells = vt.tessellate(dev(pts), vt.Params(precision="fp64", threads_per_cell=tpc, emit=("nbr", "vol", "cen")))
+    cells = vt.tessellate(dev(pts), vt.Params(precision="fp64", threads_per_cell=tpc, k0=k0, k_max=k_max,
+                                              emit=("nbr", "vol", "cen")))
     check_fp64(cells, want)
 
 

@@ -3,9 +3,13 @@ wrong: lists that hold every other generator, lists shorter and longer than the
 planes of a group, cells with more vertices than its slots, cells that every
 round leaves open, degenerate vertices (the certificate refuses them), point
 counts that leave groups and blocks partly empty, and small sets in a batch.
+Calls of up to 12,288 points build every cell by a warp ("warps"); the same
+points in a batch beside enough others go through the groups of 8 lanes, the
+walk of their open cells and the warps for what these leave ("groups").
 Both forms against the FP64 oracle, to the tolerances of the other parity tests
-(FP32: 1e-5 relative, about 150 roundings of the volume's terms; FP64: 1e-12,
-the oracle's own bound on cells of clumps)."""
+(FP32: 1e-5 relative, about 150 roundings of the volume's terms, neighbours but
+for faces below 1e-6 V^(2/3); FP64: 1e-12, the oracle's own bound on cells of
+clumps, neighbours exact)."""
 import itertools
 
 import numpy as np
@@ -15,52 +19,119 @@ torch = pytest.importorskip("torch")
 
 import oracle
 import paper_2412_04514_gb300 as vt
+from geometry_match import emitted_cell, match_cell, oracle_cell
 from paper_2412_04514_gb300 import workloads as W
 
 pytestmark = pytest.mark.gpu
 
 TOL = {"fp32": 1e-5, "fp64": 1e-12}
+GEO = ("vtx_off", "vtx", "face_off", "face_nbr", "face_vtx_off", "face_vtx")
+ROUTES = pytest.mark.parametrize("route", ["warps", "groups"])
+PRECS = pytest.mark.parametrize("prec", ["fp32", "fp64"])
 
 
-def check(pts, prec, want=None, periodic=False, **kw):
-    if want is None:
-        want = oracle.tessellate(pts, periodic=periodic)
-    cells = vt.tessellate(torch.from_numpy(pts).cuda(),
-                          vt.Params(precision=prec, emit=("nbr", "vol", "cen", "geom"), periodic=periodic, **kw))
-    np.testing.assert_allclose(cells.vol.cpu().numpy(), want["vol"], rtol=TOL[prec])
-    np.testing.assert_allclose(cells.cen.cpu().numpy(), want["cen"], rtol=TOL[prec], atol=TOL[prec] * 1e-2)
+def run(pts, prec, route, emit, **kw):
+    """The cells of ``pts`` as numpy arrays: of a call of their own, or of a
+    batch whose second set makes it large enough for the groups."""
+    p = vt.Params(precision=prec, emit=emit, **kw)
+    n = len(pts)
+    if route == "warps":
+        c = vt.tessellate(torch.from_numpy(pts).cuda(), p)
+    else:
+        both = np.concatenate([pts, W.uniform(12_301, 77)])
+        c = vt.tessellate_batch(torch.from_numpy(both).cuda(), [0, n, len(both)], p)
+        assert c.stats["clip_launches"] >= 4  # two rounds of groups, the warps, the clipper
+    assert c.stats["status"] == "VT_OK"
+    out = {}
+    for name in ("vol", "cen", "nbr_off", "nbr") + GEO:
+        t = getattr(c, name)
+        if t is not None:
+            out[name] = t.cpu().numpy()
+    out["vol"], out["cen"] = out["vol"][:n], out["cen"][:n]
+    if "nbr" in out:
+        out["nbr_off"] = out["nbr_off"][:n + 1]
+        out["nbr"] = out["nbr"][:out["nbr_off"][-1]]
+    return out
+
+
+def least_det(V, faces):
+    """The smallest |det| of three faces' unit normals over the vertices of a cell (1e-7 at least)."""
+    normal = []
+    for _, loop in faces:
+        P = V[loop] - V[loop[0]]
+        a = np.cross(P[1:-1], P[2:]).sum(0)
+        normal.append(a / max(np.linalg.norm(a), 1e-300))
+    at = [[normal[f] for f, (_, loop) in enumerate(faces) if k in loop] for k in range(len(V))]
+    return max(1e-7, min(abs(np.linalg.det(np.stack(n[:3]))) for n in at if len(n) >= 3))
+
+
+def check(pts, prec, route="warps", periodic=False, generic=True, **kw):
+    want = oracle.tessellate(pts, periodic=periodic, geometry=generic)
+    n = len(pts)
+    c = run(pts, prec, route, ("nbr", "vol", "cen") + (("geom",) if generic else ()), periodic=periodic, **kw)
+    np.testing.assert_allclose(c["vol"], want["vol"], rtol=TOL[prec])
+    np.testing.assert_allclose(c["cen"], want["cen"], rtol=TOL[prec], atol=TOL[prec] * 1e-2)
+    if not generic:
+        return
+    differ = set()
     if prec == "fp64":
-        assert np.array_equal(cells.nbr_off.cpu().numpy(), want["nbr_off"])
-        assert np.array_equal(cells.nbr.cpu().numpy(), want["nbr"])
+        assert np.array_equal(c["nbr_off"], want["nbr_off"]) and np.array_equal(c["nbr"], want["nbr"])
+    else:
+        for i in range(n):
+            got, ref = (sorted(x["nbr"][x["nbr_off"][i]:x["nbr_off"][i + 1]].tolist()) for x in (c, want))
+            if got == ref:
+                continue
+            differ.add(i)
+            faces = slice(want["face_off"][i], want["face_off"][i + 1])
+            for j in set(got) ^ set(ref):
+                areas = want["face_area"][faces][want["face_tag"][faces] == j]
+                assert len(areas) == 0 or areas.min() < 1e-6 * want["vol"][i] ** (2 / 3), (i, j, areas)
+        assert len(differ) <= max(2, 1e-3 * n)
     # every cell is a simple polyhedron: V = 2 F - 4, three faces at each vertex
-    v, f = torch.diff(cells.vtx_off), torch.diff(cells.face_off)
-    assert torch.equal(v, 2 * f - 4)
-    deg = torch.diff(cells.face_vtx_off)
-    assert int(deg.min()) >= 3 and int(deg.sum()) == 3 * int(v.sum())
-    return cells
+    v, f = np.diff(c["vtx_off"])[:n], np.diff(c["face_off"])[:n]
+    assert np.array_equal(v, 2 * f - 4)
+    deg = np.diff(c["face_vtx_off"])[:c["face_off"][n]]
+    assert deg.min() >= 3 and deg.sum() == 3 * v.sum()
+    # vertices and loops of some cells, matched one to one
+    geo = [c[g] for g in GEO]
+    for i in range(0, n, max(1, n // 40)):
+        if i in differ:
+            continue
+        V, faces = emitted_cell(geo, i)
+        Wv, wfaces = oracle_cell(want, i)
+        amax = max(1.0, np.abs(Wv).max())
+        # (Cramer's rule leaves 32 roundings / |det| of a vertex's distance from the generator)
+        atol = 32 * 2.0 ** -53 / least_det(Wv, wfaces) * np.linalg.norm(Wv - pts[i], axis=1).max() + 1e-15 * amax
+        if prec == "fp32":
+            atol += 1e-5 * np.cbrt(want["vol"][i]) + 4 * np.finfo(np.float32).eps * amax
+        match_cell(V, faces, Wv, wfaces, atol)
 
 
-@pytest.mark.parametrize("prec", ["fp32", "fp64"])
+@ROUTES
+@PRECS
 @pytest.mark.parametrize("n", [1, 2, 3, 5, 31, 32, 33, 34, 35, 63, 65, 127, 129, 515])
-def test_small_counts(n, prec):
-    check(W.uniform(n, 100 + n), prec)
+def test_small_counts(n, prec, route):
+    check(W.uniform(n, 100 + n), prec, route)
 
 
-@pytest.mark.parametrize("prec", ["fp32", "fp64"])
+@ROUTES
+@PRECS
 @pytest.mark.parametrize("k0,k_max", [(6, 12), (12, 12), (16, 31), (17, 34), (17, 40), (18, 36), (40, 70), (64, 64)])
-def test_list_lengths(k0, k_max, prec):
-    check(W.mixed(3001, 5, n_clumps=3), prec, k0=k0, k_max=k_max)
+def test_list_lengths(k0, k_max, prec, route):
+    check(W.mixed(3001, 5, n_clumps=3), prec, route, k0=k0, k_max=k_max)
 
 
-@pytest.mark.parametrize("prec", ["fp32", "fp64"])
+@ROUTES
+@PRECS
 @pytest.mark.parametrize("n", [40, 300, 1201])
-def test_periodic(n, prec):
-    check(W.mixed(n, 9, n_clumps=2, periodic=True), prec, periodic=True)
+def test_periodic(n, prec, route):
+    check(W.mixed(n, 9, n_clumps=2, periodic=True), prec, route, periodic=True)
 
 
-@pytest.mark.parametrize("prec", ["fp32", "fp64"])
+@ROUTES
+@PRECS
 @pytest.mark.parametrize("around", [20, 26, 27, 40, 60])
-def test_many_faced_cells(around, prec):
+def test_many_faced_cells(around, prec, route):
     # a generator inside a shell of `around` others at about one distance: its
     # cell has up to around faces (26 fill the vertex slots of a group)
     rng = np.random.default_rng(around)
@@ -68,10 +139,10 @@ def test_many_faced_cells(around, prec):
     shell = 0.5 + (0.2 + 1e-3 * rng.random((around, 1))) * d / np.linalg.norm(d, axis=1, keepdims=True)
     far = rng.random((400, 3))
     far = far[np.linalg.norm(far - 0.5, axis=1) > 0.4]
-    check(np.concatenate([[[0.5, 0.5, 0.5]], shell, far]).astype(np.float32), prec)
+    check(np.concatenate([[[0.5, 0.5, 0.5]], shell, far]).astype(np.float32), prec, route)
 
 
-@pytest.mark.parametrize("prec", ["fp32", "fp64"])
+@PRECS
 @pytest.mark.parametrize("m,move", [(25, 1e-3), (25, 1e-4), (25, 1e-5), (12, 1e-4)])
 def test_lattices_that_moved_little(m, move, prec):
     # most cells have planes within float32 round-off of their vertices. Where
@@ -112,29 +183,28 @@ def test_sums_of_many_edges():
     assert (rms[True] < 1.03 * rms[False]).all(), rms
 
 
-@pytest.mark.parametrize("prec", ["fp32", "fp64"])
-def test_sparse_cells_beside_a_dense_clump(prec):
+@ROUTES
+@PRECS
+def test_sparse_cells_beside_a_dense_clump(prec, route):
     # the lists of the sparse points end inside the clump; thousands of its
     # points lie within twice their radius and the rounds cut them back
     rng = np.random.default_rng(4)
     clump = 0.5 + 2e-3 * rng.standard_normal((6000, 3))
-    check(np.concatenate([clump, rng.random((60, 3))]).astype(np.float32), prec)
+    check(np.concatenate([clump, rng.random((60, 3))]).astype(np.float32), prec, route)
 
 
-@pytest.mark.parametrize("prec", ["fp32", "fp64"])
-@pytest.mark.parametrize("make", [lambda: W.cubic_lattice(8), lambda: W.bcc_lattice(6)])
-def test_lattices(make, prec):
+@ROUTES
+@PRECS
+@pytest.mark.parametrize("make", [lambda: W.cubic_lattice(8), lambda: W.bcc_lattice(6)], ids=["cubic", "bcc"])
+def test_lattices(make, prec, route):
     # every vertex of the cubic lattice and the walls' of the BCC lattice have
     # more than three planes: the certificate sends the cells to the clipper
-    pts = make()
-    want = oracle.tessellate(pts)
-    cells = vt.tessellate(torch.from_numpy(pts).cuda(), vt.Params(precision=prec, emit=("nbr", "vol", "cen")))
-    np.testing.assert_allclose(cells.vol.cpu().numpy(), want["vol"], rtol=TOL[prec])
-    np.testing.assert_allclose(cells.cen.cpu().numpy(), want["cen"], rtol=TOL[prec])
+    check(make(), prec, route, generic=False)
 
 
-@pytest.mark.parametrize("prec", ["fp32", "fp64"])
-def test_more_equal_distances_than_a_list_holds(prec):
+@ROUTES
+@PRECS
+def test_more_equal_distances_than_a_list_holds(prec, route):
     # 48 generators at one exact distance around the middle one: no limit keeps
     # between a list's length less one and a list's length of them. (Nothing
     # else: the middle cell's vertices have up to eight planes, and beside
@@ -143,13 +213,10 @@ def test_more_equal_distances_than_a_list_holds(prec):
     ring = [0.5 + np.array(s) * d[list(o)] for o in itertools.permutations(range(3))
             for s in itertools.product([-1, 1], repeat=3)]
     pts = np.concatenate([[[0.5, 0.5, 0.5]], ring]).astype(np.float32)
-    want = oracle.tessellate(pts)
-    cells = vt.tessellate(torch.from_numpy(pts).cuda(), vt.Params(precision=prec, emit=("nbr", "vol", "cen")))
-    np.testing.assert_allclose(cells.vol.cpu().numpy(), want["vol"], rtol=TOL[prec])
-    np.testing.assert_allclose(cells.cen.cpu().numpy(), want["cen"], rtol=TOL[prec])
+    check(pts, prec, route, generic=False)
 
 
-@pytest.mark.parametrize("prec", ["fp32", "fp64"])
+@PRECS
 @pytest.mark.parametrize("n", [3, 20, 300])
 def test_box_whose_plane_products_overflow(n, prec):
     # a box of 2^40: the float32 products of a vertex's three planes overflow,
@@ -176,7 +243,7 @@ def test_small_scales(n, clumps, k):
     np.testing.assert_allclose(cells.vol.cpu().numpy() / scale ** 3, want["vol"], rtol=TOL["fp32"])
 
 
-@pytest.mark.parametrize("prec", ["fp32", "fp64"])
+@PRECS
 @pytest.mark.parametrize("spacing", [1e-20, 1e-19, 1e-18, 1e-13])
 def test_generators_whose_squares_underflow(spacing, prec):
     # three generators on a line: the cell between two others is a slab of the
@@ -207,9 +274,10 @@ def test_box_beyond_float_squares():
         assert np.array_equal(cells.nbr.cpu().numpy(), want["nbr"])
 
 
-@pytest.mark.parametrize("prec", ["fp32", "fp64"])
-def test_batch_of_small_sets(prec):
-    sizes = [1, 2, 0, 7, 33, 34, 35, 200, 1, 1500]
+@ROUTES
+@PRECS
+def test_batch_of_small_sets(prec, route):
+    sizes = [1, 2, 0, 7, 33, 34, 35, 200, 1, 1500] + [11_001] * (route == "groups")
     parts = [W.uniform(n, 40 + i) for i, n in enumerate(sizes)]
     off = np.concatenate([[0], np.cumsum(sizes)])
     b = vt.Batch(torch.from_numpy(np.concatenate(parts)).cuda(), off, vt.Params(precision=prec, emit=("nbr", "vol", "cen")))
@@ -233,10 +301,10 @@ def test_repeats_bit_for_bit():
                 assert torch.equal(getattr(a, name), getattr(b, name)), (prec, name)
 
 
-@pytest.mark.parametrize("prec", ["fp32", "fp64"])
+@PRECS
 @pytest.mark.parametrize("lattice", [False, True])
 def test_fused_schedule_in_parts(lattice, prec):
-    # two parts; of the lattice every cell fails its certificate, more than the
+    # three parts of the cloud, four of the lattice; of the lattice every cell fails its certificate, more than the
     # slots that outlive a part. The list schedule builds the same cells at once
     # (but which of the lattice's faces without area it lists is round-off)
     x = torch.from_numpy(W.cubic_lattice(60) if lattice else W.mixed(200_000, 2, n_clumps=100)).cuda()
