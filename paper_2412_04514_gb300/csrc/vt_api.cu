@@ -480,10 +480,10 @@ int clip_pass(const Ctx& c, const vt_params* p, const int32_t* list, int64_t m, 
 }
 
 // Whether the list pass with lists of `kl` entries builds whole cells by edge
-// tracing (trace_impl.cuh): the pass after it would be the last one anyway (the
-// tracing finishes every open cell by its own walk, so a caller's further
-// doubling passes stay as they are), and the list is long enough that what it
-// leaves to the walk is small.
+// tracing (trace_impl.cuh): the pass after it would be the last one anyway, and
+// the list is long enough that what it leaves to the walk is small. With more
+// doublings to come (k_max >= 2 kl) a caller asks for the plane-by-plane passes,
+// whose counts by pass are part of the results.
 bool traced_pass(const vt_params* p, int kl) { return kl >= 12 && 2 * kl > p->k_max; }
 
 // Whether the box is one the traced pass may run in: it compares float32 squares
@@ -497,11 +497,20 @@ bool traced_box(const vt_params* p)
     return true;
 }
 
-// point counts up to which every cell goes to the warp-per-cell kernel at once
-// (the latency of a few launches less; above it the 8-lane groups' throughput
-// counts). With neighbours, ms: 3,000 uniform points 0.34 against 0.43 (half in
-// clumps 0.56 against 0.68), 8,000 0.44 against 0.48 (0.68 and 0.81), 11,000 0.48
-// and 0.48 (0.81 and 1.02), 15,000 0.59 and 0.54 (0.89 and 0.85)
+// point counts (all sets of a batch together) up to which every cell goes to the
+// warp-per-cell kernel at once (the latency of a few launches less; above it the
+// 8-lane groups' throughput counts). ms by groups / by warps, with neighbours:
+//                      3,000        8,000        11,000       15,000       30,000
+//   uniform FP32     0.45 / 0.36  0.48 / 0.46  0.52 / 0.51  0.57 / 0.61  0.71 / 0.96
+//     half in clumps 0.76 / 0.62  0.88 / 0.74  0.97 / 0.86  0.90 / 0.91  1.15 / 1.39
+//   uniform FP64     0.53 / 0.39  0.68 / 0.59  0.75 / 0.70  0.81 / 0.86  1.20 / 1.51
+//     half in clumps 0.89 / 0.63  1.13 / 0.85  1.22 / 0.99  1.21 / 1.18  1.79 / 2.08
+//   periodic FP32    0.52 / 0.40  0.55 / 0.54  0.60 / 0.62  0.65 / 0.74  0.82 / 1.19
+//     half in clumps 0.99 / 0.76  1.11 / 0.95  1.12 / 1.01  1.10 / 1.11  1.35 / 1.68
+//   batch of sets of about 1,000, FP32
+//                    0.37 / 0.30  0.44 / 0.43  0.47 / 0.48  0.50 / 0.55  0.59 / 0.84
+//     half in clumps 0.92 / 0.75  1.12 / 1.01  1.12 / 1.12  1.18 / 1.22  1.37 / 1.66
+// (the fused schedule as the lists): one line within 4% of every form's own
 constexpr int64_t TRACE_SMALL = 12288;
 
 // The cells by edge tracing: unordered lists, two rounds of groups of 8 lanes
