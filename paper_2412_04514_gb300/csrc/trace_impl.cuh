@@ -1108,6 +1108,10 @@ static_assert(sizeof(OpenCell) <= StateLayout<float, 64, 64>::BYTES, "an open ce
 // 2 limits: 139, 85 and 74 thousand turns of the warp-per-cell kernel on 1M
 // points half in clumps)
 constexpr int WALK_ENOUGH = 8, WALK_PAST = 2;
+// after a limit whose rows held more than WALK_DENSE generators (a clump inside one
+// grid cell: every limit reads all of it again) the next lies WALK_WIDE times farther
+constexpr unsigned WALK_DENSE = 4096;
+constexpr float WALK_WIDE = 16.0f;
 // a warp's list of cutting generators: the ones kept, and a batch
 constexpr int CUT_LIST = 64;
 
@@ -1187,6 +1191,7 @@ __device__ __forceinline__ int walk(const TraceArgs& A, const GridDesc& grid, in
     // it: 30,000 points in one clump and 60 around it 17.6 -> 16.6 ms, 500,000 half in
     // clumps, fused, 7.82 -> 7.51, 120,000 2.53 -> 2.50 ms)
     float nearest = FLT_MAX;
+    unsigned before = cands;
     bool more = false, end = !SPREAD && nf == 0;
     if (SPREAD) {
         l0 = l1 = l2 = -FLT_MAX;
@@ -1201,7 +1206,8 @@ __device__ __forceinline__ int walk(const TraceArgs& A, const GridDesc& grid, in
     // last one takes the whole ball)
 #pragma unroll 1
     for (int it = 0, past = 0; !end && (ns == 0 || (ns < WALK_ENOUGH && past++ < WALK_PAST)); ++it) {
-        const float lim2 = it < 40 ? fminf(all2, 2.25f * reach) : all2;
+        const float lim2 = it < 40 ? fminf(all2, (cands - before > WALK_DENSE ? WALK_WIDE : 2.25f) * reach) : all2;
+        before = cands;
         const float r_out2 = lim2 * (1.0f + 1e-4f), r_in2 = reach * (1.0f - 1e-4f);
         const float rr = sqrt_fast(r_out2) * (1.0f + 1e-5f);
         const float z_lo = pi.z + fmaxf(l2, -rr) - m, z_hi = pi.z + fminf(h2, rr) + m;
@@ -1417,10 +1423,14 @@ __device__ __forceinline__ int far_vertices(const Sub<TT>& G, const S& sm, bool 
     return nf;
 }
 
-// the walk of a round's open cells, a warp per cell
+// The walk of a round's open cells, a warp per cell. Waits for the generators'
+// loads: four blocks per SM (64 registers, 40 bytes of spills in the rows' set-up)
+// against three: 8M points half in clumps 78.6 -> 76.0 ms, FP64 form of 1M 30.6 ->
+// 30.3; 100,000 points in one clump and 1,000 around it, the walks alone 39.9 -> 29.1
+// with the wider limits above (34.3 by these alone; the clipper's range lists 20.7)
 constexpr int CUT_BLOCK = 256;
 template <bool PER>
-__global__ void __launch_bounds__(CUT_BLOCK) k_cutters(const __grid_constant__ TraceArgs A)
+__global__ void __launch_bounds__(CUT_BLOCK, 4) k_cutters(const __grid_constant__ TraceArgs A)
 {
     __shared__ float4 s_far[CUT_BLOCK / 32][48];
     __shared__ float s_key[CUT_BLOCK / 32][CUT_LIST];
