@@ -60,20 +60,54 @@ FP32_PEAK_TFLOPS = 152 * 128 * 2 * 2.070e9 / 1e12
 L2_FLUSH_BYTES = 256 << 20
 
 
-def _clip_traffic(n_cells: int):
-    """DRAM bytes of the clip stage per step from a committed ncu capture,
-    scaled to n_cells; None when the kernel source changed since the capture."""
+def _trace_traffic(n_cells: int):
+    """DRAM bytes of the tracing and its walks per step from a committed ncu
+    capture, scaled to n_cells; None when the kernel source changed since."""
     import hashlib
 
     try:
-        with open(os.path.join(ROOT, "profiles", "clip_traffic.json")) as f:
+        with open(os.path.join(ROOT, "profiles", "trace_traffic.json")) as f:
             rec = json.load(f)
-        src = open(os.path.join(ROOT, "paper_2412_04514_gb300", "csrc", "clip_impl.cuh"), "rb").read()
+        src = open(os.path.join(ROOT, "paper_2412_04514_gb300", "csrc", "trace_impl.cuh"), "rb").read()
     except OSError:
         return None
-    if hashlib.sha256(src).hexdigest() != rec.get("clip_impl_sha256"):
+    if hashlib.sha256(src).hexdigest() != rec.get("trace_impl_sha256"):
         return None
     return rec["bytes_per_cell"] * n_cells
+
+
+def cells_roofline(n: int, cells, st: dict, k0: int, k_max: int, cpu, args, traffic=None) -> dict:
+    """The cells' kernels against the FP32 peak, from the CUDA-event stage times ``st``.
+
+    Traced calls (the lists the library builds whole cells from, k_max below
+    four times the list's first half): every cell built once from its list, a
+    ray per vertex and one more of a plane test (10 flops) per plane, the
+    certificate (6 flops per vertex and plane), the vertices (60 each) and the
+    moments (25 per triangle, three triangles per vertex), over the time of
+    tracing and walks; cells built again and the walks count as time only. Other
+    calls: the clipper's flops, counted by the instrumented oracle on its sample."""
+    kl = 2 * k0 if 2 * k0 <= k_max else k0
+    if kl >= 12 and 2 * kl > k_max:
+        if cells.vtx_off is not None:
+            verts = cells.vtx.shape[0] / n
+        else:  # V = 2 F - 4 of a simple polyhedron (its walls are not among the neighbours)
+            verts = 2 * cells.nbr.numel() / n - 4
+        planes = 6 + min(kl, 34)
+        flops = 10 * planes * (verts + 1) + 6 * planes * verts + (60 + 3 * 25) * verts
+        ms = st["ms_clip"] + st["ms_knn"] - st["ms_knn_lists"]
+        kernel = "k_trace<float>, k_cutters, k_trace_tail<float>; k_clip for the cells these refuse"
+        units = f"{n} cells of {verts:.1f} vertices, each built once from {planes} planes: {flops:.0f} FP32 flops/cell"
+    else:
+        flops = cpu["flops_per_cell"] if cpu else args.flops_per_cell
+        ms = st["ms_clip"]
+        kernel = "k_clip<float> (all passes of one step)"
+        traffic = None
+        units = f"{n} validated cells x {flops:.0f} algorithmic FP32 flops/cell"
+    achieved = n * flops / (ms / 1e3) / 1e12
+    return {"kernel": kernel, "bound": "alu", "achieved": achieved, "peak": FP32_PEAK_TFLOPS, "unit": "TFLOP/s",
+            "frac": achieved / FP32_PEAK_TFLOPS, "traffic": traffic, "ms": ms, "units": units,
+            "peak_source": "152 SMs x 128 FP32 lanes x 2 x 2.070 GHz (unit counts and max SM clock)",
+            "stage_ms": {k: st[k] for k in ("ms_grid", "ms_knn", "ms_knn_lists", "ms_clip", "ms_emit")}}
 
 
 def _peaks():
@@ -455,8 +489,8 @@ def run_gpu(args, rank: int, world: int, local: int):
     if rank != 0:
         return
 
-    # roofline of the dominant stage (the clipper), from the live event times
-    stage = {k: statistics.mean(s[k] for s in st32) for k in ("ms_grid", "ms_knn", "ms_clip", "ms_emit")}
+    # roofline of the dominant stages (the cells), from the live event times
+    stage = {k: statistics.mean(s[k] for s in st32) for k in ("ms_grid", "ms_knn", "ms_knn_lists", "ms_clip", "ms_emit")}
     peaks = _peaks()
     probe32, probe64 = vt.probe_fma("fp32"), vt.probe_fma("fp64")  # measured FMA rates (after the timed region)
     cpu = None
@@ -471,21 +505,10 @@ def run_gpu(args, rank: int, world: int, local: int):
         if cellsF is not None:
             errors["fused_fp32_recheck"] = errors_vs_oracle(cellsF, cpu)
         errors["sample"] = cpu["sample"]
-    flops_per_cell = cpu["flops_per_cell"] if cpu else args.flops_per_cell
-    clip_launches = statistics.mean(s["clip_launches"] for s in st32)
-    achieved = n * flops_per_cell / (stage["ms_clip"] / 1e3) / 1e12
-    roofline = {
-        "kernel": "k_clip<float,32,2,64>%s (all passes of one step)" % (", periodic" if periodic else ""),
-        "bound": "alu", "achieved": achieved, "peak": FP32_PEAK_TFLOPS, "unit": "TFLOP/s",
-        "frac": achieved / FP32_PEAK_TFLOPS, "traffic": None if periodic else _clip_traffic(n),
-        "peak_source": "152 SMs x 128 FP32 lanes x 2 x 2.070 GHz (unit counts and max SM clock)",
-        "peak_probe": {"fp32_tflops": probe32, "fp64_tflops": probe64,
-                       "source": "vt_probe_fma: measured float32 / float64 FMA throughput of this GPU"},
-        "units": f"{n} validated cells x {flops_per_cell:.0f} algorithmic FP32 flops/cell over {clip_launches:.1f} "
-                 f"clip launches",
-        "stage_ms": stage,
-        "hbm_peak_gbs": peaks.get("hbm_gbs"),
-    }
+    roofline = cells_roofline(n, cells, stage, args.k0, args.k_max, cpu, args, None if periodic else _trace_traffic(n))
+    roofline["peak_probe"] = {"fp32_tflops": probe32, "fp64_tflops": probe64,
+                              "source": "vt_probe_fma: measured float32 / float64 FMA throughput of this GPU"}
+    roofline["hbm_peak_gbs"] = peaks.get("hbm_gbs")
     # every stage against its own roofline (stage times of the timed FP32 steps)
     hbm = peaks.get("hbm_gbs") or 6764.0
     csr_bytes = sum(getattr(cells, f).numel() * getattr(cells, f).element_size()
@@ -498,7 +521,7 @@ def run_gpu(args, rank: int, world: int, local: int):
         return {"bound": "hbm", "bytes": int(nbytes), "ms": ms, "achieved_gbs": gbs, "peak_gbs": hbm,
                 "frac": gbs / hbm, "bytes_are": what}
 
-    # the k-nearest-neighbour kernels against the FP32 peak: one squared
+    # the lists' kernels against the FP32 peak: one squared
     # distance per candidate examined (3 subtractions, a product, two fused
     # multiply-adds: 8 flops), over their own CUDA-event time
     kl_ms = statistics.mean(s["ms_knn_lists"] for s in st32)
@@ -508,17 +531,16 @@ def run_gpu(args, rank: int, world: int, local: int):
     knn_alu = {"bound": "alu", "ms": kl_ms, "candidates_per_query": cands / max(queries, 1), "queries": int(queries),
                "flops_per_candidate": 8, "achieved_tflops": knn_tflops, "peak_tflops": FP32_PEAK_TFLOPS,
                "frac": None if knn_tflops is None else knn_tflops / FP32_PEAK_TFLOPS,
-               "range_lists_ms": stage["ms_knn"] - kl_ms}
+               "walks_ms": stage["ms_knn"] - kl_ms}
     stage_rooflines = {
         "grid_sort": hbm_line(52 * n, stage["ms_grid"], "52 B per point: points read twice, cell id and ticket "
                                                          "written and read, sorted float4 and permutation written"),
-        "knn_and_range": hbm_line(n * (16 + 8 * kpre), stage["ms_knn"],
-                                  f"the {kpre}-entry lists: 16 B query read + {kpre} x (4 B index + 4 B key) written "
-                                  "(the stage also holds the range-list kernels, whose I/O is not counted; the "
-                                  "stage is ALU- and latency-bound)"),
-        "knn_alu": knn_alu,
-        "clip": {"bound": "alu", "achieved_tflops": achieved, "peak_tflops": FP32_PEAK_TFLOPS,
-                 "frac": achieved / FP32_PEAK_TFLOPS, "ms": stage["ms_clip"]},
+        "lists": hbm_line(n * (16 + 4 * min(kpre, 34) + 4), kl_ms,
+                          f"16 B query read, up to {min(kpre, 34)} x 4 B index and a 4 B reach written (the stage is "
+                          "bound by instruction issue)"),
+        "lists_alu": knn_alu,
+        "cells": {"bound": "alu", "achieved_tflops": roofline["achieved"], "peak_tflops": FP32_PEAK_TFLOPS,
+                  "frac": roofline["frac"], "ms": roofline["ms"]},
         "emit": hbm_line(2 * csr_bytes + 16 * n, stage["ms_emit"],
                          "the per-cell records read (the outputs' bytes + a 16 B header) and the outputs written"),
     }
@@ -647,8 +669,6 @@ def run_batch(args, rank: int, world: int, local: int):
         sub = pts_np[off[big]:off[big + 1]]
         cpu = cpu_oracle_rate(sub, min(args.cpu_cells, len(sub)))
         cpu["sample"] += f" (set {big} of the batch, {len(sub)} points)"
-    flops_per_cell = cpu["flops_per_cell"] if cpu else args.flops_per_cell
-    achieved = n * flops_per_cell / (sync["ms_clip"] / 1e3) / 1e12
     tr = b.tune_report
     line = {
         "metric": METRIC, "value": value, "unit": "cells/s", "n_gpus": world, "steps": len(ms),
@@ -663,12 +683,7 @@ def run_batch(args, rank: int, world: int, local: int):
         "e2e": None if not e2e_ms else {
             "value": n * world * len(e2e_ms) / (e2e_tot / 1e3), "unit": "cells/s", "h2d_bytes_per_step": n * 12,
             "d2h_bytes_per_step": int(d2h), "ms_per_step": e2e_tot / len(e2e_ms)},
-        "roofline": {
-            "kernel": f"k_clip<float,{b.params.threads_per_cell},...> (all passes, stage-timed synchronising run)",
-            "bound": "alu", "achieved": achieved, "peak": FP32_PEAK_TFLOPS, "unit": "TFLOP/s",
-            "frac": achieved / FP32_PEAK_TFLOPS, "traffic": None,
-            "peak_source": "152 SMs x 128 FP32 lanes x 2 x 2.070 GHz (unit counts and max SM clock)",
-            "stage_ms": {k: sync[k] for k in ("ms_grid", "ms_knn", "ms_clip", "ms_emit")}},
+        "roofline": cells_roofline(n, cells, sync, b.params.k0, b.params.k_max, cpu, args),
         "cpu_baseline": None if cpu is None else {"value": cpu["value"], "unit": "cells/s", "cores": cpu["cores"],
                                                   "kind": "oracle", "sample": cpu["sample"],
                                                   "one_core": cpu["one_core"]},
@@ -731,12 +746,10 @@ def run_lloyd(args, rank: int, world: int, local: int):
     if rank != 0:
         return
     # stage split of the forward tessellation of the current points (stage-timed)
-    st = vt.tessellate(p, vt.Params(precision="fp32", emit=("vol", "cen", "m2", "geom"), stage_times=True)).stats
+    last = vt.tessellate(p, vt.Params(precision="fp32", emit=("vol", "cen", "m2", "geom"), stage_times=True))
     cpu = None
     if world == 1 and not args.no_cpu_baseline:
         cpu = cpu_oracle_rate(p.cpu().numpy(), args.cpu_cells)
-    flops_per_cell = cpu["flops_per_cell"] if cpu else args.flops_per_cell
-    achieved = n * flops_per_cell / (st["ms_clip"] / 1e3) / 1e12
     line = {
         "metric": METRIC, "value": value, "unit": "cells/s", "n_gpus": world, "steps": len(ms),
         "warmup": args.warmup, "ms_per_step": tot / len(ms), "higher_is_better": True, "scaling": "weak",
@@ -749,12 +762,7 @@ def run_lloyd(args, rank: int, world: int, local: int):
         "e2e": None if not e2e_ms else {
             "value": n * world * len(e2e_ms) / (e2e_tot / 1e3), "unit": "cells/s", "h2d_bytes_per_step": n * 12,
             "d2h_bytes_per_step": n * 12 + 8, "ms_per_step": e2e_tot / len(e2e_ms)},
-        "roofline": {
-            "kernel": "k_clip<float,32,2,64> of the forward tessellation (stage-timed run)",
-            "bound": "alu", "achieved": achieved, "peak": FP32_PEAK_TFLOPS, "unit": "TFLOP/s",
-            "frac": achieved / FP32_PEAK_TFLOPS, "traffic": None,
-            "peak_source": "152 SMs x 128 FP32 lanes x 2 x 2.070 GHz (unit counts and max SM clock)",
-            "stage_ms": {k: st[k] for k in ("ms_grid", "ms_knn", "ms_clip", "ms_emit")}},
+        "roofline": cells_roofline(n, last, last.stats, prm.k0, prm.k_max, cpu, args),
         "cpu_baseline": None if cpu is None else {"value": cpu["value"], "unit": "cells/s", "cores": cpu["cores"],
                                                   "kind": "oracle", "sample": cpu["sample"] + " (tessellation only)",
                                                   "one_core": cpu["one_core"]},

@@ -74,7 +74,12 @@ typedef enum {
     VT_ERR_INTERNAL = 8          /* a bounds check of a debug build (VT_CHECKS) failed */
 } vt_status;
 
-enum { VT_FP64 = 0, VT_FP32_RECHECK = 1 };          /* vt_params.precision */
+/* vt_params.precision: the arithmetic of vertices and moments. VT_FP64 forms and decides
+ * everything in FP64, but for what a bound guards: the rays that find a traced cell's vertices,
+ * its list's keys and reach and its certificate's tests run in float32 with a bound on their
+ * error, and closer calls are decided in FP64. VT_FP32_RECHECK forms vertices and terms in
+ * float32, re-decides near-zero tests in FP64 and adds moments in FP64. */
+enum { VT_FP64 = 0, VT_FP32_RECHECK = 1 };
 enum { VT_INDEX_ORIGINAL = 0, VT_INDEX_SORTED = 1 }; /* vt_params.index_space */
 
 /* vt_params.emit bitmask */

@@ -25,7 +25,8 @@ _PREC = {"fp64": L.VT_FP64, "fp32": L.VT_FP32_RECHECK}
 @dataclass
 class Params:
     """Run-time parameters (vt_params). ``precision`` is ``"fp32"`` (float32
-    clipping with FP64 rechecks) or ``"fp64"`` (plain FP64). ``periodic``:
+    vertices with FP64 rechecks) or ``"fp64"`` (vertices, moments and decisions in
+    FP64; float32 only where a bound on its error guards the result). ``periodic``:
     the box [box_lo, box_hi) is periodic (VT_FLAG_PERIODIC). ``fused``: no
     neighbour lists or saved cells for all points, a quarter of the workspace:
     the cells are built in parts (VT_FLAG_FUSED)."""
