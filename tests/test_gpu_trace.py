@@ -161,6 +161,15 @@ def test_lattices_that_moved_little(m, move, prec):
             assert cells.stats["precision_retries"] < len(x) // 16
 
 
+def test_rays_that_meet_two_planes_within_float_rounding():
+    # of so many cells with nearly coincident vertices none may be left to the
+    # clipper for an order of two planes along a ray that float32 cannot tell
+    rng = np.random.default_rng(0)
+    x = (W.cubic_lattice(50) + rng.uniform(-2e-5, 2e-5, (125_000, 3))).astype(np.float32)
+    s = vt.tessellate(torch.from_numpy(x).cuda(), vt.Params(precision="fp64", emit=("vol",))).stats
+    assert s["knn_queries"] == len(x), s  # (the clipper's cells ask for lists of their own)
+
+
 def test_sums_of_many_edges():
     # the FP32 form's moments of cells of up to 60 faces (22 edges to a lane) are
     # no further off than the clipper's (k_max = 4 k0 is not traced), whose lanes
