@@ -17,11 +17,13 @@
 // others are). Each lane holds every eighth plane in registers; a ray is NR
 // plane tests per lane and a minimum over the 8 lanes. Wider groups repeat the
 // per-ray bookkeeping on more lanes, narrower ones hold more of the planes and
-// of shared memory per warp. Bound by instruction issue (4,400 warp
-// instructions per cell of the first round against 14,900 of the clipper) and
-// by instruction fetch. 1M points on a GB300, list and last pass with
-// neighbours: uniform 17.0 -> 7.3 ms, half in clumps 20.2 -> 11.0 ms in the
-// FP32 form, 126 -> 22.6 and 141 -> 35.4 ms in the FP64 form.
+// of shared memory per warp. Bound by instruction issue (3,000 warp
+// instructions per cell of the first round, 3,400 with geometry, 9,100 in all
+// against 14,900 of the clipper) and by instruction fetch; the FP64 form by the
+// FP64 pipe (77% busy). 1M points on a GB300, cells and walks with neighbours
+// against the clipper and its range lists: uniform 17.1 -> 7.1 ms, half in
+// clumps 20.2 -> 10.7 ms in the FP32 form, 126 -> 20.5 and 141 -> 27.6 ms in the
+// FP64 form.
 //
 // Certificate. The rays run in float32 and decide nothing by themselves: the
 // vertices are solved again from their three planes, and the cell is accepted

@@ -526,9 +526,10 @@ constexpr int64_t TRACE_SMALL = 12288;
 // eighth cell. The parts' tail cells keep their slots behind the lists for one
 // launch over all of them (a tail per part: each leaves the device to its last
 // few cells, 10.3 against 8.4 ms at 500,000 points half in clumps), and the slow
-// cells walk from the box. Against every cell walked from the box, at 1M points:
-// uniform 19.5 -> 8.2 ms, clumps 28.1 -> 13.5, FP64 154 -> 20.4 and 229 -> 26.9;
-// the list schedule takes 7.8, 12.0, 19.8 and 25.5 ms.
+// cells walk from the box. A state slot is 960 bytes: eight parts from 524,288
+// points on, one up to 69,905. Against every cell walked from the box, at 1M points,
+// moments: uniform 19.5 -> 8.1 ms, half in clumps 28.2 -> 13.1, FP64 154 -> 19.9 and
+// 229 -> 26.4.
 int trace_pass(const Ctx& c, const vt_params* p, int64_t n, int k, int k_list, int variant, vt_cells_out* out,
                int32_t* slow, int32_t* open, int32_t* next, int32_t* tail, int32_t* fail_next, int32_t* ctr_next,
                int32_t* fail_robust, int32_t* ctr_robust)
