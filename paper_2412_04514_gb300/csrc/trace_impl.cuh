@@ -1641,11 +1641,12 @@ __global__ void __launch_bounds__(TRACE_BLOCK, (sizeof(Real) == 4 ? TRACE_MINB :
 // of 32 planes instead of five of 8. A cell comes out the same bit for bit from
 // either kernel.
 constexpr int TAIL_BLOCK = 128;
-constexpr int TAIL_TURNS = 16, HARD_TURNS = 2;
-// close vertices of a cell in a call whose cells all run here, with no count to
-// go by, from which it is taken as one of a lattice (one degenerate vertex of a generic
-// cloud gives at most three): 8,000 points moved by 1e-5, 2.2 -> 1.4 ms
-constexpr int MANY_CLOSE = 6;
+constexpr int TAIL_TURNS = 64;
+// close vertices of a cell in a call whose cells all run here, with no count to go by, from
+// which it is taken as one of a lattice (one degenerate vertex of a generic cloud gives at
+// most three; from 8 on, rare cells of filaments went to the clipper that it cannot
+// validate): 8,000 points moved by 1e-5, 2.5 -> 1.6 ms
+constexpr int MANY_CLOSE = 10;
 constexpr int TAIL_KEEP = 32;  // cutting generators taken at once from the third turn on
 template <typename Real, bool PER>
 struct TailSmem {
@@ -1716,11 +1717,12 @@ __global__ void __launch_bounds__(TAIL_BLOCK, 4) k_trace_tail(const __grid_const
         t.st = A.st;
         t.rows = NR;
         bool done = false, spread = false;
-        int hard = 0;  // turns that took FP64 rays
-        // (every turn adds a generator that cuts; generic cells take fewer than
-        // TAIL_TURNS, and HARD_TURNS is what FP64 rays are worth: the 5,000 cells of a
-        // sphere's points, whose planes all pass within round-off of its centre, took 176 ms
-        // FP32 and 85 FP64 with 200 turns, with the clipper alone 123 and 34, now 123 and 30)
+        // (every turn adds a generator that cuts. Cells of filaments take tens of turns, and
+        // the clipper cannot validate all of those: of 9,000 points 56 cells stayed
+        // unvalidated with 16 turns, 54 with 64 or 200. What has not ended after 64 is a
+        // cell whose planes all pass within round-off of one point: 5,000 points of a
+        // sphere 268 ms FP32 and 157 FP64 with 200 turns, 183 and 76 with 64, 134 and 31
+        // with 16, 137 and 35 by the clipper alone)
 #pragma unroll 1
         for (int turn = A.round == 0 ? 0 : h->turns; turn < TAIL_TURNS && !done; ++turn) {
 #pragma unroll
@@ -1767,7 +1769,6 @@ __global__ void __launch_bounds__(TAIL_BLOCK, 4) k_trace_tail(const __grid_const
 #pragma unroll 1
             for (int again = traced ? 0 : 1; again < 2 && !t.ok; ++again) {
                 if (again == 1) {
-                    ++hard;
                     if (!F64 && lane == 0) atomicAdd(&A.st->precision_events, 1ull);
                     t.template trace<double>(G, m.t, gen0 != 0, f0, m.pd, m.far);
                 } else {
@@ -1776,7 +1777,7 @@ __global__ void __launch_bounds__(TAIL_BLOCK, 4) k_trace_tail(const __grid_const
                 t.solve(G, m.t, pi, grid, A.sorted, 2.0f, again == 0 ? T::UNIT_MIN : -1.0f, m.far);
                 t.certify64(G, m.t, m.pd, m.far, rechecks);
             }
-            if (!t.ok || t.faces.count() > REC_FACES || hard > HARD_TURNS) break;
+            if (!t.ok || t.faces.count() > REC_FACES) break;
             bool valid = all;
             if (turn == 0) {
                 valid = all || 4.0f * FAR_R2 * t.R2 <= reach;

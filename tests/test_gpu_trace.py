@@ -107,6 +107,57 @@ def check(pts, prec, route="warps", periodic=False, generic=True, **kw):
         match_cell(V, faces, Wv, wfaces, atol)
 
 
+@pytest.mark.parametrize("periodic", [False, True])
+@pytest.mark.parametrize("make", [lambda: W.uniform(2, 1), lambda: W.uniform(20, 2), lambda: W.uniform(33, 3),
+                                  lambda: W.uniform(34, 4), lambda: W.uniform(4001, 5),
+                                  lambda: W.mixed(4001, 6, n_clumps=3),
+                                  lambda: np.concatenate([W.uniform(50, 7), np.random.default_rng(8).normal(
+                                      0.5, 1e-2, (4000, 3)).astype(np.float32)])],
+                         ids=["2", "20", "33", "34", "uniform", "clumps", "sparse beside a clump"])
+def test_lists_hold_every_generator_below_their_reach(make, periodic):
+    # the lists as the call leaves them in its workspace: found by the nearest
+    # generators, which come first, and followed by the reaches
+    pts = make()
+    n, k = len(pts), 32
+    p = vt.Params(precision="fp32", emit=("vol",), periodic=periodic)
+    ws = vt.Workspace(p, n)
+    c = vt.tessellate(torch.from_numpy(pts).cuda(), p, workspace=ws, want_perm=True)
+    assert c.stats["knn_queries"] == n  # (the clipper's lists would lie in the same place)
+    x = pts[c.perm.cpu().numpy()[:n]].astype(np.float64)
+    off = x[None] - x[:, None]
+    if periodic:  # (the nearest image stands for the others: they are farther than half a period)
+        off -= np.rint(off)
+    d2 = (off ** 2).sum(-1)
+    np.fill_diagonal(d2, np.inf)
+    buf = ws.buf[:ws.buf.numel() // 4 * 4].view(torch.int32).cpu().numpy()
+    mask = (1 << 24) - 1 if periodic else -1
+    rows = np.arange(min(n, 16))
+    near = d2[rows].min(1)
+    at = np.arange(0, len(buf) - n * k, 64)
+    for r in rows:
+        first = buf[at + k * r] & mask
+        ok = (buf[at + k * r] >= 0) & (first < n)
+        at = at[ok][np.isclose(d2[r, first[ok]], near[r], rtol=1e-5, atol=0)]
+    assert len(at) == 1, at
+    lists = buf[at[0]:at[0] + n * k].reshape(n, k)
+    size = max(n * k, 64 * 32)
+    reach = buf[at[0] + (size + 63) // 64 * 64:][:n].view(np.float32).astype(np.float64)
+    for i in range(n):
+        ids = lists[i][lists[i] != -1]
+        if periodic:
+            code = ids >> 24
+            t = np.stack([code // 25 - 2, code // 5 % 5 - 2, code % 5 - 2], 1)
+            key = ((x[ids & mask] + t - x[i]) ** 2).sum(1)
+        else:
+            key = d2[i, ids]
+        assert len(set(ids.tolist())) == len(ids) and i not in (ids & mask)
+        assert key[0] <= key.min() * (1 + 1e-5) and (key < reach[i] * (1 + 1e-5)).all()
+        below = np.flatnonzero(d2[i] < min(reach[i], 0.25 if periodic else np.inf) * (1 - 1e-5))
+        assert set(below.tolist()) <= set((ids & mask).tolist()), i
+        if not periodic:
+            assert (reach[i] > 1e30) == (len(ids) == n - 1)
+
+
 @ROUTES
 @PRECS
 @pytest.mark.parametrize("n", [1, 2, 3, 5, 31, 32, 33, 34, 35, 63, 65, 127, 129, 515])
@@ -159,6 +210,20 @@ def test_lattices_that_moved_little(m, move, prec):
             assert np.array_equal(cells.nbr.cpu().numpy(), want["nbr"])
         elif m == 25:
             assert cells.stats["precision_retries"] < len(x) // 16
+
+
+@PRECS
+@pytest.mark.parametrize("seed", [25, 33, 37])
+def test_filaments_validate(seed, prec):
+    # points along segments: far cells whose thousands of cutting generators take
+    # tens of turns, more than the clipper's slots hold on the way
+    rng = np.random.default_rng(seed)
+    a, b = 0.1 + 0.8 * rng.random((20, 3)), 0.1 + 0.8 * rng.random((20, 3))
+    x = a[:, None] + (b - a)[:, None] * np.linspace(0, 1, 200)[None, :, None] + 3e-3 * rng.standard_normal((20, 200, 3))
+    x = np.unique(x.reshape(-1, 3).astype(np.float32), axis=0)
+    c = vt.tessellate(torch.from_numpy(x).cuda(), vt.Params(precision=prec, emit=("vol",), periodic=True))
+    assert c.stats["status"] == "VT_OK"
+    assert abs(float(c.vol.sum()) - 1.0) < TOL[prec]
 
 
 def test_rays_that_meet_two_planes_within_float_rounding():
