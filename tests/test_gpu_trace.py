@@ -121,6 +121,7 @@ def test_lists_hold_every_generator_below_their_reach(make, periodic):
     n, k = len(pts), 32
     p = vt.Params(precision="fp32", emit=("vol",), periodic=periodic)
     ws = vt.Workspace(p, n)
+    ws.buf.zero_()
     c = vt.tessellate(torch.from_numpy(pts).cuda(), p, workspace=ws, want_perm=True)
     assert c.stats["knn_queries"] == n  # (the clipper's lists would lie in the same place)
     x = pts[c.perm.cpu().numpy()[:n]].astype(np.float64)
@@ -138,6 +139,8 @@ def test_lists_hold_every_generator_below_their_reach(make, periodic):
         first = buf[at + k * r] & mask
         ok = (buf[at + k * r] >= 0) & (first < n)
         at = at[ok][np.isclose(d2[r, first[ok]], near[r], rtol=1e-5, atol=0)]
+        row = buf[at[:, None] + k * r + np.arange(k)]
+        at = at[((row == -1) | ((row >= 0) & ((row & mask) < n))).all(1) & (row[:, 1:] != 0).any(1)]
     assert len(at) == 1, at
     lists = buf[at[0]:at[0] + n * k].reshape(n, k)
     size = max(n * k, 64 * 32)
